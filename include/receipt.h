@@ -24,10 +24,11 @@
  *  - No C++ exception crosses this boundary. Every entry point returns a
  *    receipt_status; receipt_last_error() gives a thread-local message for the
  *    most recent failure on the calling thread.
- *  - No kernel waits on a flag or on another CTA, and every bounded
- *    structure either is sized from exact counts or has an exact fallback
- *    (an anchor whose repeat table overflows is redone through key slices),
- *    so the decomposition calls have no device-side error path.
+ *  - Every bounded structure either is sized from exact counts or has an
+ *    exact fallback (an anchor whose repeat table overflows is redone through
+ *    key slices). The only kernel whose CTAs wait for one another (the
+ *    coarse-grained step of small sides, a cooperative launch) bounds every
+ *    wait and reports RECEIPT_ERR_INTERNAL when one runs out.
  *    RECEIPT_ERR_TIMEOUT and RECEIPT_ERR_INTERNAL come from the serving
  *    engine (a wait that ran out of time; a request whose decomposition
  *    failed in a worker); RECEIPT_ERR_INTERNAL also reports a failed
@@ -113,7 +114,10 @@ typedef struct {
     int64_t fd_heavy_w;
     /* How the synchronisation rounds of Algorithm 3 are launched.
      * 0 (default): device-driven; the rounds of a range run inside one
-     * launch of a CUDA graph whose while-node repeats the round body until
+     * launch: of one cooperative kernel for the whole coarse-grained step
+     * when the side's keys fit at most four dense windows (147,456 vertices;
+     * in a batch, every graph's one window) and no degree on it reaches
+     * 65,535; otherwise of a CUDA graph whose while-node repeats the round body until
      * a round leaves no next activeSet (at most 64 rounds a launch), each
      * round's counters going to a device record that the host reads after
      * the launch; with timing on or the activeSet found by crossings the
@@ -189,7 +193,9 @@ typedef struct {
     /* Batched peel update of the coarse-grained step, per aggregation tier
      * (0 = warp table, 1 = shared-memory hybrid over the anchor's key window,
      * 2 = global dense counters for hubs, 3 = dense counters over key slices,
-     * 4 = dense counters over a key window of at most 36,864 keys):
+     * 4 = dense counters over a key window of at most 36,864 keys; the
+     * one-launch form of round_graphs counts every anchor of more than
+     * warp_max_w wedges here, with up to four windows):
      * wedges walked, middle vertices (edge visits), anchors (peeled vertices
      * with updates), kernel launches and device time (only if timing != 0). */
     uint64_t peel_wedges[5];
@@ -330,7 +336,8 @@ receipt_status receipt_count_butterflies_noalloc(receipt_graph *g, uint64_t *d_c
  * (Definition 1).
  *   d_tip : device uint64[n_side], by original id.
  *   opt   : NULL for defaults.
- * Synchronises `stream` once per range and once per peeling round.
+ * Synchronises `stream`: once for the coarse-grained step of a small side in
+ * one launch (see round_graphs), otherwise once or twice per range.
  */
 receipt_status receipt_tip_decompose(receipt_graph *g, receipt_side side, uint64_t *d_tip,
                                      const receipt_options *opt, void *stream);

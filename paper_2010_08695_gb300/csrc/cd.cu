@@ -26,40 +26,13 @@
 #include <cstddef>
 #include <vector>
 
+#include "cd.cuh"
 #include "engine.cuh"
 #include "internal.cuh"
 
 namespace receipt {
 
 namespace {
-
-constexpr int NBUCKET = LOG_BUCKETS;
-constexpr int NTIER = 5;  // warp, hybrid, global, sliced, dense window
-constexpr double DGM_FRAC = 0.125;  // stale share of live entries that triggers a compaction
-
-__device__ __forceinline__ int bucket_of(unsigned long long k) { return log_bucket_of(k); }
-__device__ __forceinline__ unsigned long long bucket_top(int b) { return log_bucket_top(b); }
-
-struct CdDev {
-    unsigned long long hi;
-    int32_t nF, nNext, nLw, nLc, nLg, nLo, nLs, nLb, nLd;
-    int32_t par;      // device-driven rounds: which of two buffers holds the activeSet
-    int32_t burst_k;  // device-driven rounds: rounds run by the current graph launch
-    int32_t pad2;
-    int32_t work[6];
-    unsigned long long work64;  // item counter of the sliced tier
-    unsigned long long peeled_edges;  // adjacency entries of assigned vertices (for DGM)
-    int32_t n_remaining;
-    int32_t range;  // 0-based index of the range being peeled
-    unsigned long long wrem_prev;
-    double tgt_prev;
-    unsigned long long wedges;
-    // per tier: wedges, mids, anchors, nonzero pairs (support atomics)
-    unsigned long long tier_w[NTIER], tier_m[NTIER], tier_a[NTIER], tier_p[NTIER];
-    unsigned long long front_w;  // sum of wfull over a full-scan activeSet (C_peel)
-    unsigned long long hist_w[NBUCKET];
-    uint32_t hist_c[NBUCKET];
-};
 
 // wfull[x] = sum over y in N_x of d_y (wedges walked when x is peeled)
 __global__ void k_deg_of_nbr(const int32_t *__restrict__ adj, int64_t m,
@@ -100,7 +73,7 @@ __global__ void k_cd_hist(int32_t n, const int32_t *__restrict__ sub,
         if (sub[x] < 0) {
             unsigned long long v = sup[x];
             init[x] = v;
-            int b = bucket_of(v);
+            int b = log_bucket_of(v);
             atomicAdd(&hc[b], 1u);
             unsigned long long w = wfull[x] - (unsigned long long)(off[x + 1] - off[x]);
             if (w) atomicAdd(&hw[b], w);
@@ -122,7 +95,7 @@ __global__ void k_cd_hist(int32_t n, const int32_t *__restrict__ sub,
 // as distinct supports, all peeled one after another by one fine-grained
 // task.
 __global__ void __launch_bounds__(1024) k_cd_select(CdDev *st, int range, int P, int32_t cap) {
-    __shared__ unsigned long long tmpw[33];
+    __shared__ unsigned long long tmpw[33], s_goal;
     __shared__ uint32_t tmpc[33];
     __shared__ int s_pick, s_first, s_last;
     constexpr int PER = (NBUCKET + 1023) / 1024;
@@ -146,15 +119,21 @@ __global__ void __launch_bounds__(1024) k_cd_select(CdDev *st, int range, int P,
     uint32_t ctot;
     unsigned long long wpre = block_exclusive_scan<unsigned long long>(wsum, tmpw, &wtot);
     uint32_t cpre = block_exclusive_scan<uint32_t>(csum, tmpc, &ctot);
-    // adaptive target: tgt_i = s_{i-1} * W_rem / (P - i + 1)
-    double s_prev = 1.0;
-    if (range > 0) {
-        unsigned long long covered = st->wrem_prev - wtot;
-        if (covered > 0) s_prev = fmin(1.0, st->tgt_prev / (double)covered);
+    // adaptive target: tgt_i = s_{i-1} * W_rem / (P - i + 1), by one thread
+    // (64-bit floating point is slow on this chip)
+    if (threadIdx.x == 0) {
+        double s_prev = 1.0;
+        if (range > 0) {
+            const unsigned long long covered = st->wrem_prev - wtot;
+            if (covered > 0) s_prev = fmin(1.0, st->tgt_prev / (double)covered);
+        }
+        const double tgt = s_prev * (double)wtot / (double)max(1, P - range);
+        st->wrem_prev = wtot;
+        st->tgt_prev = tgt;
+        s_goal = target_weight(tgt);
     }
-    int left = P - range;
-    if (left < 1) left = 1;
-    double tgt = s_prev * (double)wtot / (double)left;
+    __syncthreads();
+    const unsigned long long goal = s_goal;
     unsigned long long run = wpre;
     uint32_t crun = cpre;
     for (int j = 0; j < PER; j++) {
@@ -164,7 +143,7 @@ __global__ void __launch_bounds__(1024) k_cd_select(CdDev *st, int range, int P,
         if (c[j]) {
             atomicMin(&s_first, b);
             atomicMax(&s_last, b);
-            if ((double)run >= tgt || (cap > 0 && crun >= (uint32_t)cap)) atomicMin(&s_pick, b);
+            if (run >= goal || (cap > 0 && crun >= (uint32_t)cap)) atomicMin(&s_pick, b);
         }
     }
     __syncthreads();
@@ -172,13 +151,11 @@ __global__ void __launch_bounds__(1024) k_cd_select(CdDev *st, int range, int P,
         st->n_remaining = (int32_t)ctot;
         if (ctot > 0) {
             int b = s_pick;
-            if (tgt <= 0.0) b = s_first;
+            if (goal == 0) b = s_first;
             if (b >= NBUCKET) b = s_last;
-            unsigned long long top = bucket_top(b);
+            unsigned long long top = log_bucket_top(b);
             st->hi = top == ~0ull ? ~0ull : top + 1ull;
         }
-        st->wrem_prev = wtot;
-        st->tgt_prev = tgt;
     }
 }
 
@@ -961,6 +938,22 @@ __global__ void k_list_lengths(const int64_t *__restrict__ off, int32_t n, int32
     if (y < n) len[y] = (int32_t)(off[y + 1] - off[y]);
 }
 
+// Packed graph of every vertex (first[i]: the first vertex of graph i).
+__global__ void k_part_of(const int32_t *__restrict__ first, int ng, int32_t n,
+                          int32_t *__restrict__ part) {
+    const int32_t x = blockIdx.x * blockDim.x + threadIdx.x;
+    if (x >= n) return;
+    int lo = 0, hi = ng - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (first[mid] <= x)
+            lo = mid;
+        else
+            hi = mid - 1;
+    }
+    part[x] = lo;
+}
+
 // kwin[y] = (first, last) key of the working list y ((INT32_MAX, -1) when
 // empty): the window the route of an anchor takes over its middle vertices.
 __global__ void k_list_window(const int64_t *__restrict__ off, const int32_t *__restrict__ len,
@@ -1096,6 +1089,12 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s) {
                               : slice_ctas == 2 ? Slice2::smem() : Slice1::smem();
     const int32_t SW = slice_ctas == 4 ? Slice4::keys : slice_ctas == 2 ? Slice2::keys : Slice1::keys;
     const bool scan_next = opt.scan_frontier >= 0;
+    // One cooperative launch for the whole step (cd_persist.cu): the default
+    // for sides that need only the warp and the dense-window tier. Forced
+    // recounts, injected bounds, per-tier timing and the other launch modes
+    // take the per-round kernels below.
+    const bool persist = opt.round_graphs == 0 && scan_next && !D.timing && opt.n_bounds <= 0 &&
+                         opt.huc <= 0 && cd_persist_fits(D);
     const int32_t slice_fetch = opt.slice_fetch > 0 ? std::min(opt.slice_fetch, SLICE_FETCH_MAX) : 1;
     // vertices per range: at most range_max_n (0: 2 n / P, -1: no bound)
     const int32_t range_cap =
@@ -1104,7 +1103,7 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s) {
                                                    : (int32_t)std::max<int64_t>(1, 2 * (int64_t)n / P));
     const int32_t C = std::max(1, ceil_div(n, SW));
     // slice table (C + 1 starts per list) only while slices are few
-    const bool table = C <= 64;
+    const bool table = C <= 64 && !persist;
     DevBuf<int32_t> soff(table ? (size_t)O.n * (C + 1) : 1, s);
     // working copy of the other side's lists, compacted between ranges
     DevBuf<int32_t> adj_w(D.m, s), len_w(O.n, s);
@@ -1125,9 +1124,11 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s) {
     if (O.n > 0) {
         k_list_lengths<<<ceil_div(O.n, 256), 256, 0, s>>>(O.off, O.n, len_w.get());
         RC_LAUNCH();
-        k_list_window<<<ceil_div(O.n, 256), 256, 0, s>>>(O.off, len_w.get(), adj_w.get(), O.n,
-                                                        kwin.get());
-        RC_LAUNCH();
+        if (!persist) {
+            k_list_window<<<ceil_div(O.n, 256), 256, 0, s>>>(O.off, len_w.get(), adj_w.get(), O.n,
+                                                            kwin.get());
+            RC_LAUNCH();
+        }
         if (table) {
             k_slice_table<<<ceil_div((int64_t)O.n * (C + 1), 256), 256, 0, s>>>(
                 O.off, len_w.get(), adj_w.get(), O.n, C, SW, soff.get());
@@ -1162,10 +1163,12 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s) {
     const size_t smem_glob = chunk_extra;
     allow_max_smem((const void *)k_cd_update_global);
     const size_t hdr = offsetof(CdDev, hist_w);
-    // pinned: C_rcnt, the state's header, the device-driven rounds' records
-    constexpr int ROUND_BURST = 64;
-    unsigned long long *hpin =
-        (unsigned long long *)pinned_scratch(64 + sizeof(CdDev) + ROUND_BURST * hdr);
+    // pinned: C_rcnt, the state's header, the device-driven rounds' records,
+    // the one-launch form's state and first records
+    constexpr int ROUND_BURST = 64, PERSIST_FIRST = 512;
+    unsigned long long *hpin = (unsigned long long *)pinned_scratch(
+        64 + sizeof(CdDev) + 8 + ROUND_BURST * hdr + sizeof(PersistDev) +
+        PERSIST_FIRST * sizeof(PersistRound));
     CdDev *hst = reinterpret_cast<CdDev *>(hpin + 8);
     unsigned long long *hrec = hpin + 8 + (sizeof(CdDev) + 7) / 8;
     unsigned long long prev_w[NTIER] = {}, prev_a[NTIER] = {};
@@ -1217,7 +1220,7 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s) {
     // body until a round leaves no next activeSet or ROUND_BURST rounds ran;
     // the rounds' headers go to device records that the host reads after the
     // launch, so a range's rounds need no host round trip between them.
-    const bool dloop = opt.round_graphs == 0 && scan_next && !D.timing;
+    const bool dloop = opt.round_graphs == 0 && scan_next && !D.timing && !persist;
     const int32_t hdr_words = (int32_t)(offsetof(CdDev, hist_w) / 8);
     DevBuf<unsigned long long> rec(dloop ? (size_t)ROUND_BURST * hdr_words : 1, s);
     cudaGraphConditionalHandle loop_cond = 0;
@@ -1433,7 +1436,124 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s) {
     int parity = 0;
     int32_t *cur = abuf[0];
     uint64_t crcnt = 0;  // C_rcnt (rule on) or 0
-    for (range = 0; range < nranges; range++) {
+    if (persist) {
+        const int ng = D.parts ? (int)D.parts->size() - 1 : 1;
+        DevBuf<PersistDev> pd(1, s);
+        DevBuf<unsigned long long> ph_w(3 * NBUCKET, s);
+        DevBuf<uint32_t> ph_c(3 * NBUCKET, s);
+        DevBuf<int32_t> pfirst(ng + 1, s), plast(3 * (size_t)ng, s);
+        DevBuf<int32_t> part_of(D.parts ? n : 1, s);
+        DevBuf<PersistAnchor> pLw(n, s);
+        // items: an anchor's whole window, or its windows of DENSE_KEYS keys
+        DevBuf<PersistAnchor> pLd((size_t)n * (D.parts ? 1 : ceil_div(n, DENSE_KEYS)), s);
+        constexpr int REC_CAP = 4096;  // rounds per launch
+        DevBuf<PersistRound> prec(REC_CAP, s);
+        std::vector<int32_t> hfirst(ng + 1, 0);
+        if (D.parts)
+            for (int i = 0; i <= ng; i++) hfirst[i] = (int32_t)(*D.parts)[i];
+        else
+            hfirst[1] = n;
+        pd.zero();
+        ph_w.zero();
+        ph_c.zero();
+        RC_CUDA(cudaMemsetAsync(plast.get(), 0xff, sizeof(int32_t) * 3 * (size_t)ng, s));
+        RC_CUDA(cudaMemcpyAsync(pfirst.get(), hfirst.data(), sizeof(int32_t) * (ng + 1),
+                                cudaMemcpyHostToDevice, s));
+        if (D.parts) {
+            k_part_of<<<ceil_div(n, 256), 256, 0, s>>>(pfirst.get(), ng, n, part_of.get());
+            RC_LAUNCH();
+        }
+        const PersistArgs pa{n, O.n, D.m, S.off, S.adj, O.off, len_w.get(), adj_w.get(), D.sup,
+                             D.init, D.wfull, D.sub, st.get(), pd.get(), ph_w.get(), ph_c.get(),
+                             D.parts ? part_of.get() : nullptr, pfirst.get(), plast.get(), ng,
+                             F.get(), pLw.get(), pLd.get(), prec.get(), REC_CAP, P, range_cap,
+                             warp_max_w, dgm && O.n > 0 ? 1 : 0, dgm_frac, huc == 0 ? 1 : 0,
+                             huc_factor, rcost.get()};
+        const int pgrid = cd_persist_grid(D.m);
+        PersistDev *hpd = (PersistDev *)(hrec + ROUND_BURST * (hdr / 8));
+        PersistRound *hrc = (PersistRound *)(hpd + 1);
+        std::vector<PersistRound> recs;
+        RC_CUDA(cudaMemcpyAsync(hpin, rcost.get(), 8, cudaMemcpyDeviceToHost, s));
+        for (;;) {
+            cd_persist_launch(pa, pgrid, s);
+            RC_CUDA(cudaMemcpyAsync(hpd, pd.get(), sizeof(PersistDev), cudaMemcpyDeviceToHost, s));
+            RC_CUDA(cudaMemcpyAsync(hrc, prec.get(), PERSIST_FIRST * sizeof(PersistRound),
+                                    cudaMemcpyDeviceToHost, s));
+            RC_CUDA(cudaStreamSynchronize(s));
+            if (hpd->err) fail(RECEIPT_ERR_INTERNAL, "coarse-grained step: a grid barrier ran out of time");
+            D.cost_recount = hpin[0];
+            const PersistDev h = *hpd;
+            recs.assign(hrc, hrc + std::min(h.nrec, PERSIST_FIRST));
+            if (h.nrec > PERSIST_FIRST) {
+                recs.resize(h.nrec);
+                RC_CUDA(cudaMemcpyAsync(recs.data() + PERSIST_FIRST, prec.get() + PERSIST_FIRST,
+                                        (h.nrec - PERSIST_FIRST) * sizeof(PersistRound),
+                                        cudaMemcpyDeviceToHost, s));
+                RC_CUDA(cudaStreamSynchronize(s));
+            }
+            for (const PersistRound &r : recs) {
+                receipt_round rr{};
+                rr.range = r.range;
+                rr.frontier = r.frontier;
+                rr.hi = r.hi;
+                for (int k = 0; k < 2; k++) {
+                    const int t = k ? 4 : 0;
+                    rr.anchors[t] = r.anchors[k] - prev_a[t];
+                    rr.wedges[t] = r.wedges[k] - prev_w[t];
+                    prev_a[t] = r.anchors[k];
+                    prev_w[t] = r.wedges[k];
+                }
+                if ((size_t)r.range + 1 == D.bounds.size()) D.bounds.push_back(r.hi);
+                D.trace.push_back(rr);
+                D.rounds++;
+                D.tier_launches[0]++;
+                D.tier_launches[4]++;
+            }
+            range = h.range;
+            if (h.stop == PERSIST_DONE) {
+                D.dgm_passes += h.dgm_passes;
+                break;
+            }
+            PersistDev next = h;
+            next.nrec = 0;
+            if (h.stop == PERSIST_RECOUNT) {
+                if ((size_t)h.range + 1 == D.bounds.size()) D.bounds.push_back(h.hi);
+                next.mode = PERSIST_PEEL;
+                if (recount_fits(D)) {
+                    // the recount round takes the activeSet that the launch
+                    // listed (and assigned); the next one is scanned afresh
+                    // (k_cd_prepare of that round counts its wedges and entries)
+                    const PersistDev::Set &fs = h.set[h.sk % 3];
+                    const int32_t hf[2] = {fs.nF, h.range};
+                    RC_CUDA(cudaMemcpyAsync(hst, st.get(), hdr, cudaMemcpyDeviceToHost, s));
+                    RC_CUDA(cudaStreamSynchronize(s));
+                    const unsigned long long w0 = hst->wedges - fs.upd_w,
+                                             e0 = hst->peeled_edges - fs.front_e;
+                    RC_CUDA(cudaMemcpyAsync(&st.get()->wedges, &w0, 8, cudaMemcpyHostToDevice, s));
+                    RC_CUDA(cudaMemcpyAsync(&st.get()->peeled_edges, &e0, 8, cudaMemcpyHostToDevice, s));
+                    RC_CUDA(cudaMemcpyAsync(&st.get()->nF, &hf[0], 4, cudaMemcpyHostToDevice, s));
+                    RC_CUDA(cudaMemcpyAsync(&st.get()->range, &hf[1], 4, cudaMemcpyHostToDevice, s));
+                    RC_CUDA(cudaMemcpyAsync(&st.get()->hi, &h.hi, 8, cudaMemcpyHostToDevice, s));
+                    huc_round(F.get(), Nx.get());
+                    RC_CUDA(cudaStreamSynchronize(s));
+                    receipt_round rr{};
+                    rr.range = h.range;
+                    rr.frontier = hf[0];
+                    rr.hi = h.hi;
+                    rr.recount = 1;
+                    D.trace.push_back(rr);
+                    D.rounds++;
+                    if (dgm) next.peeled_at_dgm = hst->peeled_edges;  // the lists were just compacted
+                    next.mode = PERSIST_SCAN;
+                    for (PersistDev::Set &ps : next.set) ps = PersistDev::Set{};
+                    next.peeled = hst->peeled_edges;
+                }
+            }
+            RC_CUDA(cudaMemcpyAsync(pd.get(), &next, sizeof(next), cudaMemcpyHostToDevice, s));
+            RC_CUDA(cudaStreamSynchronize(s));
+        }
+    }
+    for (; !persist && range < nranges; range++) {
         k_cd_new_range<<<1, 256, 0, s>>>(st.get(), range);
         RC_LAUNCH();
         k_cd_hist<<<nb, 512, 0, s>>>(n, D.sub, D.sup, D.wfull, S.off, D.init, st.get());

@@ -62,6 +62,25 @@ __device__ __forceinline__ unsigned long long log_bucket_top(int b) {
     return ((unsigned long long)(33 + mant) << (e - 5)) - 1ull;
 }
 
+// Smallest weight r with (double)r >= tgt: the comparisons with a range's
+// target are then integer ones.
+__device__ __forceinline__ unsigned long long target_weight(double tgt) {
+    if (!(tgt > 0.0)) return 0;
+    if (tgt >= 18446744073709551615.0) return ~0ull;
+    unsigned long long r = (unsigned long long)ceil(tgt);
+    while (r > 0 && (double)(r - 1) >= tgt) r--;  // beyond 2^53 (double) rounds up
+    return r;
+}
+
+// How a walk loads its keys: through the read-only path, or from L2 when
+// other CTAs may have rewritten the lists since this kernel began.
+struct KeysNc {
+    static __device__ __forceinline__ int32_t load(const int32_t *p) { return __ldg(p); }
+};
+struct KeysL2 {
+    static __device__ __forceinline__ int32_t load(const int32_t *p) { return __ldcg(p); }
+};
+
 // Visits of one walk step (key < 0: no wedge). A visitor with a many<N>()
 // member gets the whole step with all 32 lanes (for warp-level aggregation);
 // others get one call per key.
@@ -107,7 +126,7 @@ __device__ __forceinline__ void emit_many(E &e, const int32_t (&k)[N], const uin
 // lengths numbers their wedges, and each lane takes wedges lane, lane + 32,
 // ..., finding its segment by a binary search over the lanes' starts, so all
 // key loads of a step are independent (U per lane in flight). visit(key).
-template <int U, class Mids, class Visit>
+template <int U, class Keys = KeysNc, class Mids, class Visit>
 __device__ __forceinline__ void warp_walk(const Mids &M, int64_t q0, int64_t q1,
                                           const int32_t *__restrict__ keys, Visit &visit) {
     const int lane = threadIdx.x & 31;
@@ -138,7 +157,7 @@ __device__ __forceinline__ void warp_walk(const Mids &M, int64_t q0, int64_t q1,
                 }
                 const int64_t b = __shfl_sync(0xffffffffu, beg, lo);
                 const int32_t e0 = __shfl_sync(0xffffffffu, ex, lo);
-                key[u] = j < total ? __ldg(keys + b + (j - e0)) : -1;
+                key[u] = j < total ? Keys::load(keys + b + (j - e0)) : -1;
             }
 #pragma unroll
             for (int u = 0; u < U; u++)
@@ -806,7 +825,8 @@ struct NoChunkHook {
 //   __device__ void seg(int64_t q, int64_t &beg, int32_t &len) const;
 // visit(k, key): k = mid index within the chunk, key = end point.
 // Returns the number of wedges walked. All threads of the CTA must call it.
-template <bool BALANCED = true, class Mids, class Visit, class Hook = NoChunkHook>
+template <bool BALANCED = true, class Keys = KeysNc, class Mids, class Visit,
+          class Hook = NoChunkHook>
 __device__ int64_t cta_walk(const Mids &M, int64_t q0, int64_t q1, const int32_t *__restrict__ keys,
                             Chunk &ch, Visit &visit, Hook *hook = nullptr) {
     // one scan of (segment length | non-empty flag << 40) gives both the
@@ -897,7 +917,7 @@ __device__ int64_t cta_walk(const Mids &M, int64_t q0, int64_t q1, const int32_t
                         // the whole group lies in segment k0 (long lists: the
                         // common case), no shared-memory lookups
                         kk[u] = kl0;
-                        key[u] = __ldg(keys + bg0 + (j - p0));
+                        key[u] = Keys::load(keys + bg0 + (j - p0));
                     } else {
                         while (ch.pre[k0 + 1] <= base) k0++;
                         const int kn = k0 + 1 + lane;
@@ -907,7 +927,7 @@ __device__ int64_t cta_walk(const Mids &M, int64_t q0, int64_t q1, const int32_t
                         const int k = k0 + __popc(m & lanes_le);
                         if (j < total) {
                             kk[u] = ch.len[k];
-                            key[u] = __ldg(keys + ch.beg[k] + (j - ch.pre[k]));
+                            key[u] = Keys::load(keys + ch.beg[k] + (j - ch.pre[k]));
                         }
                         // continue from the segment of the group's last wedge
                         k0 = min(k0 + __popc(m), nnz - 1);

@@ -1,0 +1,60 @@
+"""The coarse-grained step in one cooperative launch (sides whose keys fit a few
+dense windows): the same tip numbers as the oracle and the same rounds as the
+per-round kernels, at the edges of its windows and of its records."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def R():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2010_08695_gb300 as R
+    R.load()
+    return R
+
+
+def _rounds(g):
+    return [(r["range"], r["frontier"], r["hi"]) for r in g.trace()]
+
+
+# one dense window has 36,864 keys, at most four windows; the last side takes
+# the per-round kernels
+@pytest.mark.parametrize("n", [1, 33, 2049, 36864, 36865, 73729, 147456, 147457])
+def test_window_edges(R, n):
+    nv = max(2, n // 40)
+    m = min(3 * n, n * nv // 2)
+    eu, ev = synth.er(n, nv, m, seed=n) if n < 100 else \
+        synth.chung_lu(n, nv, m, 2.4, 2.3, seed=n)
+    want, _ = oracle.bup(eu, ev, n, nv, 0)
+    g = R.Graph(eu, ev, n, nv)
+    for kw in ({}, {"P": 3}, {"dgm": False}, {"dgm_frac_1024": 8}, {"warp_max_w": 16}):
+        t = R.as_u64(g.tip_decompose(0, **kw))
+        assert np.array_equal(t, want), kw
+        recs = _rounds(g)
+        t = R.as_u64(g.tip_decompose(0, round_graphs=-1, **kw))
+        assert np.array_equal(t, want), kw
+        assert recs == _rounds(g), kw
+
+
+def test_more_rounds_than_one_launch_records(R):
+    # a ladder: u_i shares one butterfly with each neighbour, so below the
+    # bound 2 the peel cascades in from both ends, two vertices a round
+    k = 9000
+    i = np.arange(k, dtype=np.int32)
+    eu = np.repeat(i, 4)
+    ev = np.stack([i, i + 1, k + 1 + i, k + 2 + i], axis=1).reshape(-1).astype(np.int32)
+    want, _ = oracle.bup(eu, ev, k, 2 * (k + 1), 0)
+    g = R.Graph(eu, ev, k, 2 * (k + 1))
+    t = R.as_u64(g.tip_decompose(0, P=20000))
+    assert np.array_equal(t, want)
+    assert g.stats()["rounds_cd"] > 4096
+    recs = _rounds(g)
+    t = R.as_u64(g.tip_decompose(0, P=20000, round_graphs=-1))
+    assert np.array_equal(t, want) and recs == _rounds(g)
