@@ -195,7 +195,10 @@ typedef struct {
      * 2 = global dense counters for hubs, 3 = dense counters over key slices,
      * 4 = dense counters over a key window of at most 36,864 keys; the
      * one-launch form of round_graphs counts every anchor of more than
-     * warp_max_w wedges here, with up to four windows):
+     * warp_max_w wedges here, with up to four windows). A round whose walks
+     * are long may go through the 256 middle vertices of highest degree
+     * instead (one small matrix per round, no wedge through them walked): all
+     * its anchors count under 1, with the wedges walked past those vertices:
      * wedges walked, middle vertices (edge visits), anchors (peeled vertices
      * with updates), kernel launches and device time (only if timing != 0). */
     uint64_t peel_wedges[5];

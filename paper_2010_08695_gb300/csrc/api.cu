@@ -263,6 +263,7 @@ void tip_decompose_impl(receipt_graph *g, int side, uint64_t *d_tip, const recei
     int64_t cpoints[5] = {0, 0, 0, 0, 0};
     uint64_t wc = count_local(g, cu.get(), cv.get(), s, cpoints);
     T.mark();
+    D.wedges_bup = h_wbup;  // read before count_local synchronised the stream
     D.sup = side ? cv.get() : cu.get();
     D.init = init.get();
     D.sub = sub.get();

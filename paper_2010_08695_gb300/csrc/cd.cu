@@ -1366,6 +1366,27 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s) {
         D.huc_recounts++;
         if (dgm) D.dgm_passes++;
     };
+    // A round whose updates go through the hubs (cd_hub.cu): one list of
+    // anchors whatever their walks, the next activeSet by a full scan.
+    HubPath hub;
+    bool hub_ready = false;
+    const bool hub_ok = !persist && !D.parts && HubPath::suits(D, s);
+    auto hub_round = [&](int32_t *cur, int32_t *nxt, int32_t nF) {
+        if (!hub_ready) hub.init(D, s);
+        hub_ready = true;
+        k_cd_prepare<<<nb, 512, 0, s>>>(cur, st.get(), D.sub, D.sup, D.wfull, S.off, Lw.get(),
+                                        Lb.get(), 0);
+        RC_LAUNCH();
+        if (D.timing) RC_CUDA(cudaEventRecord(ev[0], s));
+        hub.round(D, st.get(), Lb.get(), nF, s);
+        if (D.timing) RC_CUDA(cudaEventRecord(ev[1], s));
+        k_cd_frontier<<<nb, 512, 0, s>>>(n, D.sub, D.sup, D.wfull, st.get(), &st.get()->nNext,
+                                         nxt);
+        RC_LAUNCH();
+        RC_CUDA(cudaMemcpyAsync(hst, st.get(), hdr, cudaMemcpyDeviceToHost, s));
+        k_cd_advance<<<1, 1, 0, s>>>(st.get());
+        RC_LAUNCH();
+    };
     // With round_graphs the body is captured once per activeSet parity (on a
     // private stream: the caller's may be the legacy default stream, which
     // cannot capture) and each round is one graph launch.
@@ -1580,8 +1601,22 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s) {
         bool recount = huc == 1 || (huc == 0 && crcnt > 0 &&
                                     (double)hst->front_w > huc_factor * (double)crcnt &&
                                     recount_fits(D));
+        // A round whose walks are long enough goes through the hubs. Such a
+        // round costs ~0.1 ms of launches and short kernels and ~0.1 ns per
+        // remaining vertex, the per-anchor tiers ~4.5 ps per wedge: the line
+        // lies near 10^7 + 16 n_remaining wedges (flat: the 10M-edge graph
+        // takes 120.4 ms at 1.5 10^7 + 12 n, 123.8 at 3 10^6 + 12 n, 120.7 at
+        // 3 10^7 + 12 n; the 40M-edge one 621 / 609 / 625).
+        const double hmin = 1e7 + 16.0 * (double)hst->n_remaining;
+        auto hub_due = [&](int32_t nF, uint64_t front_w, uint64_t peeled) {
+            return hub_ok && nF > 0 && nF <= HubPath::MAX_ANCHORS &&
+                   (double)front_w * (double)(D.m - peeled) >= hmin * (double)D.m;
+        };
+        bool by_hubs = !recount && hub_due(hst->nF, hst->front_w, hst->peeled_edges);
+        uint64_t front_seen = hst->front_w;
+        int32_t nF_now = hst->nF;
         // one trace record per round from a copy of the state's header
-        auto record_round = [&](const CdDev *h, bool rc) {
+        auto record_round = [&](const CdDev *h, bool rc, bool hubs_used) {
             if (!rc)
                 for (int t = 0; t < NTIER; t++) D.tier_launches[t]++;
             D.rounds++;
@@ -1603,6 +1638,9 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s) {
                     RC_CUDA(cudaEventElapsedTime(&ms, ev[NTIER + 1], ev[NTIER + 2]));
                     D.ms_recount += ms;
                 }
+            } else if (D.timing && hubs_used) {
+                RC_CUDA(cudaEventElapsedTime(&rr.ms[1], ev[0], ev[1]));
+                D.tier_ms[1] += rr.ms[1];
             } else if (D.timing) {
                 // launch order: warp, dense window, hybrid, global, sliced
                 static const int tier_of_gap[NTIER] = {0, 4, 1, 2, 3};
@@ -1616,7 +1654,7 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s) {
             D.trace.push_back(rr);
         };
         for (;;) {
-            if (!recount && dloop) {
+            if (!recount && !by_hubs && dloop) {
                 // a burst of up to ROUND_BURST rounds in one graph launch
                 k_cd_burst_begin<<<1, 1, 0, s>>>(st.get(), parity);
                 RC_LAUNCH();
@@ -1631,13 +1669,15 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s) {
                 count_launches((uint64_t)kk * round_kernels);
                 for (int32_t r = 0; r < kk; r++)
                     record_round(reinterpret_cast<const CdDev *>(hrec + (size_t)r * hdr_words),
-                                 false);
+                                 false, false);
                 parity = hst->par;
                 if (hst->nF == 0) break;  // the last round left no next activeSet
                 continue;
             }
             if (recount) {
                 huc_round(abuf[parity], abuf[parity ^ 1]);
+            } else if (by_hubs) {
+                hub_round(abuf[parity], abuf[parity ^ 1], nF_now);
             } else if (graphs) {
                 RC_CUDA(cudaGraphLaunch(round_exec[parity], s));
                 count_launches(round_kernels);
@@ -1645,10 +1685,13 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s) {
                 round_body(s, abuf[parity], abuf[parity ^ 1], false, false);
             }
             RC_CUDA(cudaStreamSynchronize(s));
-            record_round(hst, recount);
+            record_round(hst, recount, by_hubs);
             if (hst->nNext == 0) break;
             parity ^= 1;  // the next round reads the activeSet this one wrote
             recount = false;
+            nF_now = hst->nNext;
+            by_hubs = scan_next && hub_due(nF_now, hst->front_w - front_seen, hst->peeled_edges);
+            front_seen = hst->front_w;
         }
         D.bounds.push_back(hi);
         // dynamic graph maintenance: once the vertices assigned since the last

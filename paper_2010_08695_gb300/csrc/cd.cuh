@@ -111,4 +111,66 @@ int cd_persist_grid(int64_t m);
 // Enqueues one launch (state in a.pd).
 void cd_persist_launch(const PersistArgs &a, int grid, cudaStream_t s);
 
+// ---------------------------------------------------------------------
+// Updates of a large activeSet through the other side's hubs (cd_hub.cu)
+// ---------------------------------------------------------------------
+struct HubDev {
+    int32_t nA, nE;          // anchors, their edges past the hubs
+    int32_t nQs, nQ;         // rows of the quadratic form: sparse, the others
+    int32_t nR, nMid, nBig;  // pulling vertices; those of warp and of CTA size
+    int32_t nTouch, cursor, work, work_mid;
+    uint32_t flags[16];      // tiles of the second digit that are not zero
+};
+
+struct HubArgs {
+    int32_t n;
+    const int64_t *off_s;
+    const int32_t *adj_s;
+    unsigned long long *sup;
+    const int32_t *sub;
+    CdDev *st;
+    const int32_t *A;        // anchors (st->nLb of them)
+    const uint32_t *mask;    // hub masks of side s, 8 words each
+    const int32_t *plen;     // hubs among every vertex's neighbours
+    const uint32_t *heavy;   // masks of the other side over the heavy vertices
+    int2 *cb;                // per other-side vertex: adjacent anchors, start of their list
+    int32_t *touch;          // other-side vertices with an adjacent anchor
+    int32_t *Qs, *Q, *R, *mid, *big;
+    int32_t *aoff;           // per anchor: first of its edges past the hubs
+    uint32_t *amask, *cols;  // anchors' hub masks and their transpose
+    int32_t colw;
+    uint32_t *gram;          // G as B fragments, two digits
+    uint32_t *gtri;          // G's strictly lower triangle, row by row
+    int32_t *ey;             // per edge past the hubs: its middle vertex,
+    int2 *ek;                // its anchor and its place in the middle vertex's list
+    int32_t *alist;
+    HubDev *hd;
+};
+
+class HubPath {
+  public:
+    static constexpr int HUBS = 256;
+    static constexpr int32_t MAX_ANCHORS = DENSE_KEYS;  // one dense window
+    // Whether a decomposition can and should use it: half of the wedges pass
+    // through hubs, and a vertex that is not heavy has a degree below 65,535
+    // (16-bit counters). Synchronises s.
+    static bool suits(const Decomp &D, cudaStream_t s);
+    HubPath() = default;
+    ~HubPath();
+    HubPath(const HubPath &) = delete;
+    HubPath &operator=(const HubPath &) = delete;
+    // Masks and work space of one decomposition.
+    void init(const Decomp &D, cudaStream_t s);
+    // Enqueues the updates of the anchors A (st->nLb of them, at most nF,
+    // assigned to their subset already) to every remaining vertex's support.
+    void round(const Decomp &D, CdDev *st, const int32_t *A, int32_t nF, cudaStream_t s);
+
+  private:
+    DevBuf<uint32_t> mask_, heavy_, amask_, cols_, gram_, gtri_;
+    DevBuf<int32_t> plen_, touch_, Qs_, Q_, R_, mid_, big_, aoff_, ey_, alist_;
+    DevBuf<int2> cb_, ek_;
+    DevBuf<HubDev> hd_;
+    cudaEvent_t ev_[5] = {};
+};
+
 }  // namespace receipt

@@ -794,7 +794,15 @@ constexpr size_t persist_smem() { return DenseSlice::bytes() + chunk_bytes(PT); 
 
 bool cd_persist_fits(const Decomp &D) {
     if (D.max_deg_s >= 65535) return false;  // counts may need 32 bits
-    if (!D.parts) return D.n <= PERSIST_SLICES * DENSE_KEYS;
+    if (!D.parts) {
+        // several windows walk a long list once per window: only while the
+        // rounds are short (120,000 x 40,000 with 3M edges, 1.9 10^9 wedges,
+        // 4 windows: 35.3 ms here, 30.8 by the per-round kernels; 40,000 x
+        // 400,000 with 3M edges, 9 10^8, 2 windows: 21.5 against 29.3)
+        const int64_t windows = ceil_div(D.n, DENSE_KEYS);
+        return windows == 1 ||
+               (windows <= PERSIST_SLICES && (double)windows * (double)D.wedges_bup <= 3e9);
+    }
     for (size_t i = 0; i + 1 < D.parts->size(); i++)
         if ((*D.parts)[i + 1] - (*D.parts)[i] > DENSE_KEYS) return false;
     return true;

@@ -59,6 +59,7 @@ struct Decomp {
     unsigned long long *wfull = nullptr;  // sum of d_y over y in N_x
     int32_t p_eff = 0;
     std::vector<uint64_t> bounds;         // theta(1..p_eff+1)
+    uint64_t wedges_bup = 0;              // sum of d (d - 1) over the other side
     uint64_t wedges_cd = 0, wedges_fd = 0;
     int64_t rounds = 0, levels = 0;
     int32_t dgm_passes = 0;
