@@ -235,10 +235,13 @@ typedef struct {
      * remaining vertex x' that share at least two neighbours (the pairs whose
      * support changes). */
     uint64_t peel_pairs[5];
-    /* Start points of Algorithm 1 per aggregation tier, both sides: warp
-     * table, shared hash table (at most 2,048 wedges), shared-memory hybrid,
-     * global counters (degree >= 65535 or a key space beyond shared memory),
-     * global counters after the hybrid's repeat table overflowed. */
+    /* Start points of Algorithm 1 whose end points past the first 1,024 (which
+     * are counted bit-sliced) take an aggregation tier, both sides: warp
+     * table, small CTAs (at most 4,096 wedges; shared hash table or counters
+     * for the first keys and a table for the rest), larger CTAs (the same, or
+     * the shared-memory hybrid), global counters (degree >= 65535 or a key
+     * space beyond shared memory), global counters after the hybrid's repeat
+     * table overflowed. */
     int64_t count_points[5];
     /* Levels of the fine-grained step's heavy tasks whose updates were a
      * recount (see receipt_options.fd_huc), and the wedges those recounts
@@ -320,7 +323,7 @@ receipt_status receipt_count_butterflies(receipt_graph *g, uint64_t *d_cnt_u,
  *   graph must have at most 65,536 vertices on each side and at most
  *   1,048,576 edges (after duplicate removal), else RECEIPT_ERR_INVALID with
  *   a message naming the limits.
- *   Every temporary lives in one fixed array of about 11 MB inside the
+ *   Every temporary lives in one fixed array of about 19 MB inside the
  *   library's device image, held on every GPU that loads the library until
  *   the process exits. The first call on a device looks up that array's
  *   device address; make that first call before any stream capture.

@@ -430,6 +430,7 @@ void decompose_batch_impl(receipt_graph *const *gs, const receipt_side *sides, i
     U.max_deg[0] = maxdeg[0];
     U.max_deg[1] = maxdeg[1];
     U.parts = abase;
+    U.parts_o = bbase;
     DevBuf<int64_t> offA(NA + 1, s), offB(NB + 1, s);
     DevBuf<int32_t> adjA(M, s), adjB(M, s), n2oA(NA, s), n2oB(NB, s), belA(NA, s), belB(NB, s);
     DevBuf<PackSrc> dsrc(n, s);

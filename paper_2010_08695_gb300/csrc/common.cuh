@@ -116,6 +116,7 @@ struct receipt_graph {
     std::vector<receipt_round> trace;  // rounds of the last decomposition
     std::vector<receipt_subset> subsets;  // fine-grained subsets of the last decomposition
     std::vector<int64_t> parts;  // batch union: first side-0 vertex of every packed graph
+    std::vector<int64_t> parts_o;  // ... first side-1 vertex
     void *owned = nullptr;  // device allocation holding every array above
 };
 

@@ -825,7 +825,10 @@ struct NoChunkHook {
 //   __device__ void seg(int64_t q, int64_t &beg, int32_t &len) const;
 // visit(k, key): k = mid index within the chunk, key = end point.
 // Returns the number of wedges walked. All threads of the CTA must call it.
-template <bool BALANCED = true, class Keys = KeysNc, class Mids, class Visit,
+// U: groups per step. More hide the key loads' latency with few warps; fewer
+// keep the code (U copies of the visit) in the instruction cache when many
+// CTAs of a kernel are at different places of it.
+template <bool BALANCED = true, class Keys = KeysNc, int U = WALK_UNROLL, class Mids, class Visit,
           class Hook = NoChunkHook>
 __device__ int64_t cta_walk(const Mids &M, int64_t q0, int64_t q1, const int32_t *__restrict__ keys,
                             Chunk &ch, Visit &visit, Hook *hook = nullptr) {
@@ -885,9 +888,9 @@ __device__ int64_t cta_walk(const Mids &M, int64_t q0, int64_t q1, const int32_t
         const int32_t total = (int32_t)(tot2 & ((1ll << 40) - 1));
         const int32_t nnz = (int32_t)(tot2 >> 40);
         const int32_t groups = (total + 31) >> 5;
-        const int32_t g_lo = BALANCED ? (int32_t)(((int64_t)groups * warp) / nwarps) : warp * WALK_UNROLL;
+        const int32_t g_lo = BALANCED ? (int32_t)(((int64_t)groups * warp) / nwarps) : warp * U;
         const int32_t g_hi = BALANCED ? (int32_t)(((int64_t)groups * (warp + 1)) / nwarps) : groups;
-        const int32_t g_step = BALANCED ? WALK_UNROLL : nwarps * WALK_UNROLL;
+        const int32_t g_step = BALANCED ? U : nwarps * U;
         for (int32_t gb = g_lo; gb < g_hi; gb += g_step) {
             // segment of the first wedge of group gb (warp-uniform search)
             int lo = 0, hi = nnz - 1;
@@ -904,10 +907,10 @@ __device__ int64_t cta_walk(const Mids &M, int64_t q0, int64_t q1, const int32_t
             int32_t p0 = ch.pre[k0], p1 = ch.pre[k0 + 1];
             int64_t bg0 = ch.beg[k0];
             int kl0 = ch.len[k0];
-            int kk[WALK_UNROLL];
-            int32_t key[WALK_UNROLL];
+            int kk[U];
+            int32_t key[U];
 #pragma unroll
-            for (int u = 0; u < WALK_UNROLL; u++) {
+            for (int u = 0; u < U; u++) {
                 const int32_t base = (gb + u) << 5;
                 kk[u] = 0;
                 key[u] = -1;
@@ -938,7 +941,7 @@ __device__ int64_t cta_walk(const Mids &M, int64_t q0, int64_t q1, const int32_t
                     }
                 }
             }
-            visit_many<WALK_UNROLL>(visit, kk, key);
+            visit_many<U>(visit, kk, key);
         }
         walked += total;
         __syncthreads();
