@@ -103,12 +103,11 @@ typedef struct {
     /* Fine-grained step (Algorithm 4): subsets whose wedge count (the LPT key
      * of Sec. 3.2.1, sum of L(L-1) over the runs L of G_i) is at least this
      * are peeled by all CTAs level by level instead of by one CTA of the
-     * persistent queue. 0 = automatic: 8 times the total weight divided by
-     * the smaller of the CTA count and the task count, or by the CTA count
-     * when there are at most half as many tasks as CTAs; at least 2^23; and
-     * also every task whose weight plus 2^15 per member exceeds the CTA
-     * count's share of the total of those sums while its wedges are at
-     * least 4 x 2^15 per member (walk-bound). A level of such a task with at
+     * persistent queue. 0 = automatic: tasks of 2^17 members and more whose
+     * range is at most members / 2^16 wide, and tasks whose members without
+     * an update list (or all members, when the lists would not fit an eighth
+     * of the device's memory) walk at least 2^23 wedges and at least
+     * 4 x 2^15 per member of the task. A level of such a task with at
      * most 32 members with big walks spreads each one's walk over the CTAs
      * in equal wedge shares. -1 = never. Speed only. */
     int64_t fd_heavy_w;

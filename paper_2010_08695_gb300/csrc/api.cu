@@ -116,6 +116,19 @@ cudaStream_t tier_stream(int k) {
     return device_stream(1 + k);
 }
 
+size_t available_bytes() {
+    size_t free_b = 0, total = 0;
+    RC_CUDA(cudaMemGetInfo(&free_b, &total));
+    int d = 0;
+    RC_CUDA(cudaGetDevice(&d));
+    cudaMemPool_t pool;
+    uint64_t reserved = 0, used = 0;
+    RC_CUDA(cudaDeviceGetDefaultMemPool(&pool, d));
+    RC_CUDA(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved));
+    RC_CUDA(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used));
+    return free_b + (size_t)(reserved > used ? reserved - used : 0);
+}
+
 int num_sms() { return dev_info().sms; }
 int max_smem_optin() { return dev_info().smem_optin - 1024; }
 void allow_max_smem(const void *kernel) {

@@ -126,11 +126,22 @@ __device__ __forceinline__ void emit_many(E &e, const int32_t (&k)[N], const uin
 // lengths numbers their wedges, and each lane takes wedges lane, lane + 32,
 // ..., finding its segment by a binary search over the lanes' starts, so all
 // key loads of a step are independent (U per lane in flight). visit(key).
+// A group of `parts` warps shares the walk by calls with part = 0 .. parts - 1:
+// blocks of 32 middle vertices when each warp has two or more, else the wedges
+// of every block.
 template <int U, class Keys = KeysNc, class Mids, class Visit>
 __device__ __forceinline__ void warp_walk(const Mids &M, int64_t q0, int64_t q1,
-                                          const int32_t *__restrict__ keys, Visit &visit) {
+                                          const int32_t *__restrict__ keys, Visit &visit,
+                                          int part = 0, int parts = 1) {
     const int lane = threadIdx.x & 31;
-    for (int64_t qb = q0; qb < q1; qb += 32) {
+    int64_t qstep = 32;
+    if (parts > 1 && q1 - q0 >= 64 * parts) {
+        q0 += 32 * part;
+        qstep = 32 * parts;
+        part = 0;
+        parts = 1;
+    }
+    for (int64_t qb = q0; qb < q1; qb += qstep) {
         int64_t beg = 0;
         int32_t len = 0;
         if (qb + lane < q1) M.seg(qb + lane, beg, len);
@@ -142,11 +153,11 @@ __device__ __forceinline__ void warp_walk(const Mids &M, int64_t q0, int64_t q1,
         }
         const int32_t total = __shfl_sync(0xffffffffu, inc, 31);
         const int32_t ex = inc - len;
-        for (int32_t j0 = 0; j0 < total; j0 += 32 * U) {
+        for (int32_t j0 = part * 32; j0 < total; j0 += 32 * U * parts) {
             int32_t key[U];
 #pragma unroll
             for (int u = 0; u < U; u++) {
-                const int32_t j = j0 + u * 32 + lane;
+                const int32_t j = j0 + u * 32 * parts + lane;
                 // last lane whose segment starts at or before j (all lanes
                 // take part in the shuffles)
                 int lo = 0;

@@ -12,6 +12,9 @@
 //  * a task queue of subset ids in decreasing order of their wedge count
 //    (Longest Processing Time first).
 //
+// The members' updates are aggregated before the peel, all at once, into lists
+// (k_fd_pairs).
+//
 // Peeling: persistent CTAs pop subsets from the queue with one atomic each.
 // Inside a subset the CTA runs bottom-up peeling level by level: the level
 // mu = max(previous level, min support over the remaining vertices); every
@@ -38,9 +41,12 @@ using FdEngine = DenseSliceT<FD_WORDS, TOUCH_LIST>;
 static_assert(TOUCH_CAP * 2 >= LOG_BUCKETS * 4, "histogram in the touched-word list");
 // walk-size flag: the vertex's degree is >= 65535 (counts may need 32 bits)
 constexpr unsigned long long WIDE_BIT = 1ull << 63;
-// heavy subsets: automatic threshold
+// heavy tasks, automatic rule
 constexpr unsigned long long HEAVY_MIN_W = 1ull << 23;
-constexpr unsigned long long HEAVY_SHARE = 8;
+constexpr int32_t HEAVY_NI = 1 << 17;
+// list entries are at most an eighth of the walks' wedges (measured: 1/10 to
+// 1/14 on Chung-Lu graphs, far fewer on uniform ones)
+constexpr unsigned long long LIST_SHARE = 8;
 // a level of a heavy task with at most this many members with big walks
 // (and at least two CTAs for each) splits each one's walk over the CTAs
 // (partial counts summed in global counters) instead of giving each member
@@ -51,9 +57,9 @@ constexpr int FDH_SPLIT_NB = 32;
 constexpr unsigned long long HEAVY_WALK_LEVELS = 4;
 // parts of one subset are merged into tasks of at least this many members
 constexpr int32_t TASK_MIN = 8192;
-// LPT weight of one member of a task in wedges: a level of the one-CTA peel
-// costs ~20-40 us (measured on Chung-Lu graphs of 10M-100M edges), the time
-// a CTA needs for ~2^15 wedges of updates
+// LPT weight of one member of a task in wedges. A task's time is its levels',
+// 2-3 us each and at most one a member; its walks, done before the peel, tell
+// tasks of as many members apart.
 constexpr unsigned long long LEVEL_WEDGES = 1ull << 15;
 
 __global__ void k_sub_keys(const int32_t *__restrict__ sub, int32_t n, uint64_t *__restrict__ key,
@@ -158,18 +164,29 @@ __global__ void k_i32_to_i64(const int32_t *__restrict__ v, int64_t m, int64_t *
     if (q < m) out[q] = v[q];
 }
 
+// A member's edges and its walk size inside G_i, by member position.
+struct alignas(16) FdMember {
+    int64_t q0;
+    int32_t deg;
+    uint32_t w;  // saturated
+};
+
 // Walk size inside G_i of every vertex (sum of its edges' run lengths, from
 // the prefix sums `pre`), stored at its member position; WIDE_BIT marks a
-// degree >= 65535 (counts may need 32 bits).
+// degree >= 65535 (counts may need 32 bits), wide[] its subset.
 __global__ void k_fd_walk_sizes(const int64_t *__restrict__ off_s, int32_t n,
                                 const int64_t *__restrict__ pre, const int32_t *__restrict__ sub,
                                 const int32_t *__restrict__ mstart, const int32_t *__restrict__ rank,
-                                unsigned long long *__restrict__ wr) {
+                                unsigned long long *__restrict__ wr, FdMember *__restrict__ info,
+                                int32_t *__restrict__ wide) {
     int32_t x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= n) return;
     const int64_t q0 = off_s[x], q1 = off_s[x + 1];
     const unsigned long long W = (unsigned long long)(pre[q1] - pre[q0]);
-    wr[mstart[sub[x]] + rank[x]] = W | (q1 - q0 >= 65535 ? WIDE_BIT : 0ull);
+    const int32_t p = mstart[sub[x]] + rank[x];
+    wr[p] = W | (q1 - q0 >= 65535 ? WIDE_BIT : 0ull);
+    info[p] = FdMember{q0, (int32_t)(q1 - q0), (uint32_t)(W < 0xffffffffull ? W : 0xffffffffull)};
+    if (q1 - q0 >= 65535) wide[sub[x]] = 1;
 }
 
 // Task boundaries: the first member of every subset and, when the side is a
@@ -206,17 +223,19 @@ __global__ void k_flag_positions(const uint32_t *__restrict__ flag, const uint32
     if (p < n && flag[p]) out[pos[p]] = p;
 }
 
-__global__ void k_walk_plain(const unsigned long long *__restrict__ wr, int32_t n,
-                             int64_t *__restrict__ out) {
+// a member's cost: its wedges and a constant
+__global__ void k_walk_cost(const unsigned long long *__restrict__ wr, int32_t n, int64_t add,
+                            int64_t *__restrict__ out) {
     const int32_t p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p < n) out[p] = (int64_t)(wr[p] & ~WIDE_BIT);
+    if (p < n) out[p] = (int64_t)(wr[p] & ~WIDE_BIT) + add;
 }
 
 __global__ void k_task_weights(const int32_t *__restrict__ tstart, const int32_t *__restrict__ tlen,
-                               const int64_t *__restrict__ cw, int32_t T,
+                               const int64_t *__restrict__ cw, int64_t add, int32_t T,
                                unsigned long long *__restrict__ w) {
     const int32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < T) w[t] = (unsigned long long)(cw[tstart[t] + tlen[t]] - cw[tstart[t]]);
+    if (t < T)
+        w[t] = (unsigned long long)(cw[tstart[t] + tlen[t]] - cw[tstart[t]] - add * tlen[t]);
 }
 
 struct FdArgs {
@@ -227,7 +246,6 @@ struct FdArgs {
     const int32_t *tlen;       // per task: members
     const int32_t *tkb;        // per task: rank of its first member inside its subset
     const int32_t *members;
-    const int64_t *off_s;
     const int64_t *fd_beg;
     const int32_t *fd_len;
     const int32_t *fd_adj;
@@ -240,12 +258,13 @@ struct FdArgs {
     int32_t *clist;            // by member position: members inside the window (two buffers)
     int32_t *clist2;
     int32_t *plist;            // by member position
-    int32_t *blist;            // by member position: peeled vertices with big updates
+    const FdMember *info;      // by member position
+    const uint32_t *pool;      // the members' lists, and where each lies
+    const unsigned long long *rec;
     unsigned long long *tip;   // output, original ids
     unsigned long long *stats; // [0] wedges, [1] levels
     unsigned long long *sub_ns;     // per task: nanoseconds spent
     unsigned long long *sub_levels; // per task: peeling levels
-    unsigned long long *wr;    // by member position: walk size inside G_i (WIDE_BIT: degree >= 65535)
 };
 
 struct FdMids {
@@ -305,6 +324,396 @@ struct FdEmit {
     }
 };
 
+// ------------------------------------------------------------------------
+// Every member's updates, before the peel
+//
+// What peeling a member r takes from the others of its subset depends only on
+// how many middle vertices they share, not on when r is peeled: C(c, 2) for
+// each member sharing c >= 2. So the walks of all members are done first, by
+// the whole chip and in any order, and leave each member a list of (rank,
+// count) entries; a level of the peel, a chain of dependent steps on one SM,
+// then reads a list instead of walking (runs, keys, counters, sweep).
+//
+// Walks have 100 to 2,000 wedges over about ten middle vertices in the tasks
+// that take longest, and up to a million in the last ones. A member gets a
+// group of g warps (a power of two), which counts in its warps' FP_WORDS words
+// taken together, one counter per rank: a count is at most the member's
+// degree, so 4 bits do for degrees up to 15, 8 up to 255, 16 up to 65,535
+// and 32 above (neighbouring ranks lie in different words). g is the least that holds the
+// counters, and at least a warp per 4,096 wedges or 512 middle vertices. A walk much shorter than its
+// task (8 W below the words the counters need) uses a table with entries (rank
+// + 1) << 10 | count instead, at most half full: at 3/4 the longest probe of a
+// warp's 32 dominated (8 us a member of 1,000 wedges; counters 1 us). Members
+// whose counters exceed a CTA's words up to 8 times walk once per slice of them.
+// The entries lie in one pool, taken by each group in blocks; a member whose
+// list does not fit it, or that is too large for all this, has no list and
+// walks when it is peeled.
+// Two CTAs of 16 warps an SM: bound by the latency of runs and keys from L2.
+// 1.93e9 wedges of a 40M-edge graph in 9.1 ms, 3.9e8 of a 10M-edge graph in 3.0
+// ms; walked during the peel they made the whole step 101 and 26 ms (34 and 10
+// now).
+// ------------------------------------------------------------------------
+constexpr int FP_THREADS = 512;
+constexpr int FP_WARPS = FP_THREADS / 32;
+constexpr int FP_WORDS = 1024;           // counter words of a warp
+constexpr int FP_BLOCK = 1024;           // pool entries taken at a time
+constexpr int32_t FP_HASH_DEG = 1024;    // counts of the table's entries
+constexpr int32_t FP_MAX_NI = (1 << 22) - 2;  // ranks of the entries
+constexpr int64_t FP_MEMBER_COST = 128;  // a member's fixed cost in wedges
+// An entry holds the rank in its low fp_rank_bits and the count above.
+constexpr unsigned long long FP_NONE = ~0ull;  // no list; else offset << 24 | length
+__device__ __forceinline__ int fp_rank_bits(int32_t ni) {
+    return max(1, 32 - __clz(ni - 1));
+}
+
+struct FdPairArgs {
+    const int32_t *tstart, *tlen, *tkb;
+    const uint8_t *tskip;     // tasks without lists
+    int32_t T;
+    const int32_t *item_p;    // per item: first member position (nitems + 1)
+    int32_t nitems;
+    int32_t *qhead;
+    const FdMember *info;     // by member position
+    const int64_t *fd_beg;
+    const int32_t *fd_len;
+    const int32_t *fd_adj;
+    uint32_t *pool;
+    unsigned long long cap;   // entries
+    unsigned long long *head;
+    unsigned long long *rec;  // by member position
+    unsigned long long *wedges;
+};
+
+// First member position of every item of Q cost units (cw: prefix costs).
+__global__ void k_pair_items(const int64_t *__restrict__ cw, int32_t n, int64_t Q, int32_t nitems,
+                             int32_t *__restrict__ item_p) {
+    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i > nitems) return;
+    int32_t lo = 0, hi = n;
+    while (lo < hi) {
+        const int32_t mid = lo + (hi - lo) / 2;
+        if (cw[mid] < (int64_t)i * Q)
+            lo = mid + 1;
+        else
+            hi = mid;
+    }
+    item_p[i] = i == nitems ? n : lo;
+}
+
+__device__ __forceinline__ FdMember fd_load(const FdMember *p) {
+    const int4 q = __ldg((const int4 *)p);
+    return FdMember{(int64_t)(uint32_t)q.x | ((int64_t)q.y << 32), q.z, (uint32_t)q.w};
+}
+
+__device__ __forceinline__ void fp_table_add(uint32_t *slot, uint32_t mask, int32_t key) {
+    const uint32_t k = ((uint32_t)key + 1u) << 10;
+    uint32_t h = (hash_key(key) >> 8) & mask;
+    for (uint32_t p = 0; p <= mask; p++) {
+        uint32_t cur = ((volatile uint32_t *)slot)[h];
+        if (cur == 0) {
+            cur = atomicCAS(&slot[h], 0u, k | 1u);
+            if (cur == 0) return;
+        }
+        if ((cur ^ k) < 1024u) {
+            atomicAdd(&slot[h], 1u);
+            return;
+        }
+        h = (h + 1) & mask;
+    }
+}
+
+// How a member is counted: bits of its counters (0: the table), log2 of the
+// words it needs, and warps (above FP_WARPS: no list).
+struct FpPlan {
+    int bits, lw, g;
+};
+__device__ __forceinline__ FpPlan fp_plan(const FdMember &m, int32_t ni) {
+    FpPlan p;
+    p.bits = m.deg < 16 ? 4 : m.deg < 256 ? 8 : m.deg < 65536 ? 16 : 32;
+    p.lw = max(7, 32 - __clz((int)(((int64_t)ni * p.bits + 31) / 32) - 1));
+    if (m.deg < FP_HASH_DEG && m.w < FP_WARPS * FP_WORDS / 2 && (m.w << 3) < (1u << p.lw)) {
+        p.bits = 0;
+        p.lw = max(7, 33 - __clz(m.w));  // 2 W to 4 W words
+    }
+    const bool ok = (int64_t)m.deg < (1ll << (32 - fp_rank_bits(ni)));
+    // a step of a warp takes 32 middle vertices or 128 wedges
+    const uint64_t steps = (uint64_t)m.w + 8ull * (uint32_t)m.deg;
+    const int by_w = steps <= 4096 ? 0 : steps > 32768 ? 4 : 32 - __clz((uint32_t)(steps - 1) >> 12);
+    p.g = ok && p.lw <= 17 ? 1 << min(max(p.lw - 10, by_w), 4) : 2 * FP_WARPS;
+    return p;
+}
+static_assert(FP_WORDS == 1 << 10 && FP_WARPS == 1 << 4, "words and warps of a plan");
+
+// Weight of each task's members that get no list.
+__global__ void k_listless(const FdMember *__restrict__ info, int32_t n,
+                           const int32_t *__restrict__ tstart, const int32_t *__restrict__ tlen,
+                           int32_t T, int32_t ni_max, unsigned long long *__restrict__ lw) {
+    const int32_t p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= n) return;
+    const FdMember m = fd_load(info + p);
+    if (ni_max <= FP_MAX_NI && fp_plan(m, ni_max).g <= FP_WARPS) return;
+    int32_t t = 0;
+    for (int32_t hi = T - 1; t < hi;) {
+        const int32_t mid = (t + hi + 1) / 2;
+        if (tstart[mid] <= p)
+            t = mid;
+        else
+            hi = mid - 1;
+    }
+    if (tlen[t] > FP_MAX_NI || fp_plan(m, tlen[t]).g > FP_WARPS)
+        atomicAdd(&lw[t], (unsigned long long)m.w);
+}
+
+// Counters of at least 2 in a word of b-bit counters: the lowest bit of each.
+__device__ __forceinline__ uint32_t fp_repeats(uint32_t v, int bits) {
+    if (bits == 4) return ((v >> 1) | (v >> 2) | (v >> 3)) & 0x11111111u;
+    if (bits == 32) return v >= 2 ? 1u : 0u;
+    uint32_t x = v & (bits == 8 ? 0xfefefefeu : 0xfffefffeu);
+    if (bits == 16) x |= x >> 8;
+    x |= x >> 4;
+    x |= x >> 2;
+    x |= x >> 1;
+    return x & (bits == 8 ? 0x01010101u : 0x00010001u);
+}
+
+__device__ __forceinline__ void fp_sync(int grp, int g) {
+    if (g == 1)
+        __syncwarp();
+    else
+        asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(32 * g) : "memory");
+}
+
+__global__ void __launch_bounds__(FP_THREADS, 2) k_fd_pairs(FdPairArgs a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int s_item;
+    __shared__ int s_cnt[FP_WARPS];                  // entries found by each warp
+    __shared__ unsigned long long s_off[FP_WARPS];   // by group: where its list lies
+    uint32_t *tab = (uint32_t *)smem;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int j = threadIdx.x; j < FP_WARPS * FP_WORDS / 4; j += FP_THREADS)
+        ((uint4 *)tab)[j] = make_uint4(0, 0, 0, 0);
+    FdMids M{a.fd_beg, a.fd_len};
+    unsigned long long wedges = 0;             // lane 0
+    unsigned long long blk = 0, blk_end = 0;   // lane 0: this warp's pool block
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_item = atomicAdd(a.qhead, 1);
+        __syncthreads();
+        const int it = a.nitems - 1 - s_item;  // the largest walks come last in position order
+        if (it < 0) break;
+        const int32_t p0 = a.item_p[it], p1 = a.item_p[it + 1];
+        // last task starting at or before p0
+        int32_t t = 0;
+        for (int32_t hi = a.T - 1; t < hi;) {
+            const int32_t mid = (t + hi + 1) / 2;
+            if (a.tstart[mid] <= p0)
+                t = mid;
+            else
+                hi = mid - 1;
+        }
+        for (; t < a.T && a.tstart[t] < p1; t++) {
+            const int32_t ts = a.tstart[t], ni = a.tlen[t], kb = a.tkb[t];
+            if (a.tskip[t] || ni > FP_MAX_NI) continue;
+            const int32_t pa = max(p0, ts), pb = min(p1, ts + ni);
+            const int rb = fp_rank_bits(ni);
+            for (int g = 1; g <= FP_WARPS; g *= 2) {
+                const int grp = warp / g, part = warp & (g - 1);
+                uint32_t *w = tab + grp * g * FP_WORDS;
+                bool more = false;
+                for (int32_t p = pa + grp; p < pb; p += FP_WARPS / g) {
+                    const FdMember m = fd_load(a.info + p);
+                    const FpPlan pl = fp_plan(m, ni);
+                    if (pl.g != g) {
+                        more |= pl.g > g && pl.g <= FP_WARPS;
+                        continue;
+                    }
+                    if (m.w == 0) {
+                        if (part == 0 && lane == 0) a.rec[p] = 0;
+                        continue;
+                    }
+                    const int32_t self = p - ts;
+                    const int slices = pl.lw > 14 ? 1 << (pl.lw - 14) : 1;
+                    const uint32_t wmask = (1u << min(pl.lw, 14)) - 1u;
+                    unsigned long long off = 0;  // lane 0 of part 0: where the next slice's entries go
+                    unsigned found = 0;          // ... and those before
+                    for (int sc = 0; sc < slices; sc++) {
+                        if (pl.bits) {
+                            auto add = [&](int32_t key) {
+                                const int32_t k = key - kb;
+                                if (k == self) return;
+                                if (slices > 1 && ((k >> 14) & (slices - 1)) != sc) return;
+                                atomicAdd(&w[k & wmask], 1u << ((k >> pl.lw) * pl.bits));
+                            };
+                            warp_walk<4>(M, m.q0, m.q0 + m.deg, a.fd_adj, add, part, g);
+                        } else {
+                            auto add = [&](int32_t key) {
+                                const int32_t k = key - kb;
+                                if (k != self) fp_table_add(w, wmask, k);
+                            };
+                            warp_walk<4>(M, m.q0, m.q0 + m.deg, a.fd_adj, add, part, g);
+                        }
+                        fp_sync(grp, g);
+                        // entries in words 4 sl .. 4 sl + 3 of this lane
+                        int cnt = 0;
+                        for (uint32_t sl = part * 32 + lane; sl <= wmask / 4; sl += 32 * g) {
+                            const uint4 v = ((const uint4 *)w)[sl];
+                            if (!(v.x | v.y | v.z | v.w)) continue;
+                            const uint32_t e[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                            for (int x = 0; x < 4; x++)
+                                cnt += pl.bits ? __popc(fp_repeats(e[x], pl.bits))
+                                               : (e[x] & 1023u) >= 2;
+                        }
+                        int inc = cnt;
+#pragma unroll
+                        for (int o = 1; o < 32; o <<= 1) {
+                            const int y = __shfl_up_sync(0xffffffffu, inc, o);
+                            if (lane >= o) inc += y;
+                        }
+                        const int wtot = __shfl_sync(0xffffffffu, inc, 31);
+                        int before = 0, total = wtot;
+                        if (g > 1) {
+                            if (lane == 0) s_cnt[warp] = wtot;
+                            fp_sync(grp, g);
+                            const int c = lane < g ? s_cnt[grp * g + lane] : 0;
+                            total = __reduce_add_sync(0xffffffffu, c);
+                            before = __reduce_add_sync(0xffffffffu, lane < part ? c : 0);
+                        }
+                        unsigned long long dst = 0;
+                        if (part == 0 && lane == 0) {
+                            if (sc == 0) {
+                                // room for the list: its length, or with more
+                                // slices to come the most it can be
+                                const unsigned long long room =
+                                    slices == 1 ? (unsigned)total : min(m.w / 2, (uint32_t)ni);
+                                if (blk + room > blk_end) {
+                                    const unsigned long long take =
+                                        max((unsigned long long)FP_BLOCK, slices == 1 ? room : 16 * room);
+                                    blk = atomicAdd(a.head, take);
+                                    blk_end = blk + take;
+                                }
+                                off = blk_end <= a.cap ? blk : FP_NONE;
+                            }
+                            dst = off == FP_NONE ? FP_NONE : off + found;
+                            found += total;
+                            if (g > 1) s_off[grp] = dst;
+                            if (sc == slices - 1) {
+                                a.rec[p] = off == FP_NONE ? FP_NONE : (off << 24) | found;
+                                blk += found;
+                                wedges += (unsigned long long)m.w * slices;
+                            }
+                        }
+                        if (g > 1) {
+                            fp_sync(grp, g);
+                            dst = s_off[grp];
+                        } else {
+                            dst = __shfl_sync(0xffffffffu, dst, 0);
+                        }
+                        uint32_t *out = a.pool + dst + before + (inc - cnt);
+                        for (uint32_t sl = part * 32 + lane; sl <= wmask / 4; sl += 32 * g) {
+                            const uint4 v = ((const uint4 *)w)[sl];
+                            if (!(v.x | v.y | v.z | v.w)) continue;
+                            ((uint4 *)w)[sl] = make_uint4(0, 0, 0, 0);
+                            if (dst == FP_NONE) continue;
+                            const uint32_t e[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                            for (int x = 0; x < 4; x++) {
+                                if (pl.bits == 0) {
+                                    const uint32_t c = e[x] & 1023u;
+                                    if (c >= 2) *out++ = ((e[x] >> 10) - 1u) | (c << rb);
+                                    continue;
+                                }
+                                const uint32_t k0 = ((uint32_t)sc << 14) + 4 * sl + x;
+                                for (uint32_t f = fp_repeats(e[x], pl.bits); f; f &= f - 1) {
+                                    const int b = __ffs(f) - 1;
+                                    const uint32_t c = (e[x] >> b) & (0xffffffffu >> (32 - pl.bits));
+                                    *out++ = (k0 + ((uint32_t)(b / pl.bits) << pl.lw)) | (c << rb);
+                                }
+                            }
+                        }
+                        fp_sync(grp, g);
+                    }
+                }
+                if (!__syncthreads_or(more)) break;
+            }
+        }
+    }
+    if (lane == 0 && wedges) atomicAdd(a.wedges, wedges);
+}
+
+// The listed updates of one level's np members (list: ranks in the task; rec:
+// the task's records), a group of warps per member: the widest groups that
+// give each of up to 16 members one, a warp per member above. Members without
+// a list are returned in list[0, n). All threads, after a barrier; ends with
+// one.
+constexpr int FD_WARPS = FD_THREADS / 32;
+template <class List, class Emit>
+__device__ __forceinline__ int fd_lists(const uint32_t *__restrict__ pool,
+                                        const unsigned long long *__restrict__ rec, List *list,
+                                        int np, int rb, Emit &emit, int *s_nbig) {
+    constexpr uint32_t MARK = 1u << (8 * sizeof(List) - 1);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int g = np >= FD_WARPS ? 1 : np > 0 ? FD_WARPS >> (32 - __clz(np - 1)) : 1;
+    const int grp = warp / g, part = warp & (g - 1);
+    const uint32_t rmask = (1u << rb) - 1u;
+    bool left = false;
+    // the next member's record is fetched ahead
+    uint32_t rn = grp < np ? (uint32_t)list[grp] & ~MARK : 0u;
+    unsigned long long qn = grp < np ? __ldg(rec + rn) : 0ull;
+    for (int pi = grp; pi < np; pi += FD_WARPS / g) {
+        const uint32_t r = rn;
+        const unsigned long long q = qn;
+        if (pi + FD_WARPS / g < np) {
+            rn = (uint32_t)list[pi + FD_WARPS / g] & ~MARK;
+            qn = __ldg(rec + rn);
+        }
+        if (q == FP_NONE) {
+            if (part == 0 && lane == 0) list[pi] = (List)(r | MARK);
+            left = true;
+            continue;
+        }
+        const uint32_t *e = pool + (q >> 24);
+        const int len = (int)(q & 0xffffffu);
+        for (int j0 = part * 32 + lane; j0 < len; j0 += 128 * g) {
+            uint32_t v[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const int j = j0 + u * 32 * g;
+                v[u] = j < len ? __ldg(e + j) : 0u;
+            }
+            int32_t k[4];
+            uint32_t c[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                c[u] = v[u] >> rb;
+                k[u] = c[u] ? (int32_t)(v[u] & rmask) : -1;
+            }
+            emit.template many<4>(k, c);
+        }
+    }
+    if (!__syncthreads_or(left)) return 0;
+    // gather the marked: entries move to lower places only, each after the
+    // barrier behind its own read
+    for (int base = 0; base < np; base += FD_THREADS) {
+        const int j = base + threadIdx.x;
+        const uint32_t r = j < np ? (uint32_t)list[j] : 0u;
+        const unsigned bal = __ballot_sync(0xffffffffu, (r & MARK) != 0);
+        __syncthreads();
+        if (bal) {
+            int pos = 0;
+            if (lane == 0) pos = atomicAdd(s_nbig, __popc(bal));
+            pos = __shfl_sync(0xffffffffu, pos, 0) + __popc(bal & lanemask_lt());
+            if (r & MARK) list[pos] = (List)(r ^ MARK);
+        }
+    }
+    __syncthreads();
+    np = *s_nbig;
+    __syncthreads();
+    if (threadIdx.x == 0) *s_nbig = 0;
+    __syncthreads();
+    return np;
+}
+
 // Ranks of one slice [base, end) of the subset's rank space: the run of a
 // middle vertex is sorted by rank, so the slice is a sub-run found by two
 // binary searches.
@@ -337,7 +746,6 @@ struct FdSliceVisit {
 struct FdSliceEmit {
     FdEmit *e;
     int32_t base;
-    __device__ __forceinline__ void operator()(int32_t k, uint32_t c) { (*e)(k + base, c); }
     template <int N>
     __device__ __forceinline__ void many(const int32_t (&k)[N], const uint32_t (&c)[N]) {
         int32_t kk[N];
@@ -347,63 +755,9 @@ struct FdSliceEmit {
     }
 };
 
-// Several anchors of one level aggregated in one pass: anchor slot a of the
-// batch owns keys [a * ni, (a + 1) * ni) of the dense counters. The batch's
-// edges form one virtual list of middle vertices; the thread that stages a
-// middle vertex records its anchor slot for the visits.
-constexpr int FD_BATCH = 32;
 // window of the level loop: about max(MIN, min(MAX, alive / 32)) members
 constexpr int FD_WINDOW_MIN = 512;
 constexpr int FD_WINDOW_MAX = 4096;
-
-struct FdBatchMids {
-    const int64_t *fd_beg;
-    const int32_t *fd_len;
-    const int64_t *bq0;   // first edge of each anchor (shared memory)
-    const int32_t *bpre;  // prefix of the anchors' degrees (nb + 1 entries)
-    int32_t nb;
-    uint8_t *slot;        // anchor slot of the middle vertex staged by each thread
-    __device__ __forceinline__ void seg(int64_t q, int64_t &beg, int32_t &len) const {
-        int lo = 0, hi = nb - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (bpre[mid] <= q)
-                lo = mid;
-            else
-                hi = mid - 1;
-        }
-        const int64_t e = bq0[lo] + (q - bpre[lo]);
-        beg = fd_beg[e];
-        len = fd_len[e];
-        slot[threadIdx.x] = (uint8_t)lo;
-    }
-};
-
-struct FdBatchVisit {
-    FdEngine *eng;
-    const uint8_t *slot;
-    const int32_t *bself;  // rank of each anchor (task ranks)
-    int32_t ni;
-    int32_t kb;            // first subset rank of the task
-    __device__ __forceinline__ void operator()(int k, int32_t key) {
-        const int a = slot[k];
-        key -= kb;
-        if (key != bself[a]) eng->add(a * ni + key);
-    }
-};
-
-struct FdBatchEmit {
-    FdEmit *e;
-    int32_t ni;
-    __device__ __forceinline__ void operator()(int32_t w, uint32_t c) { (*e)(w % ni, c); }
-    template <int N>
-    __device__ __forceinline__ void many(const int32_t (&k)[N], const uint32_t (&c)[N]) {
-        int32_t kk[N];
-#pragma unroll
-        for (int u = 0; u < N; u++) kk[u] = k[u] >= 0 ? k[u] % ni : -1;
-        e->template many<N>(kk, c);
-    }
-};
 
 // Update of one peeled member r (anchor x, edges [q0, q1) of side s) whose
 // walk has at most WARP_MAX_W wedges: one warp with its private table.
@@ -585,7 +939,7 @@ __device__ __forceinline__ unsigned char *fd_bind_smem(unsigned char *smem, int 
 
 __global__ void __launch_bounds__(FD_THREADS, 1) k_fd_peel(FdArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int s_t, s_dn, s_np, s_nbig, s_nwide, s_nf, s_pick, s_peel, s_rk;
+    __shared__ int s_t, s_dn, s_np, s_nbig, s_nf, s_pick, s_peel, s_rk;
     // window list count and next level's minimum, by level parity: level L
     // fills set L & 1 while stragglers of level L - 1 may still read the other
     __shared__ int s_nk[2];
@@ -593,18 +947,12 @@ __global__ void __launch_bounds__(FD_THREADS, 1) k_fd_peel(FdArgs a) {
     __shared__ unsigned long long s_rmn;  // minimum of a refilled window
     __shared__ unsigned long long s_T;   // window bound
     __shared__ int32_t s_scan[33];
-    __shared__ int64_t s_bq0[FD_BATCH];
-    __shared__ int32_t s_bpre[FD_BATCH + 1], s_bself[FD_BATCH];
-    __shared__ uint8_t s_slot[FD_THREADS];
     FdEngine H;
     Chunk ch;
-    // warp-private tables after the chunk staging
-    int32_t *wkey = (int32_t *)fd_bind_smem(smem, &s_dn, H, ch);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    WarpHash WH{wkey + warp * WARP_SLOTS, (uint32_t *)(wkey + nwarps * WARP_SLOTS) + warp * WARP_SLOTS};
-    WH.clear(lane);
+    fd_bind_smem(smem, &s_dn, H, ch);
+    const int lane = threadIdx.x & 31;
     H.clear_all();
-    FdMids M{a.fd_beg, a.fd_len};
+    if (threadIdx.x == 0) s_nbig = 0;
     // per warp (lane 0): wedges walked; thread 0 also counts levels
     unsigned long long wedges = 0, levels = 0;
     __syncthreads();
@@ -631,9 +979,9 @@ __global__ void __launch_bounds__(FD_THREADS, 1) k_fd_peel(FdArgs a) {
         int32_t *clist = a.clist + mb;
         int32_t *clist_next = a.clist2 + mb;
         int32_t *plist = a.plist + mb;
-        int32_t *blist = a.blist + mb;
         const int32_t *mem = a.members + mb;
-        unsigned long long *wr = a.wr + mb;
+        const FdMember *info = a.info + mb;
+        const int rb = fp_rank_bits(ni);
         for (int r = threadIdx.x; r < ni; r += blockDim.x) {
             fsup[r] = a.init[mem[r]];
             alive[r] = 1;
@@ -642,8 +990,6 @@ __global__ void __launch_bounds__(FD_THREADS, 1) k_fd_peel(FdArgs a) {
         int32_t nalive = ni, nfar = ni, ncand = 0;
         unsigned long long level = 0, mn = ~0ull;
         int par = 0;
-        // anchors aggregated per pass of the batched update
-        const int32_t bk = ni <= FD_KEYS / 2 ? min(FD_BATCH, FD_KEYS / ni) : 1;
         __syncthreads();
         while (nalive > 0) {
             if (ncand == 0) {
@@ -726,8 +1072,6 @@ __global__ void __launch_bounds__(FD_THREADS, 1) k_fd_peel(FdArgs a) {
             if (threadIdx.x == 0) {
                 s_np = 0;
                 s_nk[par] = 0;
-                s_nbig = 0;
-                s_nwide = 0;
                 s_peel = 0;
                 s_mn[par] = ~0ull;
             }
@@ -752,23 +1096,13 @@ __global__ void __launch_bounds__(FD_THREADS, 1) k_fd_peel(FdArgs a) {
                     const unsigned long long v = vv[u];
                     const bool keep = r >= 0 && v > mu;
                     const bool peel = r >= 0 && !keep;
-                    unsigned long long w = 0;
                     if (peel) {
                         alive[r] = 0;
                         a.tip[a.new2old[mem[r]]] = mu;
-                        w = wr[r];
                         peeled++;
                     }
-                    // updates: small walks -> one warp each; bigger ones -> the
-                    // batched pass; degree >= 65535 (32-bit counts) or a subset
-                    // too large to batch -> one anchor per pass (end of blist)
-                    const bool upd = peel && v > 0;
-                    const bool small = upd && w <= (unsigned long long)WARP_MAX_W;
-                    const bool single = upd && !small && ((w & WIDE_BIT) || bk == 1);
                     warp_append(keep, r, &s_nk[par], clist_next);
-                    warp_append(small, r, &s_np, plist);
-                    warp_append(upd && !small && !single, r, &s_nbig, blist);
-                    if (single) blist[ni - 1 - atomicAdd(&s_nwide, 1)] = r;
+                    warp_append(peel && v > 0, r, &s_np, plist);
                     // minimum of the survivors before this level's updates
                     const unsigned long long kv = warp_min(keep ? v : ~0ull);
                     if (lane == 0 && kv != ~0ull) atomicMin(&s_mn[par], kv);
@@ -783,82 +1117,228 @@ __global__ void __launch_bounds__(FD_THREADS, 1) k_fd_peel(FdArgs a) {
                 clist = clist_next;
                 clist_next = tmp;
             }
-            int np = s_np;
-            // a level with few updates makes them all in one batched pass
-            // (one pass costs less than a warp phase followed by a pass): the
-            // pass takes blist's nbig0 anchors, then plist's np
-            const int nbig0 = s_nbig;
-            int nmerged = 0;
-            if (bk > 1 && np > 0 && np + nbig0 <= bk) {
-                nmerged = np;
-                np = 0;
-            }
-            // updates of the peeled vertices inside G_i. Phase A: one warp per
-            // peeled vertex whose update walks at most WARP_MAX_W wedges.
+            // updates of the peeled vertices inside G_i
             FdEmit emit{fsup, alive, &s_mn[par], T, clist, &s_nk[par]};
-            for (int pi = warp; pi < np; pi += nwarps) {
+            const int np = fd_lists(a.pool, a.rec + mb, plist, s_np, rb, emit, &s_nbig);
+            for (int pi = 0; pi < np; pi++) {
                 const int32_t r = plist[pi];
-                const int32_t x = mem[r];
-                fd_update_warp(WH, M, a.fd_adj, a.off_s[x], a.off_s[x + 1], r, kb, lane, emit);
-                if (lane == 0) wedges += wr[r];
+                const FdMember m = fd_load(info + r);
+                const int64_t walked = fd_update_cta(H, ch, a.fd_beg, a.fd_len, a.fd_adj, m.q0,
+                                                     m.q0 + m.deg, r, ni, kb, emit);
+                if (threadIdx.x == 0) wedges += (unsigned long long)walked;
             }
             if (np > 0) __syncthreads();
-            const int nbig = nbig0 + nmerged, nwide = s_nwide;
-            // Phase B: bk anchors per pass of the whole CTA over one dense key
-            // space of bk * ni keys
-            for (int p0 = 0; p0 < nbig; p0 += bk) {
-                const int nb = min(bk, nbig - p0);
-                if (warp == 0) {
-                    int32_t deg = 0;
-                    if (lane < nb) {
-                        const int i = p0 + lane;
-                        const int32_t r = i < nbig0 ? blist[i] : plist[i - nbig0];
-                        const int32_t x = mem[r];
-                        const int64_t q0 = a.off_s[x];
-                        deg = (int32_t)(a.off_s[x + 1] - q0);
-                        s_bq0[lane] = q0;
-                        s_bself[lane] = r;
-                    }
-                    int32_t inc = deg;
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-                        if (lane >= o) inc += y;
-                    }
-                    if (lane < nb) s_bpre[lane + 1] = inc;
-                    if (lane == 0) s_bpre[0] = 0;
-                }
-                __syncthreads();
-                H.set_width(nb * ni, false);
-                FdBatchMids BM{a.fd_beg, a.fd_len, s_bq0, s_bpre, nb, s_slot};
-                FdBatchVisit v{&H, s_slot, s_bself, ni, kb};
-                const int64_t walked = cta_walk(BM, 0, s_bpre[nb], a.fd_adj, ch, v);
-                if (threadIdx.x == 0) wedges += (unsigned long long)walked;
-                if (walked > 0) {
-                    FdBatchEmit em{&emit, ni};
-                    H.sweep<true, true>(em);
-                    __syncthreads();
-                    // the next use of the touched-word count is after the next
-                    // pass's set-up barrier (or the level's last barrier)
-                    H.reset_scalars();
-                }
-            }
-            // one anchor at a time: degree >= 65535, or a subset too large
-            // to batch (rank slices)
-            for (int pi = 0; pi < nwide; pi++) {
-                const int32_t r = blist[ni - 1 - pi];
-                const int32_t x = mem[r];
-                const int64_t walked = fd_update_cta(H, ch, a.fd_beg, a.fd_len, a.fd_adj,
-                                                     a.off_s[x], a.off_s[x + 1], r, ni, kb, emit);
-                if (threadIdx.x == 0) wedges += (unsigned long long)walked;
-            }
-            __syncthreads();
             // window survivors plus the members that fell below T
             ncand = s_nk[par];
             mn = s_mn[par];
             par ^= 1;
         }
         __syncthreads();
+        if (threadIdx.x == 0) {
+            unsigned long long t_end;
+            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t_end));
+            a.sub_ns[i] = t_end - t_start;
+            a.sub_levels[i] = levels - levels0;
+        }
+    }
+    if (lane == 0 && wedges) atomicAdd(&a.stats[0], wedges);
+    if (threadIdx.x == 0) atomicAdd(&a.stats[1], levels);
+}
+
+// ------------------------------------------------------------------------
+// Tasks of at most FS_MEMBERS members: their supports live in shared memory.
+//
+// Such a task is a chain of thousands of levels that each peel a member or
+// two, so a level's cost is its dependent steps. With supports, lists and the
+// window in global memory, and walking, a level took 7-14 us (1,268 levels of
+// a 1,552-member task 9.4 ms; 6,861 levels of 9,817 members 94 ms). Here a
+// level is one scan of the supports (peel what is <= mu, minimum of the rest),
+// two dependent loads per member (its record, its list) and two barriers: 1.6
+// us at 1,552 members, 2.4 at 9,817. Peeled members have support FS_DEAD. Of
+// 227 KB, supports and the level's list take 10 bytes a member, the counters
+// for members without a list 64 KB.
+// ------------------------------------------------------------------------
+constexpr int FS_MEMBERS = 15360;
+constexpr int FS_WORDS = 12288;  // dense counters: 24,576 keys
+using FsEngine = DenseSliceT<FS_WORDS, TOUCH_LIST>;
+static_assert(2 * FS_WORDS >= FS_MEMBERS, "one member's keys fit");
+static_assert(FS_MEMBERS <= 1 << 14, "ranks and a mark in 16 bits");
+constexpr unsigned long long FS_DEAD = ~0ull;
+constexpr size_t FS_CHUNK = (chunk_bytes(FD_THREADS) + 15) & ~(size_t)15;
+constexpr size_t FS_SMEM = FS_CHUNK + FsEngine::bytes() + (size_t)FS_MEMBERS * 10;
+
+struct FsEmit {
+    unsigned long long *sup;  // shared
+    unsigned long long mn;    // this thread's least new support
+    __device__ __forceinline__ void operator()(int32_t k, uint32_t c) {
+        if (sup[k] == FS_DEAD) return;
+        const unsigned long long d = choose2(c);
+        const unsigned long long nv = atomicAdd(&sup[k], 0ull - d) - d;
+        mn = nv < mn ? nv : mn;
+    }
+    template <int N>
+    __device__ __forceinline__ void many(const int32_t (&k)[N], const uint32_t (&c)[N]) {
+#pragma unroll
+        for (int u = 0; u < N; u++)
+            if (k[u] >= 0) (*this)(k[u], c[u]);
+    }
+};
+
+// A member alone in a pass of the whole CTA.
+struct FsVisit {
+    FsEngine *eng;
+    int32_t kb, self;  // subset ranks
+    __device__ __forceinline__ void operator()(int, int32_t key) {
+        if (key != self) eng->add(key - kb);
+    }
+};
+
+struct FsArgs {
+    const int32_t *queue;  // task ids, LPT order
+    int32_t T;
+    int32_t *qhead;
+    const int32_t *tstart, *tlen, *tkb;
+    const int32_t *members;
+    const FdMember *info;  // by member position
+    const uint32_t *pool;
+    const unsigned long long *rec;
+    const int64_t *fd_beg;
+    const int32_t *fd_len;
+    const int32_t *fd_adj;
+    const int32_t *new2old;
+    const unsigned long long *init;
+    unsigned long long *rtip;  // by member position
+    unsigned long long *tip;   // output, original ids
+    unsigned long long *stats; // [0] wedges, [1] levels
+    unsigned long long *sub_ns, *sub_levels;
+};
+
+// minimum over a warp, in every lane
+__device__ __forceinline__ unsigned long long warp_min_all(unsigned long long v) {
+    const uint32_t hi = (uint32_t)(v >> 32);
+    const uint32_t mh = __reduce_min_sync(0xffffffffu, hi);
+    const uint32_t ml = __reduce_min_sync(0xffffffffu, hi == mh ? (uint32_t)v : ~0u);
+    return ((unsigned long long)mh << 32) | ml;
+}
+
+__global__ void __launch_bounds__(FD_THREADS, 1) k_fd_small(FsArgs a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int s_t, s_dn, s_nbig;
+    // by level parity: a level's counts, and the warps' minima for the next
+    __shared__ int s_np[2], s_peel[2];
+    __shared__ unsigned long long s_mn[2][FD_WARPS];
+    Chunk ch;
+    ch.beg = (int64_t *)smem;
+    ch.pre = (int32_t *)(ch.beg + FD_THREADS);
+    ch.tmp = ch.pre + FD_THREADS + 1;
+    ch.len = chunk_len_ptr(ch.tmp);
+    FsEngine H;
+    unsigned long long *sup = (unsigned long long *)H.bind(smem + FS_CHUNK, &s_dn);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    H.clear_all();
+    if (threadIdx.x == 0) s_nbig = 0;
+    FdMids M{a.fd_beg, a.fd_len};
+    unsigned long long wedges = 0, levels = 0;  // wedges: per warp (lane 0)
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_t = atomicAdd(a.qhead, 1);
+        __syncthreads();
+        const int t = s_t;
+        if (t >= a.T) break;
+        const int32_t i = a.queue[t];
+        const int32_t mb = a.tstart[i], ni = a.tlen[i], kb = a.tkb[i];
+        const int32_t *mem = a.members + mb;
+        const FdMember *info = a.info + mb;
+        unsigned long long *rtip = a.rtip + mb;
+        unsigned long long t_start = 0;
+        if (threadIdx.x == 0) asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t_start));
+        const int rb = fp_rank_bits(ni);
+        const int32_t nip = (ni + 1) & ~1;
+        uint16_t *plist = (uint16_t *)(sup + nip);
+        unsigned long long mn = FS_DEAD;
+        for (int r = threadIdx.x; r < nip; r += FD_THREADS) {
+            const unsigned long long v = r < ni ? a.init[mem[r]] : FS_DEAD;
+            sup[r] = v;
+            mn = v < mn ? v : mn;
+        }
+        mn = warp_min_all(mn);
+        if (lane == 0) s_mn[0][warp] = mn;
+        if (threadIdx.x == 0) s_np[0] = s_peel[0] = 0;
+        const unsigned long long levels0 = levels;
+        unsigned long long level = 0;
+        int32_t nalive = ni;
+        int par = 0;
+        __syncthreads();
+        while (nalive > 0) {
+            // ---- peel every member with support <= mu; minimum of the others
+            mn = warp_min_all(s_mn[par][lane & (FD_WARPS - 1)]);
+            const unsigned long long mu = mn > level ? mn : level;
+            level = mu;
+            levels++;
+            FsEmit emit{sup, FS_DEAD};
+            int peeled = 0;
+            for (int base = 0; base < nip; base += 4 * FD_THREADS) {
+                unsigned long long v[4];
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    const int r = base + 2 * (h * FD_THREADS + threadIdx.x);
+                    const ulonglong2 x = r < nip ? *(const ulonglong2 *)(sup + r)
+                                                 : make_ulonglong2(FS_DEAD, FS_DEAD);
+                    v[2 * h] = x.x;
+                    v[2 * h + 1] = x.y;
+                }
+                bool any = false;
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    any |= v[u] <= mu;
+                    emit.mn = v[u] > mu && v[u] < emit.mn ? v[u] : emit.mn;
+                }
+                if (!__any_sync(0xffffffffu, any)) continue;
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    const int r = base + 2 * ((u >> 1) * FD_THREADS + threadIdx.x) + (u & 1);
+                    const bool peel = v[u] <= mu;
+                    if (peel) {
+                        sup[r] = FS_DEAD;
+                        rtip[r] = mu;
+                        peeled++;
+                    }
+                    const bool upd = peel && v[u] > 0;
+                    const unsigned bal = __ballot_sync(0xffffffffu, upd);
+                    if (bal) {
+                        int pos = 0;
+                        if (lane == 0) pos = atomicAdd(&s_np[par], __popc(bal));
+                        pos = __shfl_sync(0xffffffffu, pos, 0) + __popc(bal & lanemask_lt());
+                        if (upd) plist[pos] = (uint16_t)r;
+                    }
+                }
+            }
+            peeled = __reduce_add_sync(0xffffffffu, peeled);
+            if (lane == 0 && peeled) atomicAdd(&s_peel[par], peeled);
+            __syncthreads();
+            nalive -= s_peel[par];
+            if (threadIdx.x == 0) s_np[par ^ 1] = s_peel[par ^ 1] = 0;
+            // ---- updates of the peeled members inside G_i
+            const int np = fd_lists(a.pool, a.rec + mb, plist, s_np[par], rb, emit, &s_nbig);
+            if (np > 0) {
+                for (int pi = 0; pi < np; pi++) {
+                    const int32_t r = plist[pi];
+                    const FdMember m = fd_load(info + r);
+                    H.set_width(ni, m.deg >= 65535);
+                    FsVisit v{&H, kb, r + kb};
+                    const int64_t walked = cta_walk(M, m.q0, m.q0 + m.deg, a.fd_adj, ch, v);
+                    if (walked > 0) H.template sweep<true, true>(emit);
+                    __syncthreads();
+                    H.reset_scalars();
+                    if (threadIdx.x == 0) wedges += (unsigned long long)walked;
+                }
+            }
+            mn = warp_min_all(emit.mn);
+            if (lane == 0) s_mn[par ^ 1][warp] = mn;
+            par ^= 1;
+            __syncthreads();
+        }
+        for (int r = threadIdx.x; r < ni; r += FD_THREADS) a.tip[a.new2old[mem[r]]] = rtip[r];
         if (threadIdx.x == 0) {
             unsigned long long t_end;
             asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t_end));
@@ -1262,8 +1742,11 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
     DevBuf<int32_t> fd_adj(m, s), fd_len(m, s);
     DevBuf<int64_t> fd_beg(m, s), wpre;
     DevBuf<unsigned long long> wr(n, s);
+    DevBuf<FdMember> info(n, s);
+    DevBuf<int32_t> wide(P, s);
     DevBuf<unsigned long long> wsub(P, s);
     wsub.zero();
+    wide.zero();
     if (m > 0) {
         DevBuf<uint64_t> key(m, s);
         DevBuf<uint32_t> perm(m, s);
@@ -1297,14 +1780,18 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
         RC_CUDA(cudaMemsetAsync(l64.get() + m, 0, sizeof(int64_t), s));
         scan_exclusive<int64_t>(l64.get(), wpre.get(), m + 1, s);
         k_fd_walk_sizes<<<ceil_div(n, 256), 256, 0, s>>>(S.off, n, wpre.get(), D.sub, mstart.get(),
-                                                         rank.get(), wr.get());
+                                                         rank.get(), wr.get(), info.get(),
+                                                         wide.get());
         RC_LAUNCH();
     } else {
         wr.zero();
+        info.zero();
     }
     // subset sizes and wedge counts
     std::vector<int32_t> hms(P + 1);
     std::vector<unsigned long long> hw(P);
+    std::vector<int32_t> hwide(P);
+    RC_CUDA(cudaMemcpyAsync(hwide.data(), wide.get(), sizeof(int32_t) * P, cudaMemcpyDeviceToHost, s));
     RC_CUDA(cudaMemcpyAsync(hms.data(), mstart.get(), sizeof(int32_t) * (P + 1),
                             cudaMemcpyDeviceToHost, s));
     RC_CUDA(cudaMemcpyAsync(hw.data(), wsub.get(), 8 * P, cudaMemcpyDeviceToHost, s));
@@ -1354,27 +1841,34 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
     }
     const int T = (int)tstart.size();
     // task weights: walk sizes summed over the task's members (LPT key)
-    std::vector<unsigned long long> tw(T);
+    std::vector<unsigned long long> tw(T), tlw(T);  // tlw: of members without a list
+    DevBuf<int64_t> cw;  // prefix of the members' costs, by member position
     DevBuf<int32_t> d_tstart(T > 0 ? T : 1, s), d_tlen(T > 0 ? T : 1, s), d_tkb(T > 0 ? T : 1, s);
     if (T > 0) {
         RC_CUDA(cudaMemcpyAsync(d_tstart.get(), tstart.data(), 4 * (size_t)T, cudaMemcpyHostToDevice, s));
         RC_CUDA(cudaMemcpyAsync(d_tlen.get(), tlen.data(), 4 * (size_t)T, cudaMemcpyHostToDevice, s));
         RC_CUDA(cudaMemcpyAsync(d_tkb.get(), tkb.data(), 4 * (size_t)T, cudaMemcpyHostToDevice, s));
-        DevBuf<int64_t> w64(n + 1, s), cw(n + 1, s);
+        DevBuf<int64_t> w64(n + 1, s);
+        cw.alloc(n + 1, s);
         DevBuf<unsigned long long> dtw(T, s);
-        k_walk_plain<<<ceil_div(n, 256), 256, 0, s>>>(wr.get(), n, w64.get());
+        k_walk_cost<<<ceil_div(n, 256), 256, 0, s>>>(wr.get(), n, FP_MEMBER_COST, w64.get());
         RC_LAUNCH();
         RC_CUDA(cudaMemsetAsync(w64.get() + n, 0, 8, s));
         scan_exclusive<int64_t>(w64.get(), cw.get(), n + 1, s);
-        k_task_weights<<<ceil_div(T, 256), 256, 0, s>>>(d_tstart.get(), d_tlen.get(), cw.get(), T,
-                                                        dtw.get());
+        k_task_weights<<<ceil_div(T, 256), 256, 0, s>>>(d_tstart.get(), d_tlen.get(), cw.get(),
+                                                        FP_MEMBER_COST, T, dtw.get());
+        RC_LAUNCH();
+        DevBuf<unsigned long long> dlw(T, s);
+        dlw.zero();
+        k_listless<<<ceil_div(n, 256), 256, 0, s>>>(info.get(), n, d_tstart.get(), d_tlen.get(), T,
+                                                    *std::max_element(tlen.begin(), tlen.end()),
+                                                    dlw.get());
         RC_LAUNCH();
         RC_CUDA(cudaMemcpyAsync(tw.data(), dtw.get(), 8 * (size_t)T, cudaMemcpyDeviceToHost, s));
+        RC_CUDA(cudaMemcpyAsync(tlw.data(), dlw.get(), 8 * (size_t)T, cudaMemcpyDeviceToHost, s));
         RC_CUDA(cudaStreamSynchronize(s));
     }
-    // LPT order (ties by task id). A task's time is its walks plus its
-    // levels, each level a chain of dependent steps inside one CTA; levels
-    // are at most its members, so a member counts as LEVEL_WEDGES wedges.
+    // LPT order (ties by task id), a member counting as LEVEL_WEDGES wedges.
     std::vector<int32_t> hq(T);
     for (int k = 0; k < T; k++) hq[k] = k;
     std::stable_sort(hq.begin(), hq.end(), [&](int32_t x, int32_t y) {
@@ -1382,56 +1876,71 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
         const unsigned long long ky = tw[y] + LEVEL_WEDGES * (unsigned long long)tlen[y];
         return kx > ky;
     });
-    const size_t warp_tables = (size_t)(FD_THREADS / 32) * WARP_SLOTS * 8 + 16;
-    const size_t smem = FdEngine::bytes() + CHUNK_BYTES + warp_tables;
+    const size_t smem = FdEngine::bytes() + CHUNK_BYTES;
     allow_max_smem((const void *)k_fd_peel);
     int occ = 0;
     RC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_fd_peel, FD_THREADS, smem));
     const int sms = num_sms();
     const int grid_all = sms * std::max(occ, 1);
-    // Heavy tasks (peeled first by all CTAs): task weight at least the
-    // threshold. Automatic: HEAVY_SHARE times the total weight divided by
-    // min(CTAs, tasks), and at least HEAVY_MIN_W; with at most half as many
-    // tasks as CTAs (most CTAs would idle) the divisor is the CTA count.
+    // Heavy tasks (peeled first by all CTAs, ~60-110 us a level): those above
+    // the threshold in wedges. Automatic: (a) what the members without a list
+    // walk outweighs the task's levels several times (or its walks do, if its
+    // lists would not fit the pool); (b) tasks of HEAVY_NI members and more
+    // with a range so narrow that few levels peel them: a one-CTA level scans
+    // at ~8 ns a member (1.9M members, width 1, one level: 16 ms, 0.8 heavy;
+    // 132K members, width 1, 28 levels: 27 ms for the step, 29 unless heavy).
+    // With lists nothing else gains: 4,751 levels of 80K members take 36 ms in
+    // one CTA and took 590 heavy, 20,000 levels of 42K members 117 ms.
+    const unsigned long long pool_cap = [&]() {
+        unsigned long long w = 0;
+        for (int k = 0; k < T; k++) w += tw[k];
+        const unsigned long long small = 8ull * (unsigned long long)m;
+        return w / 2 <= small
+                   ? w / 2
+                   : std::min(w / 2, std::max(small, (unsigned long long)available_bytes() / 32));
+    }();
     int nheavy = 0;
     if (D.fd_heavy_w >= 0 && T > 0) {
-        unsigned long long thr = (unsigned long long)D.fd_heavy_w;
-        if (D.fd_heavy_w == 0) {
-            unsigned long long tot = 0;
-            for (int k = 0; k < T; k++) tot += tw[k];
-            const int div = 2 * T <= grid_all ? grid_all : std::min(grid_all, T);
-            thr = std::max<unsigned long long>(HEAVY_MIN_W,
-                                               tot / (unsigned long long)div * HEAVY_SHARE);
-        }
-        // Automatic rule, second part: a task above one CTA's share of the
-        // LPT weight whose walks outweigh its levels several times over (its
-        // one-CTA peel is walk-bound, and split levels spread the walks over
-        // every CTA)
-        unsigned long long share = ~0ull;
-        if (D.fd_heavy_w == 0) {
-            unsigned long long totk = 0;
-            for (int k = 0; k < T; k++) totk += tw[k] + LEVEL_WEDGES * (unsigned long long)tlen[k];
-            share = totk / (unsigned long long)grid_all;
-        }
+        unsigned long long all = 0;
+        for (int k = 0; k < T; k++) all += tw[k];
+        const bool overflow = all / LIST_SHARE > pool_cap;
         std::vector<int32_t> front, back;
         for (int k = 0; k < T; k++) {
             const int32_t t = hq[k];
             const unsigned long long lw = LEVEL_WEDGES * (unsigned long long)tlen[t];
-            const bool walk_bound = tw[t] + lw >= share && tw[t] >= HEAVY_WALK_LEVELS * lw;
-            ((tw[t] >= thr || walk_bound) && tlen[t] > 0 ? front : back).push_back(t);
+            const unsigned long long walk = overflow ? tw[t] : tlw[t];
+            const int sub_i = tsub[t];
+            const uint64_t width = (size_t)sub_i + 1 < D.bounds.size()
+                                       ? D.bounds[sub_i + 1] - D.bounds[sub_i]
+                                       : ~0ull;
+            const bool heavy =
+                D.fd_heavy_w > 0
+                    ? tw[t] >= (unsigned long long)D.fd_heavy_w
+                    : (walk >= HEAVY_MIN_W && walk >= HEAVY_WALK_LEVELS * lw) ||
+                          (tlen[t] >= HEAVY_NI && width <= (uint64_t)(tlen[t] / (HEAVY_NI / 2)));
+            (heavy && tlen[t] > 0 ? front : back).push_back(t);
         }
         nheavy = (int)front.size();
         int pos = 0;
         for (int32_t t : front) hq[pos++] = t;
         for (int32_t t : back) hq[pos++] = t;
     }
+    // Queue: the heavy tasks, then the large ones (k_fd_peel), then those of
+    // at most FS_MEMBERS members (FS_WORDS with 32-bit counts; k_fd_small),
+    // each in LPT order.
+    const int nsmall_at = (int)(std::stable_partition(hq.begin() + nheavy, hq.end(),
+                                                      [&](int32_t t) {
+                                                          return tlen[t] > (hwide[tsub[t]] ? FS_WORDS
+                                                                                          : FS_MEMBERS);
+                                                      }) -
+                                hq.begin());
     DevBuf<int32_t> queue(T > 0 ? T : 1, s);
     if (T > 0)
         RC_CUDA(cudaMemcpyAsync(queue.get(), hq.data(), 4 * (size_t)T, cudaMemcpyHostToDevice, s));
     DevBuf<unsigned long long> fsup(n, s);
     DevBuf<uint8_t> alive(n, s);
     DevBuf<int32_t> alist(n, s), alist2(n, s), clist(n, s), clist2(n, s), plist(n, s), blist(n, s),
-        qhead(1, s);
+        qhead(2, s);
     DevBuf<unsigned long long> stats(2, s), sub_ns(T > 0 ? T : 1, s), sub_lv(T > 0 ? T : 1, s);
     qhead.zero();
     stats.zero();
@@ -1526,18 +2035,88 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
         }
         RC_CUDA(cudaMemcpyAsync(qhead.get(), &nheavy, 4, cudaMemcpyHostToDevice, s));
     }
+    // the members' lists: walks in items of equal cost, 8 a CTA. The pool has
+    // an entry per two wedges (no list is longer), up to 8 an edge or an eighth
+    // of the memory there is, and each warp's last block.
+    DevBuf<uint32_t> pool;
+    DevBuf<unsigned long long> rec;
     if (nheavy < T) {
-        const int grid = std::max(1, std::min(grid_all, T - nheavy));
-        FdArgs a{queue.get(),   T,           qhead.get(),     d_tstart.get(), d_tlen.get(),
-                 d_tkb.get(),   members.get(),
-                 S.off,         fd_beg.get(), fd_len.get(),   fd_adj.get(), S.new2old,
+        unsigned long long wtot = 0;
+        for (int k = nheavy; k < T; k++) wtot += tw[hq[k]];
+        allow_max_smem((const void *)k_fd_pairs);
+        const int ctas = 2 * sms;
+        const unsigned long long cap =
+            std::min(pool_cap, wtot / 2) + (unsigned long long)ctas * FP_WARPS * FP_BLOCK;
+        pool.alloc((size_t)cap, s);
+        rec.alloc(n, s);
+        RC_CUDA(cudaMemsetAsync(rec.get(), 0xff, 8 * (size_t)n, s));
+        DevBuf<unsigned long long> head(1, s);
+        DevBuf<int32_t> pq(1, s);
+        head.zero();
+        pq.zero();
+        std::vector<uint8_t> skip(T, 0);
+        for (int k = 0; k < nheavy; k++) skip[hq[k]] = 1;
+        DevBuf<uint8_t> dskip(T, s);
+        RC_CUDA(cudaMemcpyAsync(dskip.get(), skip.data(), T, cudaMemcpyHostToDevice, s));
+        unsigned long long cost = (unsigned long long)n * FP_MEMBER_COST;
+        for (int k = 0; k < T; k++) cost += tw[k];
+        const int64_t Q = std::max<int64_t>(8192, (int64_t)(cost / (8ull * ctas)));
+        const int32_t nitems = (int32_t)(cost / Q + 1);
+        DevBuf<int32_t> items(nitems + 1, s);
+        k_pair_items<<<ceil_div(nitems + 1, 256), 256, 0, s>>>(cw.get(), n, Q, nitems, items.get());
+        RC_LAUNCH();
+        FdPairArgs a{d_tstart.get(), d_tlen.get(), d_tkb.get(), dskip.get(), T, items.get(), nitems,
+                     pq.get(), info.get(), fd_beg.get(), fd_len.get(), fd_adj.get(), pool.get(), cap,
+                     head.get(), rec.get(), stats.get()};
+        k_fd_pairs<<<std::min(ctas, nitems), FP_THREADS, FP_WARPS * FP_WORDS * 4, s>>>(a);
+        RC_LAUNCH();
+    }
+    // large and small tasks side by side
+    DevBuf<unsigned long long> rtip(nsmall_at < T ? n : 1, s);
+    const int nlarge = nsmall_at - nheavy, nsmall = T - nsmall_at;
+    cudaEvent_t fork_ev[2] = {};
+    cudaStream_t ls = s;  // the large tasks' stream
+    struct ForkGuard {
+        cudaEvent_t *e;
+        cudaStream_t &ls;
+        bool joined = true;  // else the buffers wait for the other stream
+        ~ForkGuard() {
+            if (!joined) cudaStreamSynchronize(ls);
+            for (int k = 0; k < 2; k++)
+                if (e[k]) cudaEventDestroy(e[k]);
+        }
+    } fg{fork_ev, ls};
+    if (nlarge > 0 && nsmall > 0) {
+        for (cudaEvent_t &e : fork_ev) RC_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+        ls = tier_stream(0);
+        RC_CUDA(cudaEventRecord(fork_ev[0], s));
+        RC_CUDA(cudaStreamWaitEvent(ls, fork_ev[0], 0));
+        fg.joined = false;
+    }
+    if (nlarge > 0) {
+        const int grid = std::max(1, std::min(grid_all, nlarge));
+        FdArgs a{queue.get(),   nsmall_at,   qhead.get(),     d_tstart.get(), d_tlen.get(),
+                 d_tkb.get(),   members.get(), fd_beg.get(), fd_len.get(),   fd_adj.get(), S.new2old,
                  D.init,        fsup.get(),  alive.get(),     alist.get(),  alist2.get(),
                  clist.get(),   clist2.get(),
-                 plist.get(),   blist.get(),
-                 (unsigned long long *)d_tip, stats.get(),    sub_ns.get(), sub_lv.get(),
-                 wr.get()};
-        k_fd_peel<<<grid, FD_THREADS, smem, s>>>(a);
+                 plist.get(),   info.get(),   pool.get(),      rec.get(),
+                 (unsigned long long *)d_tip, stats.get(),    sub_ns.get(), sub_lv.get()};
+        k_fd_peel<<<grid, FD_THREADS, smem, ls>>>(a);
         RC_LAUNCH();
+    }
+    if (nsmall > 0) {
+        allow_max_smem((const void *)k_fd_small);
+        FsArgs a{queue.get() + nsmall_at, nsmall, qhead.get() + 1, d_tstart.get(), d_tlen.get(),
+                 d_tkb.get(), members.get(), info.get(), pool.get(), rec.get(), fd_beg.get(),
+                 fd_len.get(), fd_adj.get(), S.new2old, D.init, rtip.get(), (unsigned long long *)d_tip, stats.get(),
+                 sub_ns.get(), sub_lv.get()};
+        k_fd_small<<<std::min(sms, nsmall), FD_THREADS, FS_SMEM, s>>>(a);
+        RC_LAUNCH();
+    }
+    if (ls != s) {
+        RC_CUDA(cudaEventRecord(fork_ev[1], ls));
+        RC_CUDA(cudaStreamWaitEvent(s, fork_ev[1], 0));
+        fg.joined = true;
     }
     unsigned long long hs[2] = {0, 0};
     RC_CUDA(cudaMemcpyAsync(hs, stats.get(), sizeof(hs), cudaMemcpyDeviceToHost, s));

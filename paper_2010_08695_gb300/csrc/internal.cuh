@@ -24,6 +24,9 @@ void count_noalloc(const receipt_graph *g, unsigned long long *d_cnt_u,
 // Page-locked host buffer of at least `bytes`, owned by the calling thread
 // and reused across calls (no allocation per call).
 void *pinned_scratch(size_t bytes);
+// Device memory a stream-ordered allocation could get: free, or kept unused by
+// the device's pool.
+size_t available_bytes();
 
 // Non-blocking auxiliary stream of the calling thread on the current device:
 // CUDA graphs are captured on it, and counting runs its second pass on it.

@@ -1,0 +1,81 @@
+"""The fine-grained step's update lists and its two peels: the oracle's tip
+numbers at the edges of what a task, a counter, a table and the list pool hold."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def R():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2010_08695_gb300 as R
+    R.load()
+    return R
+
+
+def _check(R, eu, ev, nu, nv, Ps):
+    want, _ = oracle.bup(eu, ev, nu, nv, 0)
+    g = R.Graph(eu, ev, nu, nv)
+    for P in Ps:
+        t = R.as_u64(g.tip_decompose(0, P=P, fd_heavy_w=-1))
+        assert np.array_equal(t, want), P
+
+
+# supports in shared memory up to 15,360 members, list entries of 14 rank bits
+# up to 16,384; a warp's 1,024 words hold 8,192 4-bit counters; short walks of
+# the largest task take the table
+@pytest.mark.parametrize("n", [1, 2, 31, 1024, 1025, 8192, 8193, 15360, 15361, 16384, 16385, 70000])
+def test_task_edges(R, n):
+    nv = max(2, n // 12)
+    m = min(4 * n, n * nv // 2)
+    eu, ev = synth.er(n, nv, m, seed=n) if n < 100 else \
+        synth.chung_lu(n, nv, m, 2.4, 2.3, seed=n)
+    _check(R, eu, ev, n, nv, (1, 3))
+
+
+# groups of w members that share d keys, so counts reach the degree: 4, 8 and
+# 16 bits, entries of 10 and 18 count bits; a tenth of the members has one key
+# more, shared by all of them
+@pytest.mark.parametrize("extra", [0, 17000])
+@pytest.mark.parametrize("d,w", [(1, 513), (8, 64), (8, 65), (15, 30), (16, 30), (255, 4),
+                                 (256, 4), (600, 3), (1022, 3), (1024, 3)])
+def test_full_counters(R, d, w, extra):
+    groups = 40
+    u = np.arange(groups * w, dtype=np.int32)
+    x = u[::10]
+    y = np.arange(extra, dtype=np.int32)  # members with no butterfly
+    eu = np.concatenate([np.repeat(u, d), x, u.size + y])
+    ev = np.concatenate([np.repeat(u // w, d) * d + np.tile(np.arange(d), u.size),
+                         np.full(x.size, groups * d), groups * d + 1 + y]).astype(np.int32)
+    _check(R, eu.astype(np.int32), ev, u.size + extra, groups * d + 1 + extra, (1, 4))
+
+
+# nearly complete: the lists of 3,200 members (10M entries) do not fit the pool
+def test_lists_beyond_the_pool(R):
+    n, d = 3200, 7
+    u = np.arange(n, dtype=np.int32)
+    deg = 2 + u % (d - 1)
+    eu = np.repeat(u, deg)
+    ev = np.concatenate([(k + np.arange(c)) % d for k, c in zip(u // 640, deg)]).astype(np.int32)
+    _check(R, eu, ev, n, d, (1, 2))
+
+
+# walks of 9,000 wedges and more in a task of 140,000 members: counters of 4 and
+# 8 bits in two and four slices of a CTA's words, over ranks all along the task
+def test_sliced_counters(R):
+    n, hub = 140_000, 9_000
+    rng = np.random.default_rng(3)
+    h = rng.permutation(n)[:hub].astype(np.int64)  # members of key 0
+    trio = 1 + np.arange(hub) // 3                 # a key shared by three of them
+    wide = h[::10]                                 # degree 17 and more
+    own = 1 + hub // 3 + np.arange(wide.size * 15)
+    twin = np.arange(n) // 2 + own[-1] + 1         # pairs with one key: no butterfly
+    eu = np.concatenate([h, h, np.repeat(wide, 15), np.arange(n)]).astype(np.int32)
+    ev = np.concatenate([np.zeros(hub), trio, own, twin]).astype(np.int32)
+    _check(R, eu, ev, n, int(ev.max()) + 1, (1,))
