@@ -127,11 +127,17 @@ namespace receipt {
 // ---------------------------------------------------------------------
 template <typename T>
 void scan_exclusive(const T *d_in, T *d_out, int64_t n, cudaStream_t s);
-// Stable LSD radix sort of keys in [begin_bit, end_bit); vals may be null.
-void radix_sort_pairs(uint64_t *keys, uint32_t *vals, int64_t n, int begin_bit, int end_bit,
-                      cudaStream_t s);
-void radix_sort_pairs64(uint64_t *keys, uint64_t *vals, int64_t n, int begin_bit, int end_bit,
-                        cudaStream_t s);
+// An int32 field of 64-bit keys, written out in key order.
+struct RadixField {
+    int32_t *dst = nullptr;
+    int shift = 0;
+    uint64_t mask = 0;
+};
+// Stable LSD radix sort by the key bits [begin_bit, end_bit), of fewer than
+// 2^32 - 1 keys; the buffer may be exchanged for another. With `out` the field is
+// written too; without want_keys the keys are then left in no useful state.
+void radix_sort(DevBuf<uint64_t> &keys, int64_t n, int begin_bit, int end_bit, cudaStream_t s,
+                RadixField out = RadixField{}, bool want_keys = true);
 
 inline int bits_for(uint64_t maxval) {  // bits needed to hold values 0..maxval
     int b = 0;

@@ -33,102 +33,213 @@ __global__ void k_validate_pack(const int32_t *__restrict__ eu, const int32_t *_
     if ((threadIdx.x & 31) == 0 && nbad) atomicAdd(bad, nbad);
 }
 
-__global__ void k_head_flags(const uint64_t *__restrict__ keys, int64_t m,
-                             uint32_t *__restrict__ flag) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < m) flag[i] = (i == 0 || keys[i] != keys[i - 1]) ? 1u : 0u;
-}
+// Duplicate removal from sorted keys, a tile of DD_TILE keys a block: first the
+// tiles' counts of distinct keys, then the keys to their places and V's
+// degrees (original ids). Every warp owns consecutive keys.
+constexpr int DD_THREADS = 256;
+constexpr int DD_ITEMS = 8;
+constexpr int DD_TILE = DD_THREADS * DD_ITEMS;
 
-// Compacts unique keys and counts degrees of both sides (original ids).
-__global__ void k_compact_degrees(const uint64_t *__restrict__ keys, const uint32_t *__restrict__ flag,
-                                  const uint32_t *__restrict__ pos, int64_t m, int bits_v,
-                                  uint64_t mask_v, uint64_t *__restrict__ ukeys,
-                                  uint32_t *__restrict__ deg_u, uint32_t *__restrict__ deg_v) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < m && flag[i]) {
-        uint64_t k = keys[i];
-        ukeys[pos[i]] = k;
-        atomicAdd(&deg_u[k >> bits_v], 1u);
-        atomicAdd(&deg_v[k & mask_v], 1u);
+__device__ __forceinline__ void dd_load(const uint64_t *__restrict__ keys, int64_t m, int64_t wbase,
+                                        uint64_t (&k)[DD_ITEMS], unsigned (&heads)[DD_ITEMS]) {
+    const int lane = threadIdx.x & 31;
+    uint64_t before = wbase > 0 && wbase < m ? keys[wbase - 1] : ~0ull;
+#pragma unroll
+    for (int j = 0; j < DD_ITEMS; j++) {
+        const int64_t g = wbase + j * 32 + lane;
+        k[j] = g < m ? keys[g] : 0;
+    }
+#pragma unroll
+    for (int j = 0; j < DD_ITEMS; j++) {
+        uint64_t prev = __shfl_up_sync(0xffffffffu, k[j], 1);
+        if (lane == 0) prev = before;
+        before = __shfl_sync(0xffffffffu, k[j], 31);
+        const int64_t g = wbase + j * 32 + lane;
+        heads[j] = __ballot_sync(0xffffffffu, g < m && (g == 0 || k[j] != prev));
     }
 }
 
-// key = (maxdeg - deg) so an ascending stable sort gives descending degree,
-// ties in ascending original id (the input order).
-__global__ void k_degree_keys(const uint32_t *__restrict__ deg, int32_t n, uint32_t maxdeg,
-                              uint64_t *__restrict__ key, uint32_t *__restrict__ id) {
-    int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) {
-        key[i] = (uint64_t)(maxdeg - deg[i]);
-        id[i] = (uint32_t)i;
-    }
+__global__ void k_dedup_count(const uint64_t *__restrict__ keys, int64_t m,
+                              uint32_t *__restrict__ tiles) {
+    __shared__ uint32_t s_n;
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    uint64_t k[DD_ITEMS];
+    unsigned heads[DD_ITEMS];
+    dd_load(keys, m, (int64_t)blockIdx.x * DD_TILE + (threadIdx.x >> 5) * (32 * DD_ITEMS), k, heads);
+    uint32_t c = 0;
+#pragma unroll
+    for (int j = 0; j < DD_ITEMS; j++) c += __popc(heads[j]);
+    if ((threadIdx.x & 31) == 0) atomicAdd(&s_n, c);
+    __syncthreads();
+    if (threadIdx.x == 0) tiles[blockIdx.x] = s_n;
 }
 
-__global__ void k_relabel_maps(const uint32_t *__restrict__ sorted_id, int32_t n,
-                               const uint32_t *__restrict__ deg, int32_t *__restrict__ new2old,
-                               int32_t *__restrict__ old2new, int64_t *__restrict__ deg_new) {
-    int32_t x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x < n) {
-        int32_t o = (int32_t)sorted_id[x];
-        new2old[x] = o;
-        old2new[o] = x;
-        deg_new[x] = deg[o];
+// V's hubs would take most of a plain count's time (degree 50,000 among 10M
+// edges: 0.72 ms, 0.22 so): a block counts the ids it meets first in a shared
+// table of DD_SLOTS, added at its end.
+constexpr int DD_GROUP = 8;  // tiles a block
+constexpr int DD_SLOTS = 2048;
+__global__ void k_dedup_write(const uint64_t *__restrict__ keys, int64_t m,
+                              const uint32_t *__restrict__ tiles, int64_t ntiles, uint64_t mask_v,
+                              uint64_t *__restrict__ ukeys, uint32_t *__restrict__ deg_v) {
+    __shared__ uint32_t s_w[2][DD_THREADS / 32];
+    __shared__ uint32_t s_id[DD_SLOTS], s_cnt[DD_SLOTS];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i = threadIdx.x; i < DD_SLOTS; i += DD_THREADS) {
+        s_id[i] = ~0u;
+        s_cnt[i] = 0;
     }
+    for (int t = 0; t < DD_GROUP; t++) {
+        const int64_t tile = (int64_t)blockIdx.x * DD_GROUP + t;
+        if (tile >= ntiles) break;
+        uint64_t k[DD_ITEMS];
+        unsigned heads[DD_ITEMS];
+        dd_load(keys, m, tile * DD_TILE + warp * (32 * DD_ITEMS), k, heads);
+        uint32_t c = 0;
+#pragma unroll
+        for (int j = 0; j < DD_ITEMS; j++) c += __popc(heads[j]);
+        if (lane == 0) s_w[t & 1][warp] = c;
+        __syncthreads();
+        uint32_t at = tiles[tile];
+        for (int w = 0; w < warp; w++) at += s_w[t & 1][w];
+#pragma unroll
+        for (int j = 0; j < DD_ITEMS; j++) {
+            if (heads[j] >> lane & 1u) {
+                ukeys[at + __popc(heads[j] & lanemask_lt())] = k[j];
+                const uint32_t v = (uint32_t)(k[j] & mask_v);
+                const uint32_t h = (v * 2654435761u) >> 21;
+                uint32_t id = ((volatile uint32_t *)s_id)[h];
+                if (id == ~0u) {
+                    id = atomicCAS(&s_id[h], ~0u, v);
+                    if (id == ~0u) id = v;
+                }
+                if (id == v)
+                    atomicAdd(&s_cnt[h], 1u);
+                else
+                    atomicAdd(&deg_v[v], 1u);
+            }
+            at += __popc(heads[j]);
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < DD_SLOTS; i += DD_THREADS)
+        if (s_cnt[i]) atomicAdd(&deg_v[s_id[i]], s_cnt[i]);
 }
+static_assert(DD_SLOTS == 1 << 11, "hash of 11 bits");
 
-// below[x] = number of other-side vertices ahead of x in the global order.
-// On side U (U wins ties): #{v : deg_v > deg_x}. On side V: #{u : deg_u >= deg_y}.
-// deg_other_new is the other side's degree array in its (descending) order.
-__global__ void k_below(const int64_t *__restrict__ deg_new, int32_t n,
-                        const int64_t *__restrict__ deg_other_new, int32_t n_other, int strict,
-                        int32_t *__restrict__ below) {
-    int32_t x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= n) return;
-    int64_t d = deg_new[x];
-    // first index whose degree is <= d (strict) or < d (non-strict)
-    int32_t lo = 0, hi = n_other;
+// First of the sorted distinct keys of every u (nu + 1 entries).
+__global__ void k_u_starts(const uint64_t *__restrict__ ukeys, const uint32_t *__restrict__ mu,
+                           int32_t nu, int bits_v, uint32_t *__restrict__ ustart) {
+    const int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (u > nu) return;
+    uint32_t lo = 0, hi = *mu;
+    const uint64_t want = (uint64_t)u << bits_v;
     while (lo < hi) {
-        int32_t mid = (lo + hi) >> 1;
-        bool ahead = strict ? (deg_other_new[mid] > d) : (deg_other_new[mid] >= d);
+        const uint32_t mid = lo + (hi - lo) / 2;
+        if (ukeys[mid] < want)
+            lo = mid + 1;
+        else
+            hi = mid;
+    }
+    ustart[u] = lo;
+}
+
+// Degrees of U from the starts, and both sides' largest degrees (block
+// maxima): mx[0] U, mx[1] V.
+__global__ void k_degrees(const uint32_t *__restrict__ ustart, int32_t nu, int32_t nv,
+                          uint32_t *__restrict__ deg, unsigned *__restrict__ mx) {
+    unsigned a = 0, b = 0;
+    const int64_t n = (int64_t)nu + nv, stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+        if (i < nu) {
+            const uint32_t d = ustart[i + 1] - ustart[i];
+            deg[i] = d;
+            a = max(a, d);
+        } else {
+            b = max(b, deg[i]);
+        }
+    }
+    a = __reduce_max_sync(0xffffffffu, a);
+    b = __reduce_max_sync(0xffffffffu, b);
+    if ((threadIdx.x & 31) == 0) {
+        if (a) atomicMax(&mx[0], a);
+        if (b) atomicMax(&mx[1], b);
+    }
+}
+
+// Sort keys of both sides' vertices: side, then maxdeg - deg, so that an
+// ascending stable sort gives descending degrees, ties in ascending original
+// id (the input order, in the low 32 bits).
+__global__ void k_degree_keys(const uint32_t *__restrict__ deg, int32_t nu, int32_t nv,
+                              uint32_t maxdeg, int db, uint64_t *__restrict__ key) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (int64_t)nu + nv) return;
+    const uint64_t side = i >= nu;
+    key[i] = (((side << db) | (uint64_t)(maxdeg - deg[i])) << 32) | (uint32_t)(side ? i - nu : i);
+}
+
+__global__ void k_relabel_maps(const uint64_t *__restrict__ key, int32_t nu, int32_t nv,
+                               const uint32_t *__restrict__ deg, int32_t *__restrict__ new2old_u,
+                               int32_t *__restrict__ new2old_v, int32_t *__restrict__ old2new,
+                               int64_t *__restrict__ deg_new) {
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= (int64_t)nu + nv) return;
+    const int32_t o = (int32_t)(uint32_t)key[p];
+    const int64_t base = p < nu ? 0 : nu;
+    (p < nu ? new2old_u : new2old_v)[p - base] = o;
+    old2new[base + o] = (int32_t)(p - base);
+    deg_new[p] = deg[base + o];
+}
+
+// Offsets of both sides from the scanned degrees, and below[x] = number of
+// other-side vertices ahead of x in the global order. On side U (U wins ties):
+// #{v : deg_v > deg_x}. On side V: #{u : deg_u >= deg_y}. The degrees are in
+// descending order on each side.
+__global__ void k_offsets_below(const int64_t *__restrict__ deg_new, const int64_t *__restrict__ pre,
+                                int32_t nu, int32_t nv, int64_t m, int64_t *__restrict__ off_u,
+                                int64_t *__restrict__ off_v, int32_t *__restrict__ below_u,
+                                int32_t *__restrict__ below_v) {
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p == 0) {
+        off_u[nu] = m;
+        off_v[nv] = m;
+    }
+    if (p >= (int64_t)nu + nv) return;
+    const bool u = p < nu;
+    const int64_t d = deg_new[p];
+    const int64_t *other = u ? deg_new + nu : deg_new;
+    // first index whose degree is <= d (U) or < d (V)
+    int32_t lo = 0, hi = u ? nv : nu;
+    while (lo < hi) {
+        const int32_t mid = lo + (hi - lo) / 2;
+        const bool ahead = u ? other[mid] > d : other[mid] >= d;
         if (ahead)
             lo = mid + 1;
         else
             hi = mid;
     }
-    below[x] = lo;
-}
-
-// Relabelled keys for both sides' CSR sorts.
-__global__ void k_relabel_edges(const uint64_t *__restrict__ ukeys, int64_t m, int bits_v,
-                                uint64_t mask_v, const int32_t *__restrict__ o2n_u,
-                                const int32_t *__restrict__ o2n_v, int bu, int bv,
-                                uint64_t *__restrict__ key_u, uint64_t *__restrict__ key_v) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < m) {
-        uint64_t k = ukeys[i];
-        uint64_t u = (uint64_t)o2n_u[k >> bits_v];
-        uint64_t v = (uint64_t)o2n_v[k & mask_v];
-        key_u[i] = (u << bv) | v;
-        key_v[i] = (v << bu) | u;
+    if (u) {
+        off_u[p] = pre[p];
+        below_u[p] = lo;
+    } else {
+        off_v[p - nu] = pre[p] - m;
+        below_v[p - nu] = lo;
     }
 }
 
-__global__ void k_low_bits(const uint64_t *__restrict__ key, int64_t m, uint64_t mask,
-                           int32_t *__restrict__ adj) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < m) adj[i] = (int32_t)(key[i] & mask);
-}
-
-__global__ void k_set_last(int64_t *off, int32_t n, int64_t m) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) off[n] = m;
-}
-
-__global__ void k_u32_max(const uint32_t *__restrict__ a, int32_t n, unsigned *out) {
-    unsigned mx = 0;
-    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        mx = max(mx, a[i]);
-    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if ((threadIdx.x & 31) == 0 && mx) atomicMax(out, mx);
+// Relabelled edges grouped by U's new labels: a vertex's edges move as one
+// block to its new place. key = v << bu | u.
+__global__ void k_relabel_edges(const uint64_t *__restrict__ ukeys, int64_t m, int bits_v,
+                                uint64_t mask_v, const uint32_t *__restrict__ ustart,
+                                const int32_t *__restrict__ o2n_u, const int32_t *__restrict__ o2n_v,
+                                const int64_t *__restrict__ off_u, int bu, uint64_t *__restrict__ key) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= m) return;
+    const uint64_t k = ukeys[i];
+    const int64_t uo = (int64_t)(k >> bits_v);
+    const int32_t u = o2n_u[uo], v = o2n_v[k & mask_v];
+    key[off_u[u] + (i - ustart[uo])] = ((uint64_t)v << bu) | (uint64_t)u;
 }
 
 inline unsigned blocks_for(int64_t n, int t = 256) { return (unsigned)((n + t - 1) / t); }
@@ -156,48 +267,41 @@ receipt_graph *build_graph(const int32_t *d_eu, const int32_t *d_ev, int64_t m, 
             d_eu, d_ev, m, nu, nv, bv, keys.get(), scal.get());
         RC_LAUNCH();
     }
-    radix_sort_pairs(keys.get(), nullptr, m, 0, bu + bv, s);
-    DevBuf<uint32_t> flag(m, s), pos(m + 1, s);
+    radix_sort(keys, m, 0, bu + bv, s);
+    const int64_t tiles = (m + DD_TILE - 1) / DD_TILE;
+    DevBuf<uint32_t> tile_at(tiles + 1, s);  // distinct keys of the tiles before
     DevBuf<uint64_t> ukeys(m, s);
-    DevBuf<uint32_t> deg_u(nu, s), deg_v(nv, s);
-    deg_u.zero();
-    deg_v.zero();
+    DevBuf<uint32_t> ustart((int64_t)nu + 1, s), deg((int64_t)nu + nv, s);  // deg: U, then V
+    deg.zero();
+    tile_at.zero();
     if (m > 0) {
-        k_head_flags<<<blocks_for(m), 256, 0, s>>>(keys.get(), m, flag.get());
+        k_dedup_count<<<(unsigned)tiles, DD_THREADS, 0, s>>>(keys.get(), m, tile_at.get());
         RC_LAUNCH();
-        scan_exclusive<uint32_t>(flag.get(), pos.get(), m, s);
-        k_compact_degrees<<<blocks_for(m), 256, 0, s>>>(keys.get(), flag.get(), pos.get(), m, bv,
-                                                        mask_v, ukeys.get(), deg_u.get(),
-                                                        deg_v.get());
+        scan_exclusive<uint32_t>(tile_at.get(), tile_at.get(), tiles + 1, s);
+        k_dedup_write<<<(unsigned)((tiles + DD_GROUP - 1) / DD_GROUP), DD_THREADS, 0, s>>>(
+            keys.get(), m, tile_at.get(), tiles, mask_v, ukeys.get(), deg.get() + nu);
         RC_LAUNCH();
     }
-    keys.release();
-    // number of unique edges = pos[m-1] + flag[m-1]; read together with the checks
+    // number of unique edges, read together with the checks
     unsigned long long h[4] = {0, 0, 0, 0};
-    uint32_t last_pos = 0, last_flag = 0;
+    uint32_t distinct = 0;
     unsigned *dmax = reinterpret_cast<unsigned *>(scal.get() + 1);
-    if (nu > 0) {
-        k_u32_max<<<std::min<unsigned>(blocks_for(nu), 1024), 256, 0, s>>>(deg_u.get(), nu, dmax);
-        RC_LAUNCH();
-    }
-    if (nv > 0) {
-        k_u32_max<<<std::min<unsigned>(blocks_for(nv), 1024), 256, 0, s>>>(deg_v.get(), nv,
-                                                                          dmax + 2);
+    k_u_starts<<<blocks_for((int64_t)nu + 1), 256, 0, s>>>(ukeys.get(), tile_at.get() + tiles, nu, bv,
+                                                          ustart.get());
+    RC_LAUNCH();
+    if (nu + (int64_t)nv > 0) {
+        k_degrees<<<std::min<unsigned>(blocks_for((int64_t)nu + nv), 1024), 256, 0, s>>>(
+            ustart.get(), nu, nv, deg.get(), dmax);
         RC_LAUNCH();
     }
     RC_CUDA(cudaMemcpyAsync(h, scal.get(), sizeof(h), cudaMemcpyDeviceToHost, s));
-    if (m > 0) {
-        RC_CUDA(cudaMemcpyAsync(&last_pos, pos.get() + (m - 1), 4, cudaMemcpyDeviceToHost, s));
-        RC_CUDA(cudaMemcpyAsync(&last_flag, flag.get() + (m - 1), 4, cudaMemcpyDeviceToHost, s));
-    }
+    RC_CUDA(cudaMemcpyAsync(&distinct, tile_at.get() + tiles, 4, cudaMemcpyDeviceToHost, s));
     RC_CUDA(cudaStreamSynchronize(s));
     if (h[0]) fail(RECEIPT_ERR_INVALID, std::to_string(h[0]) + " edge ids out of range");
-    const int64_t mu = m > 0 ? (int64_t)last_pos + last_flag : 0;
+    const int64_t mu = distinct;
     if (!dedup && mu != m) fail(RECEIPT_ERR_INVALID, "duplicate edges with dedup == 0");
     const uint32_t maxdeg_u = (uint32_t)(h[1] & 0xffffffffu);
-    const uint32_t maxdeg_v = (uint32_t)(h[2] & 0xffffffffu);
-    flag.release();
-    pos.release();
+    const uint32_t maxdeg_v = (uint32_t)(h[1] >> 32);
 
     // one allocation for every array the graph keeps
     auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
@@ -239,54 +343,36 @@ receipt_graph *build_graph(const int32_t *d_eu, const int32_t *d_ev, int64_t m, 
     g->max_deg[1] = (int32_t)maxdeg_v;
 
     try {
-        // relabel each side: stable sort by (maxdeg - deg)
-        DevBuf<int32_t> o2n_u(nu, s), o2n_v(nv, s);
-        DevBuf<int64_t> dn_u(nu + 1, s), dn_v(nv + 1, s);
-        for (int sd = 0; sd < 2; sd++) {
-            int32_t n = sd ? nv : nu;
-            if (n == 0) continue;
-            uint32_t mx = sd ? maxdeg_v : maxdeg_u;
-            DevBuf<uint64_t> dk(n, s);
-            DevBuf<uint32_t> id(n, s);
-            k_degree_keys<<<blocks_for(n), 256, 0, s>>>(sd ? deg_v.get() : deg_u.get(), n, mx,
-                                                        dk.get(), id.get());
+        // relabel both sides: one stable sort by (side, maxdeg - deg)
+        const int64_t nn = (int64_t)nu + nv;
+        DevBuf<int32_t> o2n(nn, s);
+        DevBuf<int64_t> dn(nn, s), pre(nn, s);
+        if (nn > 0) {
+            const uint32_t mx = std::max(maxdeg_u, maxdeg_v);
+            const int db = bits_for(mx);
+            DevBuf<uint64_t> dk(nn, s);
+            k_degree_keys<<<blocks_for(nn), 256, 0, s>>>(deg.get(), nu, nv, mx, db, dk.get());
             RC_LAUNCH();
-            radix_sort_pairs(dk.get(), id.get(), n, 0, bits_for(mx), s);
-            k_relabel_maps<<<blocks_for(n), 256, 0, s>>>(
-                id.get(), n, sd ? deg_v.get() : deg_u.get(), sd ? SV.new2old : SU.new2old,
-                sd ? o2n_v.get() : o2n_u.get(), sd ? dn_v.get() : dn_u.get());
+            // the sides are in order already
+            radix_sort(dk, nn, 32, 32 + db + (nu > 0 && nv > 0), s);
+            k_relabel_maps<<<blocks_for(nn), 256, 0, s>>>(dk.get(), nu, nv, deg.get(), SU.new2old,
+                                                          SV.new2old, o2n.get(), dn.get());
             RC_LAUNCH();
+            scan_exclusive<int64_t>(dn.get(), pre.get(), nn, s);
         }
-        if (nu > 0) {
-            k_below<<<blocks_for(nu), 256, 0, s>>>(dn_u.get(), nu, dn_v.get(), nv, 1, SU.below);
-            RC_LAUNCH();
-        }
-        if (nv > 0) {
-            k_below<<<blocks_for(nv), 256, 0, s>>>(dn_v.get(), nv, dn_u.get(), nu, 0, SV.below);
-            RC_LAUNCH();
-        }
-        // offsets from the relabelled degree arrays
-        if (nu > 0) scan_exclusive<int64_t>(dn_u.get(), SU.off, nu, s);
-        if (nv > 0) scan_exclusive<int64_t>(dn_v.get(), SV.off, nv, s);
-        k_set_last<<<1, 32, 0, s>>>(SU.off, nu, mu);
-        k_set_last<<<1, 32, 0, s>>>(SV.off, nv, mu);
+        k_offsets_below<<<blocks_for(std::max<int64_t>(nn, 1)), 256, 0, s>>>(
+            dn.get(), pre.get(), nu, nv, mu, SU.off, SV.off, SU.below, SV.below);
         RC_LAUNCH();
-        deg_u.release();
-        deg_v.release();
         if (mu > 0) {
-            DevBuf<uint64_t> ku(mu, s), kv(mu, s);
-            k_relabel_edges<<<blocks_for(mu), 256, 0, s>>>(ukeys.get(), mu, bv, mask_v,
-                                                           o2n_u.get(), o2n_v.get(), bu, bv,
-                                                           ku.get(), kv.get());
+            // Grouped by u, a stable sort by v gives V's lists; those, stably
+            // sorted by u, give U's.
+            k_relabel_edges<<<blocks_for(mu), 256, 0, s>>>(ukeys.get(), mu, bv, mask_v, ustart.get(),
+                                                           o2n.get(), o2n.get() + nu, SU.off, bu,
+                                                           keys.get());
             RC_LAUNCH();
             ukeys.release();
-            radix_sort_pairs(ku.get(), nullptr, mu, 0, bu + bv, s);
-            k_low_bits<<<blocks_for(mu), 256, 0, s>>>(ku.get(), mu, mask_v, SU.adj);
-            RC_LAUNCH();
-            ku.release();
-            radix_sort_pairs(kv.get(), nullptr, mu, 0, bu + bv, s);
-            k_low_bits<<<blocks_for(mu), 256, 0, s>>>(kv.get(), mu, mask_u, SV.adj);
-            RC_LAUNCH();
+            radix_sort(keys, mu, bu, bu + bv, s, RadixField{SV.adj, 0, mask_u});
+            radix_sort(keys, mu, 0, bu, s, RadixField{SU.adj, bu, mask_v}, false);
         }
         RC_CUDA(cudaStreamSynchronize(s));
     } catch (...) {

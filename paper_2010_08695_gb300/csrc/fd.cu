@@ -62,35 +62,44 @@ constexpr int32_t TASK_MIN = 8192;
 // tasks of as many members apart.
 constexpr unsigned long long LEVEL_WEDGES = 1ull << 15;
 
-__global__ void k_sub_keys(const int32_t *__restrict__ sub, int32_t n, uint64_t *__restrict__ key,
-                           uint32_t *__restrict__ val, int32_t *__restrict__ cnt) {
+// Sort keys: subset in the high word, vertex (or edge) in the low one.
+__global__ void k_sub_keys(const int32_t *__restrict__ sub, int32_t n, uint64_t *__restrict__ key) {
     int32_t x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x < n) {
-        key[x] = (uint64_t)sub[x];
-        val[x] = (uint32_t)x;
-        atomicAdd(&cnt[sub[x]], 1);
-    }
+    if (x < n) key[x] = ((uint64_t)(uint32_t)sub[x] << 32) | (uint32_t)x;
 }
 
-__global__ void k_members(const uint32_t *__restrict__ sorted_x, int32_t n,
-                          const int32_t *__restrict__ sub, const int32_t *__restrict__ mstart,
-                          int32_t *__restrict__ members, int32_t *__restrict__ rank) {
+// First member position of every subset (P + 1 entries) in the sorted keys.
+__global__ void k_sub_starts(const uint64_t *__restrict__ key, int32_t n, int32_t P,
+                             int32_t *__restrict__ mstart) {
+    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i > P) return;
+    int32_t lo = 0, hi = n;
+    while (lo < hi) {
+        const int32_t mid = lo + (hi - lo) / 2;
+        if ((int64_t)(key[mid] >> 32) < i)
+            lo = mid + 1;
+        else
+            hi = mid;
+    }
+    mstart[i] = lo;
+}
+
+__global__ void k_members(const uint64_t *__restrict__ key, int32_t n,
+                          const int32_t *__restrict__ mstart, int32_t *__restrict__ members,
+                          int32_t *__restrict__ rank) {
     int32_t p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p < n) {
-        int32_t x = (int32_t)sorted_x[p];
+        const uint64_t k = key[p];
+        const int32_t x = (int32_t)(uint32_t)k;
         members[p] = x;
-        rank[x] = p - mstart[sub[x]];
+        rank[x] = p - mstart[k >> 32];
     }
 }
 
 __global__ void k_edge_sub_keys(const int32_t *__restrict__ adj_o, int64_t m,
-                                const int32_t *__restrict__ sub, uint64_t *__restrict__ key,
-                                uint32_t *__restrict__ val) {
+                                const int32_t *__restrict__ sub, uint64_t *__restrict__ key) {
     int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < m) {
-        key[k] = (uint64_t)sub[adj_o[k]];
-        val[k] = (uint32_t)k;
-    }
+    if (k < m) key[k] = ((uint64_t)(uint32_t)sub[adj_o[k]] << 32) | (uint32_t)k;
 }
 
 __device__ __forceinline__ int32_t owner_of(const int64_t *off, int32_t n, int64_t q) {
@@ -105,27 +114,26 @@ __device__ __forceinline__ int32_t owner_of(const int64_t *off, int32_t n, int64
     return lo;
 }
 
-// For sorted position p: y, sub, rank, and run head flag.
-__global__ void k_fd_fill(const uint32_t *__restrict__ perm, int64_t m, const int32_t *__restrict__ adj_o,
+// For sorted position p: y, rank, and run head flag (the position before is
+// the lane before's, but for a warp's first lane).
+__global__ void k_fd_fill(const uint64_t *__restrict__ key, int64_t m, const int32_t *__restrict__ adj_o,
                           const int64_t *__restrict__ off_o, int32_t n_o,
-                          const int32_t *__restrict__ sub, const int32_t *__restrict__ rank,
-                          int32_t *__restrict__ fd_adj, int32_t *__restrict__ fd_y,
-                          uint32_t *__restrict__ head) {
-    int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+                          const int32_t *__restrict__ rank, int32_t *__restrict__ fd_adj,
+                          int32_t *__restrict__ fd_y, uint32_t *__restrict__ head) {
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint64_t k = p < m ? key[p] : 0;
+    const int32_t y = p < m ? owner_of(off_o, n_o, (int64_t)(uint32_t)k) : 0;
+    int32_t sub = (int32_t)(k >> 32);
+    int32_t y1 = __shfl_up_sync(0xffffffffu, y, 1), sub1 = __shfl_up_sync(0xffffffffu, sub, 1);
     if (p >= m) return;
-    int64_t k = perm[p];
-    int32_t x = adj_o[k];
-    int32_t y = owner_of(off_o, n_o, k);
-    fd_adj[p] = rank[x];
-    fd_y[p] = y;
-    uint32_t h = 1;
-    if (p > 0) {
-        int64_t k2 = perm[p - 1];
-        int32_t x2 = adj_o[k2];
-        int32_t y2 = owner_of(off_o, n_o, k2);
-        h = (sub[x2] != sub[x] || y2 != y) ? 1u : 0u;
+    if ((threadIdx.x & 31) == 0 && p > 0) {
+        const uint64_t k1 = key[p - 1];
+        y1 = owner_of(off_o, n_o, (int64_t)(uint32_t)k1);
+        sub1 = (int32_t)(k1 >> 32);
     }
-    head[p] = h;
+    fd_adj[p] = rank[adj_o[(uint32_t)k]];
+    fd_y[p] = y;
+    head[p] = p == 0 || sub1 != sub || y1 != y ? 1u : 0u;
 }
 
 __global__ void k_run_starts(const uint32_t *__restrict__ head, const uint32_t *__restrict__ hpos,
@@ -134,29 +142,24 @@ __global__ void k_run_starts(const uint32_t *__restrict__ head, const uint32_t *
     if (p < m && head[p]) run_start[hpos[p]] = p;
 }
 
-// Run of every side-s edge (x, y), and each subset's wedge count.
-__global__ void k_fd_edges(const uint32_t *__restrict__ perm, int64_t m,
+// Run of every side-s edge (x, y).
+__global__ void k_fd_edges(const uint64_t *__restrict__ key, int64_t m,
                            const int32_t *__restrict__ adj_o, const int32_t *__restrict__ fd_y,
                            const uint32_t *__restrict__ head, const uint32_t *__restrict__ hpos,
                            const int64_t *__restrict__ run_start, int64_t nruns,
                            const int64_t *__restrict__ off_s, const int32_t *__restrict__ adj_s,
-                           const int32_t *__restrict__ sub, int64_t *__restrict__ fd_beg,
-                           int32_t *__restrict__ fd_len, unsigned long long *__restrict__ wsub) {
+                           int64_t *__restrict__ fd_beg, int32_t *__restrict__ fd_len) {
     int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= m) return;
     int64_t r = (int64_t)hpos[p] + head[p] - 1;  // run id
     int64_t rs = run_start[r];
     int64_t re = r + 1 < nruns ? run_start[r + 1] : m;
-    int32_t x = adj_o[perm[p]];
+    int32_t x = adj_o[(uint32_t)key[p]];
     int32_t y = fd_y[p];
     int64_t b = off_s[x];
     int64_t ps = b + lower_bound_i32(adj_s + b, off_s[x + 1] - b, y);
     fd_beg[ps] = rs;
     fd_len[ps] = (int32_t)(re - rs);
-    if (head[p]) {
-        unsigned long long L = (unsigned long long)(re - rs);
-        if (L > 1) atomicAdd(&wsub[sub[x]], L * (L - 1));
-    }
 }
 
 __global__ void k_i32_to_i64(const int32_t *__restrict__ v, int64_t m, int64_t *__restrict__ out) {
@@ -223,11 +226,27 @@ __global__ void k_flag_positions(const uint32_t *__restrict__ flag, const uint32
     if (p < n && flag[p]) out[pos[p]] = p;
 }
 
-// a member's cost: its wedges and a constant
+// a member's cost: its wedges and a constant; and each subset's wedge count,
+// the sum of L (L - 1) over its runs L (a member's walk counts itself once per
+// edge)
 __global__ void k_walk_cost(const unsigned long long *__restrict__ wr, int32_t n, int64_t add,
-                            int64_t *__restrict__ out) {
+                            const FdMember *__restrict__ info, const int32_t *__restrict__ members,
+                            const int32_t *__restrict__ sub, int64_t *__restrict__ out,
+                            unsigned long long *__restrict__ wsub) {
     const int32_t p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p < n) out[p] = (int64_t)(wr[p] & ~WIDE_BIT) + add;
+    const bool in = p < n;
+    const unsigned long long w = in ? wr[p] & ~WIDE_BIT : 0;
+    const unsigned long long others = in && w ? w - (unsigned)info[p].deg : 0;
+    const int32_t sb = in ? sub[members[p]] : -1;
+    if (in) out[p] = (int64_t)w + add;
+    // members of one subset are together
+    const int32_t s0 = __shfl_sync(0xffffffffu, sb, 0);
+    if (__all_sync(0xffffffffu, sb == s0 || sb < 0)) {
+        const unsigned long long t = warp_sum(others);
+        if ((threadIdx.x & 31) == 0 && t) atomicAdd(&wsub[s0], t);
+    } else if (others) {
+        atomicAdd(&wsub[sb], others);
+    }
 }
 
 __global__ void k_task_weights(const int32_t *__restrict__ tstart, const int32_t *__restrict__ tlen,
@@ -1725,16 +1744,15 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
     const Side &S = *D.S;
     const Side &O = *D.O;
     // members and ranks
-    DevBuf<int32_t> cnt(P + 1, s), mstart(P + 1, s), members(n, s), rank(n, s);
-    cnt.zero();
+    DevBuf<int32_t> mstart(P + 1, s), members(n, s), rank(n, s);
     {
         DevBuf<uint64_t> key(n, s);
-        DevBuf<uint32_t> val(n, s);
-        k_sub_keys<<<ceil_div(n, 256), 256, 0, s>>>(D.sub, n, key.get(), val.get(), cnt.get());
+        k_sub_keys<<<ceil_div(n, 256), 256, 0, s>>>(D.sub, n, key.get());
         RC_LAUNCH();
-        radix_sort_pairs(key.get(), val.get(), n, 0, bits_for((uint64_t)P), s);
-        scan_exclusive<int32_t>(cnt.get(), mstart.get(), P + 1, s);
-        k_members<<<ceil_div(n, 256), 256, 0, s>>>(val.get(), n, D.sub, mstart.get(), members.get(),
+        radix_sort(key, n, 32, 32 + bits_for((uint64_t)P), s);
+        k_sub_starts<<<ceil_div(P + 1, 256), 256, 0, s>>>(key.get(), n, P, mstart.get());
+        RC_LAUNCH();
+        k_members<<<ceil_div(n, 256), 256, 0, s>>>(key.get(), n, mstart.get(), members.get(),
                                                    rank.get());
         RC_LAUNCH();
     }
@@ -1749,15 +1767,13 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
     wide.zero();
     if (m > 0) {
         DevBuf<uint64_t> key(m, s);
-        DevBuf<uint32_t> perm(m, s);
-        k_edge_sub_keys<<<ceil_div(m, 256), 256, 0, s>>>(O.adj, m, D.sub, key.get(), perm.get());
+        k_edge_sub_keys<<<ceil_div(m, 256), 256, 0, s>>>(O.adj, m, D.sub, key.get());
         RC_LAUNCH();
-        radix_sort_pairs(key.get(), perm.get(), m, 0, bits_for((uint64_t)P), s);
-        key.release();
+        radix_sort(key, m, 32, 32 + bits_for((uint64_t)P), s);
         DevBuf<int32_t> fd_y(m, s);
         DevBuf<uint32_t> head(m + 1, s), hpos(m + 1, s);
-        k_fd_fill<<<ceil_div(m, 256), 256, 0, s>>>(perm.get(), m, O.adj, O.off, O.n, D.sub,
-                                                   rank.get(), fd_adj.get(), fd_y.get(), head.get());
+        k_fd_fill<<<ceil_div(m, 256), 256, 0, s>>>(key.get(), m, O.adj, O.off, O.n, rank.get(),
+                                                   fd_adj.get(), fd_y.get(), head.get());
         RC_LAUNCH();
         RC_CUDA(cudaMemsetAsync(head.get() + m, 0, 4, s));
         scan_exclusive<uint32_t>(head.get(), hpos.get(), m + 1, s);
@@ -1767,9 +1783,9 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
         DevBuf<int64_t> run_start(nruns + 1, s);
         k_run_starts<<<ceil_div(m, 256), 256, 0, s>>>(head.get(), hpos.get(), m, run_start.get());
         RC_LAUNCH();
-        k_fd_edges<<<ceil_div(m, 256), 256, 0, s>>>(perm.get(), m, O.adj, fd_y.get(), head.get(),
+        k_fd_edges<<<ceil_div(m, 256), 256, 0, s>>>(key.get(), m, O.adj, fd_y.get(), head.get(),
                                                     hpos.get(), run_start.get(), nruns, S.off, S.adj,
-                                                    D.sub, fd_beg.get(), fd_len.get(), wsub.get());
+                                                    fd_beg.get(), fd_len.get());
         RC_LAUNCH();
         // walk sizes of all vertices: prefix sums of the run lengths (kept
         // for the split levels of heavy tasks)
@@ -1794,7 +1810,6 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
     RC_CUDA(cudaMemcpyAsync(hwide.data(), wide.get(), sizeof(int32_t) * P, cudaMemcpyDeviceToHost, s));
     RC_CUDA(cudaMemcpyAsync(hms.data(), mstart.get(), sizeof(int32_t) * (P + 1),
                             cudaMemcpyDeviceToHost, s));
-    RC_CUDA(cudaMemcpyAsync(hw.data(), wsub.get(), 8 * P, cudaMemcpyDeviceToHost, s));
     // Tasks: a subset, or, in a batch's disjoint union, each packed graph's
     // part of a subset (parts share no butterfly, so each is peeled on its
     // own; consecutive small parts of one subset are merged up to TASK_MIN
@@ -1851,7 +1866,8 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
         DevBuf<int64_t> w64(n + 1, s);
         cw.alloc(n + 1, s);
         DevBuf<unsigned long long> dtw(T, s);
-        k_walk_cost<<<ceil_div(n, 256), 256, 0, s>>>(wr.get(), n, FP_MEMBER_COST, w64.get());
+        k_walk_cost<<<ceil_div(n, 256), 256, 0, s>>>(wr.get(), n, FP_MEMBER_COST, info.get(),
+                                                     members.get(), D.sub, w64.get(), wsub.get());
         RC_LAUNCH();
         RC_CUDA(cudaMemsetAsync(w64.get() + n, 0, 8, s));
         scan_exclusive<int64_t>(w64.get(), cw.get(), n + 1, s);
@@ -1865,6 +1881,7 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
                                                     dlw.get());
         RC_LAUNCH();
         RC_CUDA(cudaMemcpyAsync(tw.data(), dtw.get(), 8 * (size_t)T, cudaMemcpyDeviceToHost, s));
+        RC_CUDA(cudaMemcpyAsync(hw.data(), wsub.get(), 8 * P, cudaMemcpyDeviceToHost, s));
         RC_CUDA(cudaMemcpyAsync(tlw.data(), dlw.get(), 8 * (size_t)T, cudaMemcpyDeviceToHost, s));
         RC_CUDA(cudaStreamSynchronize(s));
     }
