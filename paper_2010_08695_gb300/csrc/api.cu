@@ -228,7 +228,7 @@ struct Timer {
 }  // namespace
 
 void tip_decompose_impl(receipt_graph *g, int side, uint64_t *d_tip, const receipt_options *optp,
-                        cudaStream_t s) {
+                        cudaStream_t s, bool list_bound) {
     if (!g) fail(RECEIPT_ERR_INVALID, "null graph");
     if (side != 0 && side != 1) fail(RECEIPT_ERR_INVALID, "side must be 0 (U) or 1 (V)");
     receipt_options opt;
@@ -257,6 +257,7 @@ void tip_decompose_impl(receipt_graph *g, int side, uint64_t *d_tip, const recei
     D.n = n;
     D.m = g->m;
     D.timing = opt.timing != 0;
+    D.list_bound = list_bound;
     D.max_deg_s = g->max_deg[side];
     D.fd_heavy_w = opt.fd_heavy_w;
     D.fd_huc = opt.fd_huc;
@@ -400,7 +401,8 @@ __global__ void k_split_tips(const unsigned long long *__restrict__ cat, const i
 }  // namespace
 
 void decompose_batch_impl(receipt_graph *const *gs, const receipt_side *sides, int32_t n,
-                          uint64_t *const *d_tips, const receipt_options *opt, cudaStream_t s) {
+                          uint64_t *const *d_tips, const receipt_options *opt, cudaStream_t s,
+                          bool list_bound) {
     if (n < 0 || (n > 0 && (!gs || !sides || !d_tips))) fail(RECEIPT_ERR_INVALID, "bad batch");
     if (n == 0) return;
     std::vector<PackSrc> src(n);
@@ -478,7 +480,7 @@ void decompose_batch_impl(receipt_graph *const *gs, const receipt_side *sides, i
     U.side[0] = Side{(int32_t)NA, offA.get(), adjA.get(), n2oA.get(), belA.get(), nullptr};
     U.side[1] = Side{(int32_t)NB, offB.get(), adjB.get(), n2oB.get(), belB.get(), nullptr};
     DevBuf<unsigned long long> cat(NA, s);
-    tip_decompose_impl(&U, 0, (uint64_t *)cat.get(), opt, s);
+    tip_decompose_impl(&U, 0, (uint64_t *)cat.get(), opt, s, list_bound);
     if (NA > 0) {
         DevBuf<unsigned long long *> outs(n, s);
         RC_CUDA(cudaMemcpyAsync(outs.get(), d_tips, sizeof(void *) * n, cudaMemcpyHostToDevice, s));
@@ -620,9 +622,9 @@ receipt_status receipt_decompose_batch(receipt_graph *const *gs, const receipt_s
     return guarded([&] {
         if (n > 0 && gs && gs[0]) {
             DeviceGuard dg(gs[0]->device);
-            decompose_batch_impl(gs, sides, n, d_tips, opt, (cudaStream_t)stream);
+            decompose_batch_impl(gs, sides, n, d_tips, opt, (cudaStream_t)stream, false);
         } else {
-            decompose_batch_impl(gs, sides, n, d_tips, opt, (cudaStream_t)stream);
+            decompose_batch_impl(gs, sides, n, d_tips, opt, (cudaStream_t)stream, false);
         }
     });
 }

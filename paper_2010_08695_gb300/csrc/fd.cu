@@ -1911,10 +1911,10 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
     const unsigned long long pool_cap = [&]() {
         unsigned long long w = 0;
         for (int k = 0; k < T; k++) w += tw[k];
-        const unsigned long long small = 8ull * (unsigned long long)m;
-        return w / 2 <= small
-                   ? w / 2
-                   : std::min(w / 2, std::max(small, (unsigned long long)available_bytes() / 32));
+        const unsigned long long small = (unsigned long long)(FD_LIST_BYTES / 4 * m);
+        if (w / 2 <= small) return w / 2;
+        if (D.list_bound) return small;
+        return std::min(w / 2, std::max(small, (unsigned long long)available_bytes() / 32));
     }();
     int nheavy = 0;
     if (D.fd_heavy_w >= 0 && T > 0) {
@@ -2053,8 +2053,8 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
         RC_CUDA(cudaMemcpyAsync(qhead.get(), &nheavy, 4, cudaMemcpyHostToDevice, s));
     }
     // the members' lists: walks in items of equal cost, 8 a CTA. The pool has
-    // an entry per two wedges (no list is longer), up to 8 an edge or an eighth
-    // of the memory there is, and each warp's last block.
+    // an entry per two wedges (no list is longer), up to FD_LIST_BYTES an edge
+    // or an eighth of the memory there is, and each warp's last block.
     DevBuf<uint32_t> pool;
     DevBuf<unsigned long long> rec;
     if (nheavy < T) {

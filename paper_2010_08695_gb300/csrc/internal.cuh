@@ -40,9 +40,12 @@ cudaStream_t tier_stream(int k);
 // opt-in shared memory of one CTA (capped at `want`); 0 if none.
 int64_t max_cta_keyspace(int64_t want, size_t extra);
 
-// Full tip decomposition of side `side` of g into d_tip (original ids).
+// Full tip decomposition of side `side` of g into d_tip (original ids). The
+// fine-grained step's update lists take at most FD_LIST_BYTES an edge, or,
+// unless list_bound, an eighth of the device's memory where that is more.
+constexpr int64_t FD_LIST_BYTES = 32;
 void tip_decompose_impl(receipt_graph *g, int side, uint64_t *d_tip, const receipt_options *opt,
-                        cudaStream_t s);
+                        cudaStream_t s, bool list_bound = false);
 
 }  // namespace receipt
 
@@ -56,6 +59,7 @@ struct Decomp {
     int32_t n = 0;
     int64_t m = 0;
     int32_t max_deg_s = 0;                // largest degree on side s
+    bool list_bound = false;              // update lists within FD_LIST_BYTES an edge
     unsigned long long *sup = nullptr;    // raw supports
     unsigned long long *init = nullptr;   // support when the vertex's range began
     int32_t *sub = nullptr;               // subset index, -1 while remaining

@@ -17,7 +17,8 @@
 
 namespace receipt {
 void decompose_batch_impl(receipt_graph *const *gs, const receipt_side *sides, int32_t n,
-                          uint64_t *const *d_tips, const receipt_options *opt, cudaStream_t s);
+                          uint64_t *const *d_tips, const receipt_options *opt, cudaStream_t s,
+                          bool list_bound);
 }
 
 using namespace receipt;
@@ -49,8 +50,9 @@ struct Request {
 // of Sec. 4.1 allocates when the rule picks one (the remaining subgraph's
 // lists, offsets and counts, the counting pass's temporaries and its
 // global-tier counters per CTA, a copy of the other side's lists: the sizes
-// the decomposition itself checks before recounting) and the fine-grained
-// step's global counters of split heavy levels (32 members x the side).
+// the decomposition itself checks before recounting), the fine-grained
+// step's global counters of split heavy levels (32 members x the side) and its
+// update lists (FD_LIST_BYTES an edge, 24 a vertex, a block a warp).
 size_t estimate_bytes(int64_t m, int32_t nu, int32_t nv, int side, int sms) {
     const int64_t ns = side ? nv : nu;
     size_t b = (size_t)160 * (size_t)m + (size_t)400 * (size_t)(nu + nv) + ((size_t)32 << 20);
@@ -59,6 +61,7 @@ size_t estimate_bytes(int64_t m, int32_t nu, int32_t nv, int side, int sms) {
     b += (size_t)40 * (size_t)m + (size_t)48 * (size_t)(nu + nv) + (size_t)8 * (size_t)sms * n_max +
          ((size_t)64 << 20);
     b += (size_t)8 * 32 * (size_t)ns;
+    b += (size_t)FD_LIST_BYTES * (size_t)m + (size_t)24 * (size_t)ns + ((size_t)32 << 20);
     return b;
 }
 
@@ -141,7 +144,7 @@ void receipt_server::run(std::vector<Request *> &batch, cudaStream_t s) {
             tips.emplace_back((size_t)(r->side ? r->nv : r->nu), s);
         }
         if (batch.size() == 1) {
-            tip_decompose_impl(gs[0], batch[0]->side, (uint64_t *)tips[0].get(), &opt, s);
+            tip_decompose_impl(gs[0], batch[0]->side, (uint64_t *)tips[0].get(), &opt, s, true);
         } else {
             std::vector<receipt_side> sides;
             std::vector<uint64_t *> outs;
@@ -149,7 +152,8 @@ void receipt_server::run(std::vector<Request *> &batch, cudaStream_t s) {
                 sides.push_back((receipt_side)batch[i]->side);
                 outs.push_back((uint64_t *)tips[i].get());
             }
-            decompose_batch_impl(gs.data(), sides.data(), (int32_t)gs.size(), outs.data(), &opt, s);
+            decompose_batch_impl(gs.data(), sides.data(), (int32_t)gs.size(), outs.data(), &opt, s,
+                                 true);
         }
         for (size_t i = 0; i < batch.size(); i++) {
             Request *r = batch[i];
