@@ -661,10 +661,13 @@ __global__ void __launch_bounds__(FP_THREADS, 2) k_fd_pairs(FdPairArgs a) {
 }
 
 // The listed updates of one level's np members (list: ranks in the task; rec:
-// the task's records), a group of warps per member: the widest groups that
-// give each of up to 16 members one, a warp per member above. Members without
-// a list are returned in list[0, n). All threads, after a barrier; ends with
-// one.
+// the task's records). Up to 16 members get a group of warps each, the widest
+// groups there are enough of. More members go in blocks of up to 32 to the
+// warps, whose lanes take a block's entries as one list: with a warp a member
+// the short lists of wide levels cost a chain of loads each (uniform graphs of
+// 1M and 5M edges, a few levels: the step took 2.9 and 3.7 ms, 1.3 and 1.8 so).
+// Members without a list are returned in list[0, n). All threads, after a
+// barrier; ends with one.
 constexpr int FD_WARPS = FD_THREADS / 32;
 template <class List, class Emit>
 __device__ __forceinline__ int fd_lists(const uint32_t *__restrict__ pool,
@@ -672,42 +675,73 @@ __device__ __forceinline__ int fd_lists(const uint32_t *__restrict__ pool,
                                         int np, int rb, Emit &emit, int *s_nbig) {
     constexpr uint32_t MARK = 1u << (8 * sizeof(List) - 1);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int g = np >= FD_WARPS ? 1 : np > 0 ? FD_WARPS >> (32 - __clz(np - 1)) : 1;
-    const int grp = warp / g, part = warp & (g - 1);
     const uint32_t rmask = (1u << rb) - 1u;
     bool left = false;
-    // the next member's record is fetched ahead
-    uint32_t rn = grp < np ? (uint32_t)list[grp] & ~MARK : 0u;
-    unsigned long long qn = grp < np ? __ldg(rec + rn) : 0ull;
-    for (int pi = grp; pi < np; pi += FD_WARPS / g) {
-        const uint32_t r = rn;
-        const unsigned long long q = qn;
-        if (pi + FD_WARPS / g < np) {
-            rn = (uint32_t)list[pi + FD_WARPS / g] & ~MARK;
-            qn = __ldg(rec + rn);
-        }
-        if (q == FP_NONE) {
-            if (part == 0 && lane == 0) list[pi] = (List)(r | MARK);
-            left = true;
-            continue;
-        }
-        const uint32_t *e = pool + (q >> 24);
-        const int len = (int)(q & 0xffffffu);
-        for (int j0 = part * 32 + lane; j0 < len; j0 += 128 * g) {
-            uint32_t v[4];
+    auto apply = [&](const uint32_t (&v)[4]) {  // entries, 0: none
+        int32_t k[4];
+        uint32_t c[4];
 #pragma unroll
-            for (int u = 0; u < 4; u++) {
-                const int j = j0 + u * 32 * g;
-                v[u] = j < len ? __ldg(e + j) : 0u;
+        for (int u = 0; u < 4; u++) {
+            c[u] = v[u] >> rb;
+            k[u] = c[u] ? (int32_t)(v[u] & rmask) : -1;
+        }
+        emit.template many<4>(k, c);
+    };
+    if (np <= FD_WARPS) {
+        const int g = np > 0 ? FD_WARPS >> (32 - __clz(np - 1)) : FD_WARPS;
+        const int pi = warp / g, part = warp & (g - 1);
+        if (pi < np) {
+            const uint32_t r = (uint32_t)list[pi] & ~MARK;
+            const unsigned long long q = __ldg(rec + r);
+            const uint32_t *e = pool + (q >> 24);
+            const int len = q == FP_NONE ? 0 : (int)(q & 0xffffffu);
+            if (q == FP_NONE) {
+                if (part == 0 && lane == 0) list[pi] = (List)(r | MARK);
+                left = true;
             }
-            int32_t k[4];
-            uint32_t c[4];
+            for (int j0 = part * 32 + lane; j0 < len; j0 += 128 * g) {
+                uint32_t v[4];
 #pragma unroll
-            for (int u = 0; u < 4; u++) {
-                c[u] = v[u] >> rb;
-                k[u] = c[u] ? (int32_t)(v[u] & rmask) : -1;
+                for (int u = 0; u < 4; u++) {
+                    const int j = j0 + u * 32 * g;
+                    v[u] = j < len ? __ldg(e + j) : 0u;
+                }
+                apply(v);
             }
-            emit.template many<4>(k, c);
+        }
+    } else {
+        const int bs = min(32, (np + FD_WARPS - 1) / FD_WARPS);
+        for (int base = warp * bs; base < np; base += FD_WARPS * bs) {
+            const bool in = lane < bs && base + lane < np;
+            const uint32_t r = in ? (uint32_t)list[base + lane] & ~MARK : 0u;
+            const unsigned long long q = in ? __ldg(rec + r) : 0ull;
+            if (q == FP_NONE) {
+                list[base + lane] = (List)(r | MARK);
+                left = true;
+            }
+            const int len = q == FP_NONE ? 0 : (int)(q & 0xffffffu);
+            int inc = len;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += y;
+            }
+            const int total = __shfl_sync(0xffffffffu, inc, 31), ex = inc - len;
+            for (int j0 = lane; j0 - lane < total; j0 += 128) {
+                uint32_t v[4];
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    const int j = j0 + u * 32;
+                    int lo = 0;  // last lane whose list starts at or before j
+#pragma unroll
+                    for (int step = 16; step > 0; step >>= 1)
+                        if (__shfl_sync(0xffffffffu, ex, lo + step) <= j) lo += step;
+                    const unsigned long long b = __shfl_sync(0xffffffffu, q >> 24, lo);
+                    const int e0 = __shfl_sync(0xffffffffu, ex, lo);
+                    v[u] = j < total ? __ldg(pool + b + (j - e0)) : 0u;
+                }
+                apply(v);
+            }
         }
     }
     if (!__syncthreads_or(left)) return 0;
