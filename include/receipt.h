@@ -115,8 +115,8 @@ typedef struct {
      * 0 (default): device-driven; the rounds of a range run inside one
      * launch: of one cooperative kernel for the whole coarse-grained step
      * when the side's keys fit at most four dense windows (147,456 vertices;
-     * in a batch, every graph's one window) and no degree on it reaches
-     * 65,535; otherwise of a CUDA graph whose while-node repeats the round body until
+     * sixteen, 589,824, where the mean walk is below 8,192 wedges; in a
+     * batch, every graph's one window) and no degree on it reaches 65,535; otherwise of a CUDA graph whose while-node repeats the round body until
      * a round leaves no next activeSet (at most 64 rounds a launch), each
      * round's counters going to a device record that the host reads after
      * the launch; with timing on or the activeSet found by crossings the

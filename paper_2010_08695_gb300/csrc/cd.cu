@@ -1459,14 +1459,17 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s) {
     uint64_t crcnt = 0;  // C_rcnt (rule on) or 0
     if (persist) {
         const int ng = D.parts ? (int)D.parts->size() - 1 : 1;
+        const bool wide = cd_persist_wide(D);
         DevBuf<PersistDev> pd(1, s);
         DevBuf<unsigned long long> ph_w(3 * NBUCKET, s);
         DevBuf<uint32_t> ph_c(3 * NBUCKET, s);
         DevBuf<int32_t> pfirst(ng + 1, s), plast(3 * (size_t)ng, s);
         DevBuf<int32_t> part_of(D.parts ? n : 1, s);
-        DevBuf<PersistAnchor> pLw(n, s);
+        DevBuf<PersistAnchor> pLw(n, s), pLg(wide ? 3 * (size_t)n : 1, s);
         // items: an anchor's whole window, or its windows of DENSE_KEYS keys
-        DevBuf<PersistAnchor> pLd((size_t)n * (D.parts ? 1 : ceil_div(n, DENSE_KEYS)), s);
+        // (wide: of anchors with 1,024 wedges and more)
+        const size_t many = wide ? std::min<size_t>(n, (D.wedges_bup + D.m) / 1024 + 1) : n;
+        DevBuf<PersistAnchor> pLd(many * (D.parts ? 1 : ceil_div(n, DENSE_KEYS)), s);
         constexpr int REC_CAP = 4096;  // rounds per launch
         DevBuf<PersistRound> prec(REC_CAP, s);
         std::vector<int32_t> hfirst(ng + 1, 0);
@@ -1487,16 +1490,16 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s) {
         const PersistArgs pa{n, O.n, D.m, S.off, S.adj, O.off, len_w.get(), adj_w.get(), D.sup,
                              D.init, D.wfull, D.sub, st.get(), pd.get(), ph_w.get(), ph_c.get(),
                              D.parts ? part_of.get() : nullptr, pfirst.get(), plast.get(), ng,
-                             F.get(), pLw.get(), pLd.get(), prec.get(), REC_CAP, P, range_cap,
+                             F.get(), pLw.get(), pLd.get(), pLg.get(), prec.get(), REC_CAP, P, range_cap,
                              warp_max_w, dgm && O.n > 0 ? 1 : 0, dgm_frac, huc == 0 ? 1 : 0,
                              huc_factor, rcost.get()};
-        const int pgrid = cd_persist_grid(D.m);
+        const int pgrid = cd_persist_grid(D.m, wide);
         PersistDev *hpd = (PersistDev *)(hrec + ROUND_BURST * (hdr / 8));
         PersistRound *hrc = (PersistRound *)(hpd + 1);
         std::vector<PersistRound> recs;
         RC_CUDA(cudaMemcpyAsync(hpin, rcost.get(), 8, cudaMemcpyDeviceToHost, s));
         for (;;) {
-            cd_persist_launch(pa, pgrid, s);
+            cd_persist_launch(pa, pgrid, wide, s);
             RC_CUDA(cudaMemcpyAsync(hpd, pd.get(), sizeof(PersistDev), cudaMemcpyDeviceToHost, s));
             RC_CUDA(cudaMemcpyAsync(hrc, prec.get(), PERSIST_FIRST * sizeof(PersistRound),
                                     cudaMemcpyDeviceToHost, s));

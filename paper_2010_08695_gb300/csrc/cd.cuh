@@ -42,9 +42,11 @@ struct CdDev {
 // keys, several (`part` numbers them, -1 for the only one).
 struct alignas(16) PersistAnchor {
     int64_t q0;
-    int32_t x, deg, kb, w, part, pad;
+    int32_t x, deg, kb, w, part;
+    uint32_t wedges;  // of group anchors
 };
-constexpr int PERSIST_SLICES = 4;  // items of one anchor, at most
+constexpr int PERSIST_SLICES = 4;        // items of one anchor, at most
+constexpr int PERSIST_WIDE_SLICES = 16;  // with groups for the short walks
 
 // One round of the one-launch form, counters cumulative over the call
 // (warp-table anchors, dense-window anchors).
@@ -69,7 +71,7 @@ struct PersistDev {
     // sets in turn: the current scan's, the next one's (cleared), the last
     // one's (perhaps still being read by a CTA that has yet to go on)
     struct Set {
-        int32_t nF, nLw, nLd, workW, workD, pad;
+        int32_t nF, nLw, nLd, workW, workD, nG[3];
         unsigned long long front_w, front_e, upd_w;
     } set[3];
 };
@@ -95,6 +97,7 @@ struct PersistArgs {
     int32_t nparts;
     int32_t *F;
     PersistAnchor *Lw, *Ld;
+    PersistAnchor *Lg;  // 3 x n: anchors for groups of 1, up to 4, up to 16 warps
     PersistRound *rec;
     int32_t rec_cap;
     int32_t P, range_cap, warp_max_w, dgm;
@@ -106,10 +109,12 @@ struct PersistArgs {
 
 // Whether a decomposition can run in the one-launch form.
 bool cd_persist_fits(const Decomp &D);
+// ... with the short walks counted by groups of warps (`wide` below).
+bool cd_persist_wide(const Decomp &D);
 // CTAs of the one-launch form for m edges.
-int cd_persist_grid(int64_t m);
+int cd_persist_grid(int64_t m, bool wide);
 // Enqueues one launch (state in a.pd).
-void cd_persist_launch(const PersistArgs &a, int grid, cudaStream_t s);
+void cd_persist_launch(const PersistArgs &a, int grid, bool wide, cudaStream_t s);
 
 // ---------------------------------------------------------------------
 // Updates of a large activeSet through the other side's hubs (cd_hub.cu)

@@ -14,7 +14,10 @@
 // with the last two repeated until the activeSet is empty. Sides whose key
 // space (or, in a union of packed graphs, every graph's) fits one dense
 // window take this form: their anchors need only the warp table and the
-// dense-window engine. Same ranges, rounds and counters as cd.cu.
+// dense-window engine. Same ranges, rounds and counters as cd.cu. Sides with
+// short walks (cd_persist_wide) count them by groups of warps instead; that is
+// a kernel of its own (WIDE), because its code and lists alone cost the others
+// (256 packed graphs: 44 ms without, 47 with).
 //
 // What bounds it: the latency of a round's chain of dependent steps. On a
 // 20,000 x 5,000 graph of 200k edges (V side, 312 rounds in 149 ranges; us):
@@ -37,6 +40,8 @@ namespace {
 
 constexpr int PT = 512;  // threads per CTA (two CTAs per SM)
 constexpr int GROUP = 8;  // dense-window anchors side by side in one pass
+// With groups (WIDE), walks of more wedges still take the whole CTA.
+constexpr unsigned long long GROUP_MAX_W = 32768;
 // Polls of a barrier wait before it gives up (each takes at least an L2 round
 // trip: ~10 s in all; a peel step takes milliseconds).
 constexpr unsigned BAR_POLLS = 1u << 24;
@@ -108,6 +113,7 @@ struct WarpTable {
     }
 };
 static_assert(PT / 32 * WARP_SLOTS * 2 <= DENSE_WORDS, "warp tables fit the dense counters");
+static_assert(PT == FP_WARPS * 32 && FP_WARPS * FP_WORDS <= DENSE_WORDS, "group counters");
 static_assert(3 * NBUCKET <= DENSE_WORDS, "range histogram fits the dense counters");
 
 // Support decrements of remaining vertices (N at once so the loads overlap).
@@ -323,9 +329,93 @@ __device__ __forceinline__ PersistAnchor load_anchor(const PersistAnchor *p) {
     an.kb = hi.x;
     an.w = hi.y;
     an.part = hi.z;
+    an.wedges = (uint32_t)hi.w;
     return an;
 }
 
+// Updates of the anchors listed in classes [c0, c1] (na[c] each), a group of
+// at least `need` warps per anchor: as many as leave every anchor a group.
+// words: FP_WARPS * FP_WORDS zeroed counter words, zero again on return. cw, cm,
+// ca: wedges (all lanes), middle vertices and anchors (lane 0 of a group's
+// first warp).
+__device__ __forceinline__ void group_items(const PersistArgs &a, const PersistMids &M,
+                                            uint32_t *words, int c0, int c1, const int (&na)[3],
+                                            int need, PersistEmit &emit, unsigned long long &cw,
+                                            unsigned long long &cm, unsigned long long &ca) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int n = 0;
+    for (int c = c0; c <= c1; c++) n += na[c];
+    int g = need;
+    while (g < FP_WARPS && (int64_t)n * 2 * g <= (int64_t)FP_WARPS * gridDim.x) g *= 2;
+    const int grp = warp / g, part = warp & (g - 1);
+    uint32_t *w = words + grp * g * FP_WORDS;
+    for (int i = grp * gridDim.x + blockIdx.x; i < n; i += gridDim.x * (FP_WARPS / g)) {
+        int c = c0, j = i;
+        while (j >= na[c]) j -= na[c++];
+        const PersistAnchor an = load_anchor(a.Lg + (size_t)c * a.n + j);
+        const FpPlan pl = fp_plan(an.deg, an.wedges, an.w);
+        const uint32_t wmask = (1u << pl.lw) - 1u;
+        const int32_t ke = an.kb + an.w;
+        // keys past the window are assigned vertices still in the lists
+        if (pl.bits) {
+            auto add = [&](int32_t key) {
+                cw++;
+                if (key < an.kb || key >= ke || key == an.x) return;
+                const int32_t k = key - an.kb;
+                atomicAdd(&w[k & wmask], 1u << ((k >> pl.lw) * pl.bits));
+            };
+            warp_walk<4, KeysL2>(M, an.q0, an.q0 + an.deg, a.adj_o, add, part, g);
+        } else {
+            auto add = [&](int32_t key) {
+                cw++;
+                if (key >= an.kb && key < ke && key != an.x) fp_table_add(w, wmask, key - an.kb);
+            };
+            warp_walk<4, KeysL2>(M, an.q0, an.q0 + an.deg, a.adj_o, add, part, g);
+        }
+        fp_sync(grp, g);
+        for (uint32_t sl = part * 32 + lane; sl <= wmask / 4; sl += 32 * g) {
+            const uint4 v = ((const uint4 *)w)[sl];
+            if (!(v.x | v.y | v.z | v.w)) continue;
+            ((uint4 *)w)[sl] = make_uint4(0, 0, 0, 0);
+            const uint32_t e[4] = {v.x, v.y, v.z, v.w};
+            if (pl.bits == 0) {
+                int32_t k[4];
+                uint32_t cc[4];
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    cc[u] = e[u] & 1023u;
+                    k[u] = cc[u] >= 2 ? an.kb + (int32_t)(e[u] >> 10) - 1 : -1;
+                }
+                emit.many<4>(k, cc);
+                continue;
+            }
+#pragma unroll
+            for (int x = 0; x < 4; x++) {
+                uint32_t f = fp_repeats(e[x], pl.bits);
+                while (f) {
+                    int32_t k[4];
+                    uint32_t cc[4];
+#pragma unroll
+                    for (int u = 0; u < 4; u++) {
+                        const int b = f ? __ffs(f) - 1 : 0;
+                        cc[u] = (e[x] >> b) & (0xffffffffu >> (32 - pl.bits));
+                        k[u] = f ? an.kb + (int32_t)(4 * sl + x) + ((b / pl.bits) << pl.lw) : -1;
+                        f &= f - 1;
+                    }
+                    emit.many<4>(k, cc);
+                }
+            }
+        }
+        fp_sync(grp, g);
+        if (part == 0 && lane == 0) {
+            cm += (unsigned long long)an.deg;
+            ca++;
+        }
+    }
+    __syncthreads();
+}
+
+template <bool WIDE>
 __global__ void __launch_bounds__(PT, 2) k_cd_persist(PersistArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_ok, s_nt, s_idx, s_nb, s_pick, s_first, s_last, s_nF, s_due;
@@ -545,6 +635,7 @@ __global__ void __launch_bounds__(PT, 2) k_cd_persist(PersistArgs a) {
                     }
                     if (!__any_sync(0xffffffffu, take)) continue;
                     PersistAnchor an{0, x[u], 0, 0, 0, -1, 0};
+                    int cls = -1;
                     unsigned long long wf = 0;
                     if (take) {
                         wf = a.wfull[x[u]];
@@ -561,13 +652,29 @@ __global__ void __launch_bounds__(PT, 2) k_cd_persist(PersistArgs a) {
                         fw += wf;
                         fe += (unsigned long long)an.deg;
                         if (v[u]) uw += wf;
+                        if (WIDE && v[u] && wf > (unsigned long long)a.warp_max_w &&
+                            wf <= GROUP_MAX_W) {
+                            an.wedges = (uint32_t)wf;
+                            const FpPlan pl = fp_plan(an.deg, an.wedges, an.w);
+                            // a round waits for its longest walk
+                            const int load = max((int)(wf >> 10), an.deg >> 6);
+                            cls = pl.lw > 14              ? -1
+                                  : pl.g == 1 && load < 1 ? 0
+                                  : pl.g <= 4 && load < 4 ? 1
+                                                          : 2;
+                        }
                     }
                     const bool small = take && v[u] && wf <= (unsigned long long)a.warp_max_w;
-                    const bool big = take && v[u] && !small;
+                    const bool big = take && v[u] && !small && cls < 0;
                     const int pf = warp_slot(take, &set->nF);
                     const int pw = warp_slot(small, &set->nLw);
                     if (take) a.F[pf] = x[u];
                     if (small) a.Lw[pw] = an;
+#pragma unroll
+                    for (int c = 0; WIDE && c < 3; c++) {
+                        const int pg = warp_slot(cls == c, &set->nG[c]);
+                        if (cls == c) a.Lg[(size_t)c * a.n + pg] = an;
+                    }
                     const int32_t win = an.w;
                     for (int j = 0; __any_sync(0xffffffffu, big && j * DENSE_KEYS < win); j++) {
                         const bool has = big && j * DENSE_KEYS < win;
@@ -681,6 +788,27 @@ __global__ void __launch_bounds__(PT, 2) k_cd_persist(PersistArgs a) {
             cw = cm = ca = 0;
             __syncthreads();  // the tables' words become dense counters again
         }
+        const int nG[3] = {WIDE ? __ldcg(&set->nG[0]) : 0, WIDE ? __ldcg(&set->nG[1]) : 0,
+                           WIDE ? __ldcg(&set->nG[2]) : 0};
+        if (WIDE && nG[0] + nG[1] + nG[2] > 0) {
+            // in one go when the widest class leaves every anchor a group
+            const int top = nG[2] ? 2 : nG[1] ? 1 : 0;
+            if ((int64_t)(nG[0] + nG[1] + nG[2]) << (2 * top) <= (int64_t)FP_WARPS * gridDim.x) {
+                group_items(a, M, H.cnt, 0, top, nG, 1 << (2 * top), emit, cw, cm, ca);
+            } else {
+                for (int c = top; c >= 0; c--)
+                    if (nG[c]) group_items(a, M, H.cnt, c, c, nG, 1 << (2 * c), emit, cw, cm, ca);
+            }
+            cw = warp_sum(cw);
+            if (lane == 0 && cw) {
+                atomicAdd(&st->tier_w[4], cw);
+                if (ca) {
+                    atomicAdd(&st->tier_m[4], cm);
+                    atomicAdd(&st->tier_a[4], ca);
+                }
+            }
+            cw = cm = ca = 0;
+        }
         // items per fetch: more than one only when the round has more items
         // than CTAs
         const int G = max(1, min(GROUP, nD / (int)gridDim.x));
@@ -792,26 +920,45 @@ constexpr size_t persist_smem() { return DenseSlice::bytes() + chunk_bytes(PT); 
 
 }  // namespace
 
+// Groups of warps pay where the mean walk is short: with several windows below
+// the 8,192 wedges their tables hold (100,000 x 30,000, 1M edges, 2,000 wedges:
+// 11.9 against 14.3 ms for the step; 40,000 x 400,000, 3M edges, 22,000: 23.6
+// against 22.1; uniform graphs of 1M and 5M edges 0.8 against 2.2, 1.0 against
+// 2.9), with one below 1,024 (2,000 x 500, 20k edges, 400: 2.2 against
+// 2.4 the whole call; 5,000 x 20,000, 200k edges, 3,800: 7.8 against 6.8).
+bool cd_persist_wide(const Decomp &D) {
+    const uint64_t mean = D.n > 0 ? D.wedges_bup / (uint64_t)D.n : 0;
+    return !D.parts && mean < (D.n > DENSE_KEYS ? 8192u : 1024u);
+}
+
 bool cd_persist_fits(const Decomp &D) {
     if (D.max_deg_s >= 65535) return false;  // counts may need 32 bits
     if (!D.parts) {
         // several windows walk a long list once per window: only while the
         // rounds are short (120,000 x 40,000 with 3M edges, 1.9 10^9 wedges,
         // 4 windows: 35.3 ms here, 30.8 by the per-round kernels; 40,000 x
-        // 400,000 with 3M edges, 9 10^8, 2 windows: 21.5 against 29.3)
+        // 400,000 with 3M edges, 9 10^8, 2 windows: 21.5 against 29.3), and
+        // past PERSIST_SLICES only where groups count the short walks
+        // (500,000 x 120,000 uniform, 5M edges, 14 windows: 0.9 against 3.1)
         const int64_t windows = ceil_div(D.n, DENSE_KEYS);
         return windows == 1 ||
-               (windows <= PERSIST_SLICES && (double)windows * (double)D.wedges_bup <= 3e9);
+               (windows <= (cd_persist_wide(D) ? PERSIST_WIDE_SLICES : PERSIST_SLICES) &&
+                (double)windows * (double)D.wedges_bup <= 3e9);
     }
     for (size_t i = 0; i + 1 < D.parts->size(); i++)
         if ((*D.parts)[i + 1] - (*D.parts)[i] > DENSE_KEYS) return false;
     return true;
 }
 
-int cd_persist_grid(int64_t m) {
-    allow_max_smem((const void *)k_cd_persist);
+static const void *persist_kernel(bool wide) {
+    return wide ? (const void *)k_cd_persist<true> : (const void *)k_cd_persist<false>;
+}
+
+int cd_persist_grid(int64_t m, bool wide) {
+    const void *kernel = persist_kernel(wide);
+    allow_max_smem(kernel);
     int occ = 0;
-    RC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cd_persist, PT, persist_smem()));
+    RC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, PT, persist_smem()));
     if (occ < 1) fail(RECEIPT_ERR_INTERNAL, "the one-launch form does not fit an SM");
     // One CTA per 4,096 edges: fewer leave a round's anchors queueing (30,000 x
     // 9,000, 300k edges: 14.4 ms a call with 8,192 edges per CTA, 10.8 with
@@ -822,10 +969,10 @@ int cd_persist_grid(int64_t m) {
     return (int)std::min<int64_t>(num_sms() * std::min(occ, 2), std::max<int64_t>(16, m / 4096));
 }
 
-void cd_persist_launch(const PersistArgs &a, int grid, cudaStream_t s) {
+void cd_persist_launch(const PersistArgs &a, int grid, bool wide, cudaStream_t s) {
     void *args[] = {(void *)&a};
     RC_CUDA(cudaMemsetAsync(&a.pd->bar, 0, sizeof(unsigned), s));
-    RC_CUDA(cudaLaunchCooperativeKernel((const void *)k_cd_persist, dim3(grid), dim3(PT), args,
+    RC_CUDA(cudaLaunchCooperativeKernel(persist_kernel(wide), dim3(grid), dim3(PT), args,
                                         persist_smem(), s));
     RC_LAUNCH();
 }

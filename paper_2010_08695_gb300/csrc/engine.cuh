@@ -178,6 +178,84 @@ __device__ __forceinline__ void warp_walk(const Mids &M, int64_t q0, int64_t q1,
 }
 
 // ------------------------------------------------------------------
+// Counting by groups of warps
+// ------------------------------------------------------------------
+// A walk of 100 to some 10,000 wedges keeps a warp busy for microseconds and a
+// whole CTA for one step of its chunk loop, so it gets a group of g warps (a
+// power of two), which counts in its warps' FP_WORDS words taken together, one
+// counter per key: a count is at most the start point's degree, so 4 bits do
+// for degrees up to 15, 8 up to 255, 16 up to 65,535 and 32 above
+// (neighbouring keys lie in different words). g is the least that holds the
+// counters, and at least a warp per 4,096 wedges or 512 middle vertices. A walk
+// much shorter than its key space (8 W below the words the counters need) uses
+// a table with entries (key + 1) << 10 | count instead, at most half full: at
+// 3/4 the longest probe of a warp's 32 dominated (8 us a walk of 1,000 wedges;
+// counters 1 us).
+constexpr int FP_WARPS = 16;             // of a CTA
+constexpr int FP_WORDS = 1024;           // counter words of a warp
+constexpr int32_t FP_HASH_DEG = 1024;    // counts of the table's entries
+constexpr int32_t FP_MAX_NI = (1 << 22) - 2;  // keys of the table's entries
+
+__device__ __forceinline__ void fp_table_add(uint32_t *slot, uint32_t mask, int32_t key) {
+    const uint32_t k = ((uint32_t)key + 1u) << 10;
+    uint32_t h = (hash_key(key) >> 8) & mask;
+    for (uint32_t p = 0; p <= mask; p++) {
+        uint32_t cur = ((volatile uint32_t *)slot)[h];
+        if (cur == 0) {
+            cur = atomicCAS(&slot[h], 0u, k | 1u);
+            if (cur == 0) return;
+        }
+        if ((cur ^ k) < 1024u) {
+            atomicAdd(&slot[h], 1u);
+            return;
+        }
+        h = (h + 1) & mask;
+    }
+}
+
+// How a walk is counted: bits of its counters (0: the table), log2 of the
+// words it needs (up to 8 times a CTA's), and warps (above FP_WARPS: none of
+// these ways).
+struct FpPlan {
+    int bits, lw, g;
+};
+// deg, w: the start point's degree and wedges; ni: keys.
+__device__ __forceinline__ FpPlan fp_plan(int32_t deg, uint32_t w, int32_t ni) {
+    FpPlan p;
+    p.bits = deg < 16 ? 4 : deg < 256 ? 8 : deg < 65536 ? 16 : 32;
+    p.lw = max(7, 32 - __clz((int)(((int64_t)ni * p.bits + 31) / 32) - 1));
+    if (deg < FP_HASH_DEG && ni <= FP_MAX_NI && w < FP_WARPS * FP_WORDS / 2 && (w << 3) < (1u << p.lw)) {
+        p.bits = 0;
+        p.lw = max(7, 33 - __clz(w));  // 2 W to 4 W words
+    }
+    // a step of a warp takes 32 middle vertices or 128 wedges
+    const uint64_t steps = (uint64_t)w + 8ull * (uint32_t)deg;
+    const int by_w = steps <= 4096 ? 0 : steps > 32768 ? 4 : 32 - __clz((uint32_t)(steps - 1) >> 12);
+    p.g = p.lw <= 17 ? 1 << min(max(p.lw - 10, by_w), 4) : 2 * FP_WARPS;
+    return p;
+}
+static_assert(FP_WORDS == 1 << 10 && FP_WARPS == 1 << 4, "words and warps of a plan");
+
+// Counters of at least 2 in a word of b-bit counters: the lowest bit of each.
+__device__ __forceinline__ uint32_t fp_repeats(uint32_t v, int bits) {
+    if (bits == 4) return ((v >> 1) | (v >> 2) | (v >> 3)) & 0x11111111u;
+    if (bits == 32) return v >= 2 ? 1u : 0u;
+    uint32_t x = v & (bits == 8 ? 0xfefefefeu : 0xfffefffeu);
+    if (bits == 16) x |= x >> 8;
+    x |= x >> 4;
+    x |= x >> 2;
+    x |= x >> 1;
+    return x & (bits == 8 ? 0x01010101u : 0x00010001u);
+}
+
+__device__ __forceinline__ void fp_sync(int grp, int g) {
+    if (g == 1)
+        __syncwarp();
+    else
+        asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(32 * g) : "memory");
+}
+
+// ------------------------------------------------------------------
 // Warp-private table
 // ------------------------------------------------------------------
 struct WarpHash {

@@ -354,16 +354,9 @@ struct FdEmit {
 // then reads a list instead of walking (runs, keys, counters, sweep).
 //
 // Walks have 100 to 2,000 wedges over about ten middle vertices in the tasks
-// that take longest, and up to a million in the last ones. A member gets a
-// group of g warps (a power of two), which counts in its warps' FP_WORDS words
-// taken together, one counter per rank: a count is at most the member's
-// degree, so 4 bits do for degrees up to 15, 8 up to 255, 16 up to 65,535
-// and 32 above (neighbouring ranks lie in different words). g is the least that holds the
-// counters, and at least a warp per 4,096 wedges or 512 middle vertices. A walk much shorter than its
-// task (8 W below the words the counters need) uses a table with entries (rank
-// + 1) << 10 | count instead, at most half full: at 3/4 the longest probe of a
-// warp's 32 dominated (8 us a member of 1,000 wedges; counters 1 us). Members
-// whose counters exceed a CTA's words up to 8 times walk once per slice of them.
+// that take longest, and up to a million in the last ones: each is counted by
+// a group of warps (FpPlan). Members whose counters exceed a CTA's words up to
+// 8 times walk once per slice of them.
 // The entries lie in one pool, taken by each group in blocks; a member whose
 // list does not fit it, or that is too large for all this, has no list and
 // walks when it is peeled.
@@ -372,12 +365,8 @@ struct FdEmit {
 // ms; walked during the peel they made the whole step 101 and 26 ms (34 and 10
 // now).
 // ------------------------------------------------------------------------
-constexpr int FP_THREADS = 512;
-constexpr int FP_WARPS = FP_THREADS / 32;
-constexpr int FP_WORDS = 1024;           // counter words of a warp
+constexpr int FP_THREADS = FP_WARPS * 32;
 constexpr int FP_BLOCK = 1024;           // pool entries taken at a time
-constexpr int32_t FP_HASH_DEG = 1024;    // counts of the table's entries
-constexpr int32_t FP_MAX_NI = (1 << 22) - 2;  // ranks of the entries
 constexpr int64_t FP_MEMBER_COST = 128;  // a member's fixed cost in wedges
 // An entry holds the rank in its low fp_rank_bits and the count above.
 constexpr unsigned long long FP_NONE = ~0ull;  // no list; else offset << 24 | length
@@ -424,44 +413,12 @@ __device__ __forceinline__ FdMember fd_load(const FdMember *p) {
     return FdMember{(int64_t)(uint32_t)q.x | ((int64_t)q.y << 32), q.z, (uint32_t)q.w};
 }
 
-__device__ __forceinline__ void fp_table_add(uint32_t *slot, uint32_t mask, int32_t key) {
-    const uint32_t k = ((uint32_t)key + 1u) << 10;
-    uint32_t h = (hash_key(key) >> 8) & mask;
-    for (uint32_t p = 0; p <= mask; p++) {
-        uint32_t cur = ((volatile uint32_t *)slot)[h];
-        if (cur == 0) {
-            cur = atomicCAS(&slot[h], 0u, k | 1u);
-            if (cur == 0) return;
-        }
-        if ((cur ^ k) < 1024u) {
-            atomicAdd(&slot[h], 1u);
-            return;
-        }
-        h = (h + 1) & mask;
-    }
-}
-
-// How a member is counted: bits of its counters (0: the table), log2 of the
-// words it needs, and warps (above FP_WARPS: no list).
-struct FpPlan {
-    int bits, lw, g;
-};
-__device__ __forceinline__ FpPlan fp_plan(const FdMember &m, int32_t ni) {
-    FpPlan p;
-    p.bits = m.deg < 16 ? 4 : m.deg < 256 ? 8 : m.deg < 65536 ? 16 : 32;
-    p.lw = max(7, 32 - __clz((int)(((int64_t)ni * p.bits + 31) / 32) - 1));
-    if (m.deg < FP_HASH_DEG && m.w < FP_WARPS * FP_WORDS / 2 && (m.w << 3) < (1u << p.lw)) {
-        p.bits = 0;
-        p.lw = max(7, 33 - __clz(m.w));  // 2 W to 4 W words
-    }
-    const bool ok = (int64_t)m.deg < (1ll << (32 - fp_rank_bits(ni)));
-    // a step of a warp takes 32 middle vertices or 128 wedges
-    const uint64_t steps = (uint64_t)m.w + 8ull * (uint32_t)m.deg;
-    const int by_w = steps <= 4096 ? 0 : steps > 32768 ? 4 : 32 - __clz((uint32_t)(steps - 1) >> 12);
-    p.g = ok && p.lw <= 17 ? 1 << min(max(p.lw - 10, by_w), 4) : 2 * FP_WARPS;
+// A member's plan in a task of ni; g above FP_WARPS: no list.
+__device__ __forceinline__ FpPlan fd_plan(const FdMember &m, int32_t ni) {
+    FpPlan p = fp_plan(m.deg, m.w, ni);
+    if ((int64_t)m.deg >= 1ll << (32 - fp_rank_bits(ni))) p.g = 2 * FP_WARPS;
     return p;
 }
-static_assert(FP_WORDS == 1 << 10 && FP_WARPS == 1 << 4, "words and warps of a plan");
 
 // Weight of each task's members that get no list.
 __global__ void k_listless(const FdMember *__restrict__ info, int32_t n,
@@ -470,7 +427,7 @@ __global__ void k_listless(const FdMember *__restrict__ info, int32_t n,
     const int32_t p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
     const FdMember m = fd_load(info + p);
-    if (ni_max <= FP_MAX_NI && fp_plan(m, ni_max).g <= FP_WARPS) return;
+    if (ni_max <= FP_MAX_NI && fd_plan(m, ni_max).g <= FP_WARPS) return;
     int32_t t = 0;
     for (int32_t hi = T - 1; t < hi;) {
         const int32_t mid = (t + hi + 1) / 2;
@@ -479,27 +436,8 @@ __global__ void k_listless(const FdMember *__restrict__ info, int32_t n,
         else
             hi = mid - 1;
     }
-    if (tlen[t] > FP_MAX_NI || fp_plan(m, tlen[t]).g > FP_WARPS)
+    if (tlen[t] > FP_MAX_NI || fd_plan(m, tlen[t]).g > FP_WARPS)
         atomicAdd(&lw[t], (unsigned long long)m.w);
-}
-
-// Counters of at least 2 in a word of b-bit counters: the lowest bit of each.
-__device__ __forceinline__ uint32_t fp_repeats(uint32_t v, int bits) {
-    if (bits == 4) return ((v >> 1) | (v >> 2) | (v >> 3)) & 0x11111111u;
-    if (bits == 32) return v >= 2 ? 1u : 0u;
-    uint32_t x = v & (bits == 8 ? 0xfefefefeu : 0xfffefffeu);
-    if (bits == 16) x |= x >> 8;
-    x |= x >> 4;
-    x |= x >> 2;
-    x |= x >> 1;
-    return x & (bits == 8 ? 0x01010101u : 0x00010001u);
-}
-
-__device__ __forceinline__ void fp_sync(int grp, int g) {
-    if (g == 1)
-        __syncwarp();
-    else
-        asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(32 * g) : "memory");
 }
 
 __global__ void __launch_bounds__(FP_THREADS, 2) k_fd_pairs(FdPairArgs a) {
@@ -541,7 +479,7 @@ __global__ void __launch_bounds__(FP_THREADS, 2) k_fd_pairs(FdPairArgs a) {
                 bool more = false;
                 for (int32_t p = pa + grp; p < pb; p += FP_WARPS / g) {
                     const FdMember m = fd_load(a.info + p);
-                    const FpPlan pl = fp_plan(m, ni);
+                    const FpPlan pl = fd_plan(m, ni);
                     if (pl.g != g) {
                         more |= pl.g > g && pl.g <= FP_WARPS;
                         continue;

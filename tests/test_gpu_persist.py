@@ -58,3 +58,29 @@ def test_more_rounds_than_one_launch_records(R):
     recs = _rounds(g)
     t = R.as_u64(g.tip_decompose(0, P=20000, round_graphs=-1))
     assert np.array_equal(t, want) and recs == _rounds(g)
+
+
+# short walks counted by groups of warps: degrees around the 4-, 8- and 16-bit
+# counters, members with d keys shared by w of them, in one and several windows
+@pytest.mark.parametrize("pad", [0, 40_000, 200_000])
+@pytest.mark.parametrize("d,w", [(2, 300), (15, 40), (16, 40), (255, 5), (256, 5), (1024, 2)])
+def test_short_walks(R, d, w, pad):
+    groups = 30
+    u = np.arange(groups * w)
+    x = u[::7]  # one more key, shared by them all
+    y = np.arange(pad)  # pairs without a butterfly
+    rng = np.random.default_rng(d)
+    lab = rng.permutation(u.size + pad)
+    eu = lab[np.concatenate([np.repeat(u, d), x, u.size + y])].astype(np.int32)
+    ev = np.concatenate([np.repeat(u // w, d) * d + np.tile(np.arange(d), u.size),
+                         np.full(x.size, groups * d), groups * d + 1 + y // 2]).astype(np.int32)
+    nv = int(ev.max()) + 1
+    want, _ = oracle.bup(eu, ev, u.size + pad, nv, 0)
+    g = R.Graph(eu, ev, u.size + pad, nv)
+    for kw in ({}, {"P": 4}, {"dgm_frac_1024": 8}, {"warp_max_w": 16}):
+        t = R.as_u64(g.tip_decompose(0, **kw))
+        assert np.array_equal(t, want), kw
+        recs = _rounds(g)
+        t = R.as_u64(g.tip_decompose(0, round_graphs=-1, **kw))
+        assert np.array_equal(t, want), kw
+        assert recs == _rounds(g), kw
