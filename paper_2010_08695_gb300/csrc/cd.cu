@@ -1469,7 +1469,10 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s) {
         // items: an anchor's whole window, or its windows of DENSE_KEYS keys
         // (wide: of anchors with 1,024 wedges and more)
         const size_t many = wide ? std::min<size_t>(n, (D.wedges_bup + D.m) / 1024 + 1) : n;
-        DevBuf<PersistAnchor> pLd(many * (D.parts ? 1 : ceil_div(n, DENSE_KEYS)), s);
+        // a CTA loads the item of its index before the round's counts are known
+        const int pgrid = cd_persist_grid(D.m, wide);
+        DevBuf<PersistAnchor> pLd(
+            std::max<size_t>(many * (D.parts ? 1 : ceil_div(n, DENSE_KEYS)), pgrid), s);
         constexpr int REC_CAP = 4096;  // rounds per launch
         DevBuf<PersistRound> prec(REC_CAP, s);
         std::vector<int32_t> hfirst(ng + 1, 0);
@@ -1493,7 +1496,6 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s) {
                              F.get(), pLw.get(), pLd.get(), pLg.get(), prec.get(), REC_CAP, P, range_cap,
                              warp_max_w, dgm && O.n > 0 ? 1 : 0, dgm_frac, huc == 0 ? 1 : 0,
                              huc_factor, rcost.get()};
-        const int pgrid = cd_persist_grid(D.m, wide);
         PersistDev *hpd = (PersistDev *)(hrec + ROUND_BURST * (hdr / 8));
         PersistRound *hrc = (PersistRound *)(hpd + 1);
         std::vector<PersistRound> recs;
