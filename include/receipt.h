@@ -116,8 +116,11 @@ typedef struct {
      * launch: of one cooperative kernel for the whole coarse-grained step
      * when the side's keys fit at most four dense windows (147,456 vertices;
      * sixteen, 589,824, where the mean walk is below 8,192 wedges; in a
-     * batch, every graph's one window) and no degree on it reaches 65,535; otherwise of a CUDA graph whose while-node repeats the round body until
-     * a round leaves no next activeSet (at most 64 rounds a launch), each
+     * batch, every graph's one window) and no degree on it reaches 65,535
+     * (sides of at most two windows and 1.2e9 wedges, or 3e9 in a batch, read
+     * every vertex's updates from lists made beforehand; the records count the
+     * walks that saves); otherwise of a CUDA graph whose while-node repeats
+     * the round body until a round leaves no next activeSet (at most 64 rounds a launch), each
      * round's counters going to a device record that the host reads after
      * the launch; with timing on or the activeSet found by crossings the
      * rounds run as with -1. 1: every round is one launch of a CUDA graph

@@ -1090,11 +1090,14 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s) {
     const int32_t SW = slice_ctas == 4 ? Slice4::keys : slice_ctas == 2 ? Slice2::keys : Slice1::keys;
     const bool scan_next = opt.scan_frontier >= 0;
     // One cooperative launch for the whole step (cd_persist.cu): the default
-    // for sides that need only the warp and the dense-window tier. Forced
-    // recounts, injected bounds, per-tier timing and the other launch modes
-    // take the per-round kernels below.
-    const bool persist = opt.round_graphs == 0 && scan_next && !D.timing && opt.n_bounds <= 0 &&
-                         opt.huc <= 0 && cd_persist_fits(D);
+    // where it fits (its rules stand there). Forced recounts, injected bounds,
+    // per-tier timing and the other launch modes take the per-round kernels
+    // below.
+    const bool one_launch = opt.round_graphs == 0 && scan_next && !D.timing && opt.n_bounds <= 0 &&
+                            opt.huc <= 0;
+    PairLists pairs;
+    const bool lists = one_launch && cd_persist_by_lists(D) && side_pair_lists(D, pairs, s);
+    const bool persist = one_launch && (lists || cd_persist_fits(D));
     const int32_t slice_fetch = opt.slice_fetch > 0 ? std::min(opt.slice_fetch, SLICE_FETCH_MAX) : 1;
     // vertices per range: at most range_max_n (0: 2 n / P, -1: no bound)
     const int32_t range_cap =
@@ -1459,7 +1462,8 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s) {
     uint64_t crcnt = 0;  // C_rcnt (rule on) or 0
     if (persist) {
         const int ng = D.parts ? (int)D.parts->size() - 1 : 1;
-        const bool wide = cd_persist_wide(D);
+        const bool wide = !lists && cd_persist_wide(D);
+        const int form = lists ? PERSIST_LISTS : wide ? PERSIST_GROUPS : PERSIST_WINDOWS;
         DevBuf<PersistDev> pd(1, s);
         DevBuf<unsigned long long> ph_w(3 * NBUCKET, s);
         DevBuf<uint32_t> ph_c(3 * NBUCKET, s);
@@ -1468,11 +1472,11 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s) {
         DevBuf<PersistAnchor> pLw(n, s), pLg(wide ? 3 * (size_t)n : 1, s);
         // items: an anchor's whole window, or its windows of DENSE_KEYS keys
         // (wide: of anchors with 1,024 wedges and more)
-        const size_t many = wide ? std::min<size_t>(n, (D.wedges_bup + D.m) / 1024 + 1) : n;
+        const size_t many = lists ? 1 : wide ? std::min<size_t>(n, (D.wedges_bup + D.m) / 1024 + 1) : n;
         // a CTA loads the item of its index before the round's counts are known
-        const int pgrid = cd_persist_grid(D.m, wide);
+        const int pgrid = cd_persist_grid(D.m, form);
         DevBuf<PersistAnchor> pLd(
-            std::max<size_t>(many * (D.parts ? 1 : ceil_div(n, DENSE_KEYS)), pgrid), s);
+            std::max<size_t>(many * (D.parts || lists ? 1 : ceil_div(n, DENSE_KEYS)), pgrid), s);
         constexpr int REC_CAP = 4096;  // rounds per launch
         DevBuf<PersistRound> prec(REC_CAP, s);
         std::vector<int32_t> hfirst(ng + 1, 0);
@@ -1495,13 +1499,13 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s) {
                              D.parts ? part_of.get() : nullptr, pfirst.get(), plast.get(), ng,
                              F.get(), pLw.get(), pLd.get(), pLg.get(), prec.get(), REC_CAP, P, range_cap,
                              warp_max_w, dgm && O.n > 0 ? 1 : 0, dgm_frac, huc == 0 ? 1 : 0,
-                             huc_factor, rcost.get()};
+                             huc_factor, rcost.get(), pairs.pool.get(), pairs.rec.get()};
         PersistDev *hpd = (PersistDev *)(hrec + ROUND_BURST * (hdr / 8));
         PersistRound *hrc = (PersistRound *)(hpd + 1);
         std::vector<PersistRound> recs;
         RC_CUDA(cudaMemcpyAsync(hpin, rcost.get(), 8, cudaMemcpyDeviceToHost, s));
         for (;;) {
-            cd_persist_launch(pa, pgrid, wide, s);
+            cd_persist_launch(pa, pgrid, form, s);
             RC_CUDA(cudaMemcpyAsync(hpd, pd.get(), sizeof(PersistDev), cudaMemcpyDeviceToHost, s));
             RC_CUDA(cudaMemcpyAsync(hrc, prec.get(), PERSIST_FIRST * sizeof(PersistRound),
                                     cudaMemcpyDeviceToHost, s));

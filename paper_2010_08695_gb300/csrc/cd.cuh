@@ -55,6 +55,9 @@ struct PersistRound {
     unsigned long long hi, anchors[2], wedges[2];
 };
 
+// How anchors are counted: dense windows, groups of warps too, or by lists made
+// beforehand.
+enum { PERSIST_WINDOWS = 0, PERSIST_GROUPS = 1, PERSIST_LISTS = 2 };
 enum { PERSIST_RANGE = 0, PERSIST_PEEL = 1, PERSIST_SCAN = 2 };          // where to go on
 enum { PERSIST_DONE = 0, PERSIST_RECOUNT = 1, PERSIST_RECORDS_FULL = 2 };  // why it stopped
 
@@ -105,16 +108,20 @@ struct PersistArgs {
     int32_t huc;  // the recount rule is on
     double huc_factor;
     const unsigned long long *crcnt;
+    const uint32_t *pool;            // update lists (PERSIST_LISTS)
+    const unsigned long long *list;  // where each vertex's lies
 };
 
 // Whether a decomposition can run in the one-launch form.
 bool cd_persist_fits(const Decomp &D);
+// ... and whether lists of every vertex's updates should be made for it.
+bool cd_persist_by_lists(const Decomp &D);
 // ... with the short walks counted by groups of warps (`wide` below).
 bool cd_persist_wide(const Decomp &D);
 // CTAs of the one-launch form for m edges.
-int cd_persist_grid(int64_t m, bool wide);
+int cd_persist_grid(int64_t m, int form);
 // Enqueues one launch (state in a.pd).
-void cd_persist_launch(const PersistArgs &a, int grid, bool wide, cudaStream_t s);
+void cd_persist_launch(const PersistArgs &a, int grid, int form, cudaStream_t s);
 
 // ---------------------------------------------------------------------
 // Updates of a large activeSet through the other side's hubs (cd_hub.cu)

@@ -14,18 +14,22 @@
 // with the last two repeated until the activeSet is empty. Sides whose key
 // space (or, in a union of packed graphs, every graph's) fits one dense
 // window take this form: their anchors need only the warp table and the
-// dense-window engine. Same ranges, rounds and counters as cd.cu. Sides with
-// short walks (cd_persist_wide) count them by groups of warps instead; that is
-// a kernel of its own (WIDE), because its code and lists alone cost the others
-// (256 packed graphs: 44 ms without, 47 with).
+// dense-window engine. Same ranges, rounds and counters as cd.cu.
+//
+// Three forms of the peel: dense windows, a CTA per item; groups of warps for
+// sides with short walks (cd_persist_wide); and, on sides small enough to make
+// every vertex's list of updates beforehand (cd_persist_by_lists), reading those
+// lists, which leaves a round two dependent loads and no walk. Each is a kernel
+// of its own: the groups' code and lists alone cost the others (256 packed
+// graphs: 44 ms without, 47 with).
 //
 // What bounds it: the latency of a round's chain of dependent steps. On a
 // 20,000 x 5,000 graph of 200k edges (V side, 312 rounds in 149 ranges; us):
 // scan 3.4, barrier 1.9, counters and first item 1.6, walk 4.3, sweep 1.2,
-// barrier 2.1; bound 3.3 a range. That step took 17.5 ms by the per-round
-// kernels and takes 5.9 so (whole call 17.4 -> 7.2 ms); 2,000 x 500 with 20k
-// edges 4.5 -> 1.8 (5.3 -> 2.9), 30,000 x 9,000 with 300k edges from host
-// buffers 20.1 -> 10.8 the whole call, 256 packed graphs 76 -> 54.
+// barrier 2.1; bound 3.3 a range. That call took 17.4 ms by the per-round
+// kernels, 7.0 by windows and takes 5.4 by lists; 2,000 x 500 with 20k edges 5.3,
+// 2.4 (2.2 by groups) and 1.9; 30,000 x 9,000 with 300k edges from host buffers
+// 20.1, 9.7 and 7.0; 256 packed graphs 76, 44 and 36.5.
 //
 // What changes during the launch (supports, subsets, working lists, the
 // activeSet) is read from L2 (ld.cg): another CTA may have written it since
@@ -415,14 +419,16 @@ __device__ __forceinline__ void group_items(const PersistArgs &a, const PersistM
     __syncthreads();
 }
 
-template <bool WIDE>
+template <int FORM>
 __global__ void __launch_bounds__(PT, 2) k_cd_persist(PersistArgs a) {
+    constexpr bool WIDE = FORM == PERSIST_GROUPS, LISTS = FORM == PERSIST_LISTS;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_ok, s_nt, s_idx, s_nb, s_pick, s_first, s_last, s_nF, s_due;
     __shared__ unsigned long long s_tmp[33], s_goal, s_wrem, s_peeled;
     __shared__ uint32_t s_tmpc[33];
     __shared__ double s_tgt;
     __shared__ PersistGroup s_g;
+    __shared__ uint32_t s_tier[8];  // a CTA's counters of a round by lists, per tier
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // global numbers with the CTA index fastest: a few items spread over CTAs
     const int gwarp = warp * gridDim.x + blockIdx.x, nwarps = (PT / 32) * gridDim.x;
@@ -451,6 +457,7 @@ __global__ void __launch_bounds__(PT, 2) k_cd_persist(PersistArgs a) {
     unsigned long long hi = pd->hi, peeled = pd->peeled, peeled_at_dgm = pd->peeled_at_dgm;
     // last remaining vertex when the range began (one graph)
     int32_t last = fused && mode != PERSIST_RANGE ? a.n - 1 : -1;
+    if (threadIdx.x < 8) s_tier[threadIdx.x] = 0;
     if (threadIdx.x == 0) {
         s_ok = 1;
         s_wrem = pd->wrem_prev;
@@ -664,7 +671,15 @@ __global__ void __launch_bounds__(PT, 2) k_cd_persist(PersistArgs a) {
                                                           : 2;
                         }
                     }
-                    const bool small = take && v[u] && wf <= (unsigned long long)a.warp_max_w;
+                    if (LISTS && take) {
+                        // rank bits and first vertex of its graph
+                        const int32_t pt = fused ? 0 : a.part_of[x[u]];
+                        an.kb = a.pfirst[pt];
+                        an.part = fp_rank_bits(a.pfirst[pt + 1] - an.kb);
+                        an.w = wf <= (unsigned long long)a.warp_max_w ? 0 : 4;  // tier
+                    }
+                    const bool small =
+                        take && v[u] && (LISTS || wf <= (unsigned long long)a.warp_max_w);
                     const bool big = take && v[u] && !small && cls < 0;
                     const int pf = warp_slot(take, &set->nF);
                     const int pw = warp_slot(small, &set->nLw);
@@ -758,7 +773,61 @@ __global__ void __launch_bounds__(PT, 2) k_cd_persist(PersistArgs a) {
         const int32_t nW = __ldcg(&set->nLw), nD = __ldcg(&set->nLd), nF = __ldcg(&set->nF);
         PersistEmit emit{a.sup, a.sub, 0};
         unsigned long long cw = 0, cm = 0, ca = 0;
-        if (nW > 0) {
+        if (LISTS && nW > 0) {
+            // a group of warps per anchor: as many as leave every anchor a group.
+            // The counters are those of the walks this saves (their lists are
+            // kept and compacted as ever): sums of the working lists' lengths.
+            int g = 1;
+            while (g < PT / 32 && (int64_t)nW * 2 * g <= nwarps) g *= 2;
+            const int grp = warp / g, part = warp & (g - 1);
+            for (int i = grp * gridDim.x + blockIdx.x; i < nW; i += nwarps / g) {
+                const PersistAnchor an = load_anchor(a.Lw + i);
+                const unsigned long long q = __ldg(a.list + an.x);
+                // (the first lengths are on their way while the list is read)
+                int j1 = part * 32 + lane;
+                uint32_t walk =
+                    j1 < an.deg ? (uint32_t)__ldcg(a.len_o + __ldg(a.adj_s + an.q0 + j1)) : 0u;
+                const uint32_t *e = a.pool + (q >> 24);
+                const int len = (int)(q & 0xffffffu);
+                const uint32_t rmask = (1u << an.part) - 1u;
+                for (int j0 = part * 32 + lane; j0 < len; j0 += 128 * g) {
+                    uint32_t c[4];
+                    int32_t k[4];
+#pragma unroll
+                    for (int u = 0; u < 4; u++) {
+                        const int j = j0 + u * 32 * g;
+                        c[u] = j < len ? __ldg(e + j) : 0u;
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; u++) {
+                        k[u] = c[u] ? an.kb + (int32_t)(c[u] & rmask) : -1;
+                        c[u] >>= an.part;
+                    }
+                    emit.many<4>(k, c);
+                }
+                for (j1 += 32 * g; j1 < an.deg; j1 += 32 * g)
+                    walk += (uint32_t)__ldcg(a.len_o + __ldg(a.adj_s + an.q0 + j1));
+                walk = __reduce_add_sync(0xffffffffu, walk);
+                const uint32_t pr = __reduce_add_sync(0xffffffffu, (uint32_t)emit.pairs);
+                emit.pairs = 0;
+                if (lane == 0) {
+                    uint32_t *t = s_tier + an.w;  // 0: the warp tier's, 4: the windows'
+                    atomicAdd(t, walk);
+                    if (pr) atomicAdd(t + 1, pr);
+                    if (part == 0) {
+                        atomicAdd(t + 2, (uint32_t)an.deg);
+                        atomicAdd(t + 3, 1u);
+                    }
+                }
+            }
+            __syncthreads();
+            if (threadIdx.x < 8 && s_tier[threadIdx.x]) {
+                unsigned long long *to[4] = {st->tier_w, st->tier_p, st->tier_m, st->tier_a};
+                atomicAdd(to[threadIdx.x & 3] + (threadIdx.x & 4), (unsigned long long)s_tier[threadIdx.x]);
+                s_tier[threadIdx.x] = 0;
+            }
+        }
+        if (!LISTS && nW > 0) {
             WarpTable T{H.cnt + warp * (2 * WARP_SLOTS), H.cnt + warp * (2 * WARP_SLOTS) + WARP_SLOTS};
             for (int i = gwarp; i < nW;) {
                 const PersistAnchor an = load_anchor(a.Lw + i);
@@ -812,7 +881,7 @@ __global__ void __launch_bounds__(PT, 2) k_cd_persist(PersistArgs a) {
         // items per fetch: more than one only when the round has more items
         // than CTAs
         const int G = max(1, min(GROUP, nD / (int)gridDim.x));
-        for (int base = blockIdx.x * G; base < nD;) {
+        for (int base = blockIdx.x * G; !LISTS && base < nD;) {
             const int gcount = min(G, nD - base);
             for (int i0 = 0; i0 < gcount;) {
                 if (warp == 0) {
@@ -931,6 +1000,31 @@ bool cd_persist_wide(const Decomp &D) {
     return !D.parts && mean < (D.n > DENSE_KEYS ? 8192u : 1024u);
 }
 
+// Lists pay where a vertex's key space is at most two windows and the walks of
+// all vertices at once (5 ms per 10^9 wedges; with the working lists compacted
+// between ranges the rounds walk a third to a half of them) cost less than what
+// the rounds save: 2 to 5 us each, of some 400, or 1,300 in a large union.
+// 5,000 x 20,000, 200k edges: the whole call 5.7 ms, 7.0 without; 30,000 x 9,000,
+// 300k, from the host 7.2 / 9.7; 2,000 x 500, 20k, 1.8 / 2.3; 256 packed graphs
+// (1.9 10^9 wedges) 36 / 44; 40,000 x 400,000, 3M (9 10^8) 23.5 / 25.4; but 36,000
+// x 1M, 10M (over 2 10^9) 44 / 42. Larger sides count a walk in slices and lose
+// more: 120,000 x 40,000, 3M, 36 / 30 for the step; 140,000 x 14,000, 2M, 60 / 31.
+// Sides of several windows with short walks keep the groups (100,000 x 30,000
+// uniform, 1M edges: 1.1 / 0.8). Not beside other units of the serving engine
+// (list_bound): the walks take every SM, and the other units' cooperative
+// launches wait for them (24 requests of 10k-1M edges: 57.4 / 56.4).
+bool cd_persist_by_lists(const Decomp &D) {
+    // (the counters of a round by lists are 32 bits wide)
+    if (D.list_bound || D.max_deg_s >= 65535 ||
+        D.wedges_bup + (uint64_t)D.m > (D.parts ? 3000000000ull : 1200000000ull))
+        return false;
+    if (!D.parts)
+        return D.n <= 2 * DENSE_KEYS && (D.n <= DENSE_KEYS || !cd_persist_wide(D));
+    for (size_t i = 0; i + 1 < D.parts->size(); i++)
+        if ((*D.parts)[i + 1] - (*D.parts)[i] > DENSE_KEYS) return false;
+    return true;
+}
+
 bool cd_persist_fits(const Decomp &D) {
     if (D.max_deg_s >= 65535) return false;  // counts may need 32 bits
     if (!D.parts) {
@@ -950,12 +1044,14 @@ bool cd_persist_fits(const Decomp &D) {
     return true;
 }
 
-static const void *persist_kernel(bool wide) {
-    return wide ? (const void *)k_cd_persist<true> : (const void *)k_cd_persist<false>;
+static const void *persist_kernel(int form) {
+    return form == PERSIST_LISTS    ? (const void *)k_cd_persist<PERSIST_LISTS>
+           : form == PERSIST_GROUPS ? (const void *)k_cd_persist<PERSIST_GROUPS>
+                                    : (const void *)k_cd_persist<PERSIST_WINDOWS>;
 }
 
-int cd_persist_grid(int64_t m, bool wide) {
-    const void *kernel = persist_kernel(wide);
+int cd_persist_grid(int64_t m, int form) {
+    const void *kernel = persist_kernel(form);
     allow_max_smem(kernel);
     int occ = 0;
     RC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, PT, persist_smem()));
@@ -969,10 +1065,10 @@ int cd_persist_grid(int64_t m, bool wide) {
     return (int)std::min<int64_t>(num_sms() * std::min(occ, 2), std::max<int64_t>(16, m / 4096));
 }
 
-void cd_persist_launch(const PersistArgs &a, int grid, bool wide, cudaStream_t s) {
+void cd_persist_launch(const PersistArgs &a, int grid, int form, cudaStream_t s) {
     void *args[] = {(void *)&a};
     RC_CUDA(cudaMemsetAsync(&a.pd->bar, 0, sizeof(unsigned), s));
-    RC_CUDA(cudaLaunchCooperativeKernel(persist_kernel(wide), dim3(grid), dim3(PT), args,
+    RC_CUDA(cudaLaunchCooperativeKernel(persist_kernel(form), dim3(grid), dim3(PT), args,
                                         persist_smem(), s));
     RC_LAUNCH();
 }

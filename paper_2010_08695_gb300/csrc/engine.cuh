@@ -196,6 +196,12 @@ constexpr int FP_WORDS = 1024;           // counter words of a warp
 constexpr int32_t FP_HASH_DEG = 1024;    // counts of the table's entries
 constexpr int32_t FP_MAX_NI = (1 << 22) - 2;  // keys of the table's entries
 
+// An entry of an update list holds the rank in its low fp_rank_bits, the count
+// above.
+__device__ __forceinline__ int fp_rank_bits(int32_t ni) {
+    return max(1, 32 - __clz(ni - 1));
+}
+
 __device__ __forceinline__ void fp_table_add(uint32_t *slot, uint32_t mask, int32_t key) {
     const uint32_t k = ((uint32_t)key + 1u) << 10;
     uint32_t h = (hash_key(key) >> 8) & mask;

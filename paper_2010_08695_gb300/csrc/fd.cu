@@ -287,6 +287,7 @@ struct FdArgs {
 };
 
 struct FdMids {
+    static constexpr bool LARGE_FIRST = false;
     const int64_t *fd_beg;
     const int32_t *fd_len;
     __device__ __forceinline__ void seg(int64_t q, int64_t &beg, int32_t &len) const {
@@ -370,9 +371,6 @@ constexpr int FP_BLOCK = 1024;           // pool entries taken at a time
 constexpr int64_t FP_MEMBER_COST = 128;  // a member's fixed cost in wedges
 // An entry holds the rank in its low fp_rank_bits and the count above.
 constexpr unsigned long long FP_NONE = ~0ull;  // no list; else offset << 24 | length
-__device__ __forceinline__ int fp_rank_bits(int32_t ni) {
-    return max(1, 32 - __clz(ni - 1));
-}
 
 struct FdPairArgs {
     const int32_t *tstart, *tlen, *tkb;
@@ -382,9 +380,7 @@ struct FdPairArgs {
     int32_t nitems;
     int32_t *qhead;
     const FdMember *info;     // by member position
-    const int64_t *fd_beg;
-    const int32_t *fd_len;
-    const int32_t *fd_adj;
+    const int32_t *keys;      // the runs' keys
     uint32_t *pool;
     unsigned long long cap;   // entries
     unsigned long long *head;
@@ -440,7 +436,8 @@ __global__ void k_listless(const FdMember *__restrict__ info, int32_t n,
         atomicAdd(&lw[t], (unsigned long long)m.w);
 }
 
-__global__ void __launch_bounds__(FP_THREADS, 2) k_fd_pairs(FdPairArgs a) {
+template <class Mids>
+__global__ void __launch_bounds__(FP_THREADS, 2) k_fd_pairs(FdPairArgs a, Mids M) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_item;
     __shared__ int s_cnt[FP_WARPS];                  // entries found by each warp
@@ -449,15 +446,15 @@ __global__ void __launch_bounds__(FP_THREADS, 2) k_fd_pairs(FdPairArgs a) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int j = threadIdx.x; j < FP_WARPS * FP_WORDS / 4; j += FP_THREADS)
         ((uint4 *)tab)[j] = make_uint4(0, 0, 0, 0);
-    FdMids M{a.fd_beg, a.fd_len};
     unsigned long long wedges = 0;             // lane 0
     unsigned long long blk = 0, blk_end = 0;   // lane 0: this warp's pool block
     for (;;) {
         __syncthreads();
         if (threadIdx.x == 0) s_item = atomicAdd(a.qhead, 1);
         __syncthreads();
-        const int it = a.nitems - 1 - s_item;  // the largest walks come last in position order
-        if (it < 0) break;
+        if (s_item >= a.nitems) break;
+        // the largest walks first: last in a task's order, first in a side's
+        const int it = Mids::LARGE_FIRST ? s_item : a.nitems - 1 - s_item;
         const int32_t p0 = a.item_p[it], p1 = a.item_p[it + 1];
         // last task starting at or before p0
         int32_t t = 0;
@@ -501,13 +498,13 @@ __global__ void __launch_bounds__(FP_THREADS, 2) k_fd_pairs(FdPairArgs a) {
                                 if (slices > 1 && ((k >> 14) & (slices - 1)) != sc) return;
                                 atomicAdd(&w[k & wmask], 1u << ((k >> pl.lw) * pl.bits));
                             };
-                            warp_walk<4>(M, m.q0, m.q0 + m.deg, a.fd_adj, add, part, g);
+                            warp_walk<4>(M, m.q0, m.q0 + m.deg, a.keys, add, part, g);
                         } else {
                             auto add = [&](int32_t key) {
                                 const int32_t k = key - kb;
                                 if (k != self) fp_table_add(w, wmask, k);
                             };
-                            warp_walk<4>(M, m.q0, m.q0 + m.deg, a.fd_adj, add, part, g);
+                            warp_walk<4>(M, m.q0, m.q0 + m.deg, a.keys, add, part, g);
                         }
                         fp_sync(grp, g);
                         // entries in words 4 sl .. 4 sl + 3 of this lane
@@ -2032,7 +2029,7 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
     if (nheavy < T) {
         unsigned long long wtot = 0;
         for (int k = nheavy; k < T; k++) wtot += tw[hq[k]];
-        allow_max_smem((const void *)k_fd_pairs);
+        allow_max_smem((const void *)k_fd_pairs<FdMids>);
         const int ctas = 2 * sms;
         const unsigned long long cap =
             std::min(pool_cap, wtot / 2) + (unsigned long long)ctas * FP_WARPS * FP_BLOCK;
@@ -2055,9 +2052,10 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
         k_pair_items<<<ceil_div(nitems + 1, 256), 256, 0, s>>>(cw.get(), n, Q, nitems, items.get());
         RC_LAUNCH();
         FdPairArgs a{d_tstart.get(), d_tlen.get(), d_tkb.get(), dskip.get(), T, items.get(), nitems,
-                     pq.get(), info.get(), fd_beg.get(), fd_len.get(), fd_adj.get(), pool.get(), cap,
-                     head.get(), rec.get(), stats.get()};
-        k_fd_pairs<<<std::min(ctas, nitems), FP_THREADS, FP_WARPS * FP_WORDS * 4, s>>>(a);
+                     pq.get(), info.get(), fd_adj.get(), pool.get(), cap, head.get(), rec.get(),
+                     stats.get()};
+        k_fd_pairs<<<std::min(ctas, nitems), FP_THREADS, FP_WARPS * FP_WORDS * 4, s>>>(
+            a, FdMids{fd_beg.get(), fd_len.get()});
         RC_LAUNCH();
     }
     // large and small tasks side by side
@@ -2145,6 +2143,97 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
     D.fd_max_n = worst >= 0 ? tlen[worst] : 0;
     D.fd_max_levels = worst >= 0 ? (int64_t)hlv[worst] : 0;
     D.fd_tasks = T;
+}
+
+namespace {
+
+// Middle vertices of a side's vertices, whole lists.
+struct SideMids {
+    static constexpr bool LARGE_FIRST = true;
+    const int32_t *adj_s;
+    const int64_t *off_o;
+    __device__ __forceinline__ void seg(int64_t q, int64_t &beg, int32_t &len) const {
+        const int32_t y = adj_s[q];
+        beg = off_o[y];
+        len = (int32_t)(off_o[y + 1] - beg);
+    }
+};
+
+__global__ void k_side_members(const int64_t *__restrict__ off_s,
+                               const unsigned long long *__restrict__ wfull, int32_t n, int64_t add,
+                               FdMember *__restrict__ info, int64_t *__restrict__ cost) {
+    const int32_t x = blockIdx.x * blockDim.x + threadIdx.x;
+    if (x >= n) return;
+    const unsigned long long w = wfull[x];
+    info[x] = FdMember{off_s[x], (int32_t)(off_s[x + 1] - off_s[x]),
+                       (uint32_t)(w < 0xffffffffull ? w : 0xffffffffull)};
+    cost[x] = (int64_t)w + add;
+}
+
+}  // namespace
+
+bool side_pair_lists(const Decomp &D, PairLists &L, cudaStream_t s) {
+    const int32_t n = D.n;
+    const int64_t m = D.m;
+    if (n > FP_MAX_NI || m == 0) return false;
+    const int T = D.parts ? (int)D.parts->size() - 1 : 1;
+    std::vector<int32_t> ts(T), tl(T);
+    for (int t = 0; t < T; t++) {
+        ts[t] = D.parts ? (int32_t)(*D.parts)[t] : 0;
+        tl[t] = (D.parts ? (int32_t)(*D.parts)[t + 1] : n) - ts[t];
+    }
+    const int ctas = 2 * num_sms();
+    const unsigned long long w = D.wedges_bup + (unsigned long long)m;  // sum of wfull
+    const unsigned long long small = (unsigned long long)(FD_LIST_BYTES / 4 * m);
+    const unsigned long long cap =
+        (w / 2 <= small
+             ? w / 2
+             : std::min(w / 2, std::max(small, (unsigned long long)available_bytes() / 32))) +
+        (unsigned long long)ctas * FP_WARPS * FP_BLOCK;
+    DevBuf<FdMember> info(n, s);
+    DevBuf<int64_t> cost(n + 1, s), cw(n + 1, s);
+    DevBuf<int32_t> dts(T, s), dtl(T, s), pq(1, s);
+    DevBuf<uint8_t> skip(T, s);
+    DevBuf<unsigned long long> scal(2 + T, s);  // pool head, wedges, weights without lists
+    RC_CUDA(cudaMemcpyAsync(dts.get(), ts.data(), 4 * (size_t)T, cudaMemcpyHostToDevice, s));
+    RC_CUDA(cudaMemcpyAsync(dtl.get(), tl.data(), 4 * (size_t)T, cudaMemcpyHostToDevice, s));
+    skip.zero();
+    scal.zero();
+    pq.zero();
+    RC_CUDA(cudaMemsetAsync(cost.get() + n, 0, 8, s));
+    k_side_members<<<ceil_div(n, 256), 256, 0, s>>>(D.S->off, D.wfull, n, FP_MEMBER_COST, info.get(),
+                                                    cost.get());
+    RC_LAUNCH();
+    scan_exclusive<int64_t>(cost.get(), cw.get(), n + 1, s);
+    const unsigned long long total = w + (unsigned long long)n * FP_MEMBER_COST;
+    const int64_t Q = std::max<int64_t>(8192, (int64_t)(total / (8ull * ctas)));
+    const int32_t nitems = (int32_t)(total / Q + 1);
+    DevBuf<int32_t> items(nitems + 1, s);
+    k_pair_items<<<ceil_div(nitems + 1, 256), 256, 0, s>>>(cw.get(), n, Q, nitems, items.get());
+    RC_LAUNCH();
+    k_listless<<<ceil_div(n, 256), 256, 0, s>>>(info.get(), n, dts.get(), dtl.get(), T,
+                                                *std::max_element(tl.begin(), tl.end()),
+                                                scal.get() + 2);
+    RC_LAUNCH();
+    L.pool.alloc((size_t)cap, s);
+    L.rec.alloc(n, s);
+    allow_max_smem((const void *)k_fd_pairs<SideMids>);
+    // keys are vertices: a task's first key is its first vertex
+    FdPairArgs a{dts.get(), dtl.get(), dts.get(), skip.get(), T, items.get(), nitems, pq.get(),
+                 info.get(), D.O->adj, L.pool.get(), cap, scal.get(), L.rec.get(), scal.get() + 1};
+    k_fd_pairs<<<std::min(ctas, nitems), FP_THREADS, FP_WARPS * FP_WORDS * 4, s>>>(
+        a, SideMids{D.S->adj, D.O->off});
+    RC_LAUNCH();
+    std::vector<unsigned long long> h(2 + T);
+    RC_CUDA(cudaMemcpyAsync(h.data(), scal.get(), 8 * (size_t)(2 + T), cudaMemcpyDeviceToHost, s));
+    RC_CUDA(cudaStreamSynchronize(s));
+    unsigned long long listless = 0;
+    for (int t = 0; t < T; t++) listless += h[2 + t];
+    L.wedges = h[1];
+    if (h[0] <= cap && listless == 0) return true;
+    L.pool.release();
+    L.rec.release();
+    return false;
 }
 
 }  // namespace receipt

@@ -134,4 +134,15 @@ void compact_lists(const int64_t *off_o, int32_t *len_w, int32_t *adj_w, int32_t
 void list_lengths(const int64_t *off, int32_t n, int32_t *len, cudaStream_t s);
 void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s);
 
+// Every vertex's updates of the others on its side (in a union: of its graph's):
+// rec[x] = offset << 24 | length of its entries in the pool, rank of the other
+// in its graph and shared neighbours (>= 2) above pair_rank_bits.
+struct PairLists {
+    DevBuf<uint32_t> pool;
+    DevBuf<unsigned long long> rec;
+    unsigned long long wedges = 0;  // walked
+};
+// False (and nothing kept) unless every vertex could get a list. Synchronises s.
+bool side_pair_lists(const Decomp &D, PairLists &L, cudaStream_t s);
+
 }  // namespace receipt

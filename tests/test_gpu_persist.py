@@ -84,3 +84,26 @@ def test_short_walks(R, d, w, pad):
         t = R.as_u64(g.tip_decompose(0, round_graphs=-1, **kw))
         assert np.array_equal(t, want), kw
         assert recs == _rounds(g), kw
+
+
+# updates by lists made beforehand, counters of 16 bits in slices of a CTA's
+# words; two windows' keys are the most a listed side has
+@pytest.mark.parametrize("n", [3000, 40_000, 73_728, 73_729])
+def test_lists_of_hubs(R, n):
+    nv, hubs, deg = 2000, 40, 600
+    rng = np.random.default_rng(n)
+    hu = rng.choice(n, hubs, replace=False)
+    ru, rv = synth.er(n, nv, 2 * n, seed=n)
+    eu = np.concatenate([np.repeat(hu, deg), ru]).astype(np.int32)
+    ev = np.concatenate([rng.choice(nv, deg, replace=False) for _ in range(hubs)] + [rv]).astype(np.int32)
+    key = np.unique(eu.astype(np.int64) * nv + ev)
+    eu, ev = (key // nv).astype(np.int32), (key % nv).astype(np.int32)
+    want, _ = oracle.bup(eu, ev, n, nv, 0)
+    g = R.Graph(eu, ev, n, nv)
+    for kw in ({}, {"P": 5}, {"huc": -1}):
+        t = R.as_u64(g.tip_decompose(0, **kw))
+        assert np.array_equal(t, want), kw
+        recs = _rounds(g)
+        t = R.as_u64(g.tip_decompose(0, round_graphs=-1, **kw))
+        assert np.array_equal(t, want), kw
+        assert recs == _rounds(g), kw
