@@ -124,8 +124,10 @@ __device__ __forceinline__ void emit_many(E &e, const int32_t (&k)[N], const uin
 // Walks the segments of the middle vertices q in [q0, q1) with one warp, 32
 // middle vertices at a time: lane i fetches segment i, a warp scan of the
 // lengths numbers their wedges, and each lane takes wedges lane, lane + 32,
-// ..., finding its segment by a binary search over the lanes' starts, so all
-// key loads of a step are independent (U per lane in flight). visit(key).
+// ..., finding its segment by one vote and one reduction over the starts (with
+// a binary search by shuffles the list walks of 256 packed graphs took 8.6 ms,
+// 7.6 so), so all key loads of a step are independent (U per lane in flight).
+// visit(key).
 // A group of `parts` warps shares the walk by calls with part = 0 .. parts - 1:
 // blocks of 32 middle vertices when each warp has two or more, else the wedges
 // of every block.
@@ -145,6 +147,18 @@ __device__ __forceinline__ void warp_walk(const Mids &M, int64_t q0, int64_t q1,
         int64_t beg = 0;
         int32_t len = 0;
         if (qb + lane < q1) M.seg(qb + lane, beg, len);
+        // non-empty segments to the front
+        const unsigned nz = __ballot_sync(0xffffffffu, len > 0);
+        const int ns = __popc(nz);
+        if (nz & (nz + 1)) {
+            int src = 0;  // lane of the lane-th non-empty segment
+#pragma unroll
+            for (int step = 16; step > 0; step >>= 1)
+                if (__popc(nz & ((1u << (src + step)) - 1u)) <= lane) src += step;
+            beg = __shfl_sync(0xffffffffu, beg, src);
+            const int32_t l = __shfl_sync(0xffffffffu, len, src);
+            len = lane < ns ? l : 0;
+        }
         int32_t inc = len;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -152,23 +166,22 @@ __device__ __forceinline__ void warp_walk(const Mids &M, int64_t q0, int64_t q1,
             if (lane >= o) inc += y;
         }
         const int32_t total = __shfl_sync(0xffffffffu, inc, 31);
-        const int32_t ex = inc - len;
+        const int32_t ex = lane < ns ? inc - len : INT32_MAX;
+        const int64_t at = beg - (inc - len);  // of wedge 0, were it in this segment
         for (int32_t j0 = part * 32; j0 < total; j0 += 32 * U * parts) {
             int32_t key[U];
 #pragma unroll
             for (int u = 0; u < U; u++) {
-                const int32_t j = j0 + u * 32 * parts + lane;
-                // last lane whose segment starts at or before j (all lanes
-                // take part in the shuffles)
-                int lo = 0;
-#pragma unroll
-                for (int step = 16; step > 0; step >>= 1) {
-                    const int32_t e = __shfl_sync(0xffffffffu, ex, lo + step);
-                    if (e <= j) lo += step;
-                }
-                const int64_t b = __shfl_sync(0xffffffffu, beg, lo);
-                const int32_t e0 = __shfl_sync(0xffffffffu, ex, lo);
-                key[u] = j < total ? Keys::load(keys + b + (j - e0)) : -1;
+                const int32_t base = j0 + u * 32 * parts, j = base + lane;
+                // segments that start at or before `base`, and those that start
+                // further on among the step's 32 wedges (all lanes take part)
+                const int before = __popc(__ballot_sync(0xffffffffu, ex <= base));
+                const uint32_t d = (uint32_t)(ex - base);
+                const uint32_t in =
+                    __reduce_or_sync(0xffffffffu, ex > base && d < 32u ? 1u << d : 0u);
+                const int seg = before - 1 + __popc(in & (lanemask_lt() | (1u << lane)));
+                const int64_t a = __shfl_sync(0xffffffffu, at, seg);
+                key[u] = j < total ? Keys::load(keys + a + j) : -1;
             }
 #pragma unroll
             for (int u = 0; u < U; u++)

@@ -361,7 +361,8 @@ struct FdEmit {
 // The entries lie in one pool, taken by each group in blocks; a member whose
 // list does not fit it, or that is too large for all this, has no list and
 // walks when it is peeled.
-// Two CTAs of 16 warps an SM: bound by the latency of runs and keys from L2.
+// Two CTAs of 16 warps an SM: bound by instruction issue (60% of the slots, the
+// rest mostly fixed-latency waits and group barriers; DRAM under 1%).
 // 1.93e9 wedges of a 40M-edge graph in 9.1 ms, 3.9e8 of a 10M-edge graph in 3.0
 // ms; walked during the peel they made the whole step 101 and 26 ms (34 and 10
 // now).
