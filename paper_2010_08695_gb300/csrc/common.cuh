@@ -64,16 +64,21 @@ class DevBuf {
         return *this;
     }
     void alloc(size_t n, cudaStream_t s) {
+        if (!try_alloc(n, s))
+            fail(RECEIPT_ERR_OOM,
+                 "device allocation of " + std::to_string((n ? n : 1) * sizeof(T)) + " bytes failed");
+    }
+    // False, and empty, when there is no memory.
+    bool try_alloc(size_t n, cudaStream_t s) {
         release();
         s_ = s;
-        n_ = n;
-        size_t bytes = (n ? n : 1) * sizeof(T);
-        cudaError_t e = cudaMallocAsync((void **)&p_, bytes, s);
-        if (e != cudaSuccess) {
+        if (cudaMallocAsync((void **)&p_, (n ? n : 1) * sizeof(T), s) != cudaSuccess) {
             cudaGetLastError();
             p_ = nullptr;
-            fail(RECEIPT_ERR_OOM, "device allocation of " + std::to_string(bytes) + " bytes failed");
+            return false;
         }
+        n_ = n;
+        return true;
     }
     void zero() {
         if (p_) RC_CUDA(cudaMemsetAsync(p_, 0, (n_ ? n_ : 1) * sizeof(T), s_));

@@ -2022,6 +2022,7 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
         }
         RC_CUDA(cudaMemcpyAsync(qhead.get(), &nheavy, 4, cudaMemcpyHostToDevice, s));
     }
+    DevBuf<unsigned long long> rtip(nsmall_at < T ? n : 1, s);
     // the members' lists: walks in items of equal cost, 8 a CTA. The pool has
     // an entry per two wedges (no list is longer), up to FD_LIST_BYTES an edge
     // or an eighth of the memory there is, and each warp's last block.
@@ -2032,10 +2033,13 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
         for (int k = nheavy; k < T; k++) wtot += tw[hq[k]];
         allow_max_smem((const void *)k_fd_pairs<FdMids>);
         const int ctas = 2 * sms;
-        const unsigned long long cap =
+        unsigned long long cap =
             std::min(pool_cap, wtot / 2) + (unsigned long long)ctas * FP_WARPS * FP_BLOCK;
-        pool.alloc((size_t)cap, s);
         rec.alloc(n, s);
+        if (!pool.try_alloc((size_t)cap, s)) {
+            cap = 0;  // no memory: members walk when they are peeled
+            pool.alloc(1, s);
+        }
         RC_CUDA(cudaMemsetAsync(rec.get(), 0xff, 8 * (size_t)n, s));
         DevBuf<unsigned long long> head(1, s);
         DevBuf<int32_t> pq(1, s);
@@ -2055,12 +2059,13 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
         FdPairArgs a{d_tstart.get(), d_tlen.get(), d_tkb.get(), dskip.get(), T, items.get(), nitems,
                      pq.get(), info.get(), fd_adj.get(), pool.get(), cap, head.get(), rec.get(),
                      stats.get()};
-        k_fd_pairs<<<std::min(ctas, nitems), FP_THREADS, FP_WARPS * FP_WORDS * 4, s>>>(
-            a, FdMids{fd_beg.get(), fd_len.get()});
-        RC_LAUNCH();
+        if (cap > 0) {
+            k_fd_pairs<<<std::min(ctas, nitems), FP_THREADS, FP_WARPS * FP_WORDS * 4, s>>>(
+                a, FdMids{fd_beg.get(), fd_len.get()});
+            RC_LAUNCH();
+        }
     }
     // large and small tasks side by side
-    DevBuf<unsigned long long> rtip(nsmall_at < T ? n : 1, s);
     const int nlarge = nsmall_at - nheavy, nsmall = T - nsmall_at;
     cudaEvent_t fork_ev[2] = {};
     cudaStream_t ls = s;  // the large tasks' stream
@@ -2216,8 +2221,10 @@ bool side_pair_lists(const Decomp &D, PairLists &L, cudaStream_t s) {
                                                 *std::max_element(tl.begin(), tl.end()),
                                                 scal.get() + 2);
     RC_LAUNCH();
-    L.pool.alloc((size_t)cap, s);
-    L.rec.alloc(n, s);
+    if (!L.pool.try_alloc((size_t)cap, s) || !L.rec.try_alloc(n, s)) {
+        L.pool.release();
+        return false;
+    }
     allow_max_smem((const void *)k_fd_pairs<SideMids>);
     // keys are vertices: a task's first key is its first vertex
     FdPairArgs a{dts.get(), dtl.get(), dts.get(), skip.get(), T, items.get(), nitems, pq.get(),
