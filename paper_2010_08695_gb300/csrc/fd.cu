@@ -1706,6 +1706,70 @@ static void fdh_levels_with_recount(Decomp &D, const FdhArgs &ha, FdhDev *dst, F
     RC_CUDA(cudaMemcpyAsync(hst_out, dst, sizeof(FdhDev), cudaMemcpyDeviceToHost, s));
 }
 
+// A task peeled from lists: its members, its walks' wedges, its range.
+struct ListTask {
+    int32_t id, n;
+    unsigned long long w;
+    uint64_t lo, hi;
+};
+
+// Tasks that all CTAs peel sooner than one CTA applies their lists. One CTA
+// takes 2.5 us a level and 0.85 ns an entry, all CTAs ~70 us a level and 3 ps a
+// wedge (the lists themselves 1.7 ps), so what decides is the entries a level
+// peels: heavy wins from ~10^5. Power-law graphs have at most 1.5 10^4, a level
+// a member or two; uniform and dense ones, whose supports lie so close that one
+// level sets off the next, 10^5 to 10^7 (20M edges, 30,000 members, 524 levels,
+// 3.8 10^8 entries: 317 ms in one CTA, 109 heavy; 6M edges, 37,500 members, 92
+// levels: 1,301 / 174; 2M edges, 4,700 members, 52 levels: 18.8 / 7.2; but 2M
+// edges, 18,000 members, 39 levels: 1.8 / 2.2).
+// Neither is known before the peel. Levels: at most a member each, and while
+// every peeled member sets off others as many as the range's share of its bound
+// (the narrowest ranges, one bucket, hold 1/32), or 16 to each support of a
+// range of few supports (measured: 1.2 to 14 times fewer). Entries: a fourth of
+// the wedges (measured: up to 0.3), at most one for every two members, and what
+// pairs of members that share c << 1 middle vertices on average make of them,
+// c^2 / 2 each.
+// One CTA a task peels the tasks left side by side, the heavy ones come one by
+// one: the longest go first while the sum falls.
+static std::vector<int32_t> heavy_by_lists(std::vector<ListTask> t, int ctas) {
+    auto levels = [](const ListTask &k) {
+        const double span = (double)(k.hi - k.lo);
+        return std::max(1.0, std::min((double)k.n * std::min(1.0, span / (double)k.hi),
+                                      std::min((double)k.n, 16.0 * span)));
+    };
+    auto by_list = [&](const ListTask &k) {
+        const double w = (double)k.w, pairs = (double)k.n * (double)k.n;
+        const double e = std::min({w / 4, pairs, w * (w / pairs) / 2});
+        return 2500.0 * levels(k) + 0.85 * e;
+    };
+    auto heavy = [&](const ListTask &k) { return 7e4 * levels(k) + 0.003 * (double)k.w; };
+    std::stable_sort(t.begin(), t.end(),
+                     [&](const ListTask &a, const ListTask &b) { return by_list(a) > by_list(b); });
+    double left = 0, walks = 0;  // of the tasks not heavy
+    for (const ListTask &k : t) {
+        left += by_list(k);
+        walks += 0.0017 * (double)k.w;
+    }
+    double first = 0, best = 0, sum = 0;
+    size_t n = 0;
+    for (size_t k = 0; k <= t.size(); k++) {
+        const double now = sum + walks + std::max(k < t.size() ? by_list(t[k]) : 0.0, left / ctas);
+        if (k == 0) first = best = now;
+        if (now < best && now < 0.9 * first) {
+            best = now;
+            n = k;
+        }
+        if (k == t.size()) break;
+        sum += heavy(t[k]);
+        left -= by_list(t[k]);
+        walks -= 0.0017 * (double)t[k].w;
+        if (sum > best) break;
+    }
+    std::vector<int32_t> out;
+    for (size_t k = 0; k < n; k++) out.push_back(t[k].id);
+    return out;
+}
+
 void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
     const int32_t n = D.n;
     const int64_t m = D.m;
@@ -1875,9 +1939,10 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
     // lists would not fit the pool); (b) tasks of HEAVY_NI members and more
     // with a range so narrow that few levels peel them: a one-CTA level scans
     // at ~8 ns a member (1.9M members, width 1, one level: 16 ms, 0.8 heavy;
-    // 132K members, width 1, 28 levels: 27 ms for the step, 29 unless heavy).
-    // With lists nothing else gains: 4,751 levels of 80K members take 36 ms in
-    // one CTA and took 590 heavy, 20,000 levels of 42K members 117 ms.
+    // 132K members, width 1, 28 levels: 27 ms for the step, 29 unless heavy);
+    // (c) tasks whose lists are long for their levels (heavy_by_lists).
+    // Otherwise one CTA is faster: 4,751 levels of 80K members take 36 ms
+    // there and took 590 heavy, 20,000 levels of 42K members 117 ms.
     const unsigned long long pool_cap = [&]() {
         unsigned long long w = 0;
         for (int k = 0; k < T; k++) w += tw[k];
@@ -1906,6 +1971,21 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
                     : (walk >= HEAVY_MIN_W && walk >= HEAVY_WALK_LEVELS * lw) ||
                           (tlen[t] >= HEAVY_NI && width <= (uint64_t)(tlen[t] / (HEAVY_NI / 2)));
             (heavy && tlen[t] > 0 ? front : back).push_back(t);
+        }
+        if (D.fd_heavy_w == 0) {
+            std::vector<ListTask> lt;
+            for (int32_t t : back) {
+                const int sub_i = tsub[t];
+                const bool open = (size_t)sub_i + 1 >= D.bounds.size();
+                lt.push_back(ListTask{t, tlen[t], tw[t], open ? 0 : D.bounds[sub_i],
+                                      open ? ~0ull : D.bounds[sub_i + 1]});
+            }
+            const std::vector<int32_t> more = heavy_by_lists(lt, sms);
+            std::vector<bool> is(T, false);
+            for (int32_t t : more) is[t] = true;
+            front.insert(front.end(), more.begin(), more.end());
+            back.erase(std::remove_if(back.begin(), back.end(), [&](int32_t t) { return is[t]; }),
+                       back.end());
         }
         nheavy = (int)front.size();
         int pos = 0;

@@ -79,3 +79,20 @@ def test_sliced_counters(R):
     eu = np.concatenate([h, h, np.repeat(wide, 15), np.arange(n)]).astype(np.int32)
     ev = np.concatenate([np.zeros(hub), trio, own, twin]).astype(np.int32)
     _check(R, eu, ev, n, int(ev.max()) + 1, (1,))
+
+
+# supports so close together that one level sets off the next: a level then
+# peels more list entries than one CTA applies in the time of a level by all
+# CTAs (uniform and dense graphs, odd sizes); on power-law graphs a level peels
+# a member or two
+@pytest.mark.parametrize("n,nv,m,gamma,P,heavy", [
+    (5_000, 20_001, 2_000_000, 0, 150, True), (6_001, 150, 300_000, 0, 150, True),
+    (100_000, 30_000, 1_000_000, 2.4, 5, False),
+    (20_000, 30_000, 1_000_000, 2.4, 1, False)])
+def test_wide_levels_take_all_ctas(R, n, nv, m, gamma, P, heavy):
+    eu, ev = synth.chung_lu(n, nv, m, gamma, gamma, 4) if gamma else synth.er(n, nv, m, 4)
+    want, _ = oracle.bup(eu, ev, n, nv, 0)
+    g = R.Graph(eu, ev, n, nv)
+    t = R.as_u64(g.tip_decompose(0, P=P))
+    assert np.array_equal(t, want)
+    assert (g.stats()["fd_heavy_subsets"] > 0) == heavy
