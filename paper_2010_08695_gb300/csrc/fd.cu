@@ -44,9 +44,10 @@ constexpr unsigned long long WIDE_BIT = 1ull << 63;
 // heavy tasks, automatic rule
 constexpr unsigned long long HEAVY_MIN_W = 1ull << 23;
 constexpr int32_t HEAVY_NI = 1 << 17;
-// list entries are at most an eighth of the walks' wedges (measured: 1/10 to
-// 1/14 on Chung-Lu graphs, far fewer on uniform ones)
-constexpr unsigned long long LIST_SHARE = 8;
+// All lists' entries are about a sixth of their walks' wedges at most: 1/8 to
+// 1/16 on Chung-Lu graphs of 1M to 40M edges; uniform and dense graphs have up to
+// 1/3, but all CTAs peel their long tasks without lists.
+constexpr unsigned long long LIST_SHARE = 6;
 // a level of a heavy task with at most this many members with big walks
 // (and at least two CTAs for each) splits each one's walk over the CTAs
 // (partial counts summed in global counters) instead of giving each member
@@ -372,6 +373,14 @@ constexpr int FP_BLOCK = 1024;           // pool entries taken at a time
 constexpr int64_t FP_MEMBER_COST = 128;  // a member's fixed cost in wedges
 // An entry holds the rank in its low fp_rank_bits and the count above.
 constexpr unsigned long long FP_NONE = ~0ull;  // no list; else offset << 24 | length
+
+// Pool entries of the lists of n vertices of w wedges together, at most: one for
+// two wedges, one for each other vertex (twice that where a block's end may stay
+// unused because the next list is longer).
+inline unsigned long long lists_at_most(unsigned long long w, int32_t n) {
+    const unsigned long long pairs = (unsigned long long)n * (unsigned long long)n;
+    return std::min(w / 2, n < 2 * FP_BLOCK ? 2 * pairs : pairs);
+}
 
 struct FdPairArgs {
     const int32_t *tstart, *tlen, *tkb;
@@ -1943,19 +1952,21 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
     // (c) tasks whose lists are long for their levels (heavy_by_lists).
     // Otherwise one CTA is faster: 4,751 levels of 80K members take 36 ms
     // there and took 590 heavy, 20,000 levels of 42K members 117 ms.
-    const unsigned long long pool_cap = [&]() {
-        unsigned long long w = 0;
-        for (int k = 0; k < T; k++) w += tw[k];
-        const unsigned long long small = (unsigned long long)(FD_LIST_BYTES / 4 * m);
-        if (w / 2 <= small) return w / 2;
-        if (D.list_bound) return small;
-        return std::min(w / 2, std::max(small, (unsigned long long)available_bytes() / 32));
-    }();
+    // The pool has room for the most entries the lists can have as long as that
+    // is cheap (FD_LIST_BYTES an edge), else for about as many as they do have
+    // (LIST_SHARE), up to an eighth of the memory there is; members past it walk.
+    unsigned long long entries_max = 0, entries = 0;
+    for (int k = 0; k < T; k++) {
+        entries_max += lists_at_most(tw[k], tlen[k]);
+        entries += std::min(tw[k] / LIST_SHARE, lists_at_most(tw[k], tlen[k]));
+    }
+    unsigned long long pool_cap = (unsigned long long)(FD_LIST_BYTES / 4 * m);
+    if (entries_max > pool_cap && entries > pool_cap && !D.list_bound)
+        pool_cap = std::max(pool_cap, std::min<unsigned long long>(entries, available_bytes() / 32));
+    pool_cap = std::min(pool_cap, entries_max);
     int nheavy = 0;
     if (D.fd_heavy_w >= 0 && T > 0) {
-        unsigned long long all = 0;
-        for (int k = 0; k < T; k++) all += tw[k];
-        const bool overflow = all / LIST_SHARE > pool_cap;
+        const bool overflow = entries > pool_cap;
         std::vector<int32_t> front, back;
         for (int k = 0; k < T; k++) {
             const int32_t t = hq[k];
@@ -2103,18 +2114,17 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
         RC_CUDA(cudaMemcpyAsync(qhead.get(), &nheavy, 4, cudaMemcpyHostToDevice, s));
     }
     DevBuf<unsigned long long> rtip(nsmall_at < T ? n : 1, s);
-    // the members' lists: walks in items of equal cost, 8 a CTA. The pool has
-    // an entry per two wedges (no list is longer), up to FD_LIST_BYTES an edge
-    // or an eighth of the memory there is, and each warp's last block.
+    // the members' lists: walks in items of equal cost, 8 a CTA. The pool also
+    // has room for each warp's last block.
     DevBuf<uint32_t> pool;
     DevBuf<unsigned long long> rec;
     if (nheavy < T) {
-        unsigned long long wtot = 0;
-        for (int k = nheavy; k < T; k++) wtot += tw[hq[k]];
+        unsigned long long most = 0;
+        for (int k = nheavy; k < T; k++) most += lists_at_most(tw[hq[k]], tlen[hq[k]]);
         allow_max_smem((const void *)k_fd_pairs<FdMids>);
         const int ctas = 2 * sms;
         unsigned long long cap =
-            std::min(pool_cap, wtot / 2) + (unsigned long long)ctas * FP_WARPS * FP_BLOCK;
+            std::min(pool_cap, most) + (unsigned long long)ctas * FP_WARPS * FP_BLOCK;
         rec.alloc(n, s);
         if (!pool.try_alloc((size_t)cap, s)) {
             cap = 0;  // no memory: members walk when they are peeled
@@ -2270,11 +2280,15 @@ bool side_pair_lists(const Decomp &D, PairLists &L, cudaStream_t s) {
     }
     const int ctas = 2 * num_sms();
     const unsigned long long w = D.wedges_bup + (unsigned long long)m;  // sum of wfull
+    // every vertex must get its list, so there is room for them all
+    unsigned long long most = 0;
+    for (int t = 0; t < T; t++) most += lists_at_most(w, tl[t]);
+    most = std::min(most, w / 2);
     const unsigned long long small = (unsigned long long)(FD_LIST_BYTES / 4 * m);
     const unsigned long long cap =
-        (w / 2 <= small
-             ? w / 2
-             : std::min(w / 2, std::max(small, (unsigned long long)available_bytes() / 32))) +
+        (most <= small
+             ? most
+             : std::min(most, std::max(small, (unsigned long long)available_bytes() / 32))) +
         (unsigned long long)ctas * FP_WARPS * FP_BLOCK;
     DevBuf<FdMember> info(n, s);
     DevBuf<int64_t> cost(n + 1, s), cw(n + 1, s);

@@ -96,3 +96,34 @@ def test_wide_levels_take_all_ctas(R, n, nv, m, gamma, P, heavy):
     t = R.as_u64(g.tip_decompose(0, P=P))
     assert np.array_equal(t, want)
     assert (g.stats()["fd_heavy_subsets"] > 0) == heavy
+
+
+def _pool_high(reset=False):
+    """Most bytes in use in the device's default memory pool since the reset."""
+    import ctypes
+    import torch
+    cu, pool, v = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(), ctypes.c_uint64(0)
+    assert cu.cuDeviceGetDefaultMemPool(ctypes.byref(pool), torch.cuda.current_device()) == 0
+    if reset:  # CU_MEMPOOL_ATTR_USED_MEM_HIGH
+        assert cu.cuMemPoolSetAttribute(pool, 8, ctypes.byref(v)) == 0
+    assert cu.cuMemPoolGetAttribute(pool, 8, ctypes.byref(v)) == 0
+    return v.value
+
+
+# the lists' pool follows what they can hold: a member of a dense graph has an
+# entry for every other member however many wedges it walks, and power-law
+# graphs an entry for six wedges or more
+@pytest.mark.parametrize("nu,nv,m,gamma,P,mb", [(3_000, 3_000, 2_000_000, 0, 150, 400),
+                                                (600, 2_000, 600_000, 0, 150, 150),
+                                                (300_000, 90_000, 2_000_000, 2.3, 4, 600)])
+def test_pool_follows_the_lists(R, nu, nv, m, gamma, P, mb):
+    import torch
+    eu, ev = synth.chung_lu(nu, nv, m, gamma, gamma, 6) if gamma else synth.er(nu, nv, m, 6)
+    g = R.Graph(eu, ev, nu, nv)
+    torch.cuda.synchronize()
+    _pool_high(True)
+    t = R.as_u64(g.tip_decompose(0, P=P))
+    assert _pool_high() < mb << 20
+    if not gamma:
+        want, _ = oracle.bup(eu, ev, nu, nv, 0)
+        assert np.array_equal(t, want)
