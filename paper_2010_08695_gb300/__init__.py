@@ -138,6 +138,7 @@ def load(build_if_missing: bool = True):
         lib.receipt_last_error.restype = ctypes.c_char_p
         lib.receipt_options_default.argtypes = [ctypes.POINTER(Options)]
         lib.receipt_kernel_launches.restype = ctypes.c_uint64
+        lib.receipt_optional_memory.argtypes = [i64]
         lib.receipt_get_trace.argtypes = [vp, ctypes.POINTER(Round), i32, ctypes.POINTER(i32)]
         lib.receipt_get_trace.restype = ctypes.c_int
         lib.receipt_get_subsets.argtypes = [vp, ctypes.POINTER(Subset), i32, ctypes.POINTER(i32)]
@@ -301,6 +302,12 @@ def receipt_support_bound(n_side: int, max_deg_side: int, max_deg_other: int, m:
 def receipt_kernel_launches() -> int:
     """Kernels launched by libreceipt in this process so far."""
     return int(load().receipt_kernel_launches())
+
+
+def receipt_optional_memory(bytes: int = -1) -> None:
+    """Bounds every optional work space (it only saves time) of this thread's
+    later calls; -1: no bound, 0: none."""
+    _check(load().receipt_optional_memory(int(bytes)))
 
 
 class Graph:

@@ -14,9 +14,11 @@
 namespace receipt {
 
 static thread_local std::string g_last_error;
+static thread_local size_t g_optional = ~(size_t)0;
 static std::atomic<uint64_t> g_launches{0};
 
 void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
+size_t optional_memory() { return g_optional; }
 void count_launches(uint64_t n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 void uncount_launches(uint64_t n) { g_launches.fetch_sub(n, std::memory_order_relaxed); }
 
@@ -696,6 +698,11 @@ receipt_status receipt_get_subsets(const receipt_graph *g, receipt_subset *out, 
         for (int32_t i = 0; i < n && i < cap; i++) out[i] = g->subsets[i];
         if (n_subsets) *n_subsets = n;
     });
+}
+
+receipt_status receipt_optional_memory(int64_t bytes) {
+    g_optional = bytes < 0 ? ~(size_t)0 : (size_t)bytes;
+    return RECEIPT_OK;
 }
 
 const char *receipt_last_error(void) { return g_last_error.c_str(); }

@@ -42,6 +42,9 @@ int max_smem_optin();
 // concurrent callers cannot lower it under one another's launches.
 void allow_max_smem(const void *kernel);
 
+// Largest optional work space the calling thread may take (bytes).
+size_t optional_memory();
+
 // Stream-ordered device buffer (cudaMallocAsync / cudaFreeAsync on one stream).
 template <typename T>
 class DevBuf {
@@ -64,21 +67,18 @@ class DevBuf {
         return *this;
     }
     void alloc(size_t n, cudaStream_t s) {
-        if (!try_alloc(n, s))
+        if (!get_memory(n, s))
             fail(RECEIPT_ERR_OOM,
                  "device allocation of " + std::to_string((n ? n : 1) * sizeof(T)) + " bytes failed");
     }
-    // False, and empty, when there is no memory.
+    // For optional work space: false, and empty, when there is no memory (or not
+    // as much as the thread may take).
     bool try_alloc(size_t n, cudaStream_t s) {
-        release();
-        s_ = s;
-        if (cudaMallocAsync((void **)&p_, (n ? n : 1) * sizeof(T), s) != cudaSuccess) {
-            cudaGetLastError();
-            p_ = nullptr;
+        if ((n ? n : 1) * sizeof(T) > optional_memory()) {
+            release();
             return false;
         }
-        n_ = n;
-        return true;
+        return get_memory(n, s);
     }
     void zero() {
         if (p_) RC_CUDA(cudaMemsetAsync(p_, 0, (n_ ? n_ : 1) * sizeof(T), s_));
@@ -92,6 +92,17 @@ class DevBuf {
     size_t size() const { return n_; }
 
   private:
+    bool get_memory(size_t n, cudaStream_t s) {
+        release();
+        s_ = s;
+        if (cudaMallocAsync((void **)&p_, (n ? n : 1) * sizeof(T), s) != cudaSuccess) {
+            cudaGetLastError();
+            p_ = nullptr;
+            return false;
+        }
+        n_ = n;
+        return true;
+    }
     T *p_ = nullptr;
     size_t n_ = 0;
     cudaStream_t s_ = 0;

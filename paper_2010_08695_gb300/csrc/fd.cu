@@ -1964,54 +1964,76 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
     if (entries_max > pool_cap && entries > pool_cap && !D.list_bound)
         pool_cap = std::max(pool_cap, std::min<unsigned long long>(entries, available_bytes() / 32));
     pool_cap = std::min(pool_cap, entries_max);
-    int nheavy = 0;
-    if (D.fd_heavy_w >= 0 && T > 0) {
-        const bool overflow = entries > pool_cap;
-        std::vector<int32_t> front, back;
-        for (int k = 0; k < T; k++) {
-            const int32_t t = hq[k];
-            const unsigned long long lw = LEVEL_WEDGES * (unsigned long long)tlen[t];
-            const unsigned long long walk = overflow ? tw[t] : tlw[t];
-            const int sub_i = tsub[t];
-            const uint64_t width = (size_t)sub_i + 1 < D.bounds.size()
-                                       ? D.bounds[sub_i + 1] - D.bounds[sub_i]
-                                       : ~0ull;
-            const bool heavy =
-                D.fd_heavy_w > 0
-                    ? tw[t] >= (unsigned long long)D.fd_heavy_w
-                    : (walk >= HEAVY_MIN_W && walk >= HEAVY_WALK_LEVELS * lw) ||
-                          (tlen[t] >= HEAVY_NI && width <= (uint64_t)(tlen[t] / (HEAVY_NI / 2)));
-            (heavy && tlen[t] > 0 ? front : back).push_back(t);
-        }
-        if (D.fd_heavy_w == 0) {
-            std::vector<ListTask> lt;
-            for (int32_t t : back) {
-                const int sub_i = tsub[t];
-                const bool open = (size_t)sub_i + 1 >= D.bounds.size();
-                lt.push_back(ListTask{t, tlen[t], tw[t], open ? 0 : D.bounds[sub_i],
-                                      open ? ~0ull : D.bounds[sub_i + 1]});
-            }
-            const std::vector<int32_t> more = heavy_by_lists(lt, sms);
-            std::vector<bool> is(T, false);
-            for (int32_t t : more) is[t] = true;
-            front.insert(front.end(), more.begin(), more.end());
-            back.erase(std::remove_if(back.begin(), back.end(), [&](int32_t t) { return is[t]; }),
-                       back.end());
-        }
-        nheavy = (int)front.size();
-        int pos = 0;
-        for (int32_t t : front) hq[pos++] = t;
-        for (int32_t t : back) hq[pos++] = t;
-    }
     // Queue: the heavy tasks, then the large ones (k_fd_peel), then those of
     // at most FS_MEMBERS members (FS_WORDS with 32-bit counts; k_fd_small),
     // each in LPT order.
-    const int nsmall_at = (int)(std::stable_partition(hq.begin() + nheavy, hq.end(),
-                                                      [&](int32_t t) {
-                                                          return tlen[t] > (hwide[tsub[t]] ? FS_WORDS
-                                                                                          : FS_MEMBERS);
-                                                      }) -
-                                hq.begin());
+    const std::vector<int32_t> lpt = hq;
+    int nheavy = 0, nsmall_at = 0;
+    auto order = [&](unsigned long long cap) {
+        hq = lpt;
+        nheavy = 0;
+        if (D.fd_heavy_w >= 0 && T > 0) {
+            const bool overflow = entries > cap;
+            std::vector<int32_t> front, back;
+            for (int32_t t : lpt) {
+                const unsigned long long lw = LEVEL_WEDGES * (unsigned long long)tlen[t];
+                const unsigned long long walk = overflow ? tw[t] : tlw[t];
+                const int sub_i = tsub[t];
+                const uint64_t width = (size_t)sub_i + 1 < D.bounds.size()
+                                           ? D.bounds[sub_i + 1] - D.bounds[sub_i]
+                                           : ~0ull;
+                const bool heavy =
+                    D.fd_heavy_w > 0
+                        ? tw[t] >= (unsigned long long)D.fd_heavy_w
+                        : (walk >= HEAVY_MIN_W && walk >= HEAVY_WALK_LEVELS * lw) ||
+                              (tlen[t] >= HEAVY_NI && width <= (uint64_t)(tlen[t] / (HEAVY_NI / 2)));
+                (heavy && tlen[t] > 0 ? front : back).push_back(t);
+            }
+            if (D.fd_heavy_w == 0 && cap > 0) {
+                std::vector<ListTask> lt;
+                for (int32_t t : back) {
+                    const int sub_i = tsub[t];
+                    const bool open = (size_t)sub_i + 1 >= D.bounds.size();
+                    lt.push_back(ListTask{t, tlen[t], tw[t], open ? 0 : D.bounds[sub_i],
+                                          open ? ~0ull : D.bounds[sub_i + 1]});
+                }
+                const std::vector<int32_t> more = heavy_by_lists(lt, sms);
+                std::vector<bool> is(T, false);
+                for (int32_t t : more) is[t] = true;
+                front.insert(front.end(), more.begin(), more.end());
+                back.erase(std::remove_if(back.begin(), back.end(), [&](int32_t t) { return is[t]; }),
+                           back.end());
+            }
+            nheavy = (int)front.size();
+            int pos = 0;
+            for (int32_t t : front) hq[pos++] = t;
+            for (int32_t t : back) hq[pos++] = t;
+        }
+        nsmall_at = (int)(std::stable_partition(hq.begin() + nheavy, hq.end(),
+                                                [&](int32_t t) {
+                                                    return tlen[t] > (hwide[tsub[t]] ? FS_WORDS
+                                                                                     : FS_MEMBERS);
+                                                }) -
+                          hq.begin());
+    };
+    // The lists' pool: room for the tasks that are not heavy, and each warp's
+    // last block. Without memory for it the order is another.
+    const int pair_ctas = 2 * sms;
+    DevBuf<uint32_t> pool;
+    unsigned long long cap = 0;
+    auto make_pool = [&]() {
+        unsigned long long most = 0;
+        for (int k = nheavy; k < T; k++) most += lists_at_most(tw[hq[k]], tlen[hq[k]]);
+        cap = std::min(pool_cap, most) + (unsigned long long)pair_ctas * FP_WARPS * FP_BLOCK;
+        return nheavy == T || pool.try_alloc((size_t)cap, s);
+    };
+    order(pool_cap);
+    if (!make_pool()) {
+        cap = 0;
+        order(0);
+    } else if (nheavy > 0) {
+        pool.release();  // the heavy tasks' recounts may want the memory
+    }
     DevBuf<int32_t> queue(T > 0 ? T : 1, s);
     if (T > 0)
         RC_CUDA(cudaMemcpyAsync(queue.get(), hq.data(), 4 * (size_t)T, cudaMemcpyHostToDevice, s));
@@ -2114,19 +2136,12 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
         RC_CUDA(cudaMemcpyAsync(qhead.get(), &nheavy, 4, cudaMemcpyHostToDevice, s));
     }
     DevBuf<unsigned long long> rtip(nsmall_at < T ? n : 1, s);
-    // the members' lists: walks in items of equal cost, 8 a CTA. The pool also
-    // has room for each warp's last block.
-    DevBuf<uint32_t> pool;
+    // the members' lists: walks in items of equal cost, 8 a CTA
     DevBuf<unsigned long long> rec;
     if (nheavy < T) {
-        unsigned long long most = 0;
-        for (int k = nheavy; k < T; k++) most += lists_at_most(tw[hq[k]], tlen[hq[k]]);
         allow_max_smem((const void *)k_fd_pairs<FdMids>);
-        const int ctas = 2 * sms;
-        unsigned long long cap =
-            std::min(pool_cap, most) + (unsigned long long)ctas * FP_WARPS * FP_BLOCK;
         rec.alloc(n, s);
-        if (!pool.try_alloc((size_t)cap, s)) {
+        if (!pool.get() && (cap == 0 || !make_pool())) {
             cap = 0;  // no memory: members walk when they are peeled
             pool.alloc(1, s);
         }
@@ -2141,7 +2156,7 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
         RC_CUDA(cudaMemcpyAsync(dskip.get(), skip.data(), T, cudaMemcpyHostToDevice, s));
         unsigned long long cost = (unsigned long long)n * FP_MEMBER_COST;
         for (int k = 0; k < T; k++) cost += tw[k];
-        const int64_t Q = std::max<int64_t>(8192, (int64_t)(cost / (8ull * ctas)));
+        const int64_t Q = std::max<int64_t>(8192, (int64_t)(cost / (8ull * pair_ctas)));
         const int32_t nitems = (int32_t)(cost / Q + 1);
         DevBuf<int32_t> items(nitems + 1, s);
         k_pair_items<<<ceil_div(nitems + 1, 256), 256, 0, s>>>(cw.get(), n, Q, nitems, items.get());
@@ -2150,7 +2165,7 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
                      pq.get(), info.get(), fd_adj.get(), pool.get(), cap, head.get(), rec.get(),
                      stats.get()};
         if (cap > 0) {
-            k_fd_pairs<<<std::min(ctas, nitems), FP_THREADS, FP_WARPS * FP_WORDS * 4, s>>>(
+            k_fd_pairs<<<std::min(pair_ctas, nitems), FP_THREADS, FP_WARPS * FP_WORDS * 4, s>>>(
                 a, FdMids{fd_beg.get(), fd_len.get()});
             RC_LAUNCH();
         }

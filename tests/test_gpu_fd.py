@@ -127,3 +127,49 @@ def test_pool_follows_the_lists(R, nu, nv, m, gamma, P, mb):
     if not gamma:
         want, _ = oracle.bup(eu, ev, nu, nv, 0)
         assert np.array_equal(t, want)
+
+
+@pytest.fixture
+def no_optional_memory(R):
+    R.receipt_optional_memory(0)
+    yield
+    R.receipt_optional_memory(-1)
+
+
+# no memory for lists: every member walks when it is peeled, in both peels, with
+# levels of one member (power law) and of thousands (uniform)
+@pytest.mark.parametrize("n", [3_000, 15_360, 15_361, 40_000])
+@pytest.mark.parametrize("uniform", [False, True])
+def test_without_lists(R, no_optional_memory, n, uniform):
+    nv = n // 12
+    eu, ev = synth.er(n, nv, 4 * n, n) if uniform else synth.chung_lu(n, nv, 4 * n, 2.4, 2.3, n)
+    _check(R, eu, ev, n, nv, (1, 4))
+
+
+# ... and tasks whose walks outweigh their levels go to all CTAs then
+def test_without_lists_long_walks_take_all_ctas(R, no_optional_memory):
+    n, nv, m = 600, 2_000, 600_000
+    eu, ev = synth.er(n, nv, m, 8)
+    want, _ = oracle.bup(eu, ev, n, nv, 0)
+    g = R.Graph(eu, ev, n, nv)
+    for lists in (False, True):
+        R.receipt_optional_memory(-1 if lists else 0)
+        t = R.as_u64(g.tip_decompose(0))
+        assert np.array_equal(t, want)
+        assert (g.stats()["fd_heavy_subsets"] > 0) == (not lists)
+
+
+# lists that overflow the serving engine's pool (eight entries an edge and 5M):
+# a part of the members has a list, the others walk
+@pytest.mark.parametrize("n,d", [(3_200, 7), (15_400, 4)])
+def test_part_of_the_lists_beyond_the_pool(R, n, d):
+    u = np.arange(n, dtype=np.int32)
+    deg = 2 + u % (d - 1)
+    eu = np.repeat(u, deg)
+    ev = np.concatenate([(k + np.arange(c)) % d for k, c in zip(u // 640, deg)]).astype(np.int32)
+    want, _ = oracle.bup(eu, ev, n, d, 0)
+    sv = R.Server(max_inflight=1)
+    rid, _ = sv.submit(eu, ev, n, d, 0)
+    got = sv.wait(rid)[0]
+    sv.close()
+    assert np.array_equal(got, want)

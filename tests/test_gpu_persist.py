@@ -107,3 +107,49 @@ def test_lists_of_hubs(R, n):
         t = R.as_u64(g.tip_decompose(0, round_graphs=-1, **kw))
         assert np.array_equal(t, want), kw
         assert recs == _rounds(g), kw
+
+
+# without memory for lists, the other two forms of one window: windows, and
+# groups of warps (short walks); the same counters as the per-round kernels
+@pytest.mark.parametrize("lists", [True, False])
+@pytest.mark.parametrize("n,nv,per,gamma", [(1, 2, 1, 0), (33, 2, 1, 0), (2_049, 51, 3, 2.4),
+                                            (36_864, 921, 3, 2.4), (36_864, 20_000, 4, 0),
+                                            (20_000, 5_000, 10, 2.3)])
+def test_one_window_forms(R, n, nv, per, gamma, lists):
+    m = min(per * n, n * nv // 2)
+    eu, ev = synth.chung_lu(n, nv, m, gamma, gamma, n) if gamma else synth.er(n, nv, m, n)
+    want, _ = oracle.bup(eu, ev, n, nv, 0)
+    g = R.Graph(eu, ev, n, nv)
+    for kw in ({}, {"P": 3}, {"dgm": False}, {"dgm_frac_1024": 8}, {"warp_max_w": 16}):
+        R.receipt_optional_memory(-1 if lists else 0)
+        try:
+            t = R.as_u64(g.tip_decompose(0, **kw))
+        finally:
+            R.receipt_optional_memory(-1)
+        assert np.array_equal(t, want), kw
+        recs, st = _rounds(g), g.stats()
+        t = R.as_u64(g.tip_decompose(0, round_graphs=-1, **kw))
+        assert np.array_equal(t, want), kw
+        assert recs == _rounds(g), kw
+        per_round = g.stats()
+        if per_round["peel_anchors"][1]:
+            continue  # hub rounds, which walk less
+        for k in ("peel_wedges", "peel_mids", "peel_anchors", "peel_pairs"):
+            assert sum(st[k]) == sum(per_round[k]), (kw, k)
+
+
+# a packed union by windows
+def test_union_by_windows(R):
+    graphs, wants = [], []
+    for i in range(5):
+        nu, nv, m = 36_864 - 9_000 * i, 2_000 + 300 * i, 90_000
+        eu, ev = synth.chung_lu(nu, nv, m, 2.3, 2.3, 60 + i)
+        graphs.append(R.Graph(eu, ev, nu, nv))
+        wants.append(oracle.bup(eu, ev, nu, nv, i % 2)[0])
+    R.receipt_optional_memory(0)
+    try:
+        outs = R.receipt_decompose_batch(graphs, [i % 2 for i in range(5)])
+    finally:
+        R.receipt_optional_memory(-1)
+    for o, w in zip(outs, wants):
+        assert np.array_equal(R.as_u64(o), w)
