@@ -1288,10 +1288,13 @@ uint64_t count_local(const receipt_graph *g, unsigned long long *cnt_u,
         RC_CUDA(cudaMemcpyAsync(first.get(), hf.data(), 4 * hf.size(), cudaMemcpyHostToDevice, s));
     }
     // masks of both sides' lists (128 bytes a vertex), unless the vertices are
-    // many for the edges
-    const bool bits = (double)n * BITS / 8 <= 64.0 * (double)m + (256 << 20);
-    DevBuf<uint32_t> mask(bits ? (size_t)n * 32 : 1, s);
-    DevBuf<int32_t> held(bits ? n : 1, s);
+    // many for the edges or there is no memory for them: then every end point
+    // is past the masks
+    DevBuf<uint32_t> mask;
+    DevBuf<int32_t> held;
+    const bool bits = (double)n * BITS / 8 <= 64.0 * (double)m + (256 << 20) &&
+                      mask.try_alloc((size_t)n * 32, s) && held.try_alloc(n, s);
+    if (!bits) mask.release();
     DevBuf<unsigned long long> hot;
     if (m >= HOT_MIN_M && !first.get()) {
         hot.alloc((size_t)2 * HOT_REPS * HOT_KEYS, s);

@@ -1,0 +1,72 @@
+"""Calls in little device memory: work space that only saves time is left out."""
+import contextlib
+import ctypes
+
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def R():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2010_08695_gb300 as R
+    R.load()
+    return R
+
+
+@contextlib.contextmanager
+def memory_left(mb):
+    """All but `mb` MB of the device's free memory is taken (what the library's
+    pool holds unused counts as free)."""
+    import torch
+    cu, pool = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p()
+    assert cu.cuDeviceGetDefaultMemPool(ctypes.byref(pool), torch.cuda.current_device()) == 0
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    assert cu.cuMemPoolTrimTo(pool, ctypes.c_size_t(0)) == 0
+    taken = [torch.empty(torch.cuda.mem_get_info()[0] - (mb << 20), dtype=torch.uint8,
+                         device="cuda")]
+    try:
+        yield
+    finally:
+        taken.clear()
+        torch.cuda.empty_cache()
+
+
+# 2M + 2M vertices: 512 MB of masks, the rest of a count about 260 MB
+def test_count_without_masks(R):
+    import torch
+    nu = nv = 2_000_000
+    eu, ev = synth.chung_lu(nu, nv, 4_000_000, 2.4, 2.4, 3)
+    g = R.Graph(eu, ev, nu, nv)
+    cu, cv = g.count_butterflies()
+    du, dv = torch.empty_like(cu), torch.empty_like(cv)
+    with memory_left(420):
+        R.receipt_count_butterflies(g.handle, du, dv)
+        torch.cuda.synchronize()
+    assert torch.equal(cu, du) and torch.equal(cv, dv)
+
+
+@pytest.mark.parametrize("nu,nv,m,gamma", [(1, 1, 1, 0), (1025, 1023, 50_000, 0), (3_000, 700, 60_000, 2.2),
+                                           (40_000, 9_000, 300_000, 2.1), (20_000, 200, 400_000, 0)])
+def test_counts_without_optional_memory(R, nu, nv, m, gamma):
+    eu, ev = synth.chung_lu(nu, nv, m, gamma, gamma, 5) if gamma else synth.er(nu, nv, m, 5)
+    cu, cv = oracle.count_vp(eu, ev, nu, nv)
+    g = R.Graph(eu, ev, nu, nv)
+    R.receipt_optional_memory(0)
+    try:
+        gu, gv = g.count_butterflies()
+        t = R.receipt_decompose_batch([g, g, g], [0, 1, 0])
+    finally:
+        R.receipt_optional_memory(-1)
+    assert np.array_equal(R.as_u64(gu), cu) and np.array_equal(R.as_u64(gv), cv)
+    want = [oracle.bup(eu, ev, nu, nv, i)[0] for i in (0, 1)]
+    for i, w in enumerate((want[0], want[1], want[0])):
+        assert np.array_equal(R.as_u64(t[i]), w)
