@@ -1254,6 +1254,21 @@ __global__ void k_scatter_both(const unsigned long long *__restrict__ cu,
 
 }  // namespace
 
+static bool masks_pay(int64_t m, int64_t n) {
+    return (double)n * BITS / 8 <= 64.0 * (double)m + (256 << 20);
+}
+
+CountMemory count_memory(int64_t m, int64_t nu, int64_t nv, int sms) {
+    const size_t n = (size_t)(nu + nv), n_max = (size_t)std::max(nu, nv);
+    CountMemory b;
+    // prefix lengths, tier lists (and first keys), hot counts, planes of the
+    // huge start points (at most 4 m / HUGE_DEG chunks), the global tier
+    b.needed = 8 * (size_t)m + 4 * (size_t)(CT_LISTS + 1) * n + 16 * (size_t)HOT_REPS * HOT_KEYS +
+               4 * (size_t)m / HUGE_DEG * HUGE_NP * 128 + 8 * (size_t)sms * n_max;
+    b.optional = masks_pay(m, (int64_t)n) ? (BITS / 8 + 4) * n : 0;
+    return b;
+}
+
 // Counts butterflies of both sides into cnt_u / cnt_v (local ids, zeroed
 // here). Returns wedges traversed.
 uint64_t count_local(const receipt_graph *g, unsigned long long *cnt_u,
@@ -1292,8 +1307,8 @@ uint64_t count_local(const receipt_graph *g, unsigned long long *cnt_u,
     // is past the masks
     DevBuf<uint32_t> mask;
     DevBuf<int32_t> held;
-    const bool bits = (double)n * BITS / 8 <= 64.0 * (double)m + (256 << 20) &&
-                      mask.try_alloc((size_t)n * 32, s) && held.try_alloc(n, s);
+    const bool bits =
+        masks_pay(m, n) && mask.try_alloc((size_t)n * 32, s) && held.try_alloc(n, s);
     if (!bits) mask.release();
     DevBuf<unsigned long long> hot;
     if (m >= HOT_MIN_M && !first.get()) {

@@ -131,20 +131,20 @@ void launch_recount_cost(const Side &S, const Side &O, int64_t m, unsigned long 
     RC_LAUNCH();
 }
 
+// The subgraph's lists, offsets (and their lengths), the counts, a copy of the
+// other side's lists, scans, and the counting pass.
+size_t recount_bytes(int64_t m, int64_t ns, int64_t no, int sms) {
+    return 12 * (size_t)m + 32 * (size_t)(ns + no) + count_memory(m, ns, no, sms).needed +
+           ((size_t)64 << 20);
+}
+
 bool recount_fits(const Decomp &D) {
     size_t fr = 0, tot = 0;
     if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    // the subgraph's lists and offsets, the counts, the counting pass's
-    // temporaries (prefix lengths and scans, tier lists, the global tier's
-    // per-CTA counters) and a copy of the other side's lists
-    const size_t n_all = (size_t)D.S->n + (size_t)D.O->n;
-    const size_t n_max = (size_t)std::max(D.S->n, D.O->n);
-    const size_t need = 40 * (size_t)D.m + 48 * n_all + 8 * (size_t)num_sms() * n_max +
-                        ((size_t)64 << 20);
-    return need <= fr;
+    return recount_bytes(D.m, D.S->n, D.O->n, num_sms()) <= fr;
 }
 
 uint64_t recount_remaining(const Decomp &D, const int32_t *len_w, const int32_t *adj_w,

@@ -15,6 +15,12 @@ void destroy_graph(receipt_graph *g);
 // repeat-table overflow.
 uint64_t count_local(const receipt_graph *g, unsigned long long *cnt_u, unsigned long long *cnt_v,
                      cudaStream_t s, int64_t *points = nullptr);
+// Device bytes of that on a device of `sms` SMs: what it needs, and the masks
+// that it leaves out when there is no memory.
+struct CountMemory {
+    size_t needed = 0, optional = 0;
+};
+CountMemory count_memory(int64_t m, int64_t nu, int64_t nv, int sms);
 void scatter_to_original(const unsigned long long *local, const int32_t *new2old, int32_t n,
                          unsigned long long *out, cudaStream_t s);
 // Counting with every temporary in a static device array (no allocation).
@@ -111,7 +117,8 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s);
 // over the edges (x, y) of min(d_x, d_y).
 void launch_recount_cost(const Side &S, const Side &O, int64_t m, unsigned long long *d_out,
                          cudaStream_t s);
-// Whether free device memory holds a recount's temporaries (upper estimate).
+// Device bytes a recount needs (upper estimate), and whether there are as many.
+size_t recount_bytes(int64_t m, int64_t ns, int64_t no, int sms);
 bool recount_fits(const Decomp &D);
 // Recounts the butterflies of the subgraph left after removing every vertex
 // with D.sub >= 0 and stores each remaining vertex's count in D.sup.

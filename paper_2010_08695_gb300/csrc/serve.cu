@@ -48,18 +48,15 @@ struct Request {
 // Device bytes a request may hold while it runs (graph, build and
 // decomposition temporaries), an upper estimate. It includes what a recount
 // of Sec. 4.1 allocates when the rule picks one (the remaining subgraph's
-// lists, offsets and counts, the counting pass's temporaries and its
-// global-tier counters per CTA, a copy of the other side's lists: the sizes
-// the decomposition itself checks before recounting), the fine-grained
-// step's global counters of split heavy levels (32 members x the side) and its
+// lists, offsets and counts, the counting pass, a copy of the other side's
+// lists: the sizes the decomposition itself checks before recounting), counting's
+// masks, the fine-grained step's global counters of split heavy levels (32 members x the side) and its
 // update lists (FD_LIST_BYTES an edge, 24 a vertex, a block a warp).
 size_t estimate_bytes(int64_t m, int32_t nu, int32_t nv, int side, int sms) {
     const int64_t ns = side ? nv : nu;
     size_t b = (size_t)160 * (size_t)m + (size_t)400 * (size_t)(nu + nv) + ((size_t)32 << 20);
     if (m >= 65535) b += (size_t)8 * 80 * (size_t)ns;  // hub slots of the global tier
-    const size_t n_max = (size_t)std::max(nu, nv);
-    b += (size_t)40 * (size_t)m + (size_t)48 * (size_t)(nu + nv) + (size_t)8 * (size_t)sms * n_max +
-         ((size_t)64 << 20);
+    b += recount_bytes(m, side ? nv : nu, side ? nu : nv, sms) + count_memory(m, nu, nv, sms).optional;
     b += (size_t)8 * 32 * (size_t)ns;
     b += (size_t)FD_LIST_BYTES * (size_t)m + (size_t)24 * (size_t)ns + ((size_t)32 << 20);
     return b;

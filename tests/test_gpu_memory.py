@@ -70,3 +70,17 @@ def test_counts_without_optional_memory(R, nu, nv, m, gamma):
     want = [oracle.bup(eu, ev, nu, nv, i)[0] for i in (0, 1)]
     for i, w in enumerate((want[0], want[1], want[0])):
         assert np.array_equal(R.as_u64(t[i]), w)
+
+
+# a recount that does not fit is left out (the global tier's counters
+# alone: 8 bytes a vertex and SM)
+def test_recount_without_memory(R):
+    nu, nv = 1_000_000, 60_000
+    eu, ev = synth.chung_lu(nu, nv, 1_000_000, 2.4, 2.2, 4)
+    g = R.Graph(eu, ev, nu, nv)
+    want = R.as_u64(g.tip_decompose(0, huc_factor_1024=1))
+    assert g.stats()["huc_recounts"] > 0
+    with memory_left(900):
+        t = R.as_u64(g.tip_decompose(0, huc_factor_1024=1))
+    assert np.array_equal(t, want)
+    assert g.stats()["huc_recounts"] == 0
