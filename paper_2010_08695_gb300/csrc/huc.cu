@@ -139,12 +139,7 @@ size_t recount_bytes(int64_t m, int64_t ns, int64_t no, int sms) {
 }
 
 bool recount_fits(const Decomp &D) {
-    size_t fr = 0, tot = 0;
-    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return recount_bytes(D.m, D.S->n, D.O->n, num_sms()) <= fr;
+    return recount_bytes(D.m, D.S->n, D.O->n, num_sms()) <= available_bytes();
 }
 
 uint64_t recount_remaining(const Decomp &D, const int32_t *len_w, const int32_t *adj_w,

@@ -72,7 +72,26 @@ def test_counts_without_optional_memory(R, nu, nv, m, gamma):
         assert np.array_equal(R.as_u64(t[i]), w)
 
 
-# a recount that does not fit is left out (the global tier's counters
+# memory that the library's pool keeps unused is there for a recount
+def test_recount_in_memory_kept_by_the_pool(R):
+    import torch
+    nu, nv = 200_000, 60_000
+    eu, ev = synth.chung_lu(nu, nv, 600_000, 2.4, 2.2, 4)
+    g = R.Graph(eu, ev, nu, nv)
+    want = R.as_u64(g.tip_decompose(0))
+    cu, p = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p()
+    with memory_left(1300):
+        assert cu.cuMemAllocAsync(ctypes.byref(p), ctypes.c_size_t(1100 << 20), ctypes.c_void_p(0)) == 0
+        assert cu.cuMemFreeAsync(p, ctypes.c_void_p(0)) == 0
+        torch.cuda.synchronize()
+        assert torch.cuda.mem_get_info()[0] < 300 << 20
+        out = torch.empty(nu, dtype=torch.int64, device="cpu").to("cuda")
+        t = R.as_u64(g.tip_decompose(0, huc_factor_1024=1, out=out))
+    assert np.array_equal(t, want)
+    assert g.stats()["huc_recounts"] > 0
+
+
+# ... and a recount that does not fit is left out (the global tier's counters
 # alone: 8 bytes a vertex and SM)
 def test_recount_without_memory(R):
     nu, nv = 1_000_000, 60_000
