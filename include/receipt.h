@@ -474,7 +474,8 @@ receipt_status receipt_get_subsets(const receipt_graph *g, receipt_subset *out, 
                                    int32_t *n_subsets);
 
 /* Work space that only saves time (the update lists of both steps, counting's
- * masks) is left out when there is no memory for it. This bounds each such allocation of the
+ * masks, the rounds through the other side's hubs) is left out when there is no
+ * memory for it. This bounds each such allocation of the
  * calling thread's later calls: bytes < 0 (the start) no bound, 0 none of it.
  * Speed only; results are the same. Always RECEIPT_OK. */
 receipt_status receipt_optional_memory(int64_t bytes);

@@ -1373,10 +1373,8 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s) {
     // anchors whatever their walks, the next activeSet by a full scan.
     HubPath hub;
     bool hub_ready = false;
-    const bool hub_ok = !persist && !D.parts && HubPath::suits(D, s);
+    bool hub_ok = !persist && !D.parts && HubPath::suits(D, s);
     auto hub_round = [&](int32_t *cur, int32_t *nxt, int32_t nF) {
-        if (!hub_ready) hub.init(D, s);
-        hub_ready = true;
         k_cd_prepare<<<nb, 512, 0, s>>>(cur, st.get(), D.sub, D.sup, D.wfull, S.off, Lw.get(),
                                         Lb.get(), 0);
         RC_LAUNCH();
@@ -1618,8 +1616,11 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s) {
         // 3 10^7 + 12 n; the 40M-edge one 621 / 609 / 625).
         const double hmin = 1e7 + 16.0 * (double)hst->n_remaining;
         auto hub_due = [&](int32_t nF, uint64_t front_w, uint64_t peeled) {
-            return hub_ok && nF > 0 && nF <= HubPath::MAX_ANCHORS &&
-                   (double)front_w * (double)(D.m - peeled) >= hmin * (double)D.m;
+            if (!hub_ok || nF <= 0 || nF > HubPath::MAX_ANCHORS ||
+                (double)front_w * (double)(D.m - peeled) < hmin * (double)D.m)
+                return false;
+            if (!hub_ready) hub_ok = hub_ready = hub.init(D, s);
+            return hub_ok;
         };
         bool by_hubs = !recount && hub_due(hst->nF, hst->front_w, hst->peeled_edges);
         uint64_t front_seen = hst->front_w;

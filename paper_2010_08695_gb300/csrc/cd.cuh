@@ -171,8 +171,10 @@ class HubPath {
     ~HubPath();
     HubPath(const HubPath &) = delete;
     HubPath &operator=(const HubPath &) = delete;
-    // Masks and work space of one decomposition.
-    void init(const Decomp &D, cudaStream_t s);
+    // Masks and work space of one decomposition, `bytes` of them at most. False
+    // (and nothing kept) when there is no memory for them.
+    bool init(const Decomp &D, cudaStream_t s);
+    static size_t bytes(int64_t m, int64_t n, int64_t n_o);
     // Enqueues the updates of the anchors A (st->nLb of them, at most nF,
     // assigned to their subset already) to every remaining vertex's support.
     void round(const Decomp &D, CdDev *st, const int32_t *A, int32_t nF, cudaStream_t s);

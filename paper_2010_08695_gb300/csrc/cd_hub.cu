@@ -839,28 +839,28 @@ constexpr size_t quad_smem() { return (size_t)2 * TILES * 256; }
 
 }  // namespace
 
-void HubPath::init(const Decomp &D, cudaStream_t s) {
+size_t HubPath::bytes(int64_t m, int64_t n, int64_t n_o) {
+    return 16 * (size_t)m + (4 * HW + 24) * (size_t)n + (4 * HW + 12) * (size_t)n_o +
+           (size_t)MAX_ANCHORS * (4 * HW + 4 + HUBS / 8) + 4 * (size_t)TRI + 512 * (size_t)TILES;
+}
+
+bool HubPath::init(const Decomp &D, cudaStream_t s) {
     const Side &S = *D.S, &O = *D.O;
     const int32_t n = D.n;
-    mask_.alloc((size_t)n * HW, s);
-    plen_.alloc(n, s);
-    heavy_.alloc((size_t)O.n * HW, s);
-    cb_.alloc(O.n, s);
-    touch_.alloc(O.n, s);
-    Qs_.alloc(n, s);
-    Q_.alloc(n, s);
-    mid_.alloc(n, s);
-    gtri_.alloc(TRI, s);
-    R_.alloc(n, s);
-    big_.alloc(n, s);
-    aoff_.alloc(MAX_ANCHORS + 1, s);
-    amask_.alloc((size_t)MAX_ANCHORS * HW, s);
-    cols_.alloc((size_t)HUBS * (MAX_ANCHORS / 32), s);
-    gram_.alloc((size_t)2 * TILES * 64, s);
-    ey_.alloc(D.m, s);
-    ek_.alloc(D.m, s);
-    alist_.alloc(D.m, s);
-    hd_.alloc(1, s);
+    if (!(mask_.try_alloc((size_t)n * HW, s) && plen_.try_alloc(n, s) &&
+          heavy_.try_alloc((size_t)O.n * HW, s) && cb_.try_alloc(O.n, s) && touch_.try_alloc(O.n, s) &&
+          Qs_.try_alloc(n, s) && Q_.try_alloc(n, s) && mid_.try_alloc(n, s) && R_.try_alloc(n, s) &&
+          big_.try_alloc(n, s) && gtri_.try_alloc(TRI, s) && aoff_.try_alloc(MAX_ANCHORS + 1, s) &&
+          amask_.try_alloc((size_t)MAX_ANCHORS * HW, s) &&
+          cols_.try_alloc((size_t)HUBS * (MAX_ANCHORS / 32), s) &&
+          gram_.try_alloc((size_t)2 * TILES * 64, s) && ey_.try_alloc(D.m, s) && ek_.try_alloc(D.m, s) &&
+          alist_.try_alloc(D.m, s) && hd_.try_alloc(1, s))) {
+        for (DevBuf<uint32_t> *b : {&mask_, &heavy_, &amask_, &cols_, &gram_, &gtri_}) b->release();
+        for (DevBuf<int32_t> *b : {&plen_, &touch_, &Qs_, &Q_, &R_, &mid_, &big_, &aoff_, &ey_, &alist_})
+            b->release();
+        for (DevBuf<int2> *b : {&cb_, &ek_}) b->release();
+        return false;
+    }
     for (cudaEvent_t &e : ev_) RC_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     cb_.zero();
     hd_.zero();
@@ -872,6 +872,7 @@ void HubPath::init(const Decomp &D, cudaStream_t s) {
     allow_max_smem((const void *)k_hub_quad_sparse);
     allow_max_smem((const void *)k_hub_quad);
     allow_max_smem((const void *)k_hub_pull_cta);
+    return true;
 }
 
 void HubPath::round(const Decomp &D, CdDev *st, const int32_t *A, int32_t nF, cudaStream_t s) {

@@ -13,6 +13,7 @@
 #include <unordered_map>
 #include <vector>
 
+#include "cd.cuh"
 #include "internal.cuh"
 
 namespace receipt {
@@ -50,13 +51,14 @@ struct Request {
 // of Sec. 4.1 allocates when the rule picks one (the remaining subgraph's
 // lists, offsets and counts, the counting pass, a copy of the other side's
 // lists: the sizes the decomposition itself checks before recounting), counting's
-// masks, the fine-grained step's global counters of split heavy levels (32 members x the side) and its
+// masks, the hub rounds' work space, the fine-grained step's global counters of split heavy levels (32 members x the side) and its
 // update lists (FD_LIST_BYTES an edge, 24 a vertex, a block a warp).
 size_t estimate_bytes(int64_t m, int32_t nu, int32_t nv, int side, int sms) {
     const int64_t ns = side ? nv : nu;
     size_t b = (size_t)160 * (size_t)m + (size_t)400 * (size_t)(nu + nv) + ((size_t)32 << 20);
     if (m >= 65535) b += (size_t)8 * 80 * (size_t)ns;  // hub slots of the global tier
     b += recount_bytes(m, side ? nv : nu, side ? nu : nv, sms) + count_memory(m, nu, nv, sms).optional;
+    b += HubPath::bytes(m, ns, side ? nu : nv);
     b += (size_t)8 * 32 * (size_t)ns;
     b += (size_t)FD_LIST_BYTES * (size_t)m + (size_t)24 * (size_t)ns + ((size_t)32 << 20);
     return b;

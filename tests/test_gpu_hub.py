@@ -55,3 +55,19 @@ def test_hub_rounds(R, name):
         assert np.array_equal(t, want), kw
         t = R.as_u64(g.tip_decompose(0, scan_frontier=-1, **kw))
         assert np.array_equal(t, want), kw
+
+
+# without memory for them, the per-anchor tiers walk every round
+def test_without_memory_for_hub_rounds(R):
+    nu, nv, eu, ev = CASES["mixed"]()
+    want, _ = oracle.bup(eu, ev, nu, nv, 0)
+    g = R.Graph(eu, ev, nu, nv)
+    R.receipt_optional_memory(0)
+    try:
+        t = R.as_u64(g.tip_decompose(0, P=4, dgm=False, huc=-1))
+    finally:
+        R.receipt_optional_memory(-1)
+    assert np.array_equal(t, want)
+    st = g.stats()
+    # all wedges (those of a hybrid anchor that overflows twice)
+    assert sum(st["peel_wedges"]) >= st["wedges_cd"]
