@@ -884,6 +884,15 @@ void HubPath::round(const Decomp &D, CdDev *st, const int32_t *A, int32_t nF, cu
     // three branches: the hub part (columns, Gram matrix, quadratic forms),
     // the heavy vertices, the pull; their decrements are atomic
     cudaStream_t sq = tier_stream(0), sh = tier_stream(1);
+    struct ForkGuard {  // left by an error, the buffers wait for the branches
+        cudaStream_t q, h;
+        bool joined = false;
+        ~ForkGuard() {
+            if (joined) return;
+            cudaStreamSynchronize(q);
+            cudaStreamSynchronize(h);
+        }
+    } fg{sq, sh};
     k_hub_begin<<<1, 1024, 0, s>>>(a);
     RC_LAUNCH();
     RC_CUDA(cudaEventRecord(ev_[0], s));
@@ -931,6 +940,7 @@ void HubPath::round(const Decomp &D, CdDev *st, const int32_t *A, int32_t nF, cu
     RC_LAUNCH();
     RC_CUDA(cudaStreamWaitEvent(s, ev_[2], 0));
     RC_CUDA(cudaStreamWaitEvent(s, ev_[4], 0));
+    fg.joined = true;
 }
 
 HubPath::~HubPath() {
