@@ -155,8 +155,9 @@ __global__ void __launch_bounds__(1024) k_hub_begin(HubArgs a) {
 // place in its middle vertex's list is the count it found.
 __global__ void k_hub_count(HubArgs a) {
     const int32_t nE = a.hd->nE, nA = a.hd->nA;
-    for (int32_t b = blockIdx.x * blockDim.x; b < nE; b += gridDim.x * blockDim.x) {
-        const int32_t e = b + threadIdx.x;
+    // (64-bit positions: one past the last step may exceed 2^31)
+    for (int64_t b = (int64_t)blockIdx.x * blockDim.x; b < nE; b += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t e = b + threadIdx.x;
         bool fresh = false;
         int32_t y = 0;
         if (e < nE) {
@@ -182,8 +183,8 @@ __global__ void k_hub_count(HubArgs a) {
 __global__ void k_hub_base(HubArgs a) {
     const int32_t n = a.hd->nTouch;
     const int lane = threadIdx.x & 31;
-    for (int32_t b = blockIdx.x * blockDim.x; b < n; b += gridDim.x * blockDim.x) {
-        const int32_t t = b + threadIdx.x;
+    for (int64_t b = (int64_t)blockIdx.x * blockDim.x; b < n; b += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t t = b + threadIdx.x;
         const int32_t y = t < n ? a.touch[t] : -1;
         const int32_t c = y >= 0 ? a.cb[y].x : 0;
         int32_t inc = c;
@@ -201,7 +202,8 @@ __global__ void k_hub_base(HubArgs a) {
 
 __global__ void k_hub_fill(HubArgs a) {
     const int32_t nE = a.hd->nE;
-    for (int32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < nE; e += gridDim.x * blockDim.x) {
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nE;
+         e += (int64_t)gridDim.x * blockDim.x) {
         const int2 k = a.ek[e];
         a.alist[a.cb[a.ey[e]].y + k.y] = k.x;
     }
@@ -209,7 +211,8 @@ __global__ void k_hub_fill(HubArgs a) {
 
 __global__ void k_hub_clear(HubArgs a) {
     const int32_t n = a.hd->nTouch;
-    for (int32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x)
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n;
+         t += (int64_t)gridDim.x * blockDim.x)
         a.cb[a.touch[t]] = make_int2(0, 0);
 }
 
@@ -296,15 +299,15 @@ __global__ void __launch_bounds__(256) k_hub_rows(HubArgs a) {
     __shared__ int32_t s_n[3], s_at[3];
     const int lane = threadIdx.x & 31;
     constexpr int U = 4;
-    for (int32_t b = blockIdx.x * 256 * U; b < a.n; b += gridDim.x * 256 * U) {
+    for (int64_t b = (int64_t)blockIdx.x * (256 * U); b < a.n; b += (int64_t)gridDim.x * (256 * U)) {
         if (threadIdx.x < 3) s_n[threadIdx.x] = 0;
         __syncthreads();
         int32_t x[U], pl[U], d[U];
         int which[U], pos[3][U];
 #pragma unroll
         for (int u = 0; u < U; u++) {
-            x[u] = b + u * 256 + threadIdx.x;
-            if (x[u] >= a.n || a.sub[x[u]] >= 0) x[u] = -1;
+            const int64_t i = b + u * 256 + threadIdx.x;
+            x[u] = i < a.n && a.sub[i] < 0 ? (int32_t)i : -1;
         }
 #pragma unroll
         for (int u = 0; u < U; u++) {
@@ -774,9 +777,9 @@ __global__ void __launch_bounds__(512) k_hub_heavy(HubArgs a) {
     int32_t b[8];
     // counts of edges e0 + 4 step, step += stride, up to e1
     auto count = [&](int32_t e0, int32_t e1, int32_t first, int32_t stride) {
-        for (int32_t e = e0 + first * 4; e < e1; e += stride * 4) {
+        for (int64_t e = e0 + first * 4; e < e1; e += stride * 4) {
             // lane: word (lane & 7) of the mask of edge e + (lane >> 3)
-            const int32_t k = e + (lane >> 3);
+            const int64_t k = e + (lane >> 3);
             const uint32_t word =
                 k < e1 ? __ldg(a.heavy + (size_t)a.ey[k] * HW + (lane & 7)) : 0u;
             if (!__any_sync(0xffffffffu, word)) continue;
