@@ -261,6 +261,7 @@ void tip_decompose_impl(receipt_graph *g, int side, uint64_t *d_tip, const recei
     D.timing = opt.timing != 0;
     D.list_bound = list_bound;
     D.max_deg_s = g->max_deg[side];
+    D.max_deg_o = g->max_deg[1 - side];
     D.fd_heavy_w = opt.fd_heavy_w;
     D.fd_huc = opt.fd_huc;
     D.huc_factor = opt.huc_factor_1024 > 0 ? opt.huc_factor_1024 / 1024.0 : 8.0;

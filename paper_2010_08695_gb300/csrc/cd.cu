@@ -1497,7 +1497,7 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s) {
                              D.parts ? part_of.get() : nullptr, pfirst.get(), plast.get(), ng,
                              F.get(), pLw.get(), pLd.get(), pLg.get(), prec.get(), REC_CAP, P, range_cap,
                              warp_max_w, dgm && O.n > 0 ? 1 : 0, dgm_frac, huc == 0 ? 1 : 0,
-                             huc_factor, rcost.get(), pairs.pool.get(), pairs.rec.get()};
+                             huc_factor, rcost.get(), pairs.pool.get(), pairs.rec.get(), cd_persist_group(D)};
         PersistDev *hpd = (PersistDev *)(hrec + ROUND_BURST * (hdr / 8));
         PersistRound *hrc = (PersistRound *)(hpd + 1);
         std::vector<PersistRound> recs;

@@ -110,6 +110,7 @@ struct PersistArgs {
     const unsigned long long *crcnt;
     const uint32_t *pool;            // update lists (PERSIST_LISTS)
     const unsigned long long *list;  // where each vertex's lies
+    int32_t group;                   // dense-window anchors per fetch, at most
 };
 
 // Whether a decomposition can run in the one-launch form.
@@ -120,6 +121,8 @@ bool cd_persist_by_lists(const Decomp &D);
 bool cd_persist_wide(const Decomp &D);
 // CTAs of the one-launch form for m edges.
 int cd_persist_grid(int64_t m, int form);
+// Dense-window anchors that a CTA may fetch at once.
+int cd_persist_group(const Decomp &D);
 // Enqueues one launch (state in a.pd).
 void cd_persist_launch(const PersistArgs &a, int grid, int form, cudaStream_t s);
 

@@ -47,8 +47,12 @@ constexpr int GROUP = 8;  // dense-window anchors side by side in one pass
 // With groups (WIDE), walks of more wedges still take the whole CTA.
 constexpr unsigned long long GROUP_MAX_W = 32768;
 // Polls of a barrier wait before it gives up (each takes at least an L2 round
-// trip: ~10 s in all; a peel step takes milliseconds).
+// trip: ~10 s in all). CTAs fetch their items as they go, so they wait for one
+// another's last fetch at most: GROUP_W wedges (1.6 s at the 1.6 10^9 wedges a
+// second of a CTA on dense graphs), or one anchor's walk, 65,534 lists of 36,864
+// keys at most and no longer.
 constexpr unsigned BAR_POLLS = 1u << 24;
+constexpr uint64_t GROUP_W = 2500000000ull;
 
 __device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
     unsigned v;
@@ -880,7 +884,7 @@ __global__ void __launch_bounds__(PT, 2) k_cd_persist(PersistArgs a) {
         }
         // items per fetch: more than one only when the round has more items
         // than CTAs
-        const int G = max(1, min(GROUP, nD / (int)gridDim.x));
+        const int G = max(1, min(a.group, nD / (int)gridDim.x));
         for (int base = blockIdx.x * G; !LISTS && base < nD;) {
             const int gcount = min(G, nD - base);
             for (int i0 = 0; i0 < gcount;) {
@@ -1048,6 +1052,11 @@ static const void *persist_kernel(int form) {
     return form == PERSIST_LISTS    ? (const void *)k_cd_persist<PERSIST_LISTS>
            : form == PERSIST_GROUPS ? (const void *)k_cd_persist<PERSIST_GROUPS>
                                     : (const void *)k_cd_persist<PERSIST_WINDOWS>;
+}
+
+int cd_persist_group(const Decomp &D) {
+    const uint64_t w = (uint64_t)D.max_deg_s * (uint64_t)D.max_deg_o;  // an anchor's, at most
+    return w > 0 ? (int)std::max<uint64_t>(1, std::min<uint64_t>(GROUP, GROUP_W / w)) : GROUP;
 }
 
 int cd_persist_grid(int64_t m, int form) {

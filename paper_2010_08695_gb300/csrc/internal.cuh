@@ -64,7 +64,7 @@ struct Decomp {
     const Side *O = nullptr;  // other side
     int32_t n = 0;
     int64_t m = 0;
-    int32_t max_deg_s = 0;                // largest degree on side s
+    int32_t max_deg_s = 0, max_deg_o = 0; // largest degrees on side s, on the other
     bool list_bound = false;              // update lists within FD_LIST_BYTES an edge
     unsigned long long *sup = nullptr;    // raw supports
     unsigned long long *init = nullptr;   // support when the vertex's range began

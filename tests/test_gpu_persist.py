@@ -153,3 +153,29 @@ def test_union_by_windows(R):
         R.receipt_optional_memory(-1)
     for o, w in zip(outs, wants):
         assert np.array_equal(R.as_u64(o), w)
+
+
+# anchors whose walks may be long are fetched fewer at a time (8, 6, 1): the
+# CTAs that have none left wait for the last fetch
+@pytest.mark.parametrize("ds,do", [(1_000, 10_000), (40_000, 10_000), (60_000, 25_000)])
+def test_anchors_per_fetch(R, ds, do):
+    n, nv = 26_001, 61_000
+    rng = np.random.default_rng(do)
+    ru, rv = synth.er(n, nv, 4 * n, do)
+    eu = np.concatenate([np.full(ds, 7), rng.choice(n, do, replace=False), ru]).astype(np.int64)
+    ev = np.concatenate([rng.choice(nv, ds, replace=False), np.full(do, 5), rv]).astype(np.int64)
+    key = np.unique(eu * nv + ev)
+    eu, ev = (key // nv).astype(np.int32), (key % nv).astype(np.int32)
+    want, _ = oracle.bup(eu, ev, n, nv, 0)
+    g = R.Graph(eu, ev, n, nv)
+    for kw in ({}, {"P": 3}, {"huc": -1}):
+        R.receipt_optional_memory(0)
+        try:
+            t = R.as_u64(g.tip_decompose(0, **kw))
+        finally:
+            R.receipt_optional_memory(-1)
+        assert np.array_equal(t, want), kw
+        recs = _rounds(g)
+        t = R.as_u64(g.tip_decompose(0, round_graphs=-1, **kw))
+        assert np.array_equal(t, want), kw
+        assert recs == _rounds(g), kw
