@@ -2293,9 +2293,15 @@ bool side_pair_lists(const Decomp &D, PairLists &L, cudaStream_t s) {
         ts[t] = D.parts ? (int32_t)(*D.parts)[t] : 0;
         tl[t] = (D.parts ? (int32_t)(*D.parts)[t + 1] : n) - ts[t];
     }
+    // every vertex must get a list (fd_plan): 16-bit counters of all keys in eight
+    // times a CTA's words, counts above the rank bits
+    const int32_t keys = *std::max_element(tl.begin(), tl.end());
+    if ((int64_t)keys * 16 > (int64_t)32 * 8 * FP_WARPS * FP_WORDS || D.max_deg_s >= 65536 ||
+        (int64_t)D.max_deg_s >= 1ll << (32 - bits_for((uint64_t)std::max(1, keys - 1))))
+        return false;
     const int ctas = 2 * num_sms();
     const unsigned long long w = D.wedges_bup + (unsigned long long)m;  // sum of wfull
-    // every vertex must get its list, so there is room for them all
+    // room for all lists
     unsigned long long most = 0;
     for (int t = 0; t < T; t++) most += lists_at_most(w, tl[t]);
     most = std::min(most, w / 2);
@@ -2309,7 +2315,7 @@ bool side_pair_lists(const Decomp &D, PairLists &L, cudaStream_t s) {
     DevBuf<int64_t> cost(n + 1, s), cw(n + 1, s);
     DevBuf<int32_t> dts(T, s), dtl(T, s), pq(1, s);
     DevBuf<uint8_t> skip(T, s);
-    DevBuf<unsigned long long> scal(2 + T, s);  // pool head, wedges, weights without lists
+    DevBuf<unsigned long long> scal(2, s);  // pool head, wedges
     RC_CUDA(cudaMemcpyAsync(dts.get(), ts.data(), 4 * (size_t)T, cudaMemcpyHostToDevice, s));
     RC_CUDA(cudaMemcpyAsync(dtl.get(), tl.data(), 4 * (size_t)T, cudaMemcpyHostToDevice, s));
     skip.zero();
@@ -2326,10 +2332,6 @@ bool side_pair_lists(const Decomp &D, PairLists &L, cudaStream_t s) {
     DevBuf<int32_t> items(nitems + 1, s);
     k_pair_items<<<ceil_div(nitems + 1, 256), 256, 0, s>>>(cw.get(), n, Q, nitems, items.get());
     RC_LAUNCH();
-    k_listless<<<ceil_div(n, 256), 256, 0, s>>>(info.get(), n, dts.get(), dtl.get(), T,
-                                                *std::max_element(tl.begin(), tl.end()),
-                                                scal.get() + 2);
-    RC_LAUNCH();
     if (!L.pool.try_alloc((size_t)cap, s) || !L.rec.try_alloc(n, s)) {
         L.pool.release();
         return false;
@@ -2341,13 +2343,10 @@ bool side_pair_lists(const Decomp &D, PairLists &L, cudaStream_t s) {
     k_fd_pairs<<<std::min(ctas, nitems), FP_THREADS, FP_WARPS * FP_WORDS * 4, s>>>(
         a, SideMids{D.S->adj, D.O->off});
     RC_LAUNCH();
-    std::vector<unsigned long long> h(2 + T);
-    RC_CUDA(cudaMemcpyAsync(h.data(), scal.get(), 8 * (size_t)(2 + T), cudaMemcpyDeviceToHost, s));
+    unsigned long long head = 0;
+    RC_CUDA(cudaMemcpyAsync(&head, scal.get(), 8, cudaMemcpyDeviceToHost, s));
     RC_CUDA(cudaStreamSynchronize(s));
-    unsigned long long listless = 0;
-    for (int t = 0; t < T; t++) listless += h[2 + t];
-    L.wedges = h[1];
-    if (h[0] <= cap && listless == 0) return true;
+    if (head <= cap) return true;
     L.pool.release();
     L.rec.release();
     return false;

@@ -147,7 +147,6 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s);
 struct PairLists {
     DevBuf<uint32_t> pool;
     DevBuf<unsigned long long> rec;
-    unsigned long long wedges = 0;  // walked
 };
 // False (and nothing kept) unless every vertex could get a list. Synchronises s.
 bool side_pair_lists(const Decomp &D, PairLists &L, cudaStream_t s);

@@ -179,3 +179,26 @@ def test_anchors_per_fetch(R, ds, do):
         t = R.as_u64(g.tip_decompose(0, round_graphs=-1, **kw))
         assert np.array_equal(t, want), kw
         assert recs == _rounds(g), kw
+
+
+# a vertex whose counts do not fit above the 17 rank bits of a side of more than
+# 65,536: no lists (degree 32,768 and more), and the edge below it
+@pytest.mark.parametrize("n", [65_536, 65_537, 73_728])
+@pytest.mark.parametrize("deg", [32_767, 32_768])
+def test_degrees_past_a_list_entry(R, n, deg):
+    nv = 33_000
+    rng = np.random.default_rng(n + deg)
+    ru, rv = synth.er(n, nv, 3 * n, n)
+    keep = ru != 9
+    eu = np.concatenate([np.full(deg, 9), ru[keep]]).astype(np.int32)
+    ev = np.concatenate([rng.choice(nv, deg, replace=False), rv[keep]]).astype(np.int32)
+    want, _ = oracle.bup(eu, ev, n, nv, 0)
+    g = R.Graph(eu, ev, n, nv)
+    assert g.max_degree[0] == deg
+    for kw in ({}, {"P": 4}):
+        t = R.as_u64(g.tip_decompose(0, **kw))
+        assert np.array_equal(t, want), kw
+        recs = _rounds(g)
+        t = R.as_u64(g.tip_decompose(0, round_graphs=-1, **kw))
+        assert np.array_equal(t, want), kw
+        assert recs == _rounds(g), kw
