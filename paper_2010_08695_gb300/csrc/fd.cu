@@ -44,10 +44,6 @@ constexpr unsigned long long WIDE_BIT = 1ull << 63;
 // heavy tasks, automatic rule
 constexpr unsigned long long HEAVY_MIN_W = 1ull << 23;
 constexpr int32_t HEAVY_NI = 1 << 17;
-// All lists' entries are about a sixth of their walks' wedges at most: 1/8 to
-// 1/16 on Chung-Lu graphs of 1M to 40M edges; uniform and dense graphs have up to
-// 1/3, but all CTAs peel their long tasks without lists.
-constexpr unsigned long long LIST_SHARE = 6;
 // a level of a heavy task with at most this many members with big walks
 // (and at least two CTAs for each) splits each one's walk over the CTAs
 // (partial counts summed in global counters) instead of giving each member
@@ -373,6 +369,20 @@ constexpr int FP_BLOCK = 1024;           // pool entries taken at a time
 constexpr int64_t FP_MEMBER_COST = 128;  // a member's fixed cost in wedges
 // An entry holds the rank in its low fp_rank_bits and the count above.
 constexpr unsigned long long FP_NONE = ~0ull;  // no list; else offset << 24 | length
+
+// Pool entries that the lists of n members of w wedges will take, about: where
+// two members share c = w / n^2 << 1 middle vertices on average, c^2 / 2 for each
+// two (uniform graphs; power-law ones have half of that), at least a twelfth of
+// the wedges (tasks of very unlike members: 300,000 members of all degrees, c =
+// 0.03, a sixteenth), at most a third; more by the ends of blocks that stay unused.
+// With lists_at_most as a bound, the tasks of whole graphs of 1M to 40M edges,
+// uniform, dense and power law, had 0.5 to 1.0 of this in entries.
+inline unsigned long long lists_about(unsigned long long w, int32_t n) {
+    const double c = (double)w / ((double)n * (double)n);
+    const double e = (double)w * std::min(1.0 / 3, std::max(1.0 / 12, c / 2));
+    const double len = e / n;
+    return (unsigned long long)(len < FP_BLOCK ? e * (1.0 + len / FP_BLOCK) : e);
+}
 
 // Pool entries of the lists of n vertices of w wedges together, at most: one for
 // two wedges, one for each other vertex (twice that where a block's end may stay
@@ -1953,12 +1963,12 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
     // Otherwise one CTA is faster: 4,751 levels of 80K members take 36 ms
     // there and took 590 heavy, 20,000 levels of 42K members 117 ms.
     // The pool has room for the most entries the lists can have as long as that
-    // is cheap (FD_LIST_BYTES an edge), else for about as many as they do have
-    // (LIST_SHARE), up to an eighth of the memory there is; members past it walk.
+    // is cheap (FD_LIST_BYTES an edge), else for about as many as they will have,
+    // up to an eighth of the memory there is; members past it walk.
     unsigned long long entries_max = 0, entries = 0;
     for (int k = 0; k < T; k++) {
         entries_max += lists_at_most(tw[k], tlen[k]);
-        entries += std::min(tw[k] / LIST_SHARE, lists_at_most(tw[k], tlen[k]));
+        entries += std::min(lists_about(tw[k], tlen[k]), lists_at_most(tw[k], tlen[k]));
     }
     unsigned long long pool_cap = (unsigned long long)(FD_LIST_BYTES / 4 * m);
     if (entries_max > pool_cap && entries > pool_cap && !D.list_bound)
