@@ -186,12 +186,33 @@ def load_workload(name):
     return eu, ev, nu, nv, side, wedges
 
 
-def roofline(st, peak, peak_kind):
+def hub_rounds(trace):
+    """Totals of an instrumented step's rounds through the other side's hubs:
+    all their device time is under tier 1, where every other round has the
+    tiers' kernels (and their times) side by side."""
+    rs = [r for r in trace if not r["recount"] and r["ms"][1] > 0
+          and not any(r["ms"][t] for t in (0, 2, 3, 4))]
+    return {"rounds": len(rs), "ms": sum(r["ms"][1] for r in rs),
+            "wedges": sum(r["wedges"][1] for r in rs), "anchors": sum(r["anchors"][1] for r in rs)}
+
+
+def roofline(st, peak, peak_kind, hub=None):
     """Roofline of the peel tier with the most device time in the
     instrumented step(s): algorithmic bytes per launch (4 B per wedge walked,
     16 B per middle-vertex visit, 16 B per support atomic, 24 B per anchor)
-    over the tier's average launch time."""
+    over the tier's average launch time. Where most of that time is rounds
+    through the hubs (`hub`, of the last step), theirs: 36 B per wedge walked
+    past the hubs (the anchor's number and its mask), 24 B per anchor."""
     tier = max(range(5), key=lambda t: st["ms_peel"][t])
+    if tier == 1 and hub and 2 * hub["ms"] > st["ms_peel"][1]:
+        lau = hub["rounds"]
+        alg_bytes = (36 * hub["wedges"] + 24 * hub["anchors"]) / lau
+        dur_s = hub["ms"] / 1e3 / lau
+        achieved = alg_bytes / dur_s / 1e9
+        return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
+                "frac": achieved / peak, "traffic": None, "kernel": "k_hub_* (the kernels of a round)",
+                "peak_source": peak_kind, "bytes_per_launch": alg_bytes, "launch_ms": dur_s * 1e3,
+                "launches": lau, "bytes_model": "36 B/wedge + 24 B/anchor"}
     lau = max(1, st["peel_launches"][tier])
     alg_bytes = (4 * st["peel_wedges"][tier] + 16 * st["peel_mids"][tier]
                  + 16 * st["peel_pairs"][tier] + 24 * st["peel_anchors"][tier]) / lau
@@ -244,7 +265,7 @@ def measure_graph(R, name, args, dist=None, world=1, local=0, clocks=True, e2e=T
             dist.barrier()
         torch.cuda.synchronize()
 
-    trace = []
+    trace, last_trace = [], []
 
     def step(timing):
         g = R.Graph(eu_d, ev_d, nu, nv, stream=stream)
@@ -252,8 +273,10 @@ def measure_graph(R, name, args, dist=None, world=1, local=0, clocks=True, e2e=T
                         round_graphs=args.round_graphs, huc=args.huc,
                         huc_factor_1024=args.huc_factor_1024)
         st = g.stats()
-        if timing and args.trace:
-            trace[:] = g.trace()
+        if timing:
+            last_trace[:] = g.trace()
+            if args.trace:
+                trace[:] = last_trace
         g.close()
         return st
 
@@ -303,6 +326,7 @@ def measure_graph(R, name, args, dist=None, world=1, local=0, clocks=True, e2e=T
         inst_ms.append(float("nan"))
     st = _mean_stats(inst)
     last = inst[-1]
+    hub = hub_rounds(last_trace)
     peak, peak_kind = _peaks()
     out = {
         "workload": DESCR.get(name, name), "nu": nu, "nv": nv, "m": int(len(eu)),
@@ -334,7 +358,7 @@ def measure_graph(R, name, args, dist=None, world=1, local=0, clocks=True, e2e=T
                 "cost_recount": last["cost_recount"]},
         "peel_tier_wedges": last["peel_wedges"], "peel_tier_anchors": last["peel_anchors"],
         "peel_tier_pairs": last["peel_pairs"], "peel_tier_mids": last["peel_mids"],
-        "roofline": roofline(st, peak, peak_kind),
+        "hub_rounds": hub, "roofline": roofline(st, peak, peak_kind, hub),
     }
     import synth
     gpath = os.path.join(ROOT, "tests", "golden", name + ".json")
@@ -705,7 +729,7 @@ def run_ours(args):
               "phase_ms_timed_steps",
               "phase_wedges_per_s", "rounds_cd", "levels_fd", "subsets", "fd_slowest_task",
               "fd_heavy", "huc", "peel_tier_wedges", "peel_tier_anchors", "peel_tier_pairs",
-              "peel_tier_mids"):
+              "peel_tier_mids", "hub_rounds"):
         line[k] = main[k]
     if world == 1 and not args.no_cpu_baseline:
         line["cpu_baseline"] = cpu_baseline(*graph, name)

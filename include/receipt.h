@@ -204,7 +204,8 @@ typedef struct {
      * instead (one small matrix per round, no wedge through them walked): all
      * its anchors count under 1, with the wedges walked past those vertices:
      * wedges walked, middle vertices (edge visits), anchors (peeled vertices
-     * with updates), kernel launches and device time (only if timing != 0). */
+     * with updates), launches (rounds in which the tier's kernel ran) and device
+     * time (only if timing != 0). */
     uint64_t peel_wedges[5];
     uint64_t peel_mids[5];
     uint64_t peel_anchors[5];
@@ -237,7 +238,8 @@ typedef struct {
     /* Support atomics of the coarse-grained peel update per tier (the same
      * tiers as peel_wedges): one per pair (x, x') of a peeled vertex x and a
      * remaining vertex x' that share at least two neighbours (the pairs whose
-     * support changes). */
+     * support changes); of a round through the hubs, one per remaining vertex
+     * that the walks past the hubs change. */
     uint64_t peel_pairs[5];
     /* Start points of Algorithm 1 whose end points past the first 1,024 (which
      * are counted bit-sliced) take an aggregation tier, both sides: warp
@@ -310,8 +312,8 @@ receipt_status receipt_graph_max_degree(const receipt_graph *g, int32_t *max_deg
 /*
  * Per-vertex butterfly counts of both sides (Algorithm 1, pvBcnt).
  *   d_cnt_u : device uint64[nu] or NULL; d_cnt_v : device uint64[nv] or NULL.
- * Counts are indexed by original id. Enqueued on `stream`; ready when the
- * stream reaches this point (no host synchronisation).
+ * Counts are indexed by original id; ready when `stream` reaches this point.
+ * Synchronises `stream` two or three times (the tiers' sizes, the wedges).
  */
 receipt_status receipt_count_butterflies(receipt_graph *g, uint64_t *d_cnt_u,
                                          uint64_t *d_cnt_v, void *stream);

@@ -1627,7 +1627,9 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s) {
         int32_t nF_now = hst->nF;
         // one trace record per round from a copy of the state's header
         auto record_round = [&](const CdDev *h, bool rc, bool hubs_used) {
-            if (!rc)
+            if (hubs_used)
+                D.tier_launches[1]++;  // the round's counters are under 1
+            else if (!rc)
                 for (int t = 0; t < NTIER; t++) D.tier_launches[t]++;
             D.rounds++;
             receipt_round rr{};

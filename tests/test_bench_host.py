@@ -32,3 +32,23 @@ def test_traffic_only_for_the_captured_sources(monkeypatch):
     assert bench.roofline(STATS, 1000.0, "measured")["traffic"] is None
     monkeypatch.setattr(bench, "NCU_TRAFFIC", {})
     assert bench.roofline(STATS, 1000.0, "measured")["traffic"] is None
+
+
+def test_roofline_of_hub_rounds():
+    """Rounds through the hubs are told from others by their times, and named
+    when they are most of tier 1's."""
+    def round_(ms, wedges, anchors, recount=0):
+        return {"recount": recount, "ms": ms, "wedges": [1, wedges, 1, 1, 1],
+                "anchors": [1, anchors, 1, 1, 1]}
+    trace = [round_([0, 3.0, 0, 0, 0], 500, 20), round_([.1, .2, .1, .1, .1], 900, 9),
+             round_([0, 0, 0, 0, 0], 0, 0, 1), round_([0, 5.0, 0, 0, 0], 700, 30)]
+    hub = bench.hub_rounds(trace)
+    assert hub == {"rounds": 2, "ms": 8.0, "wedges": 1200, "anchors": 50}
+    st = dict(STATS, ms_peel=[1.0, 15.0, 0.5, 10.0, 3.0])
+    r = bench.roofline(st, 1000.0, "measured", hub)
+    assert r["kernel"].startswith("k_hub_") and r["launches"] == 2 and r["traffic"] is None
+    assert r["bytes_per_launch"] == (36 * 1200 + 24 * 50) / 2
+    assert abs(r["achieved"] - r["bytes_per_launch"] / 4e-3 / 1e9) < 1e-9
+    st = dict(STATS, ms_peel=[1.0, 17.0, 0.5, 10.0, 3.0])
+    assert bench.roofline(st, 1000.0, "measured", hub)["kernel"] == "k_cd_update_cta"
+    assert bench.roofline(STATS, 1000.0, "measured", hub)["kernel"] == "k_cd_update_slice"

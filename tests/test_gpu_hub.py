@@ -71,3 +71,14 @@ def test_without_memory_for_hub_rounds(R):
     st = g.stats()
     # all wedges (those of a hybrid anchor that overflows twice)
     assert sum(st["peel_wedges"]) >= st["wedges_cd"]
+
+
+def test_launches_count_the_rounds_a_tier_ran(R):
+    nu, nv, eu, ev = CASES["mixed"]()
+    g = R.Graph(eu, ev, nu, nv)
+    g.tip_decompose(0, P=4, huc=-1, timing=True)
+    st = g.stats()
+    hub = sum(1 for r in g.trace() if r["ms"][1] > 0 and not any(r["ms"][t] for t in (0, 2, 3, 4)))
+    assert hub > 0
+    assert st["peel_launches"][1] == st["rounds_cd"]
+    assert all(st["peel_launches"][t] == st["rounds_cd"] - hub for t in (0, 2, 3, 4))
