@@ -28,9 +28,9 @@ __global__ void k_tile_sums(const T *__restrict__ in, int64_t n, T *__restrict__
     if (threadIdx.x == 0) sums[blockIdx.x] = tot;
 }
 
+// `in` may be `out`: a block reads its tile before it writes it, and no other.
 template <typename T>
-__global__ void k_tile_scan(const T *__restrict__ in, T *__restrict__ out, int64_t n,
-                            const T *__restrict__ offsets) {
+__global__ void k_tile_scan(const T *in, T *out, int64_t n, const T *__restrict__ offsets) {
     __shared__ T tile[SCAN_TILE];
     __shared__ T tmp[33];
     int64_t base = (int64_t)blockIdx.x * SCAN_TILE;
