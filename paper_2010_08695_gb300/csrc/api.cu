@@ -412,6 +412,7 @@ void decompose_batch_impl(receipt_graph *const *gs, const receipt_side *sides, i
     std::vector<int64_t> abase(n + 1, 0), bbase(n + 1, 0), ebase(n + 1, 0);
     int dev = -1;
     int32_t maxdeg[2] = {0, 0};
+    uint64_t walks = 0;
     for (int i = 0; i < n; i++) {
         const receipt_graph *g = gs[i];
         if (!g) fail(RECEIPT_ERR_INVALID, "null graph in batch");
@@ -433,6 +434,7 @@ void decompose_batch_impl(receipt_graph *const *gs, const receipt_side *sides, i
         abase[i + 1] = abase[i] + p.n[0];
         bbase[i + 1] = bbase[i] + p.n[1];
         ebase[i + 1] = ebase[i] + p.m;
+        walks += g->count_walks;
         maxdeg[0] = std::max(maxdeg[0], g->max_deg[a]);
         maxdeg[1] = std::max(maxdeg[1], g->max_deg[b]);
     }
@@ -445,6 +447,7 @@ void decompose_batch_impl(receipt_graph *const *gs, const receipt_side *sides, i
     U.nv = (int32_t)NB;
     U.m = M;
     U.device = dev;
+    U.count_walks = walks;
     U.max_deg[0] = maxdeg[0];
     U.max_deg[1] = maxdeg[1];
     U.parts = abase;

@@ -127,6 +127,7 @@ struct receipt_graph {
     int64_t m = 0;
     int device = 0;
     int32_t max_deg[2] = {0, 0};
+    uint64_t count_walks = ~0ull;  // wedges that counting traverses, about (~0: unknown)
     receipt::Side side[2];
     receipt_stats stats{};
     std::vector<receipt_round> trace;  // rounds of the last decomposition

@@ -13,7 +13,7 @@
 // of exponents 2.5 / 2.1 84%. Both contributions are sums over end points, so
 // the count splits by end point:
 //
-//  * The first BITS end points (k_count_bits): every vertex's list has a mask
+//  * The first BITS end points (k_count_bits; where masks_pay): every vertex's list has a mask
 //    of its first 1,024 possible entries, one word per lane of a warp. A start
 //    point adds up its middle points' masks, cut at the prefix, in bit-sliced
 //    counters (plane p holds bit p of 32 counts per lane): ~12 instructions
@@ -1254,8 +1254,14 @@ __global__ void k_scatter_both(const unsigned long long *__restrict__ cu,
 
 }  // namespace
 
-static bool masks_pay(int64_t m, int64_t n) {
-    return (double)n * BITS / 8 <= 64.0 * (double)m + (256 << 20);
+// The masks pay from about 20 wedges an edge on (the passes over them cost 128
+// bytes and some 80 instructions an edge, whatever the wedges), where their memory
+// is not many times the graph's. Counts with / without them, ms: 10M edges on 6M
+// vertices, uniform, 1.7 wedges an edge: 7.8 / 4.7; 1M on 1M, power law, 6.9: 1.24 /
+// 0.81; 10M on 6.5M, 13.6: 8.1 / 7.5; 30M on 2M, 27: 21.0 / 22.2; 10M on 670,000,
+// 32: 6.8 / 9.1; 10M on 2M, 51: 7.1 / 10.8.
+static bool masks_pay(int64_t m, int64_t n, uint64_t walks) {
+    return walks / 20 >= (uint64_t)m && (double)n * BITS / 8 <= 64.0 * (double)m + (256 << 20);
 }
 
 CountMemory count_memory(int64_t m, int64_t nu, int64_t nv, int sms) {
@@ -1265,7 +1271,7 @@ CountMemory count_memory(int64_t m, int64_t nu, int64_t nv, int sms) {
     // huge start points (at most 4 m / HUGE_DEG chunks), the global tier
     b.needed = 8 * (size_t)m + 4 * (size_t)(CT_LISTS + 1) * n + 16 * (size_t)HOT_REPS * HOT_KEYS +
                4 * (size_t)m / HUGE_DEG * HUGE_NP * 128 + 8 * (size_t)sms * n_max;
-    b.optional = masks_pay(m, (int64_t)n) ? (BITS / 8 + 4) * n : 0;
+    b.optional = masks_pay(m, (int64_t)n, ~0ull) ? (BITS / 8 + 4) * n : 0;
     return b;
 }
 
@@ -1302,13 +1308,12 @@ uint64_t count_local(const receipt_graph *g, unsigned long long *cnt_u,
         base.alloc(n, s);
         RC_CUDA(cudaMemcpyAsync(first.get(), hf.data(), 4 * hf.size(), cudaMemcpyHostToDevice, s));
     }
-    // masks of both sides' lists (128 bytes a vertex), unless the vertices are
-    // many for the edges or there is no memory for them: then every end point
-    // is past the masks
+    // masks of both sides' lists (128 bytes a vertex), unless the wedges are few
+    // or there is no memory for them: then every end point is past the masks
     DevBuf<uint32_t> mask;
     DevBuf<int32_t> held;
     const bool bits =
-        masks_pay(m, n) && mask.try_alloc((size_t)n * 32, s) && held.try_alloc(n, s);
+        masks_pay(m, n, g->count_walks) && mask.try_alloc((size_t)n * 32, s) && held.try_alloc(n, s);
     if (!bits) mask.release();
     DevBuf<unsigned long long> hot;
     if (m >= HOT_MIN_M && !first.get()) {

@@ -103,3 +103,32 @@ def test_recount_without_memory(R):
         t = R.as_u64(g.tip_decompose(0, huc_factor_1024=1))
     assert np.array_equal(t, want)
     assert g.stats()["huc_recounts"] == 0
+
+
+# counting's masks (132 bytes a vertex) pay from about 20 wedges an edge on
+@pytest.mark.parametrize("nu,nv,m,gamma,masks", [(400_000, 400_000, 600_000, 0, False),
+                                                 (300_000, 300_000, 300_000, 2.5, False),
+                                                 (100_000, 20_000, 1_000_000, 2.1, True)])
+def test_masks_where_they_pay(R, nu, nv, m, gamma, masks):
+    import torch
+    eu, ev = synth.chung_lu(nu, nv, m, gamma, gamma, 2) if gamma else synth.er(nu, nv, m, 2)
+    g = R.Graph(eu, ev, nu, nv)
+    cu, cv = oracle.count_vp(eu, ev, nu, nv)
+    lib, pool, v = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(), ctypes.c_uint64(0)
+    assert lib.cuDeviceGetDefaultMemPool(ctypes.byref(pool), torch.cuda.current_device()) == 0
+    high = []
+    for limit in (-1, 0):
+        R.receipt_optional_memory(limit)
+        torch.cuda.synchronize()
+        v.value = 0
+        assert lib.cuMemPoolSetAttribute(pool, 8, ctypes.byref(v)) == 0  # most bytes used
+        gu, gv = g.count_butterflies()
+        R.receipt_optional_memory(-1)
+        torch.cuda.synchronize()
+        assert lib.cuMemPoolGetAttribute(pool, 8, ctypes.byref(v)) == 0
+        high.append(v.value)
+        assert np.array_equal(R.as_u64(gu), cu) and np.array_equal(R.as_u64(gv), cv)
+    if not masks:
+        assert high[0] == high[1]
+    else:
+        assert high[0] != high[1]
