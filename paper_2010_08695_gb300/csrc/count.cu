@@ -70,6 +70,15 @@ constexpr int HASH_W = HASH_SLOTS / 2;
 constexpr int HASH_THREADS = 256;
 using CountHash = CtaHashT<HASH_SLOTS>;
 
+// A tier walks as many middle points a step as it has threads, ~0.9 us a step and
+// walk however few their wedges are. Hubs with few wedges (the first start points:
+// hardly an end point comes before them) of more steps than this take the next
+// larger CTA, up to the hybrid's 1,024 threads. Counts of 2M edges on 2.6M vertices
+// (degrees up to 69,633) / 1.5M on 2.7M (29,521) / 450k on 98,000 (23,327), ms: any
+// degree 2.28 / 1.92 / 0.92, 64 steps 1.72 / 1.06 / 0.68, 16 1.20 / 0.81 / 0.63, 8
+// 1.13 / 0.74 / 0.55.
+constexpr int TIER_STEPS = 8;
+
 // One side as start side A (B: the other side).
 struct CountSide {
     const int64_t *offA;
@@ -111,14 +120,15 @@ constexpr int COUNT_CTRS = 2 * CT_LISTS;
 
 __device__ __forceinline__ int32_t tier_of(const CountPlan &p, int64_t W, int64_t T, int64_t deg,
                                            int32_t sp) {
-    if (W <= WARP_MAX_W) return CT_WARP;
+    if (W <= WARP_MAX_W && deg <= 32 * TIER_STEPS) return CT_WARP;
     if (deg < 65535) {
-        if (!p.few && W <= 4096 && T <= 256) return CT_DENSE64;
-        if (W <= 65536 && T <= 1024) return CT_DENSE256;
+        if (!p.few && W <= 4096 && T <= 256 && deg <= 64 * TIER_STEPS) return CT_DENSE64;
+        if (W <= 65536 && T <= 1024 && deg <= 256 * TIER_STEPS) return CT_DENSE256;
     }
-    if (!p.few && W <= HASH_W) return CT_HASH;
+    if (!p.few && W <= HASH_W && (deg <= HASH_THREADS * TIER_STEPS || deg >= 65535)) return CT_HASH;
     if (deg < 65535) {
-        if (!p.few && T <= 2048 && W < (1ll << 32)) return CT_DENSE512;
+        if (!p.few && T <= 2048 && W < (1ll << 32) && (deg <= 512 * TIER_STEPS || sp > p.cta_keys))
+            return CT_DENSE512;
         if (sp <= p.cta_keys) return CT_HYBRID;
     }
     return CT_GLOBAL;
@@ -208,7 +218,10 @@ __global__ void __launch_bounds__(256) k_count_plan(CountPlan p) {
     if (lane == 0 && wsum) atomicAdd(p.wedges, wsum);
 }
 
-__global__ void __launch_bounds__(256) k_count_plan_wide(CountPlan p) {
+// A CTA per start point. (256 threads / 512 / 1,024: a hub of degree 69,633 196 / 99
+// / 50 us of its plan; counts of 20M edges with degrees up to 100,000 on both sides
+// 17.25 / 17.15 / 17.40 ms.)
+__global__ void __launch_bounds__(512) k_count_plan_wide(CountPlan p) {
     __shared__ unsigned long long s_w, s_t;
     const int32_t n = p.n[CT_WIDE];
     for (int32_t i = blockIdx.x; i < n; i += gridDim.x) {
@@ -220,7 +233,7 @@ __global__ void __launch_bounds__(256) k_count_plan_wide(CountPlan p) {
         const int64_t q0 = S.offA[sp], q1 = S.offA[sp + 1];
         const int32_t base = (S.first ? S.base[sp] : 0) + (S.mask ? BITS : 0);
         unsigned long long W = 0, T = 0;
-        for (int64_t q = q0 + threadIdx.x; q < q1; q += 256) {
+        for (int64_t q = q0 + threadIdx.x; q < q1; q += 512) {
             int32_t t;
             W += (unsigned long long)plan_edge(S, sp, base, q, t);
             T += (unsigned long long)t;
@@ -1346,7 +1359,7 @@ uint64_t count_local(const receipt_graph *g, unsigned long long *cnt_u,
             RC_LAUNCH();
         }
     launch_plan(p, n, s);
-    k_count_plan_wide<<<sms * 8, 256, 0, s>>>(p);
+    k_count_plan_wide<<<sms * 4, 512, 0, s>>>(p);
     RC_LAUNCH();
     if (bits) {
         k_count_bits<<<(unsigned)std::min<int64_t>((n + 7) / 8, (int64_t)sms * 32), 256, 0, s>>>(p);
@@ -1505,7 +1518,7 @@ void count_noalloc(const receipt_graph *g, unsigned long long *d_cnt_u,
                                nullptr, plen + (A ? m : 0), nullptr, nullptr, nullptr, nullptr, SA.n, 0};
         }
         launch_plan(p, n, s);
-        k_count_plan_wide<<<sms, 256, 0, s>>>(p);
+        k_count_plan_wide<<<sms, 512, 0, s>>>(p);
         RC_LAUNCH();
         launch_tiers(p, nullptr, n, s);
         const size_t gsm = MID_CHUNK * 8 + CHUNK_BYTES;

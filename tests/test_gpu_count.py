@@ -77,3 +77,22 @@ def test_union_counts_from_its_own_first_key(R):
         assert np.array_equal(R.as_u64(o), w)
     # no start point needs the global counters
     assert st["count_points"][3] == 0 and st["count_points"][4] == 0
+
+
+# hubs whose end points nearly all come after them: degrees on both sides of the
+# steps that each tier takes (32, 64, 256, 512 middle points a step, 8 steps), with
+# a few wedges (other hubs' common neighbours) and with many
+@pytest.mark.parametrize("nu,m", [(70_000, 30_000), (120_000, 400_000)])
+def test_hubs_of_few_wedges(R, nu, m):
+    degs = [d + k for d in (255, 512, 2048, 4096, 9000, 20_000, 30_000) for k in (0, 1)]
+    eu, ev = _with_degrees(nu, 20_000, degs, m, 7)
+    _check(R, eu, ev, nu, 20_000, False)
+    # ... and of degree 65,535 and more
+    eu, ev = _with_degrees(nu, 20_000, [300, 65_534, 65_535, 65_536, 66_000], m, 8)
+    _check(R, eu, ev, nu, 20_000, False)
+
+
+def test_hubs_of_few_wedges_without_allocations(R):
+    degs = [d + k for d in (255, 512, 2048, 4096, 9000, 30_000, 65_533) for k in (0, 1)]
+    eu, ev = _with_degrees(65_536, 9_000, degs, 60_000, 9)
+    _check(R, eu, ev, 65_536, 9_000, True)
