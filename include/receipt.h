@@ -107,9 +107,10 @@ typedef struct {
      * range is at most members / 2^16 wide, and tasks whose members without
      * an update list (or all members, when the lists would not fit an eighth
      * of the device's memory) walk at least 2^23 wedges and at least
-     * 4 x 2^15 per member of the task, and the longest tasks whose lists are
-     * long for their few levels (narrow ranges of many wedges, as in uniform
-     * and dense graphs) while that shortens the step. A level of such a task with at
+     * 4 x 2^15 per member of the task, and the longest dense tasks (16 wedges and
+     * more for each two members) while that shortens the step; another task goes
+     * over to all CTAs at a level whose peeled members' lists are longer than
+     * one CTA should apply (it then counts as heavy, with all its levels). A level of such a task with at
      * most 32 members with big walks spreads each one's walk over the CTAs
      * in equal wedge shares. -1 = never. Speed only. */
     int64_t fd_heavy_w;

@@ -254,6 +254,56 @@ __global__ void k_task_weights(const int32_t *__restrict__ tstart, const int32_t
         w[t] = (unsigned long long)(cw[tstart[t] + tlen[t]] - cw[tstart[t]] - add * tlen[t]);
 }
 
+// ------------------------------------------------------------------------
+// Tasks that one CTA hands over to all of them
+//
+// On graphs whose vertices are much alike (uniform ones, members of the same
+// hubs) a task's levels peel a few members each until one sets off the next, and
+// three to ten levels peel nearly all: 150 levels of 860 members, then 2,059 and
+// 1,743 with lists of 4,650 entries. A CTA applies an entry in 0.85 ns (17 ms); all
+// CTAs take ~70 us a level and 3.3 ps a wedge. When a level's lists cost more than
+// that, the hand-over (~0.6 ms) and what was handed over before (one after the
+// other), the CTA leaves the task as it was before the level, and it is peeled on
+// as a heavy task. Levels of power-law graphs stay far below (no level of 150,000
+// entries in tasks of 10M and 40M edges; the line is ~800,000).
+// Step by one CTA / handed over / heavy from the start, ms: 3.9M uniform edges,
+// 4,660 members 19.3 / 7.8 / 11.4; 20M, 30,000 members 327 / 91 / 114; 3M, 10,000
+// members 45 / 15 / 27; 1.5M power-law edges with a hub of degree 125,000 in 245
+// tasks 185 / 45 / 86; 1.7M uniform, 35,400 members 10.9 / 8.2 / 6.3.
+// ------------------------------------------------------------------------
+struct FdHandOver {
+    const unsigned long long *tw;  // per task: wedges (null: no task is handed over)
+    int32_t *count;                // [0]: tasks handed over or, for a moment, refused;
+    int32_t *list;                 // [1]: handed over; their ids
+    unsigned long long *level;     // per task: its level then
+};
+constexpr float FD_HAND_OVER_NS = 6e5f;
+
+// ns of one peeled member of a task of n: from its list (entries: all lists'), as
+// a heavy task
+__device__ __forceinline__ float2 fd_member_ns(unsigned long long entries, unsigned long long w,
+                                               int32_t n) {
+    return make_float2(0.85f * (float)entries / (float)n, 0.0033f * (float)w / (float)n);
+}
+// Members of a level from which on it may pay.
+__device__ __forceinline__ int fd_hand_over_from(float2 ns) {
+    const float gain = ns.x - ns.y;
+    return gain > 0.f ? (int)fminf(2e9f, (FD_HAND_OVER_NS + 70000.f) / gain) + 1 : INT32_MAX;
+}
+// Whether a level of np members is (one thread).
+__device__ __forceinline__ bool fd_hand_over(const FdHandOver &h, float2 ns, int np, int32_t task,
+                                             unsigned long long level) {
+    const int before = atomicAdd(h.count, 1);
+    const float cost = FD_HAND_OVER_NS + 70000.f + ns.y * (float)np;
+    if (ns.x * (float)np <= (float)(before + 1) * cost) {
+        atomicSub(h.count, 1);
+        return false;
+    }
+    h.list[atomicAdd(h.count + 1, 1)] = task;
+    h.level[task] = level;
+    return true;
+}
+
 struct FdArgs {
     const int32_t *queue;      // task ids, LPT order
     int32_t P;                 // tasks
@@ -281,6 +331,7 @@ struct FdArgs {
     unsigned long long *stats; // [0] wedges, [1] levels
     unsigned long long *sub_ns;     // per task: nanoseconds spent
     unsigned long long *sub_levels; // per task: peeling levels
+    FdHandOver ho;
 };
 
 struct FdMids {
@@ -955,6 +1006,8 @@ __global__ void __launch_bounds__(FD_THREADS, 1) k_fd_peel(FdArgs a) {
     __shared__ unsigned long long s_rmn;  // minimum of a refilled window
     __shared__ unsigned long long s_T;   // window bound
     __shared__ int32_t s_scan[33];
+    __shared__ unsigned long long s_entries;
+    __shared__ int s_over;
     FdEngine H;
     Chunk ch;
     fd_bind_smem(smem, &s_dn, H, ch);
@@ -966,7 +1019,10 @@ __global__ void __launch_bounds__(FD_THREADS, 1) k_fd_peel(FdArgs a) {
     __syncthreads();
     for (;;) {
         __syncthreads();
-        if (threadIdx.x == 0) s_t = atomicAdd(a.qhead, 1);
+        if (threadIdx.x == 0) {
+            s_t = atomicAdd(a.qhead, 1);
+            s_entries = 0;
+        }
         __syncthreads();
         const int t = s_t;
         if (t >= a.P) break;
@@ -990,15 +1046,22 @@ __global__ void __launch_bounds__(FD_THREADS, 1) k_fd_peel(FdArgs a) {
         const int32_t *mem = a.members + mb;
         const FdMember *info = a.info + mb;
         const int rb = fp_rank_bits(ni);
+        unsigned long long entries = 0;
         for (int r = threadIdx.x; r < ni; r += blockDim.x) {
             fsup[r] = a.init[mem[r]];
             alive[r] = 1;
             flist[r] = r;
+            const unsigned long long q = a.rec[mb + r];
+            entries += q == FP_NONE ? 0 : q & 0xffffffu;
         }
+        entries = warp_sum(entries);
+        if (lane == 0 && entries) atomicAdd(&s_entries, entries);
         int32_t nalive = ni, nfar = ni, ncand = 0;
         unsigned long long level = 0, mn = ~0ull;
         int par = 0;
         __syncthreads();
+        const float2 ns = a.ho.tw ? fd_member_ns(s_entries, a.ho.tw[i], ni) : make_float2(0.f, 0.f);
+        const int wide_level = fd_hand_over_from(ns);
         while (nalive > 0) {
             if (ncand == 0) {
                 // Window refill: the smallest supports among the far members,
@@ -1125,6 +1188,19 @@ __global__ void __launch_bounds__(FD_THREADS, 1) k_fd_peel(FdArgs a) {
                 clist = clist_next;
                 clist_next = tmp;
             }
+            if (s_np >= wide_level) {
+                if (threadIdx.x == 0) s_over = fd_hand_over(a.ho, ns, s_np, i, level);
+                __syncthreads();
+                if (s_over) {
+                    // back to where the level began (any support up to mu does)
+                    for (int j = threadIdx.x; j < s_np; j += blockDim.x) {
+                        fsup[plist[j]] = mu;
+                        alive[plist[j]] = 1;
+                    }
+                    levels--;
+                    break;
+                }
+            }
             // updates of the peeled vertices inside G_i
             FdEmit emit{fsup, alive, &s_mn[par], T, clist, &s_nk[par]};
             const int np = fd_lists(a.pool, a.rec + mb, plist, s_np, rb, emit, &s_nbig);
@@ -1217,8 +1293,11 @@ struct FsArgs {
     const unsigned long long *init;
     unsigned long long *rtip;  // by member position
     unsigned long long *tip;   // output, original ids
+    unsigned long long *fsup;  // supports of a task that is handed over, by member position
+    uint8_t *alive;
     unsigned long long *stats; // [0] wedges, [1] levels
     unsigned long long *sub_ns, *sub_levels;
+    FdHandOver ho;
 };
 
 // minimum over a warp, in every lane
@@ -1235,6 +1314,8 @@ __global__ void __launch_bounds__(FD_THREADS, 1) k_fd_small(FsArgs a) {
     // by level parity: a level's counts, and the warps' minima for the next
     __shared__ int s_np[2], s_peel[2];
     __shared__ unsigned long long s_mn[2][FD_WARPS];
+    __shared__ unsigned long long s_entries;
+    __shared__ int s_over;
     Chunk ch;
     ch.beg = (int64_t *)smem;
     ch.pre = (int32_t *)(ch.beg + FD_THREADS);
@@ -1249,7 +1330,10 @@ __global__ void __launch_bounds__(FD_THREADS, 1) k_fd_small(FsArgs a) {
     unsigned long long wedges = 0, levels = 0;  // wedges: per warp (lane 0)
     for (;;) {
         __syncthreads();
-        if (threadIdx.x == 0) s_t = atomicAdd(a.qhead, 1);
+        if (threadIdx.x == 0) {
+            s_t = atomicAdd(a.qhead, 1);
+            s_entries = 0;
+        }
         __syncthreads();
         const int t = s_t;
         if (t >= a.T) break;
@@ -1264,11 +1348,16 @@ __global__ void __launch_bounds__(FD_THREADS, 1) k_fd_small(FsArgs a) {
         const int32_t nip = (ni + 1) & ~1;
         uint16_t *plist = (uint16_t *)(sup + nip);
         unsigned long long mn = FS_DEAD;
+        uint32_t entries = 0;  // below FS_MEMBERS^2 in all
         for (int r = threadIdx.x; r < nip; r += FD_THREADS) {
             const unsigned long long v = r < ni ? a.init[mem[r]] : FS_DEAD;
             sup[r] = v;
             mn = v < mn ? v : mn;
+            const unsigned long long q = r < ni ? a.rec[mb + r] : 0;
+            entries += q == FP_NONE ? 0 : (uint32_t)(q & 0xffffffu);
         }
+        entries = __reduce_add_sync(0xffffffffu, entries);
+        if (lane == 0 && entries) atomicAdd(&s_entries, (unsigned long long)entries);
         mn = warp_min_all(mn);
         if (lane == 0) s_mn[0][warp] = mn;
         if (threadIdx.x == 0) s_np[0] = s_peel[0] = 0;
@@ -1277,6 +1366,9 @@ __global__ void __launch_bounds__(FD_THREADS, 1) k_fd_small(FsArgs a) {
         int32_t nalive = ni;
         int par = 0;
         __syncthreads();
+        const float2 ns = a.ho.tw ? fd_member_ns(s_entries, a.ho.tw[i], ni) : make_float2(0.f, 0.f);
+        const int wide_level = fd_hand_over_from(ns);
+        bool over = false;
         while (nalive > 0) {
             // ---- peel every member with support <= mu; minimum of the others
             mn = warp_min_all(s_mn[par][lane & (FD_WARPS - 1)]);
@@ -1326,6 +1418,18 @@ __global__ void __launch_bounds__(FD_THREADS, 1) k_fd_small(FsArgs a) {
             __syncthreads();
             nalive -= s_peel[par];
             if (threadIdx.x == 0) s_np[par ^ 1] = s_peel[par ^ 1] = 0;
+            if (s_np[par] >= wide_level) {
+                if (threadIdx.x == 0) s_over = fd_hand_over(a.ho, ns, s_np[par], i, level);
+                __syncthreads();
+                over = s_over;
+                if (over) {
+                    // back to where the level began (any support up to mu does)
+                    for (int j = threadIdx.x; j < s_np[par]; j += FD_THREADS) sup[plist[j]] = mu;
+                    levels--;
+                    __syncthreads();
+                    break;
+                }
+            }
             // ---- updates of the peeled members inside G_i
             const int np = fd_lists(a.pool, a.rec + mb, plist, s_np[par], rb, emit, &s_nbig);
             if (np > 0) {
@@ -1346,7 +1450,16 @@ __global__ void __launch_bounds__(FD_THREADS, 1) k_fd_small(FsArgs a) {
             par ^= 1;
             __syncthreads();
         }
-        for (int r = threadIdx.x; r < ni; r += FD_THREADS) a.tip[a.new2old[mem[r]]] = rtip[r];
+        for (int r = threadIdx.x; r < ni; r += FD_THREADS) {
+            if (!over) {
+                a.tip[a.new2old[mem[r]]] = rtip[r];
+                continue;
+            }
+            const unsigned long long v = sup[r];
+            a.fsup[mb + r] = v;
+            a.alive[mb + r] = v != FS_DEAD;
+            if (v == FS_DEAD) a.tip[a.new2old[mem[r]]] = rtip[r];
+        }
         if (threadIdx.x == 0) {
             unsigned long long t_end;
             asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t_end));
@@ -1441,6 +1554,25 @@ __global__ void k_fdh_init(FdhArgs a) {
         }
     }
     if (lane == 0 && mn != ~0ull) atomicMin(&a.st->mn, mn);
+}
+
+// A task that was handed over: its supports and alive members are there.
+__global__ void k_fdh_resume(FdhArgs a, const unsigned long long *__restrict__ level) {
+    unsigned long long mn = ~0ull;
+    int32_t alive = 0;
+    for (int32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < a.ni; r += gridDim.x * blockDim.x)
+        if (a.alive[r]) {
+            const unsigned long long v = a.fsup[r];
+            alive++;
+            mn = v < mn ? v : mn;
+        }
+    alive = warp_sum(alive);
+    mn = warp_min(mn);
+    if ((threadIdx.x & 31) == 0 && alive) {
+        atomicAdd(&a.st->nalive, alive);
+        atomicMin(&a.st->mn, mn);
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.st->level = *level;
 }
 
 __global__ void k_fdh_select(FdhArgs a) {
@@ -1732,24 +1864,21 @@ struct ListTask {
     uint64_t lo, hi;
 };
 
-// Tasks that all CTAs peel sooner than one CTA applies their lists. One CTA
-// takes 2.5 us a level and 0.85 ns an entry, all CTAs ~70 us a level and 3 ps a
-// wedge (the lists themselves 1.7 ps), so what decides is the entries a level
-// peels: heavy wins from ~10^5. Power-law graphs have at most 1.5 10^4, a level
-// a member or two; uniform and dense ones, whose supports lie so close that one
-// level sets off the next, 10^5 to 10^7 (20M edges, 30,000 members, 524 levels,
-// 3.8 10^8 entries: 317 ms in one CTA, 109 heavy; 6M edges, 37,500 members, 92
-// levels: 1,301 / 174; 2M edges, 4,700 members, 52 levels: 18.8 / 7.2; but 2M
-// edges, 18,000 members, 39 levels: 1.8 / 2.2).
-// Neither is known before the peel. Levels: at most a member each, and while
-// every peeled member sets off others as many as the range's share of its bound
-// (the narrowest ranges, one bucket, hold 1/32), or 16 to each support of a
-// range of few supports (measured: 1.2 to 14 times fewer). Entries: a fourth of
-// the wedges (measured: up to 0.3), at most one for every two members, and what
-// pairs of members that share c << 1 middle vertices on average make of them,
-// c^2 / 2 each.
+// Dense tasks that all CTAs peel sooner than their lists are made and applied by
+// one CTA (others are handed over when that shows, FdHandOver, after their lists
+// were made: 1.7 ps a wedge, which dense tasks have many of for an entry. 8M edges
+// on 20,000 x 1,000, 160 wedges for each two members: the step took 428 ms in one
+// CTA, 232 handed over, 152 so; 3M on 10,000 x 50,000, 1.8 wedges: 45, 15, 27; 2M on
+// 5,000 x 20,000, 8: 20, 6.8, 8.4).
+// One CTA takes 2.5 us a level and 0.85 ns an entry, all CTAs ~70 us a level and 3
+// ps a wedge. The levels are not known before the peel: at most a member each, and
+// while every peeled member sets off others as many as the range's share of its
+// bound (the narrowest ranges, one bucket, hold 1/32), or 16 to each support of a
+// range of few supports (measured: 1.2 to 14 times fewer). Entries: one for every
+// two members (all share middle vertices).
 // One CTA a task peels the tasks left side by side, the heavy ones come one by
 // one: the longest go first while the sum falls.
+constexpr double DENSE_TASK = 16;  // wedges for each two members
 static std::vector<int32_t> heavy_by_lists(std::vector<ListTask> t, int ctas) {
     auto levels = [](const ListTask &k) {
         const double span = (double)(k.hi - k.lo);
@@ -1757,8 +1886,7 @@ static std::vector<int32_t> heavy_by_lists(std::vector<ListTask> t, int ctas) {
                                       std::min((double)k.n, 16.0 * span)));
     };
     auto by_list = [&](const ListTask &k) {
-        const double w = (double)k.w, pairs = (double)k.n * (double)k.n;
-        const double e = std::min({w / 4, pairs, w * (w / pairs) / 2});
+        const double e = std::min((double)k.w / 4, (double)k.n * (double)k.n);
         return 2500.0 * levels(k) + 0.85 * e;
     };
     auto heavy = [&](const ListTask &k) { return 7e4 * levels(k) + 0.003 * (double)k.w; };
@@ -1911,6 +2039,7 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
     // task weights: walk sizes summed over the task's members (LPT key)
     std::vector<unsigned long long> tw(T), tlw(T);  // tlw: of members without a list
     DevBuf<int64_t> cw;  // prefix of the members' costs, by member position
+    DevBuf<unsigned long long> dtw;  // tw on the device
     DevBuf<int32_t> d_tstart(T > 0 ? T : 1, s), d_tlen(T > 0 ? T : 1, s), d_tkb(T > 0 ? T : 1, s);
     if (T > 0) {
         RC_CUDA(cudaMemcpyAsync(d_tstart.get(), tstart.data(), 4 * (size_t)T, cudaMemcpyHostToDevice, s));
@@ -1918,7 +2047,7 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
         RC_CUDA(cudaMemcpyAsync(d_tkb.get(), tkb.data(), 4 * (size_t)T, cudaMemcpyHostToDevice, s));
         DevBuf<int64_t> w64(n + 1, s);
         cw.alloc(n + 1, s);
-        DevBuf<unsigned long long> dtw(T, s);
+        dtw.alloc(T, s);
         k_walk_cost<<<ceil_div(n, 256), 256, 0, s>>>(wr.get(), n, FP_MEMBER_COST, info.get(),
                                                      members.get(), D.sub, w64.get(), wsub.get());
         RC_LAUNCH();
@@ -1959,9 +2088,9 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
     // with a range so narrow that few levels peel them: a one-CTA level scans
     // at ~8 ns a member (1.9M members, width 1, one level: 16 ms, 0.8 heavy;
     // 132K members, width 1, 28 levels: 27 ms for the step, 29 unless heavy);
-    // (c) tasks whose lists are long for their levels (heavy_by_lists).
-    // Otherwise one CTA is faster: 4,751 levels of 80K members take 36 ms
-    // there and took 590 heavy, 20,000 levels of 42K members 117 ms.
+    // (c) dense tasks (heavy_by_lists). Otherwise one CTA is faster (4,751
+    // levels of 80K members take 36 ms there and took 590 heavy, 20,000 levels
+    // of 42K members 117 ms), or notices that it is not (FdHandOver).
     // The pool has room for the most entries the lists can have as long as that
     // is cheap (FD_LIST_BYTES an edge), else for about as many as they will have,
     // up to an eighth of the memory there is; members past it walk.
@@ -2003,6 +2132,7 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
                 std::vector<ListTask> lt;
                 for (int32_t t : back) {
                     const int sub_i = tsub[t];
+                    if ((double)tw[t] < DENSE_TASK * (double)tlen[t] * (double)tlen[t]) continue;
                     const bool open = (size_t)sub_i + 1 >= D.bounds.size();
                     lt.push_back(ListTask{t, tlen[t], tw[t], open ? 0 : D.bounds[sub_i],
                                           open ? ~0ull : D.bounds[sub_i + 1]});
@@ -2051,7 +2181,8 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
     DevBuf<uint8_t> alive(n, s);
     DevBuf<int32_t> alist(n, s), alist2(n, s), clist(n, s), clist2(n, s), plist(n, s), blist(n, s),
         qhead(2, s);
-    DevBuf<unsigned long long> stats(2, s), sub_ns(T > 0 ? T : 1, s), sub_lv(T > 0 ? T : 1, s);
+    // stats: wedges, levels, tasks handed over (FdHandOver::count)
+    DevBuf<unsigned long long> stats(3, s), sub_ns(T > 0 ? T : 1, s), sub_lv(T > 0 ? T : 1, s);
     qhead.zero();
     stats.zero();
     sub_ns.zero();
@@ -2060,8 +2191,13 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
     D.fd_heavy_ms = 0;
     D.fd_heavy_levels = 0;
     D.fd_split_levels = 0;
-    std::vector<FdhDev> hh(nheavy);
-    if (nheavy > 0) {
+    std::vector<FdhDev> hh;  // of the heavy tasks, in the order in which they were peeled
+    std::vector<int32_t> heavy_tasks;
+    // level: null, or per task the level at which it was handed over
+    auto peel_heavy = [&](const int32_t *tasks, int count, const unsigned long long *level) {
+        heavy_tasks.insert(heavy_tasks.end(), tasks, tasks + count);
+        hh.resize(heavy_tasks.size());
+        FdhDev *hh0 = hh.data() + (hh.size() - count);
         DevBuf<FdhDev> hst(1, s);
         const size_t smem_h = FdEngine::bytes() + CHUNK_BYTES;
         allow_max_smem((const void *)k_fdh_cta);
@@ -2070,12 +2206,12 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
         const int grid_h = sms * std::max(occ_h, 1);
         // global counters of split levels, sized for the largest heavy task
         int32_t ni_max = 1;
-        for (int h = 0; h < nheavy; h++) ni_max = std::max(ni_max, tlen[hq[h]]);
+        for (int h = 0; h < count; h++) ni_max = std::max(ni_max, tlen[tasks[h]]);
         DevBuf<uint32_t> gcnt((size_t)FDH_SPLIT_NB * ni_max, s);
         DevBuf<int32_t> gtl((size_t)FDH_SPLIT_NB * ni_max, s);
         gcnt.zero();
-        for (int h = 0; h < nheavy; h++) {
-            const int32_t i = hq[h];
+        for (int h = 0; h < count; h++) {
+            const int32_t i = tasks[h];
             const int32_t mb = tstart[i], ni = tlen[i];
             FdhArgs ha{members.get() + mb, ni,           tkb[i],         S.off,
                        fd_beg.get(),       fd_len.get(), fd_adj.get(),   S.new2old,
@@ -2084,9 +2220,12 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
                        hst.get(),          gcnt.get(),   gtl.get(),      wpre.get()};
             const int gm = std::max(1, std::min(ceil_div(ni, 256), sms * 4));
             const int gi = std::max(1, std::min(ceil_div((int64_t)ni * 32, 256), sms * 16));
-            k_fdh_reset<<<1, 1, 0, s>>>(hst.get(), ni);
+            k_fdh_reset<<<1, 1, 0, s>>>(hst.get(), level ? 0 : ni);
             RC_LAUNCH();
-            k_fdh_init<<<gi, 256, 0, s>>>(ha);
+            if (level)
+                k_fdh_resume<<<gm, 256, 0, s>>>(ha, level + i);
+            else
+                k_fdh_init<<<gi, 256, 0, s>>>(ha);
             RC_LAUNCH();
             // Recount rule (Sec. 4.1) of this task: a level recounts when its
             // peeled members' walks exceed factor * C_rcnt of the task; no
@@ -2096,9 +2235,9 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
             if (D.fd_huc == 0) {
                 k_fdh_rcnt<<<gi, 256, 0, s>>>(ha);
                 RC_LAUNCH();
-                RC_CUDA(cudaMemcpyAsync(&hh[h], hst.get(), sizeof(FdhDev), cudaMemcpyDeviceToHost, s));
+                RC_CUDA(cudaMemcpyAsync(&hh0[h], hst.get(), sizeof(FdhDev), cudaMemcpyDeviceToHost, s));
                 RC_CUDA(cudaStreamSynchronize(s));
-                rcnt = hh[h].rcnt;
+                rcnt = hh0[h].rcnt;
                 may_recount = rcnt > 0 && (double)tw[i] > D.huc_factor * (double)rcnt;
             }
             // the levels in one graph launch: a while-node repeats select,
@@ -2134,15 +2273,18 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
                 RC_CUDA(cudaGraphInstantiate(&lg.e, lg.g, 0));
                 RC_CUDA(cudaGraphLaunch(lg.e, s));
             } else {
-                fdh_levels_with_recount(D, ha, hst.get(), &hh[h], rcnt, grid_h, smem_h, gm, s);
+                fdh_levels_with_recount(D, ha, hst.get(), &hh0[h], rcnt, grid_h, smem_h, gm, s);
             }
-            RC_CUDA(cudaMemcpyAsync(&hh[h], hst.get(), sizeof(FdhDev), cudaMemcpyDeviceToHost, s));
+            RC_CUDA(cudaMemcpyAsync(&hh0[h], hst.get(), sizeof(FdhDev), cudaMemcpyDeviceToHost, s));
             RC_CUDA(cudaStreamSynchronize(s));
-            if (!may_recount) count_launches(5 * (uint64_t)hh[h].levels);
-            D.fd_heavy_ms += (float)((hh[h].t1 - hh[h].t0) * 1e-6);
-            D.fd_heavy_levels += (int64_t)hh[h].levels;
-            D.fd_split_levels += (int64_t)hh[h].splits;
+            if (!may_recount) count_launches(5 * (uint64_t)hh0[h].levels);
+            D.fd_heavy_ms += (float)((hh0[h].t1 - hh0[h].t0) * 1e-6);
+            D.fd_heavy_levels += (int64_t)hh0[h].levels;
+            D.fd_split_levels += (int64_t)hh0[h].splits;
         }
+    };
+    if (nheavy > 0) {
+        peel_heavy(hq.data(), nheavy, nullptr);
         RC_CUDA(cudaMemcpyAsync(qhead.get(), &nheavy, 4, cudaMemcpyHostToDevice, s));
     }
     DevBuf<unsigned long long> rtip(nsmall_at < T ? n : 1, s);
@@ -2180,6 +2322,11 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
             RC_LAUNCH();
         }
     }
+    // tasks that go over to all CTAs after all (automatic rule)
+    DevBuf<int32_t> over(T > 0 ? T : 1, s);
+    DevBuf<unsigned long long> over_level(T > 0 ? T : 1, s);
+    const FdHandOver ho{D.fd_heavy_w == 0 ? dtw.get() : nullptr, (int32_t *)(stats.get() + 2),
+                        over.get(), over_level.get()};
     // large and small tasks side by side
     const int nlarge = nsmall_at - nheavy, nsmall = T - nsmall_at;
     cudaEvent_t fork_ev[2] = {};
@@ -2208,7 +2355,7 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
                  D.init,        fsup.get(),  alive.get(),     alist.get(),  alist2.get(),
                  clist.get(),   clist2.get(),
                  plist.get(),   info.get(),   pool.get(),      rec.get(),
-                 (unsigned long long *)d_tip, stats.get(),    sub_ns.get(), sub_lv.get()};
+                 (unsigned long long *)d_tip, stats.get(),    sub_ns.get(), sub_lv.get(), ho};
         k_fd_peel<<<grid, FD_THREADS, smem, ls>>>(a);
         RC_LAUNCH();
     }
@@ -2216,8 +2363,8 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
         allow_max_smem((const void *)k_fd_small);
         FsArgs a{queue.get() + nsmall_at, nsmall, qhead.get() + 1, d_tstart.get(), d_tlen.get(),
                  d_tkb.get(), members.get(), info.get(), pool.get(), rec.get(), fd_beg.get(),
-                 fd_len.get(), fd_adj.get(), S.new2old, D.init, rtip.get(), (unsigned long long *)d_tip, stats.get(),
-                 sub_ns.get(), sub_lv.get()};
+                 fd_len.get(), fd_adj.get(), S.new2old, D.init, rtip.get(), (unsigned long long *)d_tip,
+                 fsup.get(), alive.get(), stats.get(), sub_ns.get(), sub_lv.get(), ho};
         k_fd_small<<<std::min(sms, nsmall), FD_THREADS, FS_SMEM, s>>>(a);
         RC_LAUNCH();
     }
@@ -2226,7 +2373,7 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
         RC_CUDA(cudaStreamWaitEvent(s, fork_ev[1], 0));
         fg.joined = true;
     }
-    unsigned long long hs[2] = {0, 0};
+    unsigned long long hs[3] = {0, 0, 0};
     RC_CUDA(cudaMemcpyAsync(hs, stats.get(), sizeof(hs), cudaMemcpyDeviceToHost, s));
     std::vector<unsigned long long> hns(T), hlv(T);
     if (T > 0) {
@@ -2234,14 +2381,24 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
         RC_CUDA(cudaMemcpyAsync(hlv.data(), sub_lv.get(), 8 * (size_t)T, cudaMemcpyDeviceToHost, s));
     }
     RC_CUDA(cudaStreamSynchronize(s));
+    const int32_t nover = (int32_t)(hs[2] >> 32);
+    if (nover > 0) {
+        std::vector<int32_t> ids(nover);
+        RC_CUDA(cudaMemcpyAsync(ids.data(), over.get(), 4 * (size_t)nover, cudaMemcpyDeviceToHost, s));
+        RC_CUDA(cudaStreamSynchronize(s));
+        pool.release();
+        peel_heavy(ids.data(), nover, over_level.get());
+        D.fd_heavy += nover;
+    }
     D.wedges_fd = hs[0];
     D.levels = (int64_t)hs[1];
     std::vector<bool> heavy(T, false);
-    for (int h = 0; h < nheavy; h++) {
-        const int32_t t = hq[h];
+    for (size_t h = 0; h < hh.size(); h++) {
+        const int32_t t = heavy_tasks[h];
         heavy[t] = true;
-        hns[t] = hh[h].t1 - hh[h].t0;
-        hlv[t] = hh[h].levels;
+        D.fd_heavy_levels += (int64_t)hlv[t];  // before it was handed over
+        hns[t] += hh[h].t1 - hh[h].t0;
+        hlv[t] += hh[h].levels;
         D.wedges_fd += hh[h].wedges;
         D.levels += (int64_t)hh[h].levels;
     }

@@ -173,3 +173,40 @@ def test_part_of_the_lists_beyond_the_pool(R, n, d):
     got = sv.wait(rid)[0]
     sv.close()
     assert np.array_equal(got, want)
+
+
+# tasks whose last levels peel nearly all members go over to all CTAs there: from
+# shared memory (4,000 members) and from global memory (20,000), with vertices that
+# no level peels with updates, and several at once in a packed union
+@pytest.mark.parametrize("n,nv,m,extra", [(4_000, 60_000, 2_400_000, 0), (4_000, 9_000, 1_200_000, 9_000),
+                                          (20_000, 30_000, 3_000_000, 0)])
+def test_wide_levels_are_handed_over(R, n, nv, m, extra):
+    eu, ev = synth.er(n, nv, m, 12)
+    y = np.arange(extra, dtype=np.int32)
+    eu, ev = np.concatenate([eu, n + y]), np.concatenate([ev, nv + y // 2])
+    nu, nv = n + extra, nv + extra
+    want, _ = oracle.bup(eu, ev, nu, nv, 0)
+    g = R.Graph(eu, ev, nu, nv)
+    for P in (3, 10, 150):
+        t = R.as_u64(g.tip_decompose(0, P=P))
+        assert np.array_equal(t, want), P
+        st, subs = g.stats(), g.subsets()
+        assert st["fd_heavy_subsets"] > 0, P
+        assert sum(s["levels"] for s in subs if s["heavy"]) == st["levels_fd_heavy"]
+        levels = [s["levels"] for s in subs]
+        t = R.as_u64(g.tip_decompose(0, P=P, fd_heavy_w=-1))
+        assert np.array_equal(t, want), P
+        assert g.stats()["fd_heavy_subsets"] == 0
+        assert levels == [s["levels"] for s in g.subsets()], P
+
+
+def test_wide_levels_of_a_union(R):
+    graphs, wants = [], []
+    for i in range(3):
+        n, nv, m = 3_500 + 500 * i, 12_000, 900_000
+        eu, ev = synth.er(n, nv, m, 40 + i)
+        graphs.append(R.Graph(eu, ev, n, nv))
+        wants.append(oracle.bup(eu, ev, n, nv, 0)[0])
+    outs = R.receipt_decompose_batch(graphs, [0] * 3, P=4)
+    for o, w in zip(outs, wants):
+        assert np.array_equal(R.as_u64(o), w)
