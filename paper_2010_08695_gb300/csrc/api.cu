@@ -260,6 +260,7 @@ void tip_decompose_impl(receipt_graph *g, int side, uint64_t *d_tip, const recei
     D.m = g->m;
     D.timing = opt.timing != 0;
     D.list_bound = list_bound;
+    D.count_walks = g->count_walks;
     D.max_deg_s = g->max_deg[side];
     D.max_deg_o = g->max_deg[1 - side];
     D.fd_heavy_w = opt.fd_heavy_w;

@@ -1821,7 +1821,7 @@ static void fdh_levels_with_recount(Decomp &D, const FdhArgs &ha, FdhDev *dst, F
         RC_CUDA(cudaMemcpyAsync(adjc.get(), O.adj, sizeof(int32_t) * D.m, cudaMemcpyDeviceToDevice, s));
         list_lengths(O.off, O.n, lenc.get(), s);
         compact_lists(O.off, lenc.get(), adjc.get(), O.n, keep.get(), s);
-        return recount_masked(S, O, D.s, D.m, keep.get(), out, lenc.get(), adjc.get(), s);
+        return recount_masked(D, keep.get(), out, lenc.get(), adjc.get(), s);
     };
     for (;;) {
         k_fdh_select<<<gm, 256, 0, s>>>(ha);

@@ -144,12 +144,14 @@ bool recount_fits(const Decomp &D) {
 
 uint64_t recount_remaining(const Decomp &D, const int32_t *len_w, const int32_t *adj_w,
                            cudaStream_t s) {
-    return recount_masked(*D.S, *D.O, D.s, D.m, D.sub, D.sup, len_w, adj_w, s);
+    return recount_masked(D, D.sub, D.sup, len_w, adj_w, s);
 }
 
-uint64_t recount_masked(const Side &S, const Side &O, int side_s, int64_t m, const int32_t *sub,
-                        unsigned long long *sup, const int32_t *len_w, const int32_t *adj_w,
-                        cudaStream_t s) {
+uint64_t recount_masked(const Decomp &D, const int32_t *sub, unsigned long long *sup,
+                        const int32_t *len_w, const int32_t *adj_w, cudaStream_t s) {
+    const Side &S = *D.S, &O = *D.O;
+    const int side_s = D.s;
+    const int64_t m = D.m;
     const int32_t n = S.n, no = O.n;
     if (n == 0 || no == 0 || m == 0) return 0;
     DevBuf<int64_t> ls(n + 1, s), offs(n + 1, s), lo(no + 1, s), offo(no + 1, s);
@@ -184,6 +186,9 @@ uint64_t recount_masked(const Side &S, const Side &O, int side_s, int64_t m, con
     sg.nu = sg.side[0].n;
     sg.nv = sg.side[1].n;
     sg.m = mr;
+    // as many wedges an edge as in the whole graph
+    if (D.count_walks != ~0ull)
+        sg.count_walks = (uint64_t)((double)D.count_walks * ((double)mr / (double)m));
     DevBuf<unsigned long long> cu(sg.nu, s), cv(sg.nv, s);
     const uint64_t w = count_local(&sg, cu.get(), cv.get(), s);
     k_apply_recount<<<ceil_div(n, 256), 256, 0, s>>>(n, sub, side_s ? cv.get() : cu.get(), sup);

@@ -73,6 +73,7 @@ struct Decomp {
     int32_t p_eff = 0;
     std::vector<uint64_t> bounds;         // theta(1..p_eff+1)
     uint64_t wedges_bup = 0;              // sum of d (d - 1) over the other side
+    uint64_t count_walks = ~0ull;         // receipt_graph::count_walks
     uint64_t wedges_cd = 0, wedges_fd = 0;
     int64_t rounds = 0, levels = 0;
     int32_t dgm_passes = 0;
@@ -130,9 +131,8 @@ uint64_t recount_remaining(const Decomp &D, const int32_t *len_w, const int32_t 
 // x with sub[x] < 0 and all of the other side, of every kept vertex into
 // sup[x]. len_w/adj_w: the other side's lists (original offsets) already
 // compacted to kept vertices. Returns the wedges traversed; synchronises s.
-uint64_t recount_masked(const Side &S, const Side &O, int side_s, int64_t m, const int32_t *sub,
-                        unsigned long long *sup, const int32_t *len_w, const int32_t *adj_w,
-                        cudaStream_t s);
+uint64_t recount_masked(const Decomp &D, const int32_t *sub, unsigned long long *sup,
+                        const int32_t *len_w, const int32_t *adj_w, cudaStream_t s);
 // Drops from every list y of the other side (working copy adj_w with
 // lengths len_w, original offsets off_o) the entries x with sub[x] >= 0.
 void compact_lists(const int64_t *off_o, int32_t *len_w, int32_t *adj_w, int32_t n_o,
