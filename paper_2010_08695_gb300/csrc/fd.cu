@@ -1857,13 +1857,6 @@ static void fdh_levels_with_recount(Decomp &D, const FdhArgs &ha, FdhDev *dst, F
     RC_CUDA(cudaMemcpyAsync(hst_out, dst, sizeof(FdhDev), cudaMemcpyDeviceToHost, s));
 }
 
-// A task peeled from lists: its members, its walks' wedges, its range.
-struct ListTask {
-    int32_t id, n;
-    unsigned long long w;
-    uint64_t lo, hi;
-};
-
 // Dense tasks that all CTAs peel sooner than their lists are made and applied by
 // one CTA (others are handed over when that shows, FdHandOver, after their lists
 // were made: 1.7 ps a wedge, which dense tasks have many of for an entry. 8M edges
@@ -1878,38 +1871,40 @@ struct ListTask {
 // two members (all share middle vertices).
 // One CTA a task peels the tasks left side by side, the heavy ones come one by
 // one: the longest go first while the sum falls.
-constexpr double DENSE_TASK = 16;  // wedges for each two members
-static std::vector<int32_t> heavy_by_lists(std::vector<ListTask> t, int ctas) {
-    auto levels = [](const ListTask &k) {
-        const double span = (double)(k.hi - k.lo);
-        return std::max(1.0, std::min((double)k.n * std::min(1.0, span / (double)k.hi),
-                                      std::min((double)k.n, 16.0 * span)));
-    };
-    auto by_list = [&](const ListTask &k) {
-        const double e = std::min((double)k.w / 4, (double)k.n * (double)k.n);
-        return 2500.0 * levels(k) + 0.85 * e;
-    };
-    auto heavy = [&](const ListTask &k) { return 7e4 * levels(k) + 0.003 * (double)k.w; };
+constexpr double DENSE_TASK = 16;  // wedges for each two members, at least
+struct DenseTask {
+    int32_t id;
+    double list, heavy, walks;  // ns by one CTA, by all, to make its lists
+};
+// n members, w wedges, range [lo, hi)
+static DenseTask dense_task(int32_t id, int32_t n, unsigned long long w, uint64_t lo, uint64_t hi) {
+    const double span = (double)(hi - lo), nd = (double)n, wd = (double)w;
+    const double levels = std::max(1.0, std::min({nd * std::min(1.0, span / (double)hi), nd, 16.0 * span}));
+    const double entries = std::min(wd / 4, nd * nd);
+    return DenseTask{id, 2500.0 * levels + 0.85 * entries, 7e4 * levels + 0.003 * wd, 0.0017 * wd};
+}
+static std::vector<int32_t> heavy_by_lists(std::vector<DenseTask> t, int ctas) {
+    // (stored costs: computed in the comparison they may be rounded in two ways)
     std::stable_sort(t.begin(), t.end(),
-                     [&](const ListTask &a, const ListTask &b) { return by_list(a) > by_list(b); });
+                     [](const DenseTask &a, const DenseTask &b) { return a.list > b.list; });
     double left = 0, walks = 0;  // of the tasks not heavy
-    for (const ListTask &k : t) {
-        left += by_list(k);
-        walks += 0.0017 * (double)k.w;
+    for (const DenseTask &k : t) {
+        left += k.list;
+        walks += k.walks;
     }
     double first = 0, best = 0, sum = 0;
     size_t n = 0;
     for (size_t k = 0; k <= t.size(); k++) {
-        const double now = sum + walks + std::max(k < t.size() ? by_list(t[k]) : 0.0, left / ctas);
+        const double now = sum + walks + std::max(k < t.size() ? t[k].list : 0.0, left / ctas);
         if (k == 0) first = best = now;
         if (now < best && now < 0.9 * first) {
             best = now;
             n = k;
         }
         if (k == t.size()) break;
-        sum += heavy(t[k]);
-        left -= by_list(t[k]);
-        walks -= 0.0017 * (double)t[k].w;
+        sum += t[k].heavy;
+        left -= t[k].list;
+        walks -= t[k].walks;
         if (sum > best) break;
     }
     std::vector<int32_t> out;
@@ -2129,13 +2124,13 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
                 (heavy && tlen[t] > 0 ? front : back).push_back(t);
             }
             if (D.fd_heavy_w == 0 && cap > 0) {
-                std::vector<ListTask> lt;
+                std::vector<DenseTask> lt;
                 for (int32_t t : back) {
                     const int sub_i = tsub[t];
                     if ((double)tw[t] < DENSE_TASK * (double)tlen[t] * (double)tlen[t]) continue;
                     const bool open = (size_t)sub_i + 1 >= D.bounds.size();
-                    lt.push_back(ListTask{t, tlen[t], tw[t], open ? 0 : D.bounds[sub_i],
-                                          open ? ~0ull : D.bounds[sub_i + 1]});
+                    lt.push_back(dense_task(t, tlen[t], tw[t], open ? 0 : D.bounds[sub_i],
+                                            open ? ~0ull : D.bounds[sub_i + 1]));
                 }
                 const std::vector<int32_t> more = heavy_by_lists(lt, sms);
                 std::vector<bool> is(T, false);

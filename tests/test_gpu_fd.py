@@ -210,3 +210,14 @@ def test_wide_levels_of_a_union(R):
     outs = R.receipt_decompose_batch(graphs, [0] * 3, P=4)
     for o, w in zip(outs, wants):
         assert np.array_equal(R.as_u64(o), w)
+
+
+# many equal dense tasks: their estimated costs are equal too
+def test_equal_dense_tasks(R):
+    eu, ev = synth.er(400, 300, 30_000, 3)
+    want, _ = oracle.bup(eu, ev, 400, 300, 0)
+    g = R.Graph(eu, ev, 400, 300)
+    for k in (2, 17, 64, 150):
+        for P in (1, 5, 150):
+            for t in R.receipt_decompose_batch([g] * k, [0] * k, P=P):
+                assert np.array_equal(R.as_u64(t), want), (k, P)
