@@ -2285,6 +2285,7 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
     DevBuf<unsigned long long> rtip(nsmall_at < T ? n : 1, s);
     // the members' lists: walks in items of equal cost, 8 a CTA
     DevBuf<unsigned long long> rec;
+    std::vector<uint8_t> skip;  // (kept until the stream has passed its copy)
     if (nheavy < T) {
         allow_max_smem((const void *)k_fd_pairs<FdMids>);
         rec.alloc(n, s);
@@ -2297,7 +2298,7 @@ void fd_run(Decomp &D, uint64_t *d_tip, cudaStream_t s) {
         DevBuf<int32_t> pq(1, s);
         head.zero();
         pq.zero();
-        std::vector<uint8_t> skip(T, 0);
+        skip.assign(T, 0);
         for (int k = 0; k < nheavy; k++) skip[hq[k]] = 1;
         DevBuf<uint8_t> dskip(T, s);
         RC_CUDA(cudaMemcpyAsync(dskip.get(), skip.data(), T, cudaMemcpyHostToDevice, s));
