@@ -761,7 +761,9 @@ __global__ void __launch_bounds__(PULL_THREADS) k_hub_pull_cta(HubArgs a, int32_
 // ---- the HEAVY vertices of highest degree, anchor by anchor: lane l of a
 // warp counts b(x, x') for x' = 32 w + l, w < 8, from the masks of the
 // anchor's middle vertices over those vertices. Anchors of many edges take a
-// whole CTA (partial counts in shared memory).
+// whole CTA (partial counts in shared memory): from 256 / 1,024 / 8,192 edges on the
+// coarse-grained step of the 40M-edge graph takes 333 / 334 / 345 ms, of a 6M-edge
+// one with hubs on both sides 84.6 / 85.0 / 86.7.
 constexpr int HEAVY_DEG = 1024;
 __global__ void __launch_bounds__(512) k_hub_heavy(HubArgs a) {
     __shared__ unsigned long long s_dec[HEAVY];

@@ -44,7 +44,10 @@ namespace {
 
 constexpr int PT = 512;  // threads per CTA (two CTAs per SM)
 constexpr int GROUP = 8;  // dense-window anchors side by side in one pass
-// With groups (WIDE), walks of more wedges still take the whole CTA.
+// With groups (WIDE), walks of more wedges still take the whole CTA. (8,192, this or
+// 131,072: the same within 2% on five sides of 500k to 5M edges; the wedge counts
+// of the groups' counters end near here. So are the classes' thresholds, half or
+// four times as high: 5% on uniform graphs of 5M edges.)
 constexpr unsigned long long GROUP_MAX_W = 32768;
 // Polls of a barrier wait before it gives up (each takes at least an L2 round
 // trip: ~10 s in all). CTAs fetch their items as they go, so they wait for one
@@ -1014,7 +1017,9 @@ bool cd_persist_wide(const Decomp &D) {
 // x 1M, 10M (over 2 10^9) 44 / 42. Larger sides count a walk in slices and lose
 // more: 120,000 x 40,000, 3M, 36 / 30 for the step; 140,000 x 14,000, 2M, 60 / 31.
 // Sides of several windows with short walks keep the groups (100,000 x 30,000
-// uniform, 1M edges: 1.1 / 0.8). Not beside other units of the serving engine
+// uniform, 1M edges: 1.1 / 0.8). Large unions: 24 graphs of 3.7 10^9 wedges 35.2 ms
+// by lists, 35.8 by windows: the line may lie at 3 10^9 as well as above, and the
+// counters of a round by lists are 32 bits wide. Not beside other units of the serving engine
 // (list_bound): the walks take every SM, and the other units' cooperative
 // launches wait for them (24 requests of 10k-1M edges: 57.4 / 56.4).
 bool cd_persist_by_lists(const Decomp &D) {

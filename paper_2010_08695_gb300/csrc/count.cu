@@ -60,8 +60,13 @@ enum {
 constexpr int COUNT_HEAD = 4096;  // keys with dense 16-bit counters
 constexpr int PLAN_DEG = 256;     // larger neighbourhoods are planned by a CTA
 constexpr int BITS = 1024;        // end points of the bit-sliced part
-constexpr int BITS_DEG = 512;     // start points of at least this degree take a CTA there,
-constexpr int HUGE_DEG = 8192;    // of at least this a CTA per HUGE_DEG middle points
+// Start points of at least BITS_DEG take a CTA there, of at least HUGE_DEG one per
+// HUGE_DEG middle points. Counts with 256 / this / 1,024, ms: 300k edges 0.34 / 0.43
+// / 0.60, 1M 0.71 / 0.79 / 0.97, 10M 6.34 / 6.38 / 6.68, 20M 17.40 / 17.12 / 17.11; with
+// 2,048 / 4,096 / this: 300k 0.50 / 0.43 / 0.43, 3M 1.93 / 2.03 / 2.26, 10M 6.24 / 6.22
+// / 6.38, 20M 17.16 / 17.00 / 17.12: flat near these.
+constexpr int BITS_DEG = 512;
+constexpr int HUGE_DEG = 8192;
 
 // Start points with at most HASH_W wedges (and more than WARP_MAX_W) and too
 // many keys past the head: small CTAs, any key space, any degree.
@@ -104,7 +109,9 @@ struct CountSide {
 // the 10M-edge graph took 4.6 ms whatever its walk: all its atomics went to a
 // few cache lines.)
 constexpr int HOT_KEYS = 4096, HOT_REPS = 32;
-constexpr int64_t HOT_MIN_M = 1 << 17;  // edges from which the copies pay
+// edges from which the copies pay (with them / without, ms: 20k edges 0.100 / 0.090,
+// 130k 0.372 / 0.367, 1M 0.79 / 0.89)
+constexpr int64_t HOT_MIN_M = 1 << 17;
 
 struct CountPlan {
     CountSide s[2];
