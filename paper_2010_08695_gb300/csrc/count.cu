@@ -26,10 +26,10 @@
 //
 // Measured (both sides, ms; before: prefixes of all end points by one warp or
 // one 1,024-thread CTA per start point): 20M edges, 4.4e9 wedges, 77.1 -> 17.4
-// (bit-sliced 7.6, the rest 8.1, plan 1.1); 10M edges 14.3 -> 6.4; 1M edges
+// (bit-sliced 7.6, the rest 8.1, plan 1.0); 10M edges 14.3 -> 6.3; 1M edges
 // 1.45 -> 0.8. What bounds it now: instruction issue in the bit-sliced kernels
-// (~40 instructions per edge and pass), the chain of dependent loads per start
-// point in the others.
+// (~40 instructions per edge and pass; SMs 68% busy), the chain of dependent loads
+// per start point, barriers and instruction fetch in the others.
 #include "engine.cuh"
 #include "internal.cuh"
 
