@@ -82,7 +82,7 @@ void *pinned_scratch(size_t bytes) {
         if (g_pinned.p) cudaFreeHost(g_pinned.p);
         g_pinned.p = nullptr;
         g_pinned.n = 0;
-        size_t want = bytes < 4096 ? 4096 : bytes;
+        size_t want = bytes < PINNED_SCRATCH ? PINNED_SCRATCH : bytes;
         RC_CUDA(cudaMallocHost(&g_pinned.p, want));
         g_pinned.n = want;
     }

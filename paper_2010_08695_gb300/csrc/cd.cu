@@ -1169,9 +1169,10 @@ void cd_run(Decomp &D, const receipt_options &opt, cudaStream_t s) {
     // pinned: C_rcnt, the state's header, the device-driven rounds' records,
     // the one-launch form's state and first records
     constexpr int ROUND_BURST = 64, PERSIST_FIRST = 512;
-    unsigned long long *hpin = (unsigned long long *)pinned_scratch(
-        64 + sizeof(CdDev) + 8 + ROUND_BURST * hdr + sizeof(PersistDev) +
-        PERSIST_FIRST * sizeof(PersistRound));
+    constexpr size_t PIN_BYTES = 64 + sizeof(CdDev) + 8 + ROUND_BURST * offsetof(CdDev, hist_w) +
+                                 sizeof(PersistDev) + PERSIST_FIRST * sizeof(PersistRound);
+    static_assert(PIN_BYTES <= PINNED_SCRATCH, "taken once for every user");
+    unsigned long long *hpin = (unsigned long long *)pinned_scratch(PIN_BYTES);
     CdDev *hst = reinterpret_cast<CdDev *>(hpin + 8);
     unsigned long long *hrec = hpin + 8 + (sizeof(CdDev) + 7) / 8;
     unsigned long long prev_w[NTIER] = {}, prev_a[NTIER] = {};
