@@ -30,9 +30,10 @@
 // side, 5,000 anchors a round): pull 75 (8 lanes) + 245 (warps) + 390 (CTAs),
 // heavy 62, quadratic forms 45 + 70 and the Gram matrix 7 beside them. The pull
 // is bound by the L1 (one 32-byte mask per wedge; 68 to 74% of its throughput in
-// the larger two kernels) and by the chain of dependent loads of a vertex. The step took 664 ms by the per-anchor tiers
-// alone (1.26 10^11 wedges walked) and takes 328 so (1.2 10^10); 10M-edge
-// graph 120.6 -> 79.5 ms, 3M edges in 25 subsets 17.9 -> 12.0.
+// the larger two kernels) and by the chain of dependent loads of a vertex. The step
+// took 664 ms by the per-anchor tiers alone (1.26 10^11 wedges walked) and takes
+// 328 so (1.2 10^10); 10M-edge graph 120.6 -> 79.5 ms, 3M edges in 25 subsets
+// 17.9 -> 12.0.
 #include <cuda_fp16.h>
 
 #include <algorithm>
